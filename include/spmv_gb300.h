@@ -276,6 +276,8 @@ spmv_status spmv_check(spmv_plan_t plan, void *stream);
  * spmv_profile_enable).  kernel: 0 = chunk scatter (SpMV local), 1 = partial
  * combine, 2 = chunk dot (SpVTM local), 3 = zone fixup, 4 = dvalues,
  * 5 = row-block dot (the SpMV local step over the row-sorted copy), 6 = its zone fixup.
+ * One pass that serves both products of a spmv_pair counts as a launch of kernel 0 and of
+ * kernel 2, with half of its time each.
  * Synchronizes the device.  *ms = summed event time, *launches = number of
  * timed launches.  Timing brackets every launch with two events, which waits
  * for each kernel to drain before the next starts: a profiled sequence of
@@ -317,9 +319,10 @@ spmv_status spmv_noalloc(int64_t m, int64_t n, int64_t nnz, const int32_t *ptr, 
  *   x (n), y (m), v (m), u (n): vectors of the plan's vector type, each on the device (16-byte
  *   aligned) or in host memory (pinned or pageable); y and u are overwritten.  The four must not
  *   overlap: the two products may run at the same time.
- * With device pointers only, the call is asynchronous: the SpMV runs on `stream` and the SpVTM
- * beside it on a stream of the plan, forked after the work already queued on `stream` and joined
- * back into it (work queued on `stream` after the call sees both results).  Otherwise the
+ * With device pointers only, the call is asynchronous.  Where both short vectors fit in shared
+ * memory one reading of the matrix on `stream` serves both products; otherwise the SpMV runs on
+ * `stream` and the SpVTM beside it on a stream of the plan, forked after the work already queued
+ * on `stream` and joined back into it.  Work queued on `stream` after the call sees both results.  Otherwise the
  * library stages the host vectors through its own device buffers on `stream` and on a copy
  * stream of its own: v's copy is queued first, the copy of x to the device overlaps the SpVTM
  * kernels and the copy of u to the host overlaps the SpMV kernels, and the call returns after y

@@ -51,6 +51,53 @@ cudaError_t launch_stream(const spmv_plan_s *p, int mode, int kb, const LaunchAr
     }
 }
 
+cudaError_t launch_pass(const spmv_plan_s *p, bool sc, bool sd, const PassParams &pp, int warps, int smem,
+                        cudaStream_t s) {
+    switch (p->val_t) {
+        case SPMV_F64: return launch_pass_f64(sc, sd, pp, p->ctas, warps, smem, s);
+        case SPMV_F32: return launch_pass_f32(sc, sd, pp, p->ctas, warps, smem, s);
+        case SPMV_BF16: return launch_pass_bf16(sc, sd, pp, p->ctas, warps, smem, s);
+        default: return launch_pass_f16(sc, sd, pp, p->ctas, warps, smem, s);
+    }
+}
+
+// Shared memory of a one-vector pass: the accumulator (sc), the input vector (sd), the staging slots
+// of as many warps as fit, and what is left over for more copies of the accumulator.  Measured on
+// the 200M-nonzero wide matrix (m = 20,000; us): more warps always help (pair 420 / 481 / 537 / 627
+// at 32 / 24 / 20 / 16 warps).  The dot products alone take two slots a warp (279 against 286
+// with one); with the accumulator one slot and the room for a second copy are better (317 against
+// 345: an addition is a compare-and-swap loop, repeated when another warp got in between).
+// On the tall matrix (n = 2,000) the accumulating pass takes 438 / 378 / 335 / 306 / 276 us with
+// 1 / 2 / 4 / 8 / 16 copies, the pair 433 / 412 / 399 / 391 / 381; 32 copies add nothing.
+size_t pass_acc_bytes(const spmv_plan_s *p) { return align_up((size_t)p->n_minor * p->sa, 128); }
+size_t pass_vec_bytes(const spmv_plan_s *p) { return align_up((size_t)p->n_minor * p->sx, 128); }
+constexpr int PASS_MAX_COPIES = 16;
+struct PassGeometry {
+    int warps, slots, copies;
+    size_t smem;
+};
+// tiles of a CTA: no more warps than these can work
+int cta_tiles(const spmv_plan_s *p) { return std::max(1, (p->ntiles + p->ctas - 1) / std::max(1, p->ctas)); }
+PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd) {
+    PassGeometry g;
+    const size_t acc = sc ? pass_acc_bytes(p) : 0, vec = (sd ? pass_vec_bytes(p) : 0) + PASS_BAR_BYTES;
+    const size_t slot = pass_slot_bytes(p->sv), all = (size_t)p->smem_max;
+    const size_t fit = all > acc + vec ? (all - acc - vec) / slot : 0;
+    g.warps = (int)std::min<size_t>(std::min(pass_warps(p->sv), cta_tiles(p)), fit);
+    g.slots = g.warps > 0 ? (int)std::min<size_t>(sc ? 1 : PASS_MAX_SLOTS, fit / g.warps) : 0;
+    const size_t rest = vec + (size_t)g.warps * g.slots * slot;
+    g.copies = 1;
+    while (sc && 2 * g.copies <= std::min(g.warps, PASS_MAX_COPIES) && 2 * g.copies * acc + rest <= all) g.copies *= 2;
+    g.smem = g.copies * acc + rest;
+    return g;
+}
+// A pass runs with at least 8 warps (or all a CTA has tiles for): fewer leave it to the streaming
+// kernel.  The pair wants 20, below which its two products run faster one by one (317 + 279 us
+// with 32 warps each, against 537 with 20 and 627 with 16).
+bool pass_fits(const spmv_plan_s *p, bool sc, bool sd) {
+    return pass_geometry(p, sc, sd).warps >= std::min(sc && sd ? std::min(20, pass_warps(p->sv)) : 8, cta_tiles(p));
+}
+
 int kb_template(int kb) { return kb <= 1 ? 1 : kb <= 2 ? 2 : kb <= 4 ? 4 : 8; }
 
 // Tiles per chunk of the streaming kernels (default): a warp carries a segment across the
@@ -63,9 +110,10 @@ struct ProfScope {
     spmv_plan_s *p;
     int kernel;
     cudaStream_t s;
+    double share;  // of the bracketed time that counts for this kernel
     cudaEvent_t a = nullptr, b = nullptr;
-    ProfScope(spmv_plan_s *p_, int k, cudaStream_t s_) : p(p_), kernel(k), s(s_) {
-        if (p->prof_on.load(std::memory_order_relaxed)) {
+    ProfScope(spmv_plan_s *p_, int k, cudaStream_t s_, double share_ = 1.0) : p(p_), kernel(k), s(s_), share(share_) {
+        if (share > 0.0 && p->prof_on.load(std::memory_order_relaxed)) {
             cudaEventCreate(&a);
             cudaEventCreate(&b);
             cudaEventRecord(a, s);
@@ -75,7 +123,7 @@ struct ProfScope {
         if (a) {
             cudaEventRecord(b, s);
             std::lock_guard<std::mutex> lk(p->prof_mu);
-            p->prof.push_back({kernel, a, b});
+            p->prof.push_back({kernel, share, a, b});
         }
     }
 };
@@ -193,6 +241,52 @@ size_t plan_footprint(const spmv_plan_s *p) {
     return b;
 }
 
+// The one-vector pass of plan p: y_short += A x (sc) into the per-CTA partials, u = the dot
+// products with v (sd), or both; then the combine and the zone fix-up.
+static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *v, void *u, cudaStream_t s) {
+    const bool sc = y != nullptr, sd = u != nullptr;
+    PassParams pp;
+    std::memset(&pp, 0, sizeof(pp));
+    pp.idx = p->idx;
+    pp.vals = p->vals;
+    pp.steps = p->steps;
+    pp.seglist = p->seglist;
+    pp.rank = p->segrank;
+    pp.nnz = (int)p->nnz;
+    pp.n_minor = p->n_minor;
+    pp.ntiles = p->ntiles;
+    pp.spt = p->T / 256;
+    pp.chunk_tiles = p->chunk_tiles;
+    pp.acc_bytes = sc ? (int)pass_acc_bytes(p) : 0;
+    pp.vec_bytes = sd ? (int)pass_vec_bytes(p) : 0;
+    pp.x = x;
+    pp.v = v;
+    pp.part = p->part;
+    pp.u = u;
+    pp.rec_left = p->rec_left;
+    pp.rec_right = p->rec_right;
+    pp.err = p->err;
+    const PassGeometry g = pass_geometry(p, sc, sd);
+    pp.slots = g.slots;
+    pp.copies = g.copies;
+    const bool f64 = p->vec_t == SPMV_F64;
+    {
+        // a pass that serves both products counts as a launch of each, with half of its time
+        ProfScope ps0(p, 0, s, !sc ? 0.0 : sd ? 0.5 : 1.0), ps2(p, 2, s, !sd ? 0.0 : sc ? 0.5 : 1.0);
+        CUDA_TRY(launch_pass(p, sc, sd, pp, g.warps, (int)g.smem, s));
+    }
+    if (sc) {
+        ProfScope ps(p, 1, s);
+        CUDA_TRY(launch_combine(f64, f64, p->part, p->ctas, p->n_minor, 1, &y, s));
+    }
+    if (sd && (p->pz.z > 0 || p->nempty > 0)) {
+        ProfScope ps(p, 3, s);
+        CUDA_TRY(launch_fixup(f64, p->pz.zones, p->pz.z, p->rec_left, p->rec_right, p->pz.nproc, 1, &u, s));
+        CUDA_TRY(launch_zero_list(f64, p->emptylist, p->nempty, u, s));
+    }
+    return SPMV_OK;
+}
+
 spmv_status run_scatter(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s) {
     const size_t out_bytes = (size_t)p->n_minor * p->sx;
     if (p->nnz == 0 || p->n_major == 0) {
@@ -200,6 +294,7 @@ spmv_status run_scatter(spmv_plan_s *p, int kb, const void *const *in, void *con
             for (int b = 0; b < kb; ++b) CUDA_TRY(cudaMemsetAsync(out[b], 0, out_bytes, s));
         return SPMV_OK;
     }
+    if (kb == 1 && p->pass_sc) return run_pass(p, in[0], out[0], nullptr, nullptr, s);
     if (!p->onchip && kb > 1) {
         for (int b = 0; b < kb; ++b) {
             spmv_status st = run_scatter(p, 1, in + b, out + b, s);
@@ -292,6 +387,7 @@ static spmv_status run_segdot_impl(spmv_plan_s *p, int kb, const void *const *in
             for (int b = 0; b < kb; ++b) CUDA_TRY(cudaMemsetAsync(out[b], 0, out_bytes, s));
         return SPMV_OK;
     }
+    if (kb == 1 && p->pass_sd) return run_pass(p, nullptr, nullptr, in[0], out[0], s);
     const bool f64_onchip = p->val_t == SPMV_F64 && p->onchip && kb <= p->batch_width;
     if (kb > 1 && !f64_onchip) {
         const int grp = seg_group(p);
@@ -416,6 +512,7 @@ void plan_free(spmv_plan_s *p) {
     }
     if (p->ws) cudaFree(p->ws);
     if (p->ws2) cudaFree(p->ws2);
+    if (p->ws_seg) cudaFree(p->ws_seg);
     if (p->hin) cudaFree(p->hin);
     if (p->hout) cudaFree(p->hout);
     if (p->hv) cudaFree(p->hv);
@@ -551,8 +648,12 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     if (opts && opts->tile_items) {
         p->T = opts->tile_items;
     } else {
+        // (an unvalidated plan or one with its short vector in global memory never runs the
+        // one-vector passes, which want tiles of whole 256-position steps)
         const int64_t fill = (int64_t)sms * 16 * 2;
-        if (nnz < fill * 512) p->T = (int)std::max<int64_t>(64, std::min<int64_t>(512, (nnz / fill) & ~int64_t(7)));
+        if (!(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL)))
+            p->T = nnz < fill * 512 ? 256 : 512;
+        else if (nnz < fill * 512) p->T = (int)std::max<int64_t>(64, std::min<int64_t>(512, (nnz / fill) & ~int64_t(7)));
     }
     p->S = (opts && opts->stages) ? opts->stages : 2;
     int W = (opts && opts->warps_per_cta) ? opts->warps_per_cta : MAX_WARPS;
@@ -626,9 +727,10 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
 
     // ---- structural checks
     if (!(flags & SPMV_PLAN_NO_VALIDATE)) {
-        CUDA_TRY(launch_validate(ptr, idx, p->n_major, (int)nnz, p->n_minor, p->err, s));
+        CUDA_TRY(launch_validate(ptr, idx, p->n_major, (int)nnz, p->n_minor, p->err, p->counts + 20, s));
         int32_t e = 0;
         CUDA_TRY(cudaMemcpyAsync(&e, p->err, 4, cudaMemcpyDeviceToHost, s));
+        CUDA_TRY(cudaMemcpyAsync(&p->nempty, p->counts + 20, 4, cudaMemcpyDeviceToHost, s));
         CUDA_TRY(cudaStreamSynchronize(s));
         if (e) {
             std::string msg = "malformed matrix:";
@@ -684,14 +786,40 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
         stream_processors(nt, p->T, (int)nnz, p->ctas * p->bpc, p->chunk_tiles, pnzb.data());
         p->max_nproc = std::max(1, pz.nproc);
     }
-    const size_t part_bytes = (pi && pi->segdot_only) ? 16
-                              : p->onchip ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa
-                                          : (size_t)p->n_minor * sizeof(double);
+    // the one-vector passes serve validated plans with whole-step tiles whose short vectors fit in
+    // shared memory beside the staging slots of enough warps
+    if (!pi && nnz > 0 && p->T % 256 == 0 && !(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL))) {
+        // (the accumulating product alone of FP64 values stays with the streaming kernel: 62 us
+        // against 66 on 8M nonzeros, n = 4,000)
+        p->pass_sc = p->sv != 8 && pass_fits(p, true, false);
+        p->pass_sd = pass_fits(p, false, true);
+        p->pass_pair = pass_fits(p, true, true);
+    }
+    const size_t part_bytes =
+        (pi && pi->segdot_only) ? 16
+                                : std::max(p->onchip ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa
+                                                     : (size_t)p->n_minor * sizeof(double),
+                                           p->pass_sc || p->pass_pair ? (size_t)p->ctas * p->n_minor * p->sa : (size_t)0);
+    // ranks of the nonempty segments, when some are empty
+    int32_t *&rank = p->segrank;
+    if ((p->pass_sc || p->pass_sd || p->pass_pair) && p->nempty > 0) {
+        const int nfull = p->n_major - p->nempty, nblk = seg_rank_blocks(p->n_major);
+        const size_t seg_bytes = ((size_t)p->n_major * 2 + 1 + nblk + 4) * 4;
+        CUDA_TRY(cudaMalloc(&p->ws_seg, seg_bytes));
+        p->seglist = static_cast<int32_t *>(p->ws_seg);
+        p->emptylist = p->seglist + nfull;
+        rank = p->emptylist + p->nempty;
+        int32_t *blk = rank + p->n_major + 1;
+        CUDA_TRY(launch_seg_ranks(p->pptr, p->n_major, rank, p->seglist, p->emptylist, blk, blk + nblk, s));
+        p->ws_bytes = seg_bytes;
+    }
     const size_t rec_bytes = (size_t)VL_MAX * p->max_nproc * 2 * p->sa;  // any segmented pass: up to VL_MAX vectors
     off = 0;
     const size_t o_meta = carve((size_t)(nt + 1) * sizeof(TileMeta));
     const size_t o_masks = carve((size_t)std::max(nt, 1) * p->mwp * 4);
     const size_t o_pfx = carve((size_t)std::max(nt, 1) * p->mwq * 2);
+    const bool passes = p->pass_sc || p->pass_sd || p->pass_pair;
+    const size_t o_steps = carve(passes ? (size_t)nt * (p->T / 256) * sizeof(StepRec) : 0);
     const size_t o_pz = carve((size_t)p->max_nproc * sizeof(ZoneDev));
     const size_t o_recl = carve(rec_bytes);
     const size_t o_recr = carve(rec_bytes);
@@ -705,11 +833,12 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     const size_t o_pscr = carve(setup_scratch_bytes(p->max_nproc));
     const size_t ws2 = off;
     CUDA_TRY(cudaMalloc(&p->ws2, ws2));
-    p->ws_bytes = ws1 + ws2;
+    p->ws_bytes += ws1 + ws2;
     char *w2 = static_cast<char *>(p->ws2);
     p->meta = reinterpret_cast<TileMeta *>(w2 + o_meta);
     p->masks = reinterpret_cast<uint32_t *>(w2 + o_masks);
     p->pfx = reinterpret_cast<uint16_t *>(w2 + o_pfx);
+    p->steps = passes ? reinterpret_cast<StepRec *>(w2 + o_steps) : nullptr;
     p->rec_left = w2 + o_recl;
     p->rec_right = w2 + o_recr;
     p->part = w2 + o_part;
@@ -722,7 +851,8 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
         // execution tiles: bounds, first/last segments, owned end events; masks and descriptors
         CUDA_TRY(launch_tile_bounds(nt, p->T, (int)nnz, tnzb, s));
         CUDA_TRY(launch_chunks(p->pptr, p->n_major, (int)nnz, nt, tnzb, p->T, taux, s));
-        CUDA_TRY(launch_masks(p->pptr, taux, nt, (int)nnz, p->n_major, p->mwp, p->masks, p->mwq, p->pfx, p->meta, s));
+        CUDA_TRY(launch_masks(p->pptr, taux, nt, (int)nnz, p->n_major, p->mwp, p->masks, p->mwq, p->pfx, p->meta, rank, s));
+        if (passes) CUDA_TRY(launch_steps(p->meta, p->masks, p->mwp, nt, p->T / 256, p->seglist, p->steps, s));
         // the Sec. IV-B set-up over the processors (chunks) gives their overlap zones
         spmv_plan_s::ProcZones &pz = p->pz;
         pz.zones = reinterpret_cast<ZoneDev *>(w2 + o_pz);
@@ -883,6 +1013,11 @@ static spmv_status pair_staged(spmv_plan_s *p, const void *x, void *y, const voi
 // lets the short combine and fix-up kernels, and the tail of either pass, overlap the other.
 // Asynchronous; whatever fails, the join is recorded so that `s` never runs ahead of the fork.
 static spmv_status pair_device(spmv_plan_s *p, const void *x, void *y, const void *v, void *u, cudaStream_t s) {
+    // both short vectors on chip: one reading of the matrix serves both products
+    if (p->pass_pair && !p->tplan) {
+        const bool csc = p->layout == SPMV_CSC_WIDE;
+        return csc ? run_pass(p, x, y, v, u, s) : run_pass(p, v, u, x, y, s);
+    }
     if (!p->cstream) CUDA_TRY(cudaStreamCreateWithFlags(&p->cstream, cudaStreamNonBlocking));
     if (!p->ev_x) CUDA_TRY(cudaEventCreateWithFlags(&p->ev_x, cudaEventDisableTiming));
     if (!p->ev_u) CUDA_TRY(cudaEventCreateWithFlags(&p->ev_u, cudaEventDisableTiming));
@@ -1020,7 +1155,7 @@ spmv_status spmv_profile_read(spmv_plan_t p, int32_t kernel, double *ms, int64_t
     for (auto &pr : p->prof) {
         float t = 0.f;
         cudaEventElapsedTime(&t, pr.a, pr.b);
-        p->prof_ms[pr.kernel] += t;
+        p->prof_ms[pr.kernel] += t * pr.share;
         p->prof_n[pr.kernel] += 1;
         cudaEventDestroy(pr.a);
         cudaEventDestroy(pr.b);

@@ -12,6 +12,8 @@ constexpr int ERR_INDEX = 1;      // an index outside the short vector was met (
 constexpr int ERR_WAIT = 2;       // a staging wait ran past its time limit
 constexpr int ERR_STRUCT = 4;     // a tile descriptor was inconsistent with the chunk
 
+constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;  // 2 s per staging wait
+
 constexpr unsigned FULL = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -99,6 +101,39 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_d<__nv_bfloat16>(doubl
     return __float2bfloat16_rn(static_cast<float>(v));
 }
 template <> __device__ __forceinline__ __half from_d<__half>(double v) { return __float2half_rn(static_cast<float>(v)); }
+
+// A product rounded on its own (never fused into a following addition), so that the
+// segmented passes round every product the same way whatever code surrounds it.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+// One term of a segmented prefix: v w added to s, or alone where a segment starts.  FP64 fuses the
+// product into the addition (its pipe does 2 operations a cycle per SM, the bound of the FP64
+// passes); the 32-bit passes round the product first.
+__device__ __forceinline__ float seg_term(float v, float w, float s, bool restart) {
+    const float q = __fmul_rn(v, w);
+    return restart ? q : s + q;
+}
+__device__ __forceinline__ double seg_term(double v, double w, double s, bool restart) {
+    return fma(v, w, restart ? 0.0 : s);
+}
+// hi + lo += t, compensated (TwoSum: hi takes the rounded sum, lo gathers its rounding
+// errors).  A sum that is infinite or NaN carries no error term, so that hi + lo stays what the
+// plain sum gives (an infinity would otherwise make the error term NaN).
+template <typename AT>
+__device__ __forceinline__ void carry_in(AT &hi, AT &lo, AT t) {
+    const AT s_ = hi + t;
+    const AT bp = s_ - hi;
+    const AT err = (hi - (s_ - bp)) + (t - bp);
+    lo += isfinite(s_) ? err : AT(0);
+    hi = s_;
+}
+
+// carry records: (hi, lo) of the accumulation type, widened to FP64 by the zone fixup
+template <typename T> struct Pair;
+template <> struct Pair<float> { using type = float2; };
+template <> struct Pair<double> { using type = double2; };
+__device__ __forceinline__ float2 make_pair2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ double2 make_pair2(double a, double b) { return make_double2(a, b); }
 
 // Load 4 consecutive values at element position p (a multiple of 4) of a
 // 16-byte aligned shared-memory array into the accumulation type.

@@ -47,11 +47,12 @@ struct ZoneDev {
 
 // What the streaming kernel reads per execution tile (16 bytes).  Tile t covers
 // nonzeros [meta[t].nzb, meta[t+1].nzb) and owns the segment end events
-// [meta[t].e_begin, meta[t+1].e_begin); meta[ntiles] is the sentinel {nnz, n_major}.
+// [meta[t].e_begin, meta[t+1].e_begin); meta[ntiles] is the sentinel {nnz, n_major}
+// with the number of nonempty segments as its rank.
 struct alignas(16) TileMeta {
     int32_t nzb, e_begin;
     int32_t flags;  // bit0 needLeft, bit1 needRight, bit2 an empty segment ends in the tile
-    int32_t pad;
+    int32_t rank;   // rank among the nonempty segments of the one open before the tile's first head bit
 };
 
 // Parameters of the streaming kernel.
@@ -81,6 +82,43 @@ struct StreamParams {
                              // the input vector; the indices are offsets into the window (NULL: whole vector)
     int32_t *err;
 };
+
+// What the one-vector passes (pass_kernel.cuh) read per step of 256 nonzeros beside them.
+struct alignas(16) StepRec {
+    uint32_t heads[8];  // bit i of word j: a segment starts at position 32 j + i (the tile's masks)
+    uint8_t before[8];  // heads of the step before word j
+    int32_t first;      // the segment open before the step's first head (-1: none, leading empty ones)
+    int32_t flags;      // STEP_* bits; the heads of the step << 16
+};
+constexpr int STEP_NEED_LEFT = 1;   // the tile's first segment began before it (its first step is asked)
+constexpr int STEP_NEED_RIGHT = 2;  // the tile's last segment continues after it (its last step is asked)
+constexpr int STEP_ENDS = 4;        // the tile's last step: the open segment ends with the tile
+constexpr int STEP_GAPS = 8;        // empty segments lie between the step's segments
+
+// Parameters of the one-vector passes of a validated plan (tiles of T = 256 spt nonzeros).
+struct PassParams {
+    const int32_t *idx;
+    const void *vals;
+    const StepRec *steps;
+    // the nonempty segments in order and every segment's rank among them (read in steps with gaps)
+    const int32_t *seglist, *rank;
+    int32_t nnz, n_minor, ntiles, spt, chunk_tiles;
+    int32_t slots;           // staging slots per warp
+    int32_t copies;          // copies of the accumulator (a power of two), shared by the warps in turn
+    int32_t acc_bytes, vec_bytes;  // shared memory of one accumulator (0 without SC) and of the input (0 without SD)
+    const void *x, *v;       // the long input (SC), the short input (SD)
+    void *part;              // SC: per-CTA partials [cta][n_minor]
+    void *u;                 // SD: the long output
+    void *rec_left, *rec_right;  // SD: carry records [proc], (hi, lo) pairs
+    int32_t *err;
+};
+// Staging of a pass: a slot holds a step's indices, values, record and 16-byte header.
+constexpr int PASS_BAR_BYTES = 512;  // slot barriers, PASS_MAX_SLOTS for each of up to 32 warps
+constexpr int PASS_MAX_SLOTS = 2;
+__host__ __device__ constexpr int pass_slot_bytes(int val_bytes) { return 1024 + 256 * val_bytes + (int)sizeof(StepRec) + 16; }
+// Most warps of a pass: 32 of 64 registers a thread; FP64 needs more registers, and its passes do
+// not gain from more warps (57 us with 16 and with 24 on 8M nonzeros).
+constexpr int pass_warps(int val_bytes) { return val_bytes != 8 ? 32 : 16; }
 
 // Dynamic shared-memory limit of one kernel, raised at most once per device and
 // size: the value set so far on each device, read without a lock, raised under it.
@@ -119,6 +157,11 @@ cudaError_t launch_stream_f64(int mode, int kb, const LaunchArgs &a);
 cudaError_t launch_stream_f32(int mode, int kb, const LaunchArgs &a);
 cudaError_t launch_stream_bf16(int mode, int kb, const LaunchArgs &a);
 cudaError_t launch_stream_f16(int mode, int kb, const LaunchArgs &a);
+// One-vector pass: the accumulating product (sc), the dot products (sd) or both.
+cudaError_t launch_pass_f64(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_pass_f32(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_pass_bf16(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_pass_f16(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
 
 // Small kernels (small_kernels.cu).
 // out_b[i] = sum over parts q of part[q * qstride + b * bstride + i], in FP64, in part order
@@ -131,14 +174,25 @@ cudaError_t launch_interleave(bool f64, int kbt, int kb, const void *const *in, 
                               cudaStream_t s);
 cudaError_t launch_fixup(bool vec_f64, const ZoneDev *zones, int z, const void *rec_left, const void *rec_right,
                          int P, int kb, void *const *out, cudaStream_t s);
+// out[list[i]] = 0, i < count: the outputs of empty segments.
+cudaError_t launch_zero_list(bool vec_f64, const int32_t *list, int count, void *out, cudaStream_t s);
 // Processors of the streaming launches: the chunks of tiles of every CTA's tile range, in
 // order (the kernel's numbering, whatever the warp count).  Fills nzb[0..nproc] (if not
 // NULL) with their nonzero boundaries; returns nproc.
 int stream_processors(int ntiles, int T, int nnz, int ctas, int C, int32_t *nzb);
 
 // Plan kernels (plan.cu).
+// Structural checks (bits into *err) and the number of empty segments (into *nempty, zero on entry).
 cudaError_t launch_validate(const int32_t *ptr, const int32_t *idx, int n_major, int nnz, int n_minor, int32_t *err,
-                            cudaStream_t s);
+                            int32_t *nempty, cudaStream_t s);
+// rank[j] = nonempty segments before j (j <= n_major); seglist / emptylist: the nonempty and
+// the empty segments in order; blk: seg_rank_blocks(n_major) ints of scratch.
+cudaError_t launch_seg_ranks(const int32_t *pptr, int n_major, int32_t *rank, int32_t *seglist, int32_t *emptylist,
+                             int32_t *blk, int32_t *total, cudaStream_t s);
+int seg_rank_blocks(int n_major);
+// The step records of tiles of 256 spt nonzeros, from their masks and descriptors.
+cudaError_t launch_steps(const TileMeta *meta, const uint32_t *masks, int mwp, int ntiles, int spt,
+                         const int32_t *seglist, StepRec *steps, cudaStream_t s);
 cudaError_t launch_pad_ptr(const int32_t *ptr, int32_t *pptr, int n_major, int nnz, int padded, cudaStream_t s);
 // Per chunk: bounds by the Sec. II rule over P chunks (nzb == nullptr) or from nzb[0..P], first/last
 // segments, owned end events, and the number of execution tiles of at most tmax nonzeros.
@@ -152,8 +206,9 @@ size_t setup_scratch_bytes(int P);
 // Execution tile boundaries tile_nzb[t] = min(t * T, nnz), t = 0..ntiles.
 cudaError_t launch_tile_bounds(int ntiles, int T, int nnz, int32_t *tile_nzb, cudaStream_t s);
 // Per tile: segment-start masks and the kernel's tile descriptors (needLeft / needRight of
-// every tile from its neighbours' first and last segments).
+// every tile from its neighbours' first and last segments; rank: launch_seg_ranks' array, or
+// NULL when no segment is empty).
 cudaError_t launch_masks(const int32_t *pptr, const ChunkAux *tiles, int ntiles, int nnz, int n_major, int mwp,
-                         uint32_t *masks, int mwq, uint16_t *pfx, TileMeta *meta, cudaStream_t s);
+                         uint32_t *masks, int mwq, uint16_t *pfx, TileMeta *meta, const int32_t *rank, cudaStream_t s);
 
 }  // namespace gbk

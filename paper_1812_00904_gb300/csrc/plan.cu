@@ -11,14 +11,18 @@ namespace gbk {
 // Error bits of the structural check (plan-time; the host maps them to messages).
 // 1: ptr[0] != 0, 2: ptr decreasing or outside [0, nnz], 4: ptr[last] != nnz, 8: index out of range.
 __global__ void validate_kernel(const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx, int n_major,
-                                int nnz, int n_minor, int32_t *err) {
-    int bits = 0;
+                                int nnz, int n_minor, int32_t *err, int32_t *nempty) {
+    int bits = 0, empty = 0;
     const long stride = (long)gridDim.x * blockDim.x;
     for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j <= n_major; j += stride) {
         const int pj = ptr[j];
         if (j == 0 && pj != 0) bits |= 1;
         if (pj < 0 || pj > nnz) bits |= 2;
-        if (j < n_major && ptr[j + 1] < pj) bits |= 2;
+        if (j < n_major) {
+            const int pn = ptr[j + 1];
+            if (pn < pj) bits |= 2;
+            empty += pn == pj;
+        }
         if (j == n_major && pj != nnz) bits |= 4;
     }
     for (long k = blockIdx.x * (long)blockDim.x + threadIdx.x; k < nnz; k += stride) {
@@ -26,11 +30,13 @@ __global__ void validate_kernel(const int32_t *__restrict__ ptr, const int32_t *
         if (r < 0 || r >= n_minor) bits |= 8;
     }
     if (bits) atomicOr(err, bits);
+    empty = __reduce_add_sync(0xffffffffu, empty);
+    if (empty && (threadIdx.x & 31) == 0) atomicAdd(nempty, empty);
 }
 
 cudaError_t launch_validate(const int32_t *ptr, const int32_t *idx, int n_major, int nnz, int n_minor, int32_t *err,
-                            cudaStream_t s) {
-    validate_kernel<<<1024, 256, 0, s>>>(ptr, idx, n_major, nnz, n_minor, err);
+                            int32_t *nempty, cudaStream_t s) {
+    validate_kernel<<<1024, 256, 0, s>>>(ptr, idx, n_major, nnz, n_minor, err, nempty);
     return cudaGetLastError();
 }
 
@@ -365,6 +371,49 @@ size_t setup_scratch_bytes(int P) {
     return (size_t)((nb + 3) & ~3) * sizeof(int) + 2 * (size_t)nb * sizeof(SegPair) + 64;
 }
 
+// The nonempty segments in order and their ranks, for matrices with empty ones: every block
+// counts its SU_ITEMS segments, one block scans the counts, every block writes its part.
+__global__ void __launch_bounds__(SU_THREADS) seg_count_kernel(const int32_t *__restrict__ pptr, int n_major,
+                                                               int32_t *__restrict__ blk) {
+    const int j0 = blockIdx.x * SU_ITEMS + threadIdx.x * SU_IPT;
+    int c = 0;
+    for (int i = 0; i < SU_IPT && j0 + i < n_major; ++i) c += pptr[j0 + i + 1] > pptr[j0 + i];
+    int total;
+    block_exclusive(c, 0, AddOp(), &total);
+    if (threadIdx.x == 0) blk[blockIdx.x] = total;
+}
+__global__ void __launch_bounds__(SU_THREADS) seg_rank_kernel(const int32_t *__restrict__ pptr, int n_major,
+                                                              const int32_t *__restrict__ blk, int32_t *__restrict__ rank,
+                                                              int32_t *__restrict__ seglist,
+                                                              int32_t *__restrict__ emptylist) {
+    const int j0 = blockIdx.x * SU_ITEMS + threadIdx.x * SU_IPT;
+    int c = 0;
+    for (int i = 0; i < SU_IPT && j0 + i < n_major; ++i) c += pptr[j0 + i + 1] > pptr[j0 + i];
+    int total;
+    int r = blk[blockIdx.x] + block_exclusive(c, 0, AddOp(), &total);
+    for (int i = 0; i < SU_IPT && j0 + i < n_major; ++i) {
+        const int j = j0 + i;
+        rank[j] = r;
+        if (pptr[j + 1] > pptr[j])
+            seglist[r++] = j;
+        else
+            emptylist[j - r] = j;  // (j - r empty ones before it)
+        if (j == n_major - 1) rank[n_major] = r;
+    }
+}
+
+int seg_rank_blocks(int n_major) { return (n_major + SU_ITEMS - 1) / SU_ITEMS; }
+
+cudaError_t launch_seg_ranks(const int32_t *pptr, int n_major, int32_t *rank, int32_t *seglist, int32_t *emptylist,
+                             int32_t *blk, int32_t *total, cudaStream_t s) {
+    const int nb = seg_rank_blocks(n_major);
+    if (nb <= 0) return cudaSuccess;
+    seg_count_kernel<<<nb, SU_THREADS, 0, s>>>(pptr, n_major, blk);
+    setup_scan_add_kernel<<<1, SU_THREADS, 0, s>>>(blk, nb, total);
+    seg_rank_kernel<<<nb, SU_THREADS, 0, s>>>(pptr, n_major, blk, rank, seglist, emptylist);
+    return cudaGetLastError();
+}
+
 // Execution tile boundaries: tile t covers nonzeros [t*T, min((t+1)*T, nnz)), so
 // every tile starts on a multiple of 8 and fills whole steps of the kernels.
 __global__ void tile_bounds_kernel(int ntiles, int T, int nnz, int32_t *__restrict__ tile_nzb) {
@@ -386,7 +435,7 @@ cudaError_t launch_tile_bounds(int ntiles, int T, int nnz, int32_t *tile_nzb, cu
 // segments can start at one position and the kernels take their general path).
 __global__ void masks_kernel(const int32_t *__restrict__ pptr, const ChunkAux *__restrict__ tiles, int ntiles, int nnz,
                              int n_major, int mwp, uint32_t *__restrict__ masks, int mwq, uint16_t *__restrict__ pfx,
-                             TileMeta *__restrict__ meta) {
+                             TileMeta *__restrict__ meta, const int32_t *__restrict__ rank) {
     __shared__ uint32_t sm[8][32];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -428,23 +477,60 @@ __global__ void masks_kernel(const int32_t *__restrict__ pptr, const ChunkAux *_
         const bool need_left = t > 0 && tiles[t - 1].jl == d.jf;
         const bool need_right = t + 1 < ntiles && tiles[t + 1].jf == d.jl;
         m.flags = (need_left ? 1 : 0) | (need_right ? 2 : 0) | (dup ? 4 : 0);
-        m.pad = 0;
+        // (leading empty segments set bit 0 of the first tile: its count starts one lower)
+        m.rank = rank ? rank[d.jf] - static_cast<int>(sm[wib][0] & 1u) : d.e_begin;
         meta[t] = m;
         if (t == ntiles - 1) {
             TileMeta e;
             e.nzb = nnz;
             e.e_begin = n_major;
             e.flags = 0;
-            e.pad = 0;
+            e.rank = rank ? rank[n_major] : n_major;
             meta[ntiles] = e;
         }
     }
 }
 
 cudaError_t launch_masks(const int32_t *pptr, const ChunkAux *tiles, int ntiles, int nnz, int n_major, int mwp,
-                         uint32_t *masks, int mwq, uint16_t *pfx, TileMeta *meta, cudaStream_t s) {
+                         uint32_t *masks, int mwq, uint16_t *pfx, TileMeta *meta, const int32_t *rank, cudaStream_t s) {
     if (ntiles <= 0) return cudaSuccess;
-    masks_kernel<<<(ntiles + 7) / 8, 256, 0, s>>>(pptr, tiles, ntiles, nnz, n_major, mwp, masks, mwq, pfx, meta);
+    masks_kernel<<<(ntiles + 7) / 8, 256, 0, s>>>(pptr, tiles, ntiles, nnz, n_major, mwp, masks, mwq, pfx, meta, rank);
+    return cudaGetLastError();
+}
+
+// One thread per step: its 8 mask words, the heads before each, the segment open before its first
+// head and the flags of StepRec.  seglist: the nonempty segments, or NULL when none is empty.
+__global__ void steps_kernel(const TileMeta *__restrict__ meta, const uint32_t *__restrict__ masks, int mwp, int ntiles,
+                             int spt, const int32_t *__restrict__ seglist, StepRec *__restrict__ steps) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t ti = i / spt;
+    if (ti >= ntiles) return;
+    const int t = (int)ti, stp = (int)(i % spt);
+    const TileMeta m = meta[t];
+    const int n = meta[t + 1].nzb - m.nzb;
+    if (stp * 256 >= n) return;
+    const uint32_t *w = masks + (size_t)t * mwp;
+    int rank = m.rank, c = 0;
+    for (int j = 0; j < 8 * stp; ++j) rank += __popc(w[j]);
+    StepRec r;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        r.heads[j] = w[8 * stp + j];
+        r.before[j] = static_cast<uint8_t>(c);
+        c += __popc(r.heads[j]);
+    }
+    r.first = seglist && rank >= 0 ? seglist[rank] : rank;
+    const bool last = (stp + 1) * 256 >= n;
+    const bool gaps = seglist && (rank < 0 || seglist[rank + c] - r.first != c);
+    r.flags = (m.flags & 3) | (last && meta[t + 1].rank != rank + c ? STEP_ENDS : 0) | (gaps ? STEP_GAPS : 0) | (c << 16);
+    steps[i] = r;
+}
+
+cudaError_t launch_steps(const TileMeta *meta, const uint32_t *masks, int mwp, int ntiles, int spt,
+                         const int32_t *seglist, StepRec *steps, cudaStream_t s) {
+    if (ntiles <= 0) return cudaSuccess;
+    const int64_t n = (int64_t)ntiles * spt;
+    steps_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(meta, masks, mwp, ntiles, spt, seglist, steps);
     return cudaGetLastError();
 }
 

@@ -45,6 +45,13 @@ struct spmv_plan_s {
     int32_t *err = nullptr;
     gbk::TileMeta *meta = nullptr;         // execution tiles (ntiles + 1)
     uint32_t *masks = nullptr;
+    // one-vector passes (pass_kernel.cuh): which products they serve (the short vectors fit on chip)
+    bool pass_sc = false, pass_sd = false, pass_pair = false;
+    gbk::StepRec *steps = nullptr;
+    // nonempty / empty segments and ranks among the nonempty (when some are empty)
+    int32_t *seglist = nullptr, *emptylist = nullptr, *segrank = nullptr;
+    int nempty = 0;
+    void *ws_seg = nullptr;
     uint16_t *pfx = nullptr;    // per tile: segment starts before each mask word (then the total)
     // Overlap zones among the processors of the streaming passes: the chunks of whole tiles
     // (contiguous Sec. II groups) every CTA's tile range is cut into.
@@ -91,6 +98,7 @@ struct spmv_plan_s {
     // kernel timers (SPMV_PLAN_PROFILE)
     struct Prof {
         int kernel;
+        double share;
         cudaEvent_t a, b;
     };
     std::atomic<bool> prof_on{false};  // SPMV_PLAN_PROFILE at creation; spmv_profile_enable later

@@ -195,4 +195,19 @@ cudaError_t launch_fixup(bool vec_f64, const ZoneDev *zones, int z, const void *
     return cudaGetLastError();
 }
 
+template <typename XT>
+__global__ void __launch_bounds__(256) zero_list_kernel(const int32_t *__restrict__ list, int count, XT *__restrict__ out) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) out[list[i]] = XT(0);
+}
+
+cudaError_t launch_zero_list(bool vec_f64, const int32_t *list, int count, void *out, cudaStream_t s) {
+    if (count <= 0) return cudaSuccess;
+    const int grid = std::min((count + 255) / 256, 152 * 8);
+    if (vec_f64)
+        zero_list_kernel<double><<<grid, 256, 0, s>>>(list, count, static_cast<double *>(out));
+    else
+        zero_list_kernel<float><<<grid, 256, 0, s>>>(list, count, static_cast<float *>(out));
+    return cudaGetLastError();
+}
+
 }  // namespace gbk

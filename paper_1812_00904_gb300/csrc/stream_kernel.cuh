@@ -42,8 +42,6 @@
 
 namespace gbk {
 
-constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;   // 2 s per pipeline wait
-
 __device__ __forceinline__ void copy_elem(unsigned char *d, const unsigned char *s, int es) {
     if (es == 8) {
         *reinterpret_cast<unsigned long long *>(d) = *reinterpret_cast<const unsigned long long *>(s);
@@ -55,29 +53,6 @@ __device__ __forceinline__ void copy_elem(unsigned char *d, const unsigned char 
 }
 
 template <typename XT> __device__ __forceinline__ XT zero_of() { return XT(0); }
-
-// A product rounded on its own (never fused into a following addition), so that the
-// segmented passes round every product the same way whatever code surrounds it.
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-// hi + lo += t, compensated (TwoSum: hi takes the rounded sum, lo gathers its rounding
-// errors).  A sum that is infinite or NaN carries no error term, so that hi + lo stays what the
-// plain sum gives (an infinity would otherwise make the error term NaN).
-template <typename AT>
-__device__ __forceinline__ void carry_in(AT &hi, AT &lo, AT t) {
-    const AT s_ = hi + t;
-    const AT bp = s_ - hi;
-    const AT err = (hi - (s_ - bp)) + (t - bp);
-    lo += isfinite(s_) ? err : AT(0);
-    hi = s_;
-}
-
-// carry records: (hi, lo) of the accumulation type, widened to FP64 by the zone fixup
-template <typename T> struct Pair;
-template <> struct Pair<float> { using type = float2; };
-template <> struct Pair<double> { using type = double2; };
-__device__ __forceinline__ float2 make_pair2(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ double2 make_pair2(double a, double b) { return make_double2(a, b); }
 
 // KB consecutive vector entries at a 16-byte aligned address (KB >= 2), by vector loads
 // through the read-only path.
@@ -724,15 +699,15 @@ __global__ void __launch_bounds__(WB * 32, 1) stream_kernel(const __grid_constan
                             }
 #pragma unroll
                             for (int b = 0; b < KB; ++b) {
-                                const AT pe = mul_rn(vae, static_cast<AT>(wv[b]));
-                                rr[e][b] = (e == 0 || ((hb >> e) & 1u)) ? pe : rr[e > 0 ? e - 1 : 0][b] + pe;
+                                rr[e][b] = seg_term(vae, static_cast<AT>(wv[b]), rr[e > 0 ? e - 1 : 0][b],
+                                                    e == 0 || ((hb >> e) & 1u));
                             }
                         }
                         return;
                     }
 #pragma unroll
                     for (int b = 0; b < KB; ++b) {
-                        AT pr[8];
+                        AT wr[8];
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
                             AT w_ = AT(0);
@@ -743,12 +718,17 @@ __global__ void __launch_bounds__(WB * 32, 1) stream_kernel(const __grid_constan
                                     w_ = static_cast<AT>(__ldg(static_cast<const XT *>(p.vin[b]) + vwin + ix[e]));
                                 }
                             }
-                            pr[e] = mul_rn(va[e], w_);
+                            wr[e] = sizeof(AT) == 4 ? mul_rn(va[e], w_) : w_;  // (FP64: multiplied below)
                         }
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
-                            const AT pe = sw ? pr[e ^ 4] : pr[e];
-                            rr[e][b] = (e == 0 || ((hb >> e) & 1u)) ? pe : rr[e > 0 ? e - 1 : 0][b] + pe;
+                            if constexpr (sizeof(AT) == 4) {
+                                const AT pe = sw ? wr[e ^ 4] : wr[e];
+                                rr[e][b] = (e == 0 || ((hb >> e) & 1u)) ? pe : rr[e > 0 ? e - 1 : 0][b] + pe;
+                            } else {
+                                rr[e][b] = seg_term(sw ? va[e ^ 4] : va[e], sw ? wr[e ^ 4] : wr[e],
+                                                    rr[e > 0 ? e - 1 : 0][b], e == 0 || ((hb >> e) & 1u));
+                            }
                         }
                     }
                 };

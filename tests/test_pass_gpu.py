@@ -1,0 +1,96 @@
+"""The one-vector passes of validated plans (pass_kernel.cuh): products against the FP64 oracle,
+dot products bit for bit against the streaming kernel (an unvalidated plan of the same tiles),
+at the edges of steps and tiles, with empty segments anywhere, and from many copies of a short
+accumulator to the longest one that fits in shared memory."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import oracle  # noqa: E402
+import synth  # noqa: E402
+
+import paper_1812_00904_gb300 as pkg  # noqa: E402
+from gpu_util import DEV, TOL, assert_close, check_products, dev_vec, host_of, make_plan  # noqa: E402
+
+DTYPES = [torch.float64, torch.float32, torch.bfloat16, torch.float16]
+
+
+def _degrees(kind, nnz, rng, short):
+    if kind == "one":  # one long segment (repeated indices), empty ones before and after
+        return np.array([0, 0, nnz, 0])
+    if kind == "single":  # a head at every position
+        return np.ones(nnz, dtype=np.int64)
+    deg = []  # segments of 0 to 90 nonzeros, empty ones at both ends and in runs
+    left = nnz
+    deg += [0, 0, 0]
+    while left > 0:
+        d = int(min(left, rng.integers(0, 90) if rng.random() < 0.7 else rng.integers(0, 4)))
+        deg.append(d)
+        if rng.random() < 0.02:
+            deg += [0] * int(rng.integers(1, 40))
+        left -= d
+    return np.array(deg + [0, 0])
+
+
+def _check(A, dtype, tile_items, what):
+    plan, stored = make_plan(A, dtype, tile_items=tile_items)
+    x, v = synth.uniform_vector(A.n, 3), synth.uniform_vector(A.m, 4)
+    check_products(plan, stored, x, v, TOL[dtype], what)
+    ref, _ = make_plan(A, dtype, tile_items=tile_items, flags=pkg.SPMV_PLAN_NO_VALIDATE)
+    xd, vd = dev_vec(x, plan.vec_dtype), dev_vec(v, plan.vec_dtype)
+    dot = (lambda p: p.spvtm(vd)) if A.layout == "csc" else (lambda p: p.spmv(xd))
+    assert torch.equal(dot(plan), dot(ref)), f"{what}: dot products differ from the streaming kernel's"
+    y, u = torch.full((A.m,), 7.0, dtype=plan.vec_dtype, device=DEV), torch.full((A.n,), 7.0, dtype=plan.vec_dtype, device=DEV)
+    pkg.spmv_pair(plan.handle, xd, y, vd, u)
+    assert torch.equal(u if A.layout == "csc" else y, dot(plan)), f"{what}: the pair's dot products differ"
+    short, ref_s, scale = ((y, oracle.spmv, oracle.abs_spmv) if A.layout == "csc" else (u, oracle.spvtm, oracle.abs_spvtm))
+    arg = host_of(xd if A.layout == "csc" else vd)
+    assert_close(host_of(short), ref_s(stored, arg), scale(stored, arg), TOL[dtype], f"{what}: pair")
+    plan.check()
+
+
+@pytest.mark.parametrize("dtype", DTYPES, ids=str)
+@pytest.mark.parametrize("layout", ["csc", "csr"])
+@pytest.mark.parametrize("kind", ["one", "single", "mixed"])
+def test_edges_of_steps_and_tiles(kind, layout, dtype):
+    rng = np.random.default_rng(5)
+    for tile_items in (256, 512, 768):
+        for nnz in (1, 8, 255, 256, 257, 511, 513, 769, 60_000):
+            deg = _degrees(kind, nnz, rng, 300)
+            m, n = (300, len(deg)) if layout == "csc" else (len(deg), 300)
+            A = synth.random_matrix(m, n, layout, degrees=deg, seed=nnz, duplicates=True)
+            _check(A, dtype, tile_items, f"{kind} {layout} nnz={nnz} T={tile_items}")
+
+
+@pytest.mark.parametrize("dtype", DTYPES, ids=str)
+@pytest.mark.parametrize("short", [1, 31, 4000, 14_000, 23_000, 27_000, 48_000, 52_001, 57_000])
+def test_length_of_the_short_vector(short, dtype):
+    # from 16 copies of the accumulator to one beside the staging of a few warps, and beyond
+    rng = np.random.default_rng(short)
+    deg = np.minimum((3.0 * rng.random(20_000) ** -1.0).astype(np.int64), 3_000)
+    A = synth.random_matrix(short, 20_000, "csc", degrees=deg, seed=9, duplicates=True)
+    _check(A, dtype, 256, f"short={short}")
+
+
+def test_in_a_graph_and_with_changed_values():
+    """A captured pair replays on new vectors and on values changed in place (the plan borrows them)."""
+    rng = np.random.default_rng(8)
+    A = synth.random_matrix(2_000, 30_000, "csc", degrees=rng.integers(0, 40, 30_000), seed=2)
+    plan, stored = make_plan(A)
+    xd, vd = dev_vec(synth.uniform_vector(A.n, 1), torch.float32), dev_vec(synth.uniform_vector(A.m, 2), torch.float32)
+    y, u = torch.empty(A.m, device=DEV), torch.empty(A.n, device=DEV)
+    pkg.spmv_pair(plan.handle, xd, y, vd, u)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        pkg.spmv_pair(plan.handle, xd, y, vd, u)
+    plan.vals.mul_(-2.0)
+    xd.mul_(3.0)
+    g.replay()
+    torch.cuda.synchronize()
+    stored = synth.SparseMatrix(A.layout, A.m, A.n, A.ptr, A.idx, -2.0 * stored.vals)
+    xs, vs = host_of(xd), host_of(vd)
+    assert_close(host_of(y), oracle.spmv(stored, xs), oracle.abs_spmv(stored, xs), 1e-5, "y")
+    assert_close(host_of(u), oracle.spvtm(stored, vs), oracle.abs_spvtm(stored, vs), 1e-5, "u")
