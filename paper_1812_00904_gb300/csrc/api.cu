@@ -242,7 +242,7 @@ size_t plan_footprint(const spmv_plan_s *p) {
 }
 
 // The one-vector pass of plan p: y_short += A x (sc) into the per-CTA partials, u = the dot
-// products with v (sd), or both; then the combine and the zone fix-up.
+// products with v (sd), or both; then the combine and the zone fix-up in one launch.
 static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *v, void *u, cudaStream_t s) {
     const bool sc = y != nullptr, sd = u != nullptr;
     PassParams pp;
@@ -265,6 +265,8 @@ static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *
     pp.u = u;
     pp.rec_left = p->rec_left;
     pp.rec_right = p->rec_right;
+    pp.emptylist = p->emptylist;
+    pp.nempty = p->nempty;
     pp.err = p->err;
     const PassGeometry g = pass_geometry(p, sc, sd);
     pp.slots = g.slots;
@@ -275,14 +277,17 @@ static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *
         ProfScope ps0(p, 0, s, !sc ? 0.0 : sd ? 0.5 : 1.0), ps2(p, 2, s, !sd ? 0.0 : sc ? 0.5 : 1.0);
         CUDA_TRY(launch_pass(p, sc, sd, pp, g.warps, (int)g.smem, s));
     }
-    if (sc) {
-        ProfScope ps(p, 1, s);
-        CUDA_TRY(launch_combine(f64, f64, p->part, p->ctas, p->n_minor, 1, &y, s));
-    }
-    if (sd && (p->pz.z > 0 || p->nempty > 0)) {
-        ProfScope ps(p, 3, s);
-        CUDA_TRY(launch_fixup(f64, p->pz.zones, p->pz.z, p->rec_left, p->rec_right, p->pz.nproc, 1, &u, s));
-        CUDA_TRY(launch_zero_list(f64, p->emptylist, p->nempty, u, s));
+    const spmv_plan_s::ProcZones &pz = p->pz;
+    const bool zones = sd && pz.z > 0;
+    if (sc || zones) {
+        ProfScope ps1(p, 1, s, !sc ? 0.0 : zones ? 0.5 : 1.0), ps3(p, 3, s, !zones ? 0.0 : sc ? 0.5 : 1.0);
+        if (sc && zones)
+            CUDA_TRY(launch_combine_fixup(f64, p->part, p->ctas, p->n_minor, y, pz.zones, pz.z, p->rec_left, p->rec_right,
+                                          pz.nproc, u, s));
+        else if (sc)
+            CUDA_TRY(launch_combine(f64, f64, p->part, p->ctas, p->n_minor, 1, &y, s));
+        else
+            CUDA_TRY(launch_fixup(f64, pz.zones, pz.z, p->rec_left, p->rec_right, pz.nproc, 1, &u, s));
     }
     return SPMV_OK;
 }

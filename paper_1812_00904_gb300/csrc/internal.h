@@ -83,6 +83,24 @@ struct StreamParams {
     int32_t *err;
 };
 
+// CTA g's chunks (processors) when ntiles tiles are cut over `ctas` CTAs with chunks of C tiles:
+// tiles [ta, ta + nct), nb chunks of C tiles, then single-tile ones, nq in all, numbered from proc0.
+struct CtaChunks {
+    int ta, nct, nb, nq, proc0;
+};
+__host__ __device__ inline CtaChunks cta_chunks(int g, int ntiles, int ctas, int C) {
+    const int tq = ntiles / ctas, tr = ntiles % ctas, tail = MAX_WARPS * C + MAX_WARPS;
+    auto big = [&](int n) { return (n - (n < tail ? n : tail)) / C; };
+    auto chunks = [&](int n) { return n - (C - 1) * big(n); };
+    CtaChunks c;
+    c.ta = g * tq + (g < tr ? g : tr);
+    c.nct = tq + (g < tr ? 1 : 0);
+    c.nb = big(c.nct);
+    c.nq = chunks(c.nct);
+    c.proc0 = g * chunks(tq) + (g < tr ? g : tr) * (chunks(tq + 1) - chunks(tq));
+    return c;
+}
+
 // What the one-vector passes (pass_kernel.cuh) read per step of 256 nonzeros beside them.
 struct alignas(16) StepRec {
     uint32_t heads[8];  // bit i of word j: a segment starts at position 32 j + i (the tile's masks)
@@ -110,6 +128,8 @@ struct PassParams {
     void *part;              // SC: per-CTA partials [cta][n_minor]
     void *u;                 // SD: the long output
     void *rec_left, *rec_right;  // SD: carry records [proc], (hi, lo) pairs
+    const int32_t *emptylist;  // SD: the empty segments, whose outputs are 0
+    int32_t nempty;
     int32_t *err;
 };
 // Staging of a pass: a slot holds a step's indices, values, record and 16-byte header.
@@ -174,8 +194,10 @@ cudaError_t launch_interleave(bool f64, int kbt, int kb, const void *const *in, 
                               cudaStream_t s);
 cudaError_t launch_fixup(bool vec_f64, const ZoneDev *zones, int z, const void *rec_left, const void *rec_right,
                          int P, int kb, void *const *out, cudaStream_t s);
-// out[list[i]] = 0, i < count: the outputs of empty segments.
-cudaError_t launch_zero_list(bool vec_f64, const int32_t *list, int count, void *out, cudaStream_t s);
+// Both after a pass over one vector that served both products.
+cudaError_t launch_combine_fixup(bool f64, const void *part, int nparts, int n_minor, void *short_out, const ZoneDev *zones,
+                                 int z, const void *rec_left, const void *rec_right, int P, void *long_out,
+                                 cudaStream_t s);
 // Processors of the streaming launches: the chunks of tiles of every CTA's tile range, in
 // order (the kernel's numbering, whatever the warp count).  Fills nzb[0..nproc] (if not
 // NULL) with their nonzero boundaries; returns nproc.

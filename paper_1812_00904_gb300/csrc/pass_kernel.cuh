@@ -38,17 +38,12 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
     // head-free ones, and a fixed round-robin left warps waiting at the end (14% of warp time on
     // the 50M-nonzero wide matrix).  Whichever warp runs a chunk, its sums are the same.
     const int C = p.chunk_tiles;
-    const int tq = p.ntiles / gridDim.x, tr = p.ntiles % gridDim.x;
-    const int gb = blockIdx.x;
-    const int ta = gb * tq + min(gb, tr);
-    const int nct = tq + (gb < tr ? 1 : 0);
-    auto big_chunks = [&](int n) { return (n - min(n, MAX_WARPS * C + MAX_WARPS)) / C; };
-    auto chunks_of = [&](int n) { return n - (C - 1) * big_chunks(n); };
-    const int nb = big_chunks(nct);
-    const int nq = chunks_of(nct);
-    const int proc0 = gb * chunks_of(tq) + min(gb, tr) * (chunks_of(tq + 1) - chunks_of(tq));
+    const CtaChunks cc_ = cta_chunks(blockIdx.x, p.ntiles, gridDim.x, C);
+    const int ta = cc_.ta, nb = cc_.nb, nq = cc_.nq, proc0 = cc_.proc0;
     const int nsteps = p.nnz / 256 + (p.nnz % 256 != 0);  // of the matrix
 
+    // the combine and the zone fix-up may be launched: their blocks find room as this grid's CTAs end
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ int next_chunk;
     if (threadIdx.x == 0) next_chunk = 0;
     if (lane == 0) {
@@ -103,6 +98,8 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
         for (int i = threadIdx.x; i < n16; i += blockDim.x) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if constexpr (SD) {
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x)
+            static_cast<XT *>(p.u)[p.emptylist[i]] = XT(0);
         constexpr int xa = 16 / (int)sizeof(XT);
         const XT *src = static_cast<const XT *>(p.v);
         const int n16 = p.n_minor / xa;

@@ -9,6 +9,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "zones.cuh"
 
 namespace gbk {
 
@@ -19,120 +20,142 @@ struct InPtrs {
     const void *p[VL_MAX];
 };
 
-// An FP32 value widened to FP64 exactly, by integer operations on its bits only: the FP64
-// pipe (slow on this part) is left to the additions.  Normal numbers move the sign, the
-// exponent (rebiased from 127 to 1023) and the mantissa; a subnormal m 2^-149 is normalised
-// at its leading one bit h (exponent h - 149); zeros keep their sign; infinities and NaNs
-// take the all-ones exponent with the mantissa bits (a NaN stays a NaN).
-__device__ __forceinline__ double widen(float f) {
-    const uint32_t u = __float_as_uint(f);
-    const uint32_t e = (u >> 23) & 0xFFu;
-    const uint32_t mant = u & 0x7FFFFFu;
-    const uint64_t sign = static_cast<uint64_t>(u & 0x80000000u) << 32;
-    uint64_t d;
-    if (e == 0u) {
-        const int h = 31 - __clz(mant | 1u);
-        d = mant == 0u ? sign
-                       : sign | (static_cast<uint64_t>(h + 874) << 52) |
-                             (static_cast<uint64_t>(mant ^ (1u << h)) << (52 - h));
-    } else {
-        const uint64_t ed = e == 0xFFu ? 0x7FFull : static_cast<uint64_t>(e + 896u);
-        d = sign | (ed << 52) | (static_cast<uint64_t>(mant) << 29);
-    }
-    return __longlong_as_double(static_cast<long long>(d));
-}
-__device__ __forceinline__ double widen(double f) { return f; }
-
-// out_b[i] = sum_{q < nparts} part[q * qstride + b * bstride + i].  A block takes 32
-// consecutive elements; its 8 thread rows sum the partials q = row, row + 8, ... in
-// FP64 and the 8 row sums are added in row order: a fixed order, independent of
-// timing.  Partials of any type are widened to FP64 before they are added.
-constexpr int COMB_X = 32, COMB_Y = 8;
-template <typename XT, typename PT>
-__global__ void __launch_bounds__(COMB_X * COMB_Y) combine_kernel(const PT *__restrict__ part, int nparts, int n_minor,
-                                                                  size_t qstride, size_t bstride, OutPtrs out) {
-    __shared__ double sh_s[COMB_Y][COMB_X];
-    const int i = blockIdx.x * COMB_X + threadIdx.x;
+// The cross-CTA sums after a pass, one launch for both kinds of block:
+// - combine: out_b[i] = sum_{q < nparts} part[q * qstride + b * bstride + i].  A block takes 32
+//   consecutive elements; its 8 thread rows sum the partials q = row, row + 8, ... in FP64 and the
+//   row sums are added in row order: a fixed order, independent of timing.  Partials of any type
+//   are widened to FP64 before they are added.  The FP64 additions (2 a cycle per SM) set the
+//   floor, 5 us for 152 partials of 20,000 elements; the loads of FIN_CB partials go together.
+// - fix-up: the overlap zones' sums (zones.cuh), one thread per zone, into the zones' columns.
+// blockIdx.y is the vector.
+struct FinishArgs {
+    int comb_blocks;  // blocks [0, comb_blocks) combine, the others fix up
+    const void *part;
+    int nparts, n_minor;
+    size_t qstride, bstride;
+    const ZoneDev *zones;
+    int z, P;
+    const void *rec_left, *rec_right;
+    OutPtrs short_out, long_out;
+};
+constexpr int FIN_X = 32, FIN_ROWS = 8, FIN_CB = 10;
+template <typename XT, typename PT, typename RT>
+__global__ void __launch_bounds__(FIN_X * FIN_ROWS) finish_kernel(const __grid_constant__ FinishArgs p) {
+    __shared__ double sh_s[FIN_ROWS][FIN_X];
     const int b = blockIdx.y;
-    const int row = threadIdx.y;
-    double s = 0.0;
-    if (i < n_minor) {
-        const PT *src = part + (size_t)b * bstride + i;
-#pragma unroll 4
-        for (int q = row; q < nparts; q += COMB_Y) s += widen(__ldg(src + (size_t)q * qstride));
+    if ((int)blockIdx.x >= p.comb_blocks) {
+        const int k = (blockIdx.x - p.comb_blocks) * (FIN_X * FIN_ROWS) + threadIdx.x;
+        const ZoneDev zd = k < p.z ? p.zones[k] : ZoneDev{0, 0, 0, 0};
+        asm volatile("griddepcontrol.wait;" ::: "memory");  // the records of the pass launched before
+        const double t = zone_sum(k < p.z, zd, static_cast<const RT *>(p.rec_left) + (size_t)b * p.P,
+                                  static_cast<const RT *>(p.rec_right) + (size_t)b * p.P);
+        if (k < p.z) static_cast<XT *>(p.long_out.p[b])[zd.col] = static_cast<XT>(t);
+        return;
     }
-    sh_s[row][threadIdx.x] = s;
-    __syncthreads();
-    if (row == 0 && i < n_minor) {
-        double t = sh_s[0][threadIdx.x];
+    const int tx = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const int i = blockIdx.x * FIN_X + tx;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the partials
+    double s = 0.0;
+    if (i < p.n_minor) {
+        const PT *src = static_cast<const PT *>(p.part) + (size_t)b * p.bstride + i;
+        for (int q = row; q < p.nparts; q += FIN_CB * FIN_ROWS) {
+            PT m[FIN_CB];
 #pragma unroll
-        for (int r = 1; r < COMB_Y; ++r) t += sh_s[r][threadIdx.x];
-        static_cast<XT *>(out.p[b])[i] = static_cast<XT>(t);
+            for (int j = 0; j < FIN_CB; ++j)
+                m[j] = q + j * FIN_ROWS < p.nparts ? src[(size_t)(q + j * FIN_ROWS) * p.qstride] : PT(0);
+#pragma unroll
+            for (int j = 0; j < FIN_CB; ++j)
+                if (q + j * FIN_ROWS < p.nparts) s += widen(m[j]);
+        }
+    }
+    sh_s[row][tx] = s;
+    __syncthreads();
+    if (row == 0 && i < p.n_minor) {
+        double t = sh_s[0][tx];
+#pragma unroll
+        for (int r = 1; r < FIN_ROWS; ++r) t += sh_s[r][tx];
+        static_cast<XT *>(p.short_out.p[b])[i] = static_cast<XT>(t);
     }
 }
 
-// Zone k spans tiles S_k = [first, last]: u_{j_k} = right record of the first
-// tile + the records of the middle tiles (whole-tile sums, kept as right records)
-// + left record of the last, added in this order in FP64 (the hi and the lo
-// parts of the (hi, lo) records in two FP64 sums, added at the end).  One thread
-// per zone (most zones span two tiles); the loads of a long zone are issued
-// eight at a time.  Every zone's column is written once.
-template <typename XT, typename RT>
-__global__ void __launch_bounds__(256) fixup_kernel(const ZoneDev *__restrict__ zones, int z,
-                                                    const RT *__restrict__ rec_left, const RT *__restrict__ rec_right,
-                                                    int P, int kb, OutPtrs out) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= z) return;
-    const ZoneDev zd = zones[k];
-    for (int b = 0; b < kb; ++b) {
-        const RT *rr = rec_right + (size_t)b * P;
-        const RT l = rec_left[(size_t)b * P + zd.last];
-        // hi and lo parts summed apart in FP64 (for FP32 records both widen exactly)
-        double sh = widen(rr[zd.first].x), sl = widen(rr[zd.first].y);
-        int q = zd.first + 1;
-        for (; q + 8 <= zd.last; q += 8) {
-            RT m[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) m[e] = rr[q + e];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                sh += widen(m[e].x);
-                sl += widen(m[e].y);
-            }
-        }
-        for (; q < zd.last; ++q) {
-            sh += widen(rr[q].x);
-            sl += widen(rr[q].y);
-        }
-        sh += widen(l.x);
-        sl += widen(l.y);
-        const double s = sh + sl;
-        static_cast<XT *>(out.p[b])[zd.col] = static_cast<XT>(s);
-    }
+// Launched with programmatic serialization: its blocks may become resident while the pass before
+// drains (they wait in griddepcontrol.wait), which hides the launch.  They would all settle on
+// the SMs that come free first and share those SMs' FP64 pipes (19 us instead of 7 for 20,000
+// elements); each asks for so much shared memory that no SM takes more than its share of them.
+template <typename XT, typename PT, typename RT>
+cudaError_t launch_finish(FinishArgs &p, int kb, cudaStream_t s) {
+    constexpr int SMS = 152, ALL = 220 * 1024, RESIDENT = 2048 / (FIN_X * FIN_ROWS);
+    p.comb_blocks = (p.n_minor + FIN_X - 1) / FIN_X;
+    const int64_t blocks = p.comb_blocks + ((int64_t)p.z + FIN_X * FIN_ROWS - 1) / (FIN_X * FIN_ROWS);
+    if (blocks <= 0) return cudaSuccess;
+    const int64_t per_sm = (blocks * kb + SMS - 1) / SMS;
+    auto kern = finish_kernel<XT, PT, RT>;
+    static SmemLimit lim;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks, kb);
+    cfg.blockDim = dim3(FIN_X * FIN_ROWS);
+    cfg.dynamicSmemBytes = per_sm < RESIDENT ? ALL / per_sm - 4096 : 0;
+    const cudaError_t e = ensure_smem_limit(kern, lim, (int)cfg.dynamicSmemBytes);
+    if (e != cudaSuccess) return e;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
+static void out_ptrs(OutPtrs &o, void *const *out, int kb) {
+    for (int b = 0; b < VL_MAX; ++b) o.p[b] = b < kb ? out[b] : nullptr;
 }
 
 cudaError_t launch_combine(bool vec_f64, bool part_f64, const void *part, int nparts, int n_minor, int kb,
                            void *const *out, cudaStream_t s, size_t qstride, size_t bstride) {
     if (n_minor <= 0) return cudaSuccess;
     if (kb < 1 || kb > VL_MAX) return cudaErrorInvalidValue;
-    OutPtrs o;
-    for (int b = 0; b < VL_MAX; ++b) o.p[b] = b < kb ? out[b] : nullptr;
-    if (qstride == 0) {  // [part][vector][element]
-        qstride = (size_t)kb * n_minor;
-        bstride = (size_t)n_minor;
-    }
-    const dim3 grid((n_minor + COMB_X - 1) / COMB_X, kb), block(COMB_X, COMB_Y);
-    if (vec_f64) {
-        combine_kernel<double, double><<<grid, block, 0, s>>>(static_cast<const double *>(part), nparts, n_minor,
-                                                               qstride, bstride, o);
-    } else if (part_f64) {
-        combine_kernel<float, double><<<grid, block, 0, s>>>(static_cast<const double *>(part), nparts, n_minor,
-                                                              qstride, bstride, o);
-    } else {
-        combine_kernel<float, float><<<grid, block, 0, s>>>(static_cast<const float *>(part), nparts, n_minor,
-                                                             qstride, bstride, o);
-    }
-    return cudaGetLastError();
+    FinishArgs p = {};
+    out_ptrs(p.short_out, out, kb);
+    p.part = part;
+    p.nparts = nparts;
+    p.n_minor = n_minor;
+    p.qstride = qstride ? qstride : (size_t)kb * n_minor;  // (0: [part][vector][element])
+    p.bstride = qstride ? bstride : (size_t)n_minor;
+    if (vec_f64) return launch_finish<double, double, double2>(p, kb, s);
+    if (part_f64) return launch_finish<float, double, float2>(p, kb, s);
+    return launch_finish<float, float, float2>(p, kb, s);
+}
+
+cudaError_t launch_fixup(bool vec_f64, const ZoneDev *zones, int z, const void *rec_left, const void *rec_right,
+                         int P, int kb, void *const *out, cudaStream_t s) {
+    if (z <= 0) return cudaSuccess;
+    if (kb < 1 || kb > VL_MAX) return cudaErrorInvalidValue;
+    FinishArgs p = {};
+    out_ptrs(p.long_out, out, kb);
+    p.zones = zones;
+    p.z = z;
+    p.P = P;
+    p.rec_left = rec_left;
+    p.rec_right = rec_right;
+    return vec_f64 ? launch_finish<double, double, double2>(p, kb, s) : launch_finish<float, float, float2>(p, kb, s);
+}
+
+cudaError_t launch_combine_fixup(bool f64, const void *part, int nparts, int n_minor, void *short_out, const ZoneDev *zones,
+                                 int z, const void *rec_left, const void *rec_right, int P, void *long_out,
+                                 cudaStream_t s) {
+    FinishArgs p = {};
+    p.short_out.p[0] = short_out;
+    p.long_out.p[0] = long_out;
+    p.part = part;
+    p.nparts = nparts;
+    p.n_minor = n_minor;
+    p.qstride = (size_t)n_minor;
+    p.zones = zones;
+    p.z = z;
+    p.P = P;
+    p.rec_left = rec_left;
+    p.rec_right = rec_right;
+    return f64 ? launch_finish<double, double, double2>(p, 1, s) : launch_finish<float, float, float2>(p, 1, s);
 }
 
 // out[i * KB + b] = in_b[i] for b < kb, 0 for kb <= b < KB: k vectors interleaved for the
@@ -176,37 +199,6 @@ cudaError_t launch_interleave(bool f64, int kbt, int kb, const void *const *in, 
         else if (kbt == 4) interleave_kernel<float, 4><<<grid, 256, 0, s>>>(ip, kb, len, o);
         else interleave_kernel<float, 8><<<grid, 256, 0, s>>>(ip, kb, len, o);
     }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fixup(bool vec_f64, const ZoneDev *zones, int z, const void *rec_left, const void *rec_right,
-                         int P, int kb, void *const *out, cudaStream_t s) {
-    if (z <= 0) return cudaSuccess;
-    if (kb < 1 || kb > VL_MAX) return cudaErrorInvalidValue;
-    OutPtrs o;
-    for (int b = 0; b < VL_MAX; ++b) o.p[b] = b < kb ? out[b] : nullptr;
-    const int grid = (z + 255) / 256;
-    if (vec_f64)
-        fixup_kernel<double, double2><<<grid, 256, 0, s>>>(zones, z, static_cast<const double2 *>(rec_left),
-                                                           static_cast<const double2 *>(rec_right), P, kb, o);
-    else
-        fixup_kernel<float, float2><<<grid, 256, 0, s>>>(zones, z, static_cast<const float2 *>(rec_left),
-                                                         static_cast<const float2 *>(rec_right), P, kb, o);
-    return cudaGetLastError();
-}
-
-template <typename XT>
-__global__ void __launch_bounds__(256) zero_list_kernel(const int32_t *__restrict__ list, int count, XT *__restrict__ out) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) out[list[i]] = XT(0);
-}
-
-cudaError_t launch_zero_list(bool vec_f64, const int32_t *list, int count, void *out, cudaStream_t s) {
-    if (count <= 0) return cudaSuccess;
-    const int grid = std::min((count + 255) / 256, 152 * 8);
-    if (vec_f64)
-        zero_list_kernel<double><<<grid, 256, 0, s>>>(list, count, static_cast<double *>(out));
-    else
-        zero_list_kernel<float><<<grid, 256, 0, s>>>(list, count, static_cast<float *>(out));
     return cudaGetLastError();
 }
 
