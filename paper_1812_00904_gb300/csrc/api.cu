@@ -78,9 +78,9 @@ struct PassGeometry {
 };
 // tiles of a CTA: no more warps than these can work
 int cta_tiles(const spmv_plan_s *p) { return std::max(1, (p->ntiles + p->ctas - 1) / std::max(1, p->ctas)); }
-PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd) {
+PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1) {
     PassGeometry g;
-    const size_t acc = sc ? pass_acc_bytes(p) : 0, vec = (sd ? pass_vec_bytes(p) : 0) + PASS_BAR_BYTES;
+    const size_t acc = sc ? align_up((size_t)p->n_minor * kv * p->sa, 128) : 0, vec = (sd ? pass_vec_bytes(p) : 0) + PASS_BAR_BYTES;
     const size_t slot = pass_slot_bytes(p->sv), all = (size_t)p->smem_max;
     const size_t fit = all > acc + vec ? (all - acc - vec) / slot : 0;
     g.warps = (int)std::min<size_t>(std::min(pass_warps(p->sv), cta_tiles(p)), fit);
@@ -241,10 +241,7 @@ size_t plan_footprint(const spmv_plan_s *p) {
     return b;
 }
 
-// The one-vector pass of plan p: y_short += A x (sc) into the per-CTA partials, u = the dot
-// products with v (sd), or both; then the combine and the zone fix-up in one launch.
-static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *v, void *u, cudaStream_t s) {
-    const bool sc = y != nullptr, sd = u != nullptr;
+static PassParams pass_params(const spmv_plan_s *p) {
     PassParams pp;
     std::memset(&pp, 0, sizeof(pp));
     pp.idx = p->idx;
@@ -257,17 +254,26 @@ static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *
     pp.ntiles = p->ntiles;
     pp.spt = p->T / 256;
     pp.chunk_tiles = p->chunk_tiles;
-    pp.acc_bytes = sc ? (int)pass_acc_bytes(p) : 0;
-    pp.vec_bytes = sd ? (int)pass_vec_bytes(p) : 0;
-    pp.x = x;
-    pp.v = v;
     pp.part = p->part;
-    pp.u = u;
     pp.rec_left = p->rec_left;
     pp.rec_right = p->rec_right;
     pp.emptylist = p->emptylist;
     pp.nempty = p->nempty;
+    pp.nproc = p->pz.nproc;
     pp.err = p->err;
+    return pp;
+}
+
+// The one-vector pass of plan p: y_short += A x (sc) into the per-CTA partials, u = the dot
+// products with v (sd), or both; then the combine and the zone fix-up in one launch.
+static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *v, void *u, cudaStream_t s) {
+    const bool sc = y != nullptr, sd = u != nullptr;
+    PassParams pp = pass_params(p);
+    pp.acc_bytes = sc ? (int)pass_acc_bytes(p) : 0;
+    pp.vec_bytes = sd ? (int)pass_vec_bytes(p) : 0;
+    pp.x = x;
+    pp.v = v;
+    pp.u = u;
     const PassGeometry g = pass_geometry(p, sc, sd);
     pp.slots = g.slots;
     pp.copies = g.copies;
@@ -292,6 +298,8 @@ static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *
     return SPMV_OK;
 }
 
+static spmv_status run_mvscatter(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s);
+
 spmv_status run_scatter(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s) {
     const size_t out_bytes = (size_t)p->n_minor * p->sx;
     if (p->nnz == 0 || p->n_major == 0) {
@@ -300,6 +308,7 @@ spmv_status run_scatter(spmv_plan_s *p, int kb, const void *const *in, void *con
         return SPMV_OK;
     }
     if (kb == 1 && p->pass_sc) return run_pass(p, in[0], out[0], nullptr, nullptr, s);
+    if (p->pass_mv && p->pass_sc) return run_mvscatter(p, kb, in, out, s);
     if (!p->onchip && kb > 1) {
         for (int b = 0; b < kb; ++b) {
             spmv_status st = run_scatter(p, 1, in + b, out + b, s);
@@ -340,6 +349,61 @@ static spmv_status interleave_inputs(spmv_plan_s *p, int kbt, int kb, const void
         p->vt_bytes = need;
     }
     CUDA_TRY(launch_interleave(p->vec_t == SPMV_F64, kbt, kb, in, len, p->vt, s));
+    return SPMV_OK;
+}
+
+// The accumulating product of kb = 2 .. batch_width vectors of a plan with step records (32-bit
+// accumulation), then the combine.
+static spmv_status run_mvscatter(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s) {
+    const int kv = kb_template(kb);
+    const PassGeometry g = pass_geometry(p, true, false, kv);
+    PassParams pp = pass_params(p);
+    pp.kb = kb;
+    for (int b = 0; b < kb; ++b) pp.xv[b] = in[b];
+    pp.acc_bytes = (int)align_up((size_t)p->n_minor * kv * p->sa, 128);
+    pp.slots = g.slots;
+    pp.copies = g.copies;
+    {
+        ProfScope ps(p, 0, s);
+        CUDA_TRY(p->val_t == SPMV_F32    ? launch_mvscatter_f32(kv, pp, p->ctas, g.warps, (int)g.smem, s)
+                 : p->val_t == SPMV_BF16 ? launch_mvscatter_bf16(kv, pp, p->ctas, g.warps, (int)g.smem, s)
+                                         : launch_mvscatter_f16(kv, pp, p->ctas, g.warps, (int)g.smem, s));
+    }
+    ProfScope ps(p, 1, s);
+    CUDA_TRY(launch_combine(false, false, p->part, p->ctas, p->n_minor, kb, out, s));
+    return SPMV_OK;
+}
+
+// The dot products of kb = 2 .. 8 vectors of a plan with step records (32-bit accumulation), the
+// vectors interleaved; on chip when that leaves room for all but a quarter of the warps.
+static spmv_status run_mvdot(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s) {
+    const int kv = kb <= 2 ? 2 : kb <= 4 ? 4 : 8;
+    spmv_status st = interleave_inputs(p, kv, kb, in, p->n_minor, s);
+    if (st != SPMV_OK) return st;
+    PassParams pp = pass_params(p);
+    pp.v = p->vt;
+    pp.kb = kb;
+    for (int b = 0; b < kb; ++b) pp.uv[b] = static_cast<float *>(out[b]);
+    const size_t slot = pass_slot_bytes(p->sv), vec = align_up((size_t)p->n_minor * kv * 4, 128);
+    const int most = std::min(mvdot_warps(kv), cta_tiles(p));
+    const size_t room = (size_t)p->smem_max - PASS_BAR_BYTES;
+    const size_t fit = room > vec ? (room - vec) / slot : 0;
+    const bool onchip = fit >= (size_t)(most - most / 4);
+    const int warps = onchip ? (int)std::min<size_t>(most, fit) : most;
+    pp.slots = onchip ? (int)std::min<size_t>(PASS_MAX_SLOTS, fit / warps) : PASS_MAX_SLOTS;
+    pp.vec_bytes = onchip ? (int)vec : 0;
+    const size_t smem = pp.vec_bytes + PASS_BAR_BYTES + (size_t)warps * pp.slots * slot;
+    {
+        ProfScope ps(p, 2, s);
+        CUDA_TRY(p->val_t == SPMV_F32    ? launch_mvdot_f32(kv, onchip, pp, p->ctas, warps, (int)smem, s)
+                 : p->val_t == SPMV_BF16 ? launch_mvdot_bf16(kv, onchip, pp, p->ctas, warps, (int)smem, s)
+                                         : launch_mvdot_f16(kv, onchip, pp, p->ctas, warps, (int)smem, s));
+    }
+    const spmv_plan_s::ProcZones &pz = p->pz;
+    if (pz.z > 0) {
+        ProfScope ps(p, 3, s);
+        CUDA_TRY(launch_fixup(false, pz.zones, pz.z, p->rec_left, p->rec_right, pz.nproc, kb, out, s));
+    }
     return SPMV_OK;
 }
 
@@ -399,7 +463,8 @@ static spmv_status run_segdot_impl(spmv_plan_s *p, int kb, const void *const *in
         for (int g0 = 0; g0 < kb; g0 += grp) {
             const int kg = std::min(grp, kb - g0);
             spmv_status st = kg == 1 ? run_segdot_impl(p, 1, in + g0, out + g0, s, prof, id_dot, id_fix, in_len)
-                                     : run_segdot_global(p, kg, in + g0, out + g0, s, prof, id_dot, id_fix, in_len);
+                                : p->pass_mv ? run_mvdot(p, kg, in + g0, out + g0, s)
+                                             : run_segdot_global(p, kg, in + g0, out + g0, s, prof, id_dot, id_fix, in_len);
             if (st != SPMV_OK) return st;
         }
         return SPMV_OK;
@@ -799,15 +864,23 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
         p->pass_sc = p->sv != 8 && pass_fits(p, true, false);
         p->pass_sd = pass_fits(p, false, true);
         p->pass_pair = pass_fits(p, true, true);
+        p->pass_mv = p->sv != 8;
+        // vectors per accumulating pass: as many as leave room for nearly all of the warps' staging
+        if (p->pass_mv && p->pass_sc) {
+            const int full = std::min(pass_warps(p->sv), cta_tiles(p));
+            p->batch_width = 1;
+            for (int kv : {8, 4, 2})
+                if (p->batch_width == 1 && pass_geometry(p, true, false, kv).warps >= full - full / 8) p->batch_width = kv;
+        }
     }
     const size_t part_bytes =
         (pi && pi->segdot_only) ? 16
                                 : std::max(p->onchip ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa
                                                      : (size_t)p->n_minor * sizeof(double),
-                                           p->pass_sc || p->pass_pair ? (size_t)p->ctas * p->n_minor * p->sa : (size_t)0);
+                                           p->pass_sc || p->pass_pair ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa : (size_t)0);
     // ranks of the nonempty segments, when some are empty
     int32_t *&rank = p->segrank;
-    if ((p->pass_sc || p->pass_sd || p->pass_pair) && p->nempty > 0) {
+    if ((p->pass_sc || p->pass_sd || p->pass_pair || p->pass_mv) && p->nempty > 0) {
         const int nfull = p->n_major - p->nempty, nblk = seg_rank_blocks(p->n_major);
         const size_t seg_bytes = ((size_t)p->n_major * 2 + 1 + nblk + 4) * 4;
         CUDA_TRY(cudaMalloc(&p->ws_seg, seg_bytes));
@@ -823,7 +896,7 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     const size_t o_meta = carve((size_t)(nt + 1) * sizeof(TileMeta));
     const size_t o_masks = carve((size_t)std::max(nt, 1) * p->mwp * 4);
     const size_t o_pfx = carve((size_t)std::max(nt, 1) * p->mwq * 2);
-    const bool passes = p->pass_sc || p->pass_sd || p->pass_pair;
+    const bool passes = p->pass_sc || p->pass_sd || p->pass_pair || p->pass_mv;
     const size_t o_steps = carve(passes ? (size_t)nt * (p->T / 256) * sizeof(StepRec) : 0);
     const size_t o_pz = carve((size_t)p->max_nproc * sizeof(ZoneDev));
     const size_t o_recl = carve(rec_bytes);

@@ -10,5 +10,11 @@ cudaError_t launch_pass_bf16(bool sc, bool sd, const PassParams &p, int grid, in
                             cudaStream_t s) {
     return launch_pass<__nv_bfloat16, float>(sc, sd, p, grid, warps, smem, s);
 }
+cudaError_t launch_mvdot_bf16(int kv, bool onchip, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return launch_mvdot<__nv_bfloat16>(kv, onchip, p, grid, warps, smem, s);
+}
+cudaError_t launch_mvscatter_bf16(int kv, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return launch_mvscatter<__nv_bfloat16>(kv, p, grid, warps, smem, s);
+}
 
 }  // namespace gbk

@@ -10,5 +10,11 @@ cudaError_t launch_pass_f16(bool sc, bool sd, const PassParams &p, int grid, int
                             cudaStream_t s) {
     return launch_pass<__half, float>(sc, sd, p, grid, warps, smem, s);
 }
+cudaError_t launch_mvdot_f16(int kv, bool onchip, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return launch_mvdot<__half>(kv, onchip, p, grid, warps, smem, s);
+}
+cudaError_t launch_mvscatter_f16(int kv, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return launch_mvscatter<__half>(kv, p, grid, warps, smem, s);
+}
 
 }  // namespace gbk

@@ -10,5 +10,11 @@ cudaError_t launch_pass_f32(bool sc, bool sd, const PassParams &p, int grid, int
                             cudaStream_t s) {
     return launch_pass<float, float>(sc, sd, p, grid, warps, smem, s);
 }
+cudaError_t launch_mvdot_f32(int kv, bool onchip, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return launch_mvdot<float>(kv, onchip, p, grid, warps, smem, s);
+}
+cudaError_t launch_mvscatter_f32(int kv, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return launch_mvscatter<float>(kv, p, grid, warps, smem, s);
+}
 
 }  // namespace gbk

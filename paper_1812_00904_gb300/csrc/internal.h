@@ -128,6 +128,9 @@ struct PassParams {
     void *part;              // SC: per-CTA partials [cta][n_minor]
     void *u;                 // SD: the long output
     void *rec_left, *rec_right;  // SD: carry records [proc], (hi, lo) pairs
+    float *uv[VL_MAX];       // several vectors: their outputs (SD; v then being interleaved [entry][KV]),
+    const void *xv[VL_MAX];  // their long inputs (SC)
+    int32_t kb, nproc;       // several vectors: how many; records [b * nproc + proc]
     const int32_t *emptylist;  // SD: the empty segments, whose outputs are 0
     int32_t nempty;
     int32_t *err;
@@ -139,6 +142,9 @@ __host__ __device__ constexpr int pass_slot_bytes(int val_bytes) { return 1024 +
 // Most warps of a pass: 32 of 64 registers a thread; FP64 needs more registers, and its passes do
 // not gain from more warps (57 us with 16 and with 24 on 8M nonzeros).
 constexpr int pass_warps(int val_bytes) { return val_bytes != 8 ? 32 : 16; }
+
+// Most warps of the dot products of KV vectors (128, 96 and 80 registers a thread).
+constexpr int mvdot_warps(int kv) { return kv == 8 ? 16 : kv == 4 ? 20 : 24; }
 
 // Dynamic shared-memory limit of one kernel, raised at most once per device and
 // size: the value set so far on each device, read without a lock, raised under it.
@@ -183,6 +189,13 @@ cudaError_t launch_pass_f32(bool sc, bool sd, const PassParams &p, int grid, int
 cudaError_t launch_pass_bf16(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
 cudaError_t launch_pass_f16(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
 
+// Accumulating and dot products of up to kv = 2, 4 or 8 vectors (32-bit accumulation).
+cudaError_t launch_mvscatter_f32(int kv, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_mvdot_f32(int kv, bool onchip, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_mvscatter_bf16(int kv, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_mvdot_bf16(int kv, bool onchip, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_mvscatter_f16(int kv, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_mvdot_f16(int kv, bool onchip, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
 // Small kernels (small_kernels.cu).
 // out_b[i] = sum over parts q of part[q * qstride + b * bstride + i], in FP64, in part order
 // (qstride = 0: the layout [part][vector][element]).

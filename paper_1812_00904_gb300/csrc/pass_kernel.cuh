@@ -15,81 +15,122 @@
 
 namespace gbk {
 
+// What a warp of a pass works off: the steps of its CTA's chunks, staged by bulk copies into slots of
+// the warp's own.  The CTA's tiles [ta, ta + nct) (the Sec. II rule over the grid) form nb chunks of
+// C tiles, then single-tile ones (the streaming kernel's processors, numbered from proc0).  The
+// warps take them in this order from a counter in shared memory: steps with heads cost more than
+// head-free ones, and a fixed round-robin left warps waiting at the end (14% of warp time on the
+// 50M-nonzero wide matrix).  Whichever warp runs a chunk, its sums are the same.
+// A slot receives a step's indices, values and record, one bulk copy each (the nonzeros of a partial
+// last step are read from global memory instead), and a header: step, chunk << 2 | first << 1 |
+// last; step -1: no more work.
+template <typename VT> struct StepFeed {
+    static constexpr int SLOT = pass_slot_bytes(sizeof(VT));
+    static constexpr int OFF_VAL = 1024, OFF_REC = OFF_VAL + 256 * (int)sizeof(VT), OFF_HDR = OFF_REC + (int)sizeof(StepRec);
+    const PassParams &p;
+    const int lane;
+    uint64_t *bars;
+    unsigned char *slots;
+    int *next_chunk;
+    const CtaChunks c;
+    // cursor of the copies: steps [fs, fe) of chunk fq are still to come (lane 0 alone keeps it)
+    int fs = 0, fe = 0, fq = -1, ffirst = 0;
+    int s = 0;        // slot of the warp's next step
+    uint32_t ph = 0;  // phase parity of that slot's barrier
+
+    __device__ __forceinline__ StepFeed(const PassParams &p_, unsigned char *area, int *next_chunk_)
+        : p(p_), lane(threadIdx.x & 31), next_chunk(next_chunk_),
+          c(cta_chunks(blockIdx.x, p_.ntiles, gridDim.x, p_.chunk_tiles)) {
+        const int warp = threadIdx.x >> 5;
+        bars = reinterpret_cast<uint64_t *>(area) + warp * p.slots;
+        slots = area + PASS_BAR_BYTES + warp * p.slots * SLOT;
+        if (threadIdx.x == 0) *next_chunk = 0;
+        if (lane == 0) {
+            for (int i = 0; i < p.slots; ++i) mbar_init(&bars[i], 1);
+            fence_mbar_init();
+        }
+        __syncthreads();
+        for (int i = 0; i < p.slots; ++i) issue(i);  // the first copies fly while the vectors are staged
+    }
+
+    __device__ __forceinline__ void issue(int i) {
+        if (lane != 0) return;
+        if (fs == fe) {
+            fq = atomicAdd(next_chunk, 1);
+            if (fq < c.nq) {
+                const int C = p.chunk_tiles;
+                const int t0 = fq < c.nb ? c.ta + fq * C : c.ta + c.nb * C + (fq - c.nb);
+                fs = t0 * p.spt;
+                fe = min((t0 + (fq < c.nb ? C : 1)) * p.spt, p.nnz / 256 + (p.nnz % 256 != 0));
+                ffirst = 2;
+            }
+        }
+        unsigned char *slot = slots + i * SLOT;
+        int2 hdr = make_int2(-1, 0);
+        uint32_t bytes = 0;
+        if (fs < fe) {
+            hdr = make_int2(fs, (fq << 2) | ffirst | (fs + 1 == fe ? 1 : 0));
+            bytes = sizeof(StepRec) + ((p.nnz >> 8) > fs ? 1024u + 256u * (uint32_t)sizeof(VT) : 0u);
+        }
+        *reinterpret_cast<int2 *>(slot + OFF_HDR) = hdr;
+        mbar_arrive_expect_tx(&bars[i], bytes);  // releases the header; the bulk bytes complete the phase
+        if (fs < fe) {
+            bulk_g2s(slot + OFF_REC, p.steps + fs, sizeof(StepRec), &bars[i]);
+            if ((p.nnz >> 8) > fs) {
+                bulk_g2s(slot, p.idx + (size_t)fs * 256, 1024u, &bars[i]);
+                bulk_g2s(slot + OFF_VAL, static_cast<const VT *>(p.vals) + (size_t)fs * 256,
+                         256u * (uint32_t)sizeof(VT), &bars[i]);
+            }
+            ++fs;
+            ffirst = 0;
+        }
+    }
+
+    // The next step's slot and header, or false: no more work (or a copy did not arrive in time,
+    // which is reported; the copies still in flight are let land).
+    __device__ __forceinline__ bool next(unsigned char *&slot, int2 &hdr) {
+        slot = slots + s * SLOT;
+        bool ok = mbar_wait_bounded(&bars[s], ph, WAIT_LIMIT_NS);
+        ok = __all_sync(FULL, ok);
+        if (!ok) {
+            if (lane == 0) atomicOr(p.err, ERR_WAIT);
+            for (int r = 0; r < p.slots; ++r) {
+                const int rs = s + r < p.slots ? s + r : s + r - p.slots;
+                mbar_wait_bounded(&bars[rs], s + r < p.slots ? ph : ph ^ 1u, WAIT_LIMIT_NS);
+            }
+            return false;
+        }
+        hdr = *reinterpret_cast<const int2 *>(slot + OFF_HDR);
+        return hdr.x >= 0;  // (-1: every later slot is empty as well)
+    }
+
+    // The slot is read: its next step's copies go into it.  No lane may wait for the slot before
+    // lane 0 has armed its barrier.
+    __device__ __forceinline__ void release() {
+        __syncwarp();
+        issue(s);
+        __syncwarp();
+        if (++s == p.slots) {
+            s = 0;
+            ph ^= 1u;
+        }
+    }
+};
+
 template <typename VT, typename XT, bool SC, bool SD, int WB>
 __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant__ PassParams p) {
     using AT = typename Acc<VT>::type;
     using AT2 = typename Pair<AT>::type;
-    constexpr int SLOT = pass_slot_bytes(sizeof(VT));
-    constexpr int OFF_VAL = 1024, OFF_REC = OFF_VAL + 256 * (int)sizeof(VT), OFF_HDR = OFF_REC + (int)sizeof(StepRec);
+    using Feed = StepFeed<VT>;
     extern __shared__ __align__(128) unsigned char smem[];
     // this warp's copy of the accumulator (warps share p.copies of them)
     AT *acc = reinterpret_cast<AT *>(smem + (threadIdx.x >> 5) % p.copies * p.acc_bytes);
     XT *vs = reinterpret_cast<XT *>(smem + p.copies * p.acc_bytes);
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int W = blockDim.x >> 5;
-    const int S = p.slots;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + p.copies * p.acc_bytes + p.vec_bytes) + warp * S;
-    unsigned char *slots = smem + p.copies * p.acc_bytes + p.vec_bytes + PASS_BAR_BYTES + warp * S * SLOT;
-
-    // This CTA's tiles [ta, ta + nct) by the Sec. II rule over the grid: nb chunks of C tiles, then
-    // single-tile ones (the streaming kernel's processors, numbered from proc0).  The warps take
-    // them in this order from a counter in shared memory: steps with heads cost more than
-    // head-free ones, and a fixed round-robin left warps waiting at the end (14% of warp time on
-    // the 50M-nonzero wide matrix).  Whichever warp runs a chunk, its sums are the same.
-    const int C = p.chunk_tiles;
-    const CtaChunks cc_ = cta_chunks(blockIdx.x, p.ntiles, gridDim.x, C);
-    const int ta = cc_.ta, nb = cc_.nb, nq = cc_.nq, proc0 = cc_.proc0;
-    const int nsteps = p.nnz / 256 + (p.nnz % 256 != 0);  // of the matrix
-
     // the combine and the zone fix-up may be launched: their blocks find room as this grid's CTAs end
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ int next_chunk;
-    if (threadIdx.x == 0) next_chunk = 0;
-    if (lane == 0) {
-        for (int s = 0; s < S; ++s) mbar_init(&bars[s], 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-
-    // ---- the copies of the next step into slot s: indices, values and the step's record, one bulk
-    // copy each (a partial last step's nonzeros are read from global memory instead), and a
-    // header: step, chunk << 2 | first << 1 | last; step -1: no more work.  Cursor of the copies:
-    // steps [fs, fe) of chunk fq are still to come (lane 0 alone keeps it).
-    int fs = 0, fe = 0, fq = -1, ffirst = 0;
-    auto issue = [&](int s) {
-        if (lane == 0) {
-            if (fs == fe) {
-                fq = atomicAdd(&next_chunk, 1);
-                if (fq < nq) {
-                    const int t0 = fq < nb ? ta + fq * C : ta + nb * C + (fq - nb);
-                    fs = t0 * p.spt;
-                    fe = min((t0 + (fq < nb ? C : 1)) * p.spt, nsteps);
-                    ffirst = 2;
-                }
-            }
-            unsigned char *slot = slots + s * SLOT;
-            int2 hdr = make_int2(-1, 0);
-            uint32_t bytes = 0;
-            if (fs < fe) {
-                hdr = make_int2(fs, (fq << 2) | ffirst | (fs + 1 == fe ? 1 : 0));
-                bytes = sizeof(StepRec) + ((p.nnz >> 8) > fs ? 1024u + 256u * (uint32_t)sizeof(VT) : 0u);
-            }
-            *reinterpret_cast<int2 *>(slot + OFF_HDR) = hdr;
-            mbar_arrive_expect_tx(&bars[s], bytes);  // releases the header; the bulk bytes complete the phase
-            if (fs < fe) {
-                bulk_g2s(slot + OFF_REC, p.steps + fs, sizeof(StepRec), &bars[s]);
-                if ((p.nnz >> 8) > fs) {
-                    bulk_g2s(slot, p.idx + (size_t)fs * 256, 1024u, &bars[s]);
-                    bulk_g2s(slot + OFF_VAL, static_cast<const VT *>(p.vals) + (size_t)fs * 256,
-                             256u * (uint32_t)sizeof(VT), &bars[s]);
-                }
-                ++fs;
-                ffirst = 0;
-            }
-        }
-    };
-    for (int s = 0; s < S; ++s) issue(s);  // the first copies fly while the vectors are staged
+    Feed feed(p, smem + p.copies * p.acc_bytes + p.vec_bytes, &next_chunk);
 
     // ---- the short vectors on chip: the accumulator zeroed, the input staged
     if constexpr (SC) {
@@ -116,24 +157,11 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
 
     AT chi = AT(0), clo = AT(0);  // open segment's running sum (SD)
     int cfirst = -1;              // the chunk's first segment when its sum goes to the left record
-    int s = 0;
-    uint32_t ph = 0;
-    while (true) {
-        unsigned char *slot = slots + s * SLOT;
-        bool okw = mbar_wait_bounded(&bars[s], ph, WAIT_LIMIT_NS);
-        okw = __all_sync(FULL, okw);
-        if (!okw) {  // report, let the copies in flight land, do no more work
-            if (lane == 0) atomicOr(p.err, ERR_WAIT);
-            for (int r = 0; r < S; ++r) {
-                const int rs = s + r < S ? s + r : s + r - S;
-                mbar_wait_bounded(&bars[rs], s + r < S ? ph : ph ^ 1u, WAIT_LIMIT_NS);
-            }
-            break;
-        }
-        const int2 hdr = *reinterpret_cast<const int2 *>(slot + OFF_HDR);
-        if (hdr.x < 0) break;  // every later slot is empty as well
+    unsigned char *slot;
+    int2 hdr;
+    while (feed.next(slot, hdr)) {
         const int ps = hdr.x << 8;
-        const StepRec *rec = reinterpret_cast<const StepRec *>(slot + OFF_REC);
+        const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
         const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);  // first, flags
         // the step's segments are columns (rows of a tall matrix) first, first + 1, ..; with empty
         // ones between them they are counted by rank and looked up
@@ -149,7 +177,7 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
         AT va[8];
         if (whole && !SD) {
             const int32_t *is = reinterpret_cast<const int32_t *>(slot);
-            const VT *vv = reinterpret_cast<const VT *>(slot + OFF_VAL);
+            const VT *vv = reinterpret_cast<const VT *>(slot + Feed::OFF_VAL);
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 ix[e] = is[32 * e + lane];
@@ -157,7 +185,7 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
             }
         } else if (whole) {
             stag8_idx(reinterpret_cast<const int32_t *>(slot), 8 * lane, sw, ix);
-            Stag8<VT, AT>::run(slot + OFF_VAL, 8 * lane, sw, va);
+            Stag8<VT, AT>::run(slot + Feed::OFF_VAL, 8 * lane, sw, va);
         } else {
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -179,13 +207,7 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
             w[0] = wa.x; w[1] = wa.y; w[2] = wa.z; w[3] = wa.w;
             w[4] = wb.x; w[5] = wb.y; w[6] = wb.z; w[7] = wb.w;
         }
-        __syncwarp();  // the slot is read: its next step's copies go into it
-        issue(s);
-        __syncwarp();  // no lane may wait for the slot before lane 0 has armed its barrier
-        if (++s == S) {
-            s = 0;
-            ph ^= 1u;
-        }
+        feed.release();
         const unsigned bal = SD ? __ballot_sync(FULL, hb != 0u) : static_cast<unsigned>(bf.y >> 16);  // 0: no head
         AT a[8], c[8];
         if constexpr (SC) {  // the long vector's entries
@@ -307,7 +329,7 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
                     const AT v = f + lead;
                     const int col = col_of(L);
                     if (col == cfirst)
-                        static_cast<AT2 *>(p.rec_left)[proc0 + (hdr.y >> 2)] = make_pair2(v, AT(0));
+                        static_cast<AT2 *>(p.rec_left)[feed.c.proc0 + (hdr.y >> 2)] = make_pair2(v, AT(0));
                     else
                         static_cast<XT *>(p.u)[col] = static_cast<XT>(v);
                 }
@@ -325,11 +347,11 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
                     if (ends) {
                         const AT v = chi + clo;
                         if (last == cfirst)
-                            static_cast<AT2 *>(p.rec_left)[proc0 + (hdr.y >> 2)] = make_pair2(v, AT(0));
+                            static_cast<AT2 *>(p.rec_left)[feed.c.proc0 + (hdr.y >> 2)] = make_pair2(v, AT(0));
                         else
                             static_cast<XT *>(p.u)[last] = static_cast<XT>(v);
                     } else if (bf.y & STEP_NEED_RIGHT) {
-                        static_cast<AT2 *>(p.rec_right)[proc0 + (hdr.y >> 2)] = make_pair2(chi, clo);
+                        static_cast<AT2 *>(p.rec_right)[feed.c.proc0 + (hdr.y >> 2)] = make_pair2(chi, clo);
                     }
                 }
                 chi = AT(0);
@@ -351,6 +373,342 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
                 part[i] = t;
             }
         }
+    }
+}
+
+// KV vectors' entries of index i from the interleaved copy [entry][KV], in shared or global memory.
+// On chip the 16-byte halves of an 8-vector entry are swapped in every other group of four
+// entries, so that one load instruction's halves fall into all banks (128 lanes' worth of
+// conflicts fewer: 48M -> 34M wavefronts on 50M nonzeros).
+template <int KV, bool ONCHIP> __device__ __forceinline__ void mv_gather(const float *vt, int i, float (&w)[KV]) {
+    const float *q = vt + (size_t)i * KV;
+    const int hs = ONCHIP && KV == 8 ? (i >> 2) & 1 : 0;
+    if constexpr (!ONCHIP && KV == 8) {
+        asm volatile("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(w[0]), "=f"(w[1]), "=f"(w[2]), "=f"(w[3]), "=f"(w[4]), "=f"(w[5]), "=f"(w[6]), "=f"(w[7])
+                     : "l"(q));
+    } else if constexpr (KV == 2) {
+        const float2 t = ONCHIP ? *reinterpret_cast<const float2 *>(q) : __ldg(reinterpret_cast<const float2 *>(q));
+        w[0] = t.x;
+        w[1] = t.y;
+    } else {
+#pragma unroll
+        for (int h = 0; h < KV / 4; ++h) {
+            const float4 t = ONCHIP ? reinterpret_cast<const float4 *>(q)[h ^ hs] : __ldg(reinterpret_cast<const float4 *>(q) + h);
+            w[4 * h] = t.x;
+            w[4 * h + 1] = t.y;
+            w[4 * h + 2] = t.z;
+            w[4 * h + 3] = t.w;
+        }
+    }
+}
+
+// The dot products of up to KV = 2, 4 or 8 vectors in one reading of the matrix (32-bit
+// accumulation).  A lane carries all vectors through its 8 positions: one vector load fetches a
+// nonzero's KV entries (32 bytes for 8 vectors), GP positions' loads are in flight together, and
+// the products, prefixes and scans of a vector are those of pass_kernel, so each vector's result
+// equals its single product bit for bit.  Lane b keeps vector b's carry.  With the vectors read
+// through L2 (8 of m = 20,000 are 640 KB) the gathers set the pace.
+template <typename VT, int KV, bool ONCHIP, int WB>
+__global__ void __launch_bounds__(WB * 32, 1) mvdot_kernel(const __grid_constant__ PassParams p) {
+    using Feed = StepFeed<VT>;
+    constexpr int GP = 4;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    __shared__ int next_chunk;
+    Feed feed(p, smem + p.vec_bytes, &next_chunk);
+
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x) {
+        const int col = p.emptylist[i];
+        for (int b = 0; b < p.kb; ++b) p.uv[b][col] = 0.f;
+    }
+    const float *vt = static_cast<const float *>(p.v);
+    if constexpr (ONCHIP) {
+        const int n8 = p.n_minor * KV / 2;  // in pairs of values
+#pragma unroll 4
+        for (int i = threadIdx.x; i < n8; i += blockDim.x)
+            reinterpret_cast<float2 *>(smem)[KV == 8 ? i ^ ((i >> 3) & 2) : i] = __ldg(reinterpret_cast<const float2 *>(vt) + i);
+        vt = reinterpret_cast<const float *>(smem);
+        __syncthreads();
+    }
+    const int sh = (lane & 3) << 3;
+    const int sw = (lane >> 2) & 1;
+    float chi = 0.f, clo = 0.f;  // vector `lane`'s open segment
+    int cfirst = -1;
+    unsigned char *slot;
+    int2 hdr;
+    while (feed.next(slot, hdr)) {
+        const int ps = hdr.x << 8;
+        const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
+        const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);
+        const bool gaps = (bf.y & STEP_GAPS) != 0;
+        const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
+        auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
+        const bool whole = p.nnz - ps >= 256;
+        int ix[8];
+        float va[8];
+        if (whole) {
+            stag8_idx(reinterpret_cast<const int32_t *>(slot), 8 * lane, sw, ix);
+            Stag8<VT, float>::run(slot + Feed::OFF_VAL, 8 * lane, sw, va);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {  // into the order of the positions
+                const int i0 = sw ? ix[e + 4] : ix[e];
+                const float v0 = sw ? va[e + 4] : va[e];
+                ix[e + 4] = sw ? ix[e] : ix[e + 4];
+                va[e + 4] = sw ? va[e] : va[e + 4];
+                ix[e] = i0;
+                va[e] = v0;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int pos = ps + 8 * lane + e;
+                const bool in = pos < p.nnz;
+                ix[e] = in ? __ldg(p.idx + pos) : 0;
+                va[e] = in ? to_f<VT>(static_cast<const VT *>(p.vals)[pos]) : 0.f;
+            }
+        }
+        const uint32_t mw = rec->heads[lane >> 2];
+        const uint32_t hb = (mw >> sh) & 0xFFu;
+        const int L = base + rec->before[lane >> 2] + __popc(mw & ((1u << sh) - 1u));
+        feed.release();
+        const unsigned bal = __ballot_sync(FULL, hb != 0u);
+        const int proc = feed.c.proc0 + (hdr.y >> 2);
+        if (hdr.y & 2) cfirst = (bf.y & STEP_NEED_LEFT) ? bf.x : -1;
+
+        // the lane's prefix s, restarted at every head; f: what its first head closes; segments
+        // inside the lane are closed by its later heads
+        const uint32_t h1 = hb & (0u - hb), hr = hb ^ h1;
+        float s[KV], f[KV];
+        int cc = L;
+#pragma unroll
+        for (int b = 0; b < KV; ++b) s[b] = f[b] = 0.f;
+#pragma unroll
+        for (int e0 = 0; e0 < 8; e0 += GP) {
+            float w[GP][KV];
+#pragma unroll
+            for (int g = 0; g < GP; ++g) mv_gather<KV, ONCHIP>(vt, ix[e0 + g], w[g]);
+            if (!whole) {  // past the last nonzero (zero times an infinity is no zero)
+#pragma unroll
+                for (int g = 0; g < GP; ++g)
+                    if (8 * lane + e0 + g >= p.nnz - ps) {
+#pragma unroll
+                        for (int b = 0; b < KV; ++b) w[g][b] = 0.f;
+                    }
+            }
+#pragma unroll
+            for (int g = 0; g < GP; ++g) {
+                const int e = e0 + g;
+                if (e > 0) {
+                    if ((hr >> e) & 1u) {
+                        const int col = col_of(++cc);
+#pragma unroll
+                        for (int b = 0; b < KV; ++b)
+                            if (b < p.kb) p.uv[b][col] = s[b];
+                    }
+                    if ((h1 >> e) & 1u) {
+#pragma unroll
+                        for (int b = 0; b < KV; ++b) f[b] = s[b];
+                    }
+                }
+                const bool restart = e == 0 || ((hb >> e) & 1u);
+#pragma unroll
+                for (int b = 0; b < KV; ++b) {
+                    const float q = mul_rn(va[e], w[g][b]);
+                    s[b] = restart ? q : s[b] + q;
+                }
+            }
+        }
+        if (bal == 0u) {
+            // butterfly totals, the vectors halved between the lanes as long as there are several
+            // (the same pairs are added as by a butterfly of every vector); lane b gets vector b's
+            int n = KV, d = 16;
+#pragma unroll
+            for (; n > 1; n >>= 1, d >>= 1) {
+                const bool up = (lane & d) != 0;
+#pragma unroll
+                for (int j = 0; j < KV / 2; ++j)
+                    if (j < n / 2) {
+                        const float mine = up ? s[j + n / 2] : s[j], other = up ? s[j] : s[j + n / 2];
+                        s[j] = mine + __shfl_xor_sync(FULL, other, d);
+                    }
+            }
+#pragma unroll
+            for (; d >= 1; d >>= 1) s[0] += __shfl_xor_sync(FULL, s[0], d);
+            carry_in(chi, clo, __shfl_sync(FULL, s[0], (lane * (32 / KV)) & 31));
+        } else {
+            const unsigned le = bal & (FULL >> (31 - lane));
+            const int reach = le ? lane - (31 - __clz(le)) : lane;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                if (!__any_sync(FULL, d <= reach)) break;
+#pragma unroll
+                for (int b = 0; b < KV; ++b) {
+                    const float o = __shfl_up_sync(FULL, s[b], d);
+                    if (d <= reach) s[b] += o;
+                }
+            }
+            const float carry = chi + clo;
+            const bool own = hb && L >= 0, inner = (bal & ((1u << lane) - 1u)) != 0u;
+            const int col = own ? col_of(L) : 0;
+            clo = 0.f;
+#pragma unroll
+            for (int b = 0; b < KV; ++b) {
+                float before = __shfl_up_sync(FULL, s[b], 1);
+                if (lane == 0) before = 0.f;
+                const float cb = __shfl_sync(FULL, carry, b), end = __shfl_sync(FULL, s[b], 31);
+                if (own && b < p.kb) {
+                    const float v = f[b] + (before + (inner ? 0.f : cb));
+                    if (col == cfirst)
+                        static_cast<float2 *>(p.rec_left)[(size_t)b * p.nproc + proc] = make_float2(v, 0.f);
+                    else
+                        p.uv[b][col] = v;
+                }
+                if (lane == b) chi = end;
+            }
+        }
+        const bool ends = (bf.y & STEP_ENDS) != 0, chunk_last = (hdr.y & 1) != 0;
+        if (ends || chunk_last) {
+            if (lane < p.kb) {
+                const int last = col_of(base + (bf.y >> 16));
+                if (ends) {
+                    const float v = chi + clo;
+                    if (last == cfirst)
+                        static_cast<float2 *>(p.rec_left)[(size_t)lane * p.nproc + proc] = make_float2(v, 0.f);
+                    else
+                        p.uv[lane][last] = v;
+                } else if (bf.y & STEP_NEED_RIGHT) {
+                    static_cast<float2 *>(p.rec_right)[(size_t)lane * p.nproc + proc] = make_float2(chi, clo);
+                }
+            }
+            chi = 0.f;
+            clo = 0.f;
+        }
+    }
+}
+
+// The accumulating product of up to KV = 2, 4 or 8 vectors in one reading of the matrix (32-bit
+// accumulation), the accumulators interleaved [row][KV] on chip.  KV lanes take one nonzero, a
+// vector each, four nonzeros in a row per load; 32 / KV nonzeros per addition then meet fewer
+// bank conflicts than 32 rows of one vector do, and the nonzeros are staged once.  The partials
+// go out as [cta][vector][row].
+template <typename VT, int KV, int WB>
+__global__ void __launch_bounds__(WB * 32, 1) mvscatter_kernel(const __grid_constant__ PassParams p) {
+    using Feed = StepFeed<VT>;
+    constexpr int NG = 32 / KV;  // lane groups
+    extern __shared__ __align__(128) unsigned char smem[];
+    float *acc = reinterpret_cast<float *>(smem + (threadIdx.x >> 5) % p.copies * p.acc_bytes);
+    const int lane = threadIdx.x & 31;
+    const int g = lane / KV, b = lane % KV;
+    const bool act = b < p.kb;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    __shared__ int next_chunk;
+    Feed feed(p, smem + p.copies * p.acc_bytes, &next_chunk);
+    {
+        float4 *q = reinterpret_cast<float4 *>(smem);
+        const int n16 = p.copies * p.acc_bytes >> 4;
+        for (int i = threadIdx.x; i < n16; i += blockDim.x) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    const float *xb = static_cast<const float *>(p.xv[act ? b : 0]);
+    acc += b;
+    unsigned char *slot;
+    int2 hdr;
+    while (feed.next(slot, hdr)) {
+        const int ps = hdr.x << 8;
+        const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
+        const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);
+        const bool gaps = (bf.y & STEP_GAPS) != 0;
+        const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
+        auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
+        const int left = p.nnz - ps;  // (256 or more but in a partial last step)
+        int cprev = -1;
+        float x = 0.f;
+#pragma unroll 2
+        for (int j = 0; j < 64 / NG; ++j) {
+            const int pos = 4 * (NG * j + g);
+            const uint32_t w = rec->heads[pos >> 5];
+            const uint32_t hb = w >> (pos & 31);
+            int c = base + rec->before[pos >> 5] + __popc(w & ((1u << (pos & 31)) - 1u));
+            int row[4];
+            float v[4];
+            if (left >= 256) {
+                const int4 q = *reinterpret_cast<const int4 *>(slot + 4 * pos);
+                row[0] = q.x; row[1] = q.y; row[2] = q.z; row[3] = q.w;
+                Load4<VT, float>::run(slot + Feed::OFF_VAL, pos, v);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const bool in = pos + i < left;
+                    row[i] = in ? __ldg(p.idx + ps + pos + i) : -1;
+                    v[i] = in ? to_f<VT>(static_cast<const VT *>(p.vals)[ps + pos + i]) : 0.f;
+                }
+            }
+            float xs[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                c += (hb >> i) & 1u;
+                if (c != cprev) x = __ldg(xb + col_of(c));
+                cprev = c;
+                xs[i] = x;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (act && row[i] >= 0) atomicAdd(acc + row[i] * KV, v[i] * xs[i]);
+        }
+        feed.release();
+    }
+    __syncthreads();
+    float *part = static_cast<float *>(p.part) + (size_t)blockIdx.x * p.kb * p.n_minor;
+    const float *acc0 = reinterpret_cast<const float *>(smem);
+    for (int i = threadIdx.x; i < p.n_minor * KV; i += blockDim.x) {
+        if (i % KV >= p.kb) continue;
+        float t = acc0[i];
+        for (int r = 1; r < p.copies; ++r) t += acc0[r * (p.acc_bytes / 4) + i];
+        part[(size_t)(i % KV) * p.n_minor + i / KV] = t;
+    }
+}
+
+template <typename VT>
+cudaError_t launch_mvscatter(int kv, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    if constexpr (sizeof(VT) == 8) {
+        return cudaErrorInvalidValue;
+    } else {
+        auto go = [&](auto kern, SmemLimit &lim) {
+            const cudaError_t e = ensure_smem_limit(kern, lim, smem);
+            if (e != cudaSuccess) return e;
+            kern<<<grid, warps * 32, smem, s>>>(p);
+            return cudaGetLastError();
+        };
+        static SmemLimit lim[3];
+        return kv == 2   ? go(mvscatter_kernel<VT, 2, 32>, lim[0])
+               : kv == 4 ? go(mvscatter_kernel<VT, 4, 32>, lim[1])
+                         : go(mvscatter_kernel<VT, 8, 32>, lim[2]);
+    }
+}
+
+template <typename VT, int KV, bool ONCHIP>
+cudaError_t launch_mvdot_one(const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    auto kern = mvdot_kernel<VT, KV, ONCHIP, mvdot_warps(KV)>;
+    static SmemLimit lim;
+    const cudaError_t e = ensure_smem_limit(kern, lim, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, warps * 32, smem, s>>>(p);
+    return cudaGetLastError();
+}
+template <typename VT>
+cudaError_t launch_mvdot(int kv, bool onchip, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    if constexpr (sizeof(VT) == 8) {
+        return cudaErrorInvalidValue;
+    } else {
+        if (onchip)
+            return kv == 2   ? launch_mvdot_one<VT, 2, true>(p, grid, warps, smem, s)
+                   : kv == 4 ? launch_mvdot_one<VT, 4, true>(p, grid, warps, smem, s)
+                             : launch_mvdot_one<VT, 8, true>(p, grid, warps, smem, s);
+        return kv == 2   ? launch_mvdot_one<VT, 2, false>(p, grid, warps, smem, s)
+               : kv == 4 ? launch_mvdot_one<VT, 4, false>(p, grid, warps, smem, s)
+                         : launch_mvdot_one<VT, 8, false>(p, grid, warps, smem, s);
     }
 }
 

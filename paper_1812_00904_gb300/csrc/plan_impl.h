@@ -47,6 +47,7 @@ struct spmv_plan_s {
     uint32_t *masks = nullptr;
     // one-vector passes (pass_kernel.cuh): which products they serve (the short vectors fit on chip)
     bool pass_sc = false, pass_sd = false, pass_pair = false;
+    bool pass_mv = false;  // the dot products of several vectors run in mvdot_kernel
     gbk::StepRec *steps = nullptr;
     // nonempty / empty segments and ranks among the nonempty (when some are empty)
     int32_t *seglist = nullptr, *emptylist = nullptr, *segrank = nullptr;

@@ -94,3 +94,29 @@ def test_in_a_graph_and_with_changed_values():
     xs, vs = host_of(xd), host_of(vd)
     assert_close(host_of(y), oracle.spmv(stored, xs), oracle.abs_spmv(stored, xs), 1e-5, "y")
     assert_close(host_of(u), oracle.spvtm(stored, vs), oracle.abs_spvtm(stored, vs), 1e-5, "u")
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16, torch.float16], ids=str)
+@pytest.mark.parametrize("layout", ["csc", "csr"])
+@pytest.mark.parametrize("short", [4, 300, 5_000, 9_000, 20_000, 56_000])
+def test_several_vectors(short, layout, dtype):
+    """Batches of either direction against the oracle, on and off chip; the dot products equal the
+    single ones bit for bit."""
+    rng = np.random.default_rng(short)
+    for k, nnz in ((2, 256), (3, 257), (4, 30_011), (5, 513), (8, 30_000), (11, 12_345)):
+        deg = _degrees("mixed", nnz, rng, short)
+        deg = np.concatenate([deg, np.zeros(-len(deg) % 4, dtype=np.int64)])
+        m, n = (short, len(deg)) if layout == "csc" else (len(deg), short)
+        A = synth.random_matrix(m, n, layout, degrees=deg, seed=k, duplicates=True)
+        plan, stored = make_plan(A, dtype, tile_items=256)
+        for op, ln, ref, scale in ((pkg.SPMV_OP_AX, n, oracle.spmv, oracle.abs_spmv),
+                                   (pkg.SPMV_OP_VTA, m, oracle.spvtm, oracle.abs_spvtm)):
+            Z = torch.stack([dev_vec(synth.uniform_vector(ln, 10 + b), torch.float32) for b in range(k)])
+            R = plan.batch(op, Z)
+            plan.check()
+            dots = (op == pkg.SPMV_OP_VTA) == (layout == "csc")
+            for b in range(k):
+                z = host_of(Z[b])
+                assert_close(host_of(R[b]), ref(stored, z), scale(stored, z), TOL[dtype], f"{layout} {op} k={k} vector {b}")
+                if dots:
+                    assert torch.equal(R[b], plan.spvtm(Z[b]) if op == pkg.SPMV_OP_VTA else plan.spmv(Z[b]))
