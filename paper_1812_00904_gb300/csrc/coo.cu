@@ -42,17 +42,22 @@ __global__ void coo_ptr_kernel(const int32_t *__restrict__ major, int64_t nnz, i
 }
 
 // ---- stable LSD radix sort of 64-bit keys (major * n_minor + minor) with a 32-bit payload (the
-// triple's input position), 8 bits per pass.  A tile is 4096 keys: 256 threads x 16 rounds; in
-// round j thread t holds tile element j * 256 + t, so tile order is round-major and every load is
-// coalesced.  Deterministic: every key's destination follows from the keys alone.
-constexpr int RS_THREADS = 256, RS_ROUNDS = 16, RS_TILE = RS_THREADS * RS_ROUNDS, RS_BINS = 256;
+// value itself, or the triple's input position for 8-byte values), up to RS_BITS bits per pass.  A
+// tile is 4096 keys: warp w of 16 holds tile elements 256 w .. 256 w + 255, lane l of its round j
+// element 32 j + l of them, so that every load is coalesced.  Deterministic: every key's
+// destination follows from the keys alone.
+constexpr int RS_THREADS = 512, RS_WARPS = RS_THREADS / 32, RS_ROUNDS = 8, RS_TILE = RS_THREADS * RS_ROUNDS;
+constexpr int RS_BITS = 9, RS_BINS = 1 << RS_BITS;
+static_assert(RS_BINS == RS_THREADS, "one thread per digit in the tile's scan");
 
-__device__ __forceinline__ int digit_of(uint64_t key, int shift) { return (int)((key >> shift) & 0xFFu); }
+__device__ __forceinline__ int digit_of(uint64_t key, int shift, int mask) { return (int)(key >> shift) & mask; }
 
-// err bit 1: major index outside [0, n_major); bit 4: minor index outside [0, n_minor)
-__global__ void coo_keys_kernel(const int32_t *__restrict__ major, const int32_t *__restrict__ minor, int64_t nnz,
-                                int n_major, int n_minor, uint64_t *__restrict__ keys, int32_t *__restrict__ pay,
-                                int32_t *err) {
+// err bit 1: major index outside [0, n_major); bit 4: minor index outside [0, n_minor).  vals: the
+// values of 4 or 2 bytes that become the payload, or NULL (input positions).
+template <typename W>
+__global__ void coo_keys_kernel(const int32_t *__restrict__ major, const int32_t *__restrict__ minor,
+                                const W *__restrict__ vals, int64_t nnz, int n_major, int n_minor,
+                                uint64_t *__restrict__ keys, uint32_t *__restrict__ pay, int32_t *err) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int bits = 0;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nnz; k += stride) {
@@ -62,25 +67,27 @@ __global__ void coo_keys_kernel(const int32_t *__restrict__ major, const int32_t
         if (!okj) bits |= 1;
         if (!oki) bits |= 4;
         keys[k] = (okj && oki) ? (uint64_t)j * (uint64_t)n_minor + (uint64_t)i : 0;
-        pay[k] = (int32_t)k;
+        pay[k] = vals ? (uint32_t)vals[k] : (uint32_t)k;
     }
     if (bits) atomicOr(err, bits);
 }
 
 // hist[d * ntiles + tile] = number of keys of the tile whose digit is d
 __global__ void __launch_bounds__(RS_THREADS) rs_hist_kernel(const uint64_t *__restrict__ keys, int64_t nnz,
-                                                             int shift, int ntiles, int32_t *__restrict__ hist) {
+                                                             int shift, int mask, int ntiles,
+                                                             int32_t *__restrict__ hist) {
     __shared__ int h[RS_BINS];
     const int t = threadIdx.x;
     h[t] = 0;
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * RS_TILE;
+#pragma unroll
     for (int j = 0; j < RS_ROUNDS; ++j) {
         const int64_t k = base + (int64_t)j * RS_THREADS + t;
-        if (k < nnz) atomicAdd(&h[digit_of(keys[k], shift)], 1);
+        if (k < nnz) atomicAdd(&h[digit_of(keys[k], shift, mask)], 1);
     }
     __syncthreads();
-    hist[(int64_t)t * ntiles + blockIdx.x] = h[t];
+    if (t <= mask) hist[(int64_t)t * ntiles + blockIdx.x] = h[t];
 }
 
 // exclusive scan of n int32 values in place: per-block sums, one-block scan of the sums, block scans
@@ -154,59 +161,92 @@ __global__ void __launch_bounds__(SC_THREADS) scan_apply_kernel(int32_t *__restr
     }
 }
 
-// stable scatter: a key goes to offs[d * ntiles + tile] + (keys of digit d before it in the tile)
+// Stable scatter of a tile: every warp ranks its keys among its own of the same digit
+// (__match_any_sync, counters per warp), a scan over warps and digits gives their order in the
+// tile, and the keys go through shared memory in that order, so that the keys of a digit (8 on
+// average, 64 bytes) are written side by side to offs[d * ntiles + tile] and on.  Bound by the
+// 24 bytes a key moves; without the reordering the single 8- and 4-byte writes took 162 us a pass
+// of 10M keys.
+constexpr size_t RS_SMEM = RS_TILE * 12 + RS_WARPS * RS_BINS * 2 + RS_BINS * 8;
 __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const uint64_t *__restrict__ kin,
-                                                                const int32_t *__restrict__ pin, int64_t nnz, int shift,
-                                                                int ntiles, const int32_t *__restrict__ offs,
-                                                                uint64_t *__restrict__ kout, int32_t *__restrict__ pout,
+                                                                const uint32_t *__restrict__ pin, int64_t nnz, int shift,
+                                                                int mask, int ntiles, const int32_t *__restrict__ offs,
+                                                                uint64_t *__restrict__ kout, uint32_t *__restrict__ pout,
                                                                 int32_t *err) {
-    constexpr int NW = RS_THREADS / 32;
-    __shared__ int run[RS_BINS];        // keys of each digit placed so far in this tile
-    __shared__ int wcnt[NW][RS_BINS];   // this round: keys of each digit in each warp
+    extern __shared__ __align__(16) unsigned char sm[];
+    uint64_t *skey = reinterpret_cast<uint64_t *>(sm);
+    uint32_t *spay = reinterpret_cast<uint32_t *>(sm + RS_TILE * 8);
+    uint16_t *wcnt = reinterpret_cast<uint16_t *>(sm + RS_TILE * 12);  // [warp][digit]
+    int32_t *lstart = reinterpret_cast<int32_t *>(sm + RS_TILE * 12 + RS_WARPS * RS_BINS * 2);  // in the tile
+    int32_t *gdelta = lstart + RS_BINS;  // place in the output less place in the tile
+    __shared__ int wt[32];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    run[t] = offs[(int64_t)t * ntiles + blockIdx.x];
-    for (int q = 0; q < NW; ++q) wcnt[q][t] = 0;
-    __syncthreads();
+    for (int q = t; q < RS_WARPS * RS_BINS / 2; q += RS_THREADS) reinterpret_cast<uint32_t *>(wcnt)[q] = 0u;
     const int64_t base = (int64_t)blockIdx.x * RS_TILE;
+    const int n = nnz - base < RS_TILE ? (int)(nnz - base) : RS_TILE;
+    uint64_t key[RS_ROUNDS];
+    uint32_t pl[RS_ROUNDS];
+    uint16_t rank[RS_ROUNDS];
+#pragma unroll
     for (int j = 0; j < RS_ROUNDS; ++j) {
-        const int64_t k = base + (int64_t)j * RS_THREADS + t;
-        const bool live = k < nnz;
-        uint64_t key = 0;
-        int32_t pl = 0;
-        int d = -1;
-        if (live) {
-            key = kin[k];
-            pl = pin[k];
-            d = digit_of(key, shift);
+        const int i = w * (32 * RS_ROUNDS) + 32 * j + lane;
+        key[j] = i < n ? kin[base + i] : 0;
+        pl[j] = i < n ? pin[base + i] : 0;
+    }
+    __syncthreads();
+    uint16_t *mine = wcnt + w * RS_BINS;
+#pragma unroll
+    for (int j = 0; j < RS_ROUNDS; ++j) {
+        const bool live = w * (32 * RS_ROUNDS) + 32 * j + lane < n;
+        const int d = digit_of(key[j], shift, mask);
+        const unsigned peers = __match_any_sync(0xffffffffu, live ? d : -1);
+        const int before = __popc(peers & ((1u << lane) - 1u));
+        rank[j] = live ? (uint16_t)(mine[d] + before) : (uint16_t)0;
+        __syncwarp();
+        if (live && before == 0) mine[d] = (uint16_t)(mine[d] + __popc(peers));
+        __syncwarp();
+    }
+    __syncthreads();
+    {  // thread t: digit t
+        int c = 0;
+#pragma unroll
+        for (int q = 0; q < RS_WARPS; ++q) {
+            const int v = wcnt[q * RS_BINS + t];
+            wcnt[q * RS_BINS + t] = (uint16_t)c;
+            c += v;
         }
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const int before_in_warp = __popc(peers & ((1u << lane) - 1u));
-        if (live && before_in_warp == 0) wcnt[w][d] = __popc(peers);
-        __syncthreads();
-        if (live) {
-            int pos = run[d] + before_in_warp;
-            for (int q = 0; q < w; ++q) pos += wcnt[q][d];
-            if (pos >= 0 && pos < nnz) {
-                kout[pos] = key;
-                pout[pos] = pl;
-            } else {
-                atomicOr(err, 8);
-            }
+        int total;
+        const int ls = block_exclusive_scan(c, wt, total);
+        lstart[t] = ls;
+        gdelta[t] = t <= mask ? offs[(int64_t)t * ntiles + blockIdx.x] - ls : 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < RS_ROUNDS; ++j) {
+        if (w * (32 * RS_ROUNDS) + 32 * j + lane < n) {
+            const int d = digit_of(key[j], shift, mask);
+            const int pos = lstart[d] + mine[d] + rank[j];  // (< n: a permutation of the tile)
+            skey[pos] = key[j];
+            spay[pos] = pl[j];
         }
-        __syncthreads();
-        int add = 0;
-        for (int q = 0; q < NW; ++q) {
-            add += wcnt[q][t];
-            wcnt[q][t] = 0;
+    }
+    __syncthreads();
+    for (int i = t; i < n; i += RS_THREADS) {
+        const uint64_t k = skey[i];
+        const int64_t pos = (int64_t)gdelta[digit_of(k, shift, mask)] + i;
+        if (pos >= 0 && pos < nnz) {
+            kout[pos] = k;
+            pout[pos] = spay[i];
+        } else {
+            atomicOr(err, 8);
         }
-        run[t] += add;
-        __syncthreads();
     }
 }
 
-// sorted keys -> major (for the pointer array), minor indices and the values gathered by payload
+// sorted keys -> major (for the pointer array) and minor indices; the values from the payload, or
+// gathered by it (8-byte values: vals not NULL)
 template <typename W>
-__global__ void coo_unpack_kernel(const uint64_t *__restrict__ keys, const int32_t *__restrict__ pay, int64_t nnz,
+__global__ void coo_unpack_kernel(const uint64_t *__restrict__ keys, const uint32_t *__restrict__ pay, int64_t nnz,
                                   int n_minor, const W *__restrict__ vals, int32_t *__restrict__ major,
                                   int32_t *__restrict__ minor, W *__restrict__ ovals, int32_t *err) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -215,8 +255,10 @@ __global__ void coo_unpack_kernel(const uint64_t *__restrict__ keys, const int32
         const uint64_t j = key / (uint64_t)n_minor;
         major[k] = (int32_t)j;
         minor[k] = (int32_t)(key - j * (uint64_t)n_minor);
-        const int32_t src = pay[k];
-        if (src >= 0 && src < nnz) {
+        const uint32_t src = pay[k];
+        if (!vals) {
+            ovals[k] = (W)src;
+        } else if (src < nnz) {
             ovals[k] = vals[src];
         } else {
             ovals[k] = W(0);
@@ -252,37 +294,48 @@ spmv_status coo_sort(CooSort &cs, const int32_t *major, const int32_t *minor, co
     if (cudaMalloc(&cs.tmp, 2 * kb + 2 * pb + hb + sb) != cudaSuccess) return set_error(SPMV_ERR_OOM, "sort scratch");
     char *t = static_cast<char *>(cs.tmp);
     uint64_t *ka = reinterpret_cast<uint64_t *>(t), *kb2 = reinterpret_cast<uint64_t *>(t + kb);
-    int32_t *pa = reinterpret_cast<int32_t *>(t + 2 * kb), *pb2 = reinterpret_cast<int32_t *>(t + 2 * kb + pb);
+    uint32_t *pa = reinterpret_cast<uint32_t *>(t + 2 * kb), *pb2 = reinterpret_cast<uint32_t *>(t + 2 * kb + pb);
     int32_t *hist = reinterpret_cast<int32_t *>(t + 2 * kb + 2 * pb);
     int32_t *sums = reinterpret_cast<int32_t *>(t + 2 * kb + 2 * pb + hb);
     const size_t ib = up((size_t)nnz * 4);
     cs.own_bytes = ib + up((size_t)nnz * sv);
     if (cudaMalloc(&cs.own, cs.own_bytes) != cudaSuccess) return set_error(SPMV_ERR_OOM, "sorted triples");
 
-    coo_keys_kernel<<<grid, 256, 0, s>>>(major, minor, nnz, n_major, n_minor, ka, pa, err);
+    if (sv == 2)
+        coo_keys_kernel<uint16_t><<<grid, 256, 0, s>>>(major, minor, static_cast<const uint16_t *>(vals), nnz, n_major, n_minor, ka, pa, err);
+    else
+        coo_keys_kernel<uint32_t><<<grid, 256, 0, s>>>(major, minor, sv == 4 ? static_cast<const uint32_t *>(vals) : nullptr, nnz,
+                                                       n_major, n_minor, ka, pa, err);
     const uint64_t span = (uint64_t)n_major * (uint64_t)n_minor;
     const int bits = span > 1 ? 64 - __builtin_clzll(span - 1) : 0;
-    for (int shift = 0; shift < bits; shift += 8) {
-        rs_hist_kernel<<<ntiles, RS_THREADS, 0, s>>>(ka, nnz, shift, ntiles, hist);
-        scan_sums_kernel<<<nsc, SC_THREADS, 0, s>>>(hist, nh, sums);
-        scan_top_kernel<<<1, SC_THREADS, 0, s>>>(sums, nsc);
-        scan_apply_kernel<<<nsc, SC_THREADS, 0, s>>>(hist, nh, sums);
-        rs_scatter_kernel<<<ntiles, RS_THREADS, 0, s>>>(ka, pa, nnz, shift, ntiles, hist, kb2, pb2, err);
+    const int passes = (bits + RS_BITS - 1) / RS_BITS;
+    static SmemLimit lim;
+    if (ensure_smem_limit(rs_scatter_kernel, lim, (int)RS_SMEM) != cudaSuccess) return set_error(SPMV_ERR_CUDA, "sort launch failed");
+    for (int q = 0, shift = 0; q < passes; ++q) {  // passes of equal width, give or take a bit
+        const int width = (bits - shift + passes - q - 1) / (passes - q), mask = (1 << width) - 1;
+        const int64_t nhq = (int64_t)(mask + 1) * ntiles;
+        const int nscq = (int)((nhq + SC_CHUNK - 1) / SC_CHUNK);
+        rs_hist_kernel<<<ntiles, RS_THREADS, 0, s>>>(ka, nnz, shift, mask, ntiles, hist);
+        scan_sums_kernel<<<nscq, SC_THREADS, 0, s>>>(hist, nhq, sums);
+        scan_top_kernel<<<1, SC_THREADS, 0, s>>>(sums, nscq);
+        scan_apply_kernel<<<nscq, SC_THREADS, 0, s>>>(hist, nhq, sums);
+        rs_scatter_kernel<<<ntiles, RS_THREADS, RS_SMEM, s>>>(ka, pa, nnz, shift, mask, ntiles, hist, kb2, pb2, err);
         std::swap(ka, kb2);
         std::swap(pa, pb2);
+        shift += width;
     }
     int32_t *omin = static_cast<int32_t *>(cs.own);
     void *ovals = static_cast<char *>(cs.own) + ib;
-    int32_t *omaj = pb2;  // the free payload buffer
+    int32_t *omaj = reinterpret_cast<int32_t *>(pb2);  // the free payload buffer
     if (sv == 8)
         coo_unpack_kernel<uint64_t><<<grid, 256, 0, s>>>(ka, pa, nnz, n_minor, static_cast<const uint64_t *>(vals), omaj,
                                                          omin, static_cast<uint64_t *>(ovals), err);
     else if (sv == 4)
-        coo_unpack_kernel<uint32_t><<<grid, 256, 0, s>>>(ka, pa, nnz, n_minor, static_cast<const uint32_t *>(vals), omaj,
-                                                         omin, static_cast<uint32_t *>(ovals), err);
+        coo_unpack_kernel<uint32_t><<<grid, 256, 0, s>>>(ka, pa, nnz, n_minor, nullptr, omaj, omin,
+                                                         static_cast<uint32_t *>(ovals), err);
     else
-        coo_unpack_kernel<uint16_t><<<grid, 256, 0, s>>>(ka, pa, nnz, n_minor, static_cast<const uint16_t *>(vals), omaj,
-                                                         omin, static_cast<uint16_t *>(ovals), err);
+        coo_unpack_kernel<uint16_t><<<grid, 256, 0, s>>>(ka, pa, nnz, n_minor, nullptr, omaj, omin,
+                                                         static_cast<uint16_t *>(ovals), err);
     if (cudaGetLastError() != cudaSuccess) return set_error(SPMV_ERR_CUDA, "sort launch failed");
     *major_sorted = omaj;
     *minor_sorted = omin;

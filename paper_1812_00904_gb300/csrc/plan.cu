@@ -132,7 +132,7 @@ __device__ __forceinline__ SegPair seg_op(SegPair a, SegPair b) {
     return r;
 }
 
-constexpr int SU_THREADS = 256, SU_IPT = 8, SU_ITEMS = SU_THREADS * SU_IPT;
+constexpr int SU_THREADS = 256, SU_IPT = 2, SU_ITEMS = SU_THREADS * SU_IPT;
 
 struct AddOp {
     __device__ __forceinline__ int operator()(int a, int b) const { return a + b; }
