@@ -574,15 +574,15 @@ void plan_free(spmv_plan_s *p) {
     plan_free(p->tplan);
     if (p->vt) cudaFree(p->vt);
     if (p->ypart_k) cudaFree(p->ypart_k);
-    if (p->bws) cudaFree(p->bws);
-    if (p->bown) cudaFree(p->bown);
+    dev_free(p->bws, p->device);
+    dev_free(p->bown, p->device);
     for (auto &pr : p->prof) {
         cudaEventDestroy(pr.a);
         cudaEventDestroy(pr.b);
     }
-    if (p->ws) cudaFree(p->ws);
-    if (p->ws2) cudaFree(p->ws2);
-    if (p->ws_seg) cudaFree(p->ws_seg);
+    dev_free(p->ws, p->device);
+    dev_free(p->ws2, p->device);
+    dev_free(p->ws_seg, p->device);
     if (p->hin) cudaFree(p->hin);
     if (p->hout) cudaFree(p->hout);
     if (p->hv) cudaFree(p->hv);
@@ -592,8 +592,8 @@ void plan_free(spmv_plan_s *p) {
     if (p->cstream) cudaStreamDestroy(p->cstream);
     if (p->hg) cudaFree(p->hg);
     if (p->ynorm) cudaFree(p->ynorm);
-    if (p->owned_ptr) cudaFree(p->owned_ptr);
-    if (p->owned_nz) cudaFree(p->owned_nz);
+    dev_free(p->owned_ptr, p->device);
+    dev_free(p->owned_nz, p->device);
     delete p;
 }
 
@@ -601,9 +601,12 @@ void plan_free(spmv_plan_s *p) {
 
 namespace {
 
-struct PlanGuard {
+struct PlanGuard {  // a plan whose creation failed: its set-up may still be running
     spmv_plan_s *p;
-    ~PlanGuard() { plan_free(p); }
+    ~PlanGuard() {
+        if (p) cudaDeviceSynchronize();
+        plan_free(p);
+    }
 };
 
 // Runs `fn` on device pointers, staging host pointers through plan buffers.
@@ -784,7 +787,7 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     const size_t o_sscr = carve(setup_scratch_bytes(p->P));
     const size_t o_err = carve(16);
     const size_t ws1 = off;
-    CUDA_TRY(cudaMalloc(&p->ws, ws1));
+    CUDA_TRY(dev_alloc(&p->ws, ws1));
     char *w1 = static_cast<char *>(p->ws);
     p->pptr = reinterpret_cast<int32_t *>(w1 + o_pptr);
     p->aux = reinterpret_cast<ChunkAux *>(w1 + o_aux);
@@ -817,16 +820,18 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     if ((flags & SPMV_PLAN_BANK_ORDER) && nnz > 0) {
         const size_t ib = align_up((size_t)nnz * 4, 256);
         const size_t vb = align_up((size_t)nnz * p->sv, 256);
-        CUDA_TRY(cudaMalloc(&p->owned_nz, ib + vb));
+        CUDA_TRY(dev_alloc(&p->owned_nz, ib + vb));
         p->owned_bytes = ib + vb;
-        int32_t *slots = nullptr;
-        CUDA_TRY(cudaMalloc(&slots, (size_t)nnz * 4));
+        void *slots_mem = nullptr;
+        CUDA_TRY(dev_alloc(&slots_mem, (size_t)nnz * 4));
+        int32_t *slots = static_cast<int32_t *>(slots_mem);
         int32_t *oidx = static_cast<int32_t *>(p->owned_nz);
         void *ovals = static_cast<char *>(p->owned_nz) + ib;
         cudaError_t ce = launch_bank_order(ptr, p->n_major, (int)nnz, idx, vals, p->sv, oidx, ovals, slots, p->T,
                                            p->sx == 8 ? 16 : 32, s);
-        if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-        cudaFree(slots);
+        const cudaError_t cs = cudaStreamSynchronize(s);
+        if (ce == cudaSuccess) ce = cs;
+        dev_free(slots_mem, p->device);
         if (ce != cudaSuccess) return set_error(SPMV_ERR_CUDA, std::string("bank order: ") + cudaGetErrorString(ce));
         p->idx = oidx;
         p->vals = ovals;
@@ -883,7 +888,7 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     if ((p->pass_sc || p->pass_sd || p->pass_pair || p->pass_mv) && p->nempty > 0) {
         const int nfull = p->n_major - p->nempty, nblk = seg_rank_blocks(p->n_major);
         const size_t seg_bytes = ((size_t)p->n_major * 2 + 1 + nblk + 4) * 4;
-        CUDA_TRY(cudaMalloc(&p->ws_seg, seg_bytes));
+        CUDA_TRY(dev_alloc(&p->ws_seg, seg_bytes));
         p->seglist = static_cast<int32_t *>(p->ws_seg);
         p->emptylist = p->seglist + nfull;
         rank = p->emptylist + p->nempty;
@@ -910,7 +915,7 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     const size_t o_pdev = carve((size_t)p->max_nproc * sizeof(ChunkDev));
     const size_t o_pscr = carve(setup_scratch_bytes(p->max_nproc));
     const size_t ws2 = off;
-    CUDA_TRY(cudaMalloc(&p->ws2, ws2));
+    CUDA_TRY(dev_alloc(&p->ws2, ws2));
     p->ws_bytes += ws1 + ws2;
     char *w2 = static_cast<char *>(p->ws2);
     p->meta = reinterpret_cast<TileMeta *>(w2 + o_meta);

@@ -138,14 +138,17 @@ spmv_status build_row_blocks(spmv_plan_s *p, int sms, cudaStream_t s) {
         const int64_t max_elems = (int64_t)(budget / p->sx);
         if (max_elems < 64) continue;
         int32_t *d_max = nullptr;
-        if (cudaMalloc(&d_max, BLOCK_CANDIDATES * 4) != cudaSuccess) return set_error(SPMV_ERR_OOM, "row blocks");
+        void *mem = nullptr;
+        if (dev_alloc(&mem, BLOCK_CANDIDATES * 4) != cudaSuccess) return set_error(SPMV_ERR_OOM, "row blocks");
+        d_max = static_cast<int32_t *>(mem);
         std::vector<int32_t> mx(BLOCK_CANDIDATES, 0);
         cudaMemsetAsync(d_max, 0, BLOCK_CANDIDATES * 4, s);
         block_span_kernel<<<std::max(1, sms * 4), 256, 0, s>>>(p->pptr, p->n_major, p->nnz, nt, Tc, sms,
                                                                BLOCK_CANDIDATES, xa, d_max);
         cudaError_t ce = cudaMemcpyAsync(mx.data(), d_max, BLOCK_CANDIDATES * 4, cudaMemcpyDeviceToHost, s);
-        if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-        cudaFree(d_max);
+        const cudaError_t cs = cudaStreamSynchronize(s);
+        if (ce == cudaSuccess) ce = cs;
+        dev_free(mem, p->device);
         if (ce != cudaSuccess) return set_error(SPMV_ERR_CUDA, std::string("row blocks: ") + cudaGetErrorString(ce));
         for (int c = 0; c < BLOCK_CANDIDATES; ++c) {
             const int Gc = (c + 1) * sms;
@@ -169,20 +172,25 @@ spmv_status build_row_blocks(spmv_plan_s *p, int sms, cudaStream_t s) {
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t o_win = 0, o_bptr = up((size_t)G * 8), o_ypart = o_bptr + up((nseg + 1) * 4);
     const size_t bws_bytes = o_ypart + up(nseg * p->sx);
-    if (cudaMalloc(&p->bws, bws_bytes) != cudaSuccess) return set_error(SPMV_ERR_OOM, "row blocks");
+    if (dev_alloc(&p->bws, bws_bytes) != cudaSuccess) return set_error(SPMV_ERR_OOM, "row blocks");
     p->bws_bytes = bws_bytes;
     int2 *win = reinterpret_cast<int2 *>(static_cast<char *>(p->bws) + o_win);
     int32_t *bptr = reinterpret_cast<int32_t *>(static_cast<char *>(p->bws) + o_bptr);
     p->ypart = static_cast<char *>(p->bws) + o_ypart;
-    int32_t *keys = nullptr;  // bmaj then bmin, nnz each
-    if (cudaMalloc(&keys, (size_t)p->nnz * 8) != cudaSuccess) return set_error(SPMV_ERR_OOM, "row blocks");
+    void *keys_mem = nullptr;  // bmaj then bmin, nnz each
+    if (dev_alloc(&keys_mem, (size_t)p->nnz * 8) != cudaSuccess) return set_error(SPMV_ERR_OOM, "row blocks");
+    int32_t *keys = static_cast<int32_t *>(keys_mem);
+    auto free_keys = [&] {
+        cudaStreamSynchronize(s);
+        dev_free(keys_mem, p->device);
+    };
     int32_t *bmaj = keys, *bmin = keys + p->nnz;
     block_window_kernel<<<(G + 255) / 256, 256, 0, s>>>(p->pptr, p->n_major, p->nnz, nt, T, G, xa, win);
     block_keys_kernel<<<std::max(1, sms * 16), 256, 0, s>>>(p->pptr, p->idx, p->n_major, n_minor, nt, T, G, win, bmaj,
                                                             bmin);
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) {
-        cudaFree(keys);
+        free_keys();
         return set_error(SPMV_ERR_CUDA, std::string("row blocks: ") + cudaGetErrorString(ce));
     }
     CooSort cs;
@@ -196,7 +204,7 @@ spmv_status build_row_blocks(spmv_plan_s *p, int sms, cudaStream_t s) {
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
         if (ce != cudaSuccess) st = set_error(SPMV_ERR_CUDA, std::string("row blocks: ") + cudaGetErrorString(ce));
     }
-    cudaFree(keys);
+    free_keys();
     if (st != SPMV_OK) return st;
     int32_t e = 0;
     cudaMemcpy(&e, p->err, 4, cudaMemcpyDeviceToHost);

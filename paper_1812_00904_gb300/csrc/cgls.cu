@@ -179,12 +179,13 @@ spmv_status cgls_typed(spmv_plan_s *p, const void *b, void *x, int max_iters, do
     CG_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
     c.grid = std::max(1, sms * 4);
     const size_t m = (size_t)std::max<int64_t>(p->m, 1), n = (size_t)std::max<int64_t>(p->n, 1);
-    char *mem = nullptr;
+    void *block = nullptr;
     const size_t off_s = cg_align(m * sizeof(T), 256), off_p = off_s + cg_align(n * sizeof(T), 256);
     const size_t off_q = off_p + cg_align(n * sizeof(T), 256), off_part = off_q + cg_align(m * sizeof(T), 256);
     const size_t off_sc = off_part + cg_align(DOT_BLOCKS * sizeof(double), 256);
     const size_t total = off_sc + sizeof(CgScalars);
-    CG_TRY(cudaMalloc(&mem, total));
+    CG_TRY(dev_alloc(&block, total));
+    char *mem = static_cast<char *>(block);
     c.r = reinterpret_cast<T *>(mem);
     c.sv = reinterpret_cast<T *>(mem + off_s);
     c.pv = reinterpret_cast<T *>(mem + off_p);
@@ -196,7 +197,7 @@ spmv_status cgls_typed(spmv_plan_s *p, const void *b, void *x, int max_iters, do
                                                rel)
                                       : set_error(SPMV_ERR_CUDA, cudaGetErrorString(e));
     cudaStreamSynchronize(s);
-    cudaFree(mem);
+    dev_free(block, p->device);
     return st;
 }
 

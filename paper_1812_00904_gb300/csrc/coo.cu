@@ -270,8 +270,10 @@ __global__ void coo_unpack_kernel(const uint64_t *__restrict__ keys, const uint3
 }  // namespace
 
 CooSort::~CooSort() {
-    if (tmp) cudaFree(tmp);
-    if (own) cudaFree(own);
+    if (!tmp && !own) return;
+    cudaStreamSynchronize(s);
+    dev_free(tmp, device);
+    dev_free(own, device);
 }
 
 cudaError_t launch_coo_ptr(const int32_t *major_sorted, int64_t nnz, int n_major, int32_t *ptr, int grid,
@@ -291,7 +293,9 @@ spmv_status coo_sort(CooSort &cs, const int32_t *major, const int32_t *minor, co
     const int64_t nh = (int64_t)RS_BINS * ntiles;
     const int nsc = (int)((nh + SC_CHUNK - 1) / SC_CHUNK);
     const size_t kb = up((size_t)nnz * 8), pb = up((size_t)nnz * 4), hb = up((size_t)nh * 4), sb = up((size_t)nsc * 4);
-    if (cudaMalloc(&cs.tmp, 2 * kb + 2 * pb + hb + sb) != cudaSuccess) return set_error(SPMV_ERR_OOM, "sort scratch");
+    cs.s = s;
+    if (cudaGetDevice(&cs.device) != cudaSuccess) return set_error(SPMV_ERR_CUDA, "no current device");
+    if (dev_alloc(&cs.tmp, 2 * kb + 2 * pb + hb + sb) != cudaSuccess) return set_error(SPMV_ERR_OOM, "sort scratch");
     char *t = static_cast<char *>(cs.tmp);
     uint64_t *ka = reinterpret_cast<uint64_t *>(t), *kb2 = reinterpret_cast<uint64_t *>(t + kb);
     uint32_t *pa = reinterpret_cast<uint32_t *>(t + 2 * kb), *pb2 = reinterpret_cast<uint32_t *>(t + 2 * kb + pb);
@@ -299,7 +303,7 @@ spmv_status coo_sort(CooSort &cs, const int32_t *major, const int32_t *minor, co
     int32_t *sums = reinterpret_cast<int32_t *>(t + 2 * kb + 2 * pb + hb);
     const size_t ib = up((size_t)nnz * 4);
     cs.own_bytes = ib + up((size_t)nnz * sv);
-    if (cudaMalloc(&cs.own, cs.own_bytes) != cudaSuccess) return set_error(SPMV_ERR_OOM, "sorted triples");
+    if (dev_alloc(&cs.own, cs.own_bytes) != cudaSuccess) return set_error(SPMV_ERR_OOM, "sorted triples");
 
     if (sv == 2)
         coo_keys_kernel<uint16_t><<<grid, 256, 0, s>>>(major, minor, static_cast<const uint16_t *>(vals), nnz, n_major, n_minor, ka, pa, err);
@@ -376,10 +380,16 @@ extern "C" spmv_status spmv_plan_coo(spmv_plan_t *out, int64_t m, int64_t n, int
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int32_t *ptr = nullptr, *err = nullptr;
-    if (cudaMalloc(&ptr, ((size_t)n_major + 1) * 4 + 16) != cudaSuccess) return set_error(SPMV_ERR_OOM, "pointer array");
+    void *ptr_mem = nullptr;
+    if (dev_alloc(&ptr_mem, ((size_t)n_major + 1) * 4 + 16) != cudaSuccess) return set_error(SPMV_ERR_OOM, "pointer array");
+    ptr = static_cast<int32_t *>(ptr_mem);
+    auto free_ptr = [&] {
+        cudaStreamSynchronize(s);
+        dev_free(ptr_mem, dev);
+    };
     err = reinterpret_cast<int32_t *>(reinterpret_cast<char *>(ptr) + (((size_t)n_major + 1) * 4 + 3) / 4 * 4);
     auto fail = [&](spmv_status st, const char *msg) {
-        cudaFree(ptr);
+        free_ptr();
         return set_error(st, msg);
     };
     if (cudaMemsetAsync(err, 0, 4, s) != cudaSuccess) return fail(SPMV_ERR_CUDA, "memset");
@@ -393,7 +403,7 @@ extern "C" spmv_status spmv_plan_coo(spmv_plan_t *out, int64_t m, int64_t n, int
         const spmv_status st = coo_sort(cs, major, minor, vals, dsize(val_dtype), nnz, n_major, n_minor, grid, err, s,
                                         &maj_use, &omin, &ovals);
         if (st != SPMV_OK) {
-            cudaFree(ptr);
+            free_ptr();
             return st;
         }
         min_use = omin;
@@ -413,7 +423,7 @@ extern "C" spmv_status spmv_plan_coo(spmv_plan_t *out, int64_t m, int64_t n, int
     spmv_status st = spmv_plan_ex(out, m, n, nnz, layout, ptr, min_use, vals_use, val_dtype, vec_dtype, stream,
                                   flags, opts);
     if (st != SPMV_OK) {
-        cudaFree(ptr);
+        free_ptr();
         return st;
     }
     (*out)->owned_ptr = ptr;  // freed with the plan

@@ -1,0 +1,84 @@
+// Device memory of plans and of calls that need scratch: a private memory pool per device.
+//
+// cudaMalloc and cudaFree take about 100 us each on this machine (a plan makes eight, a CGLS call
+// two: 0.8 of the 2.4 ms of ingesting 10M triples, 0.2 of the 1.0 ms of a short CGLS run).  The
+// pool keeps up to POOL_KEEP bytes of freed memory for the next plan and gives everything beyond
+// back to the device at its next synchronisation; when an allocation fails it gives all of it back
+// and tries again.  The allocations and frees go through a stream of the pool's own: memory is
+// handed out after that stream was waited for, so it can be used on any stream, and the caller
+// frees memory only when no work that uses it is pending.  Every call is safe from any thread.
+#include <cuda_runtime.h>
+
+#include <mutex>
+
+#include "plan_impl.h"
+
+namespace gbk {
+namespace {
+
+constexpr uint64_t POOL_KEEP = 512ull << 20;
+
+struct DevicePool {
+    std::once_flag once;
+    cudaMemPool_t pool = nullptr;  // NULL: no pool could be made, plain allocations
+    cudaStream_t stream = nullptr;
+};
+DevicePool g_pools[MAX_DEVICES];
+
+DevicePool &pool_of(int device) {
+    DevicePool &P = g_pools[device];
+    std::call_once(P.once, [&] {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        cudaMemPool_t pool = nullptr;
+        cudaStream_t st = nullptr;
+        uint64_t keep = POOL_KEEP;
+        if (cudaMemPoolCreate(&pool, &props) == cudaSuccess &&
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess &&
+            cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess) {
+            P.pool = pool;
+            P.stream = st;
+        } else {
+            cudaGetLastError();
+            if (pool) cudaMemPoolDestroy(pool);
+        }
+    });
+    return P;
+}
+
+}  // namespace
+
+cudaError_t dev_alloc(void **p, size_t bytes) {
+    *p = nullptr;
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    if (device < 0 || device >= MAX_DEVICES) return cudaErrorInvalidDevice;
+    DevicePool &P = pool_of(device);
+    if (!P.pool) return cudaMalloc(p, bytes);
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        e = cudaMallocFromPoolAsync(p, bytes, P.pool, P.stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(P.stream);
+        if (e != cudaErrorMemoryAllocation) break;
+        cudaGetLastError();
+        *p = nullptr;
+        if (attempt == 0) {
+            cudaStreamSynchronize(P.stream);
+            cudaMemPoolTrimTo(P.pool, 0);
+        }
+    }
+    return e;
+}
+
+void dev_free(void *p, int device) {
+    if (!p) return;
+    if (device >= 0 && device < MAX_DEVICES && g_pools[device].pool) {
+        cudaFreeAsync(p, g_pools[device].stream);
+    } else {
+        cudaFree(p);
+    }
+}
+
+}  // namespace gbk

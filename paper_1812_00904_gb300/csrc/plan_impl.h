@@ -111,6 +111,11 @@ struct spmv_plan_s {
 
 namespace gbk {
 
+// Device memory from the current device's pool (devmem.cu): usable on any stream once returned;
+// freed when no work that uses it is pending on `device`.
+cudaError_t dev_alloc(void **p, size_t bytes);
+void dev_free(void *p, int device);
+
 // Internal overrides of a plan made by the library itself.
 struct PlanInternal {
     int ctas = 0;             // CTAs of every pass (0: one per SM, at most one per tile)
@@ -144,6 +149,8 @@ struct CooSort {
     void *tmp = nullptr;   // keys x2, payloads x2, histogram, block sums
     void *own = nullptr;   // sorted minor indices + values (handed to the plan)
     size_t own_bytes = 0;
+    int device = 0;
+    cudaStream_t s = nullptr;  // waited for before the buffers are freed
     ~CooSort();
 };
 // Stable LSD radix sort of the triples by (major, minor) on `s`: sorted minor indices and values
