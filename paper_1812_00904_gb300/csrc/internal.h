@@ -171,6 +171,23 @@ cudaError_t ensure_smem_limit(K kern, SmemLimit &lim, int smem) {
     return e;
 }
 
+// Launch with programmatic serialization: the grid may become resident, and run up to its
+// griddepcontrol.wait, while the kernel before it in the stream drains.
+template <typename... Params, typename... Args>
+cudaError_t launch_overlapped(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+}
+
 struct LaunchArgs {
     StreamParams sp;
     int grid, block, smem;

@@ -50,6 +50,7 @@ template <typename VT> struct StepFeed {
             fence_mbar_init();
         }
         __syncthreads();
+        grid_wait();  // (values and vectors may come from the kernels before)
         for (int i = 0; i < p.slots; ++i) issue(i);  // the first copies fly while the vectors are staged
     }
 
@@ -128,16 +129,16 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
     XT *vs = reinterpret_cast<XT *>(smem + p.copies * p.acc_bytes);
     const int lane = threadIdx.x & 31;
     // the combine and the zone fix-up may be launched: their blocks find room as this grid's CTAs end
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __shared__ int next_chunk;
-    Feed feed(p, smem + p.copies * p.acc_bytes + p.vec_bytes, &next_chunk);
-
-    // ---- the short vectors on chip: the accumulator zeroed, the input staged
+    grid_release();
+    // ---- the short vectors on chip: the accumulator zeroed (while the kernel before drains), the
+    // input staged
     if constexpr (SC) {
         float4 *q = reinterpret_cast<float4 *>(smem);
         const int n16 = p.copies * p.acc_bytes >> 4;
         for (int i = threadIdx.x; i < n16; i += blockDim.x) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
+    __shared__ int next_chunk;
+    Feed feed(p, smem + p.copies * p.acc_bytes + p.vec_bytes, &next_chunk);
     if constexpr (SD) {
         for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x)
             static_cast<XT *>(p.u)[p.emptylist[i]] = XT(0);
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(WB * 32, 1) mvdot_kernel(const __grid_constant
     constexpr int GP = 4;
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    grid_release();
     __shared__ int next_chunk;
     Feed feed(p, smem + p.vec_bytes, &next_chunk);
 
@@ -602,14 +603,14 @@ __global__ void __launch_bounds__(WB * 32, 1) mvscatter_kernel(const __grid_cons
     const int lane = threadIdx.x & 31;
     const int g = lane / KV, b = lane % KV;
     const bool act = b < p.kb;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __shared__ int next_chunk;
-    Feed feed(p, smem + p.copies * p.acc_bytes, &next_chunk);
+    grid_release();
     {
         float4 *q = reinterpret_cast<float4 *>(smem);
         const int n16 = p.copies * p.acc_bytes >> 4;
         for (int i = threadIdx.x; i < n16; i += blockDim.x) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
+    __shared__ int next_chunk;
+    Feed feed(p, smem + p.copies * p.acc_bytes, &next_chunk);
     __syncthreads();
     const float *xb = static_cast<const float *>(p.xv[act ? b : 0]);
     acc += b;
@@ -678,8 +679,7 @@ cudaError_t launch_mvscatter(int kv, const PassParams &p, int grid, int warps, i
         auto go = [&](auto kern, SmemLimit &lim) {
             const cudaError_t e = ensure_smem_limit(kern, lim, smem);
             if (e != cudaSuccess) return e;
-            kern<<<grid, warps * 32, smem, s>>>(p);
-            return cudaGetLastError();
+            return launch_overlapped(kern, dim3(grid), dim3(warps * 32), smem, s, p);
         };
         static SmemLimit lim[3];
         return kv == 2   ? go(mvscatter_kernel<VT, 2, 32>, lim[0])
@@ -694,8 +694,7 @@ cudaError_t launch_mvdot_one(const PassParams &p, int grid, int warps, int smem,
     static SmemLimit lim;
     const cudaError_t e = ensure_smem_limit(kern, lim, smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, warps * 32, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_overlapped(kern, dim3(grid), dim3(warps * 32), smem, s, p);
 }
 template <typename VT>
 cudaError_t launch_mvdot(int kv, bool onchip, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
@@ -719,8 +718,7 @@ cudaError_t launch_pass_one(const PassParams &p, int grid, int warps, int smem, 
     static SmemLimit lim;
     const cudaError_t e = ensure_smem_limit(kern, lim, smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, warps * 32, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_overlapped(kern, dim3(grid), dim3(warps * 32), smem, s, p);
 }
 
 template <typename VT, typename XT>

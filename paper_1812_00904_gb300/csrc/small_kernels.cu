@@ -8,6 +8,7 @@
 
 #include <algorithm>
 
+#include "device_common.cuh"
 #include "internal.h"
 #include "zones.cuh"
 
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(FIN_X * FIN_ROWS) finish_kernel(const __grid_c
     if ((int)blockIdx.x >= p.comb_blocks) {
         const int k = (blockIdx.x - p.comb_blocks) * (FIN_X * FIN_ROWS) + threadIdx.x;
         const ZoneDev zd = k < p.z ? p.zones[k] : ZoneDev{0, 0, 0, 0};
-        asm volatile("griddepcontrol.wait;" ::: "memory");  // the records of the pass launched before
+        grid_wait();  // the records of the pass launched before
         const double t = zone_sum(k < p.z, zd, static_cast<const RT *>(p.rec_left) + (size_t)b * p.P,
                                   static_cast<const RT *>(p.rec_right) + (size_t)b * p.P);
         if (k < p.z) static_cast<XT *>(p.long_out.p[b])[zd.col] = static_cast<XT>(t);
@@ -54,7 +55,7 @@ __global__ void __launch_bounds__(FIN_X * FIN_ROWS) finish_kernel(const __grid_c
     }
     const int tx = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int i = blockIdx.x * FIN_X + tx;
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the partials
+    grid_wait();  // the partials
     double s = 0.0;
     if (i < p.n_minor) {
         const PT *src = static_cast<const PT *>(p.part) + (size_t)b * p.bstride + i;
@@ -91,19 +92,10 @@ cudaError_t launch_finish(FinishArgs &p, int kb, cudaStream_t s) {
     const int64_t per_sm = (blocks * kb + SMS - 1) / SMS;
     auto kern = finish_kernel<XT, PT, RT>;
     static SmemLimit lim;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks, kb);
-    cfg.blockDim = dim3(FIN_X * FIN_ROWS);
-    cfg.dynamicSmemBytes = per_sm < RESIDENT ? ALL / per_sm - 4096 : 0;
-    const cudaError_t e = ensure_smem_limit(kern, lim, (int)cfg.dynamicSmemBytes);
+    const size_t smem = per_sm < RESIDENT ? ALL / per_sm - 4096 : 0;
+    const cudaError_t e = ensure_smem_limit(kern, lim, (int)smem);
     if (e != cudaSuccess) return e;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, p);
+    return launch_overlapped(kern, dim3((unsigned)blocks, kb), dim3(FIN_X * FIN_ROWS), smem, s, p);
 }
 
 static void out_ptrs(OutPtrs &o, void *const *out, int kb) {
@@ -167,6 +159,8 @@ __global__ void __launch_bounds__(256) interleave_kernel(InPtrs in, int kb, int6
     constexpr int IT = 256;
     constexpr int RS = KB + 1;  // padded row: no bank conflicts in either phase
     __shared__ XT sh[IT * RS];
+    grid_release();
+    grid_wait();  // (the vectors may come from the kernel before, which may also still read `out`)
     for (int64_t i0 = (int64_t)blockIdx.x * IT; i0 < len; i0 += (int64_t)gridDim.x * IT) {
         const int cnt = (int)(len - i0 < IT ? len - i0 : (int64_t)IT);
 #pragma unroll
@@ -190,14 +184,14 @@ cudaError_t launch_interleave(bool f64, int kbt, int kb, const void *const *in, 
     const int grid = (int)std::min<int64_t>((len + 255) / 256, 152 * 8);
     if (f64) {
         double *o = static_cast<double *>(out);
-        if (kbt == 2) interleave_kernel<double, 2><<<grid, 256, 0, s>>>(ip, kb, len, o);
-        else if (kbt == 4) interleave_kernel<double, 4><<<grid, 256, 0, s>>>(ip, kb, len, o);
-        else interleave_kernel<double, 8><<<grid, 256, 0, s>>>(ip, kb, len, o);
+        if (kbt == 2) return launch_overlapped(interleave_kernel<double, 2>, dim3(grid), dim3(256), 0, s, ip, kb, len, o);
+        else if (kbt == 4) return launch_overlapped(interleave_kernel<double, 4>, dim3(grid), dim3(256), 0, s, ip, kb, len, o);
+        else return launch_overlapped(interleave_kernel<double, 8>, dim3(grid), dim3(256), 0, s, ip, kb, len, o);
     } else {
         float *o = static_cast<float *>(out);
-        if (kbt == 2) interleave_kernel<float, 2><<<grid, 256, 0, s>>>(ip, kb, len, o);
-        else if (kbt == 4) interleave_kernel<float, 4><<<grid, 256, 0, s>>>(ip, kb, len, o);
-        else interleave_kernel<float, 8><<<grid, 256, 0, s>>>(ip, kb, len, o);
+        if (kbt == 2) return launch_overlapped(interleave_kernel<float, 2>, dim3(grid), dim3(256), 0, s, ip, kb, len, o);
+        else if (kbt == 4) return launch_overlapped(interleave_kernel<float, 4>, dim3(grid), dim3(256), 0, s, ip, kb, len, o);
+        else return launch_overlapped(interleave_kernel<float, 8>, dim3(grid), dim3(256), 0, s, ip, kb, len, o);
     }
     return cudaGetLastError();
 }
