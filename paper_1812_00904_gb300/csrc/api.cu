@@ -61,8 +61,8 @@ cudaError_t launch_pass(const spmv_plan_s *p, bool sc, bool sd, const PassParams
     }
 }
 
-// Shared memory of a one-vector pass: the accumulator (sc), the input vector (sd), the staging slots
-// of as many warps as fit, and what is left over for more copies of the accumulator.  Measured on
+// Shared memory of a one-vector pass: the accumulator (sc), the input vector (sd), a staging slot for
+// each of as many warps as fit, and what is left over for more copies of the accumulator.  Measured on
 // the 200M-nonzero wide matrix (m = 20,000; us): more warps always help (pair 420 / 481 / 537 / 627
 // at 32 / 24 / 20 / 16 warps).  The dot products alone take two slots a warp (279 against 286
 // with one); with the accumulator one slot and the room for a second copy are better (317 against
@@ -84,10 +84,11 @@ PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1) {
     const size_t slot = pass_slot_bytes(p->sv), all = (size_t)p->smem_max;
     const size_t fit = all > acc + vec ? (all - acc - vec) / slot : 0;
     g.warps = (int)std::min<size_t>(std::min(pass_warps(p->sv), cta_tiles(p)), fit);
-    g.slots = g.warps > 0 ? (int)std::min<size_t>(sc ? 1 : PASS_MAX_SLOTS, fit / g.warps) : 0;
+    g.slots = 1;
     const size_t rest = vec + (size_t)g.warps * g.slots * slot;
     g.copies = 1;
-    while (sc && 2 * g.copies <= std::min(g.warps, PASS_MAX_COPIES) && 2 * g.copies * acc + rest <= all) g.copies *= 2;
+    const int most = p->sv == 8 ? 2 : PASS_MAX_COPIES;  // (adding up FP64 copies costs more than they save)
+    while (sc && 2 * g.copies <= std::min(g.warps, most) && 2 * g.copies * acc + rest <= all) g.copies *= 2;
     g.smem = g.copies * acc + rest;
     return g;
 }
@@ -864,9 +865,7 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     // the one-vector passes serve validated plans with whole-step tiles whose short vectors fit in
     // shared memory beside the staging slots of enough warps
     if (!pi && nnz > 0 && p->T % 256 == 0 && !(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL))) {
-        // (the accumulating product alone of FP64 values stays with the streaming kernel: 62 us
-        // against 66 on 8M nonzeros, n = 4,000)
-        p->pass_sc = p->sv != 8 && pass_fits(p, true, false);
+        p->pass_sc = pass_fits(p, true, false);
         p->pass_sd = pass_fits(p, false, true);
         p->pass_pair = pass_fits(p, true, true);
         p->pass_mv = p->sv != 8;

@@ -241,13 +241,12 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
 #pragma unroll
             for (int e = 0; e < 8; ++e) a[e] = static_cast<AT>(vs[ix[e]]);
         }
-        if constexpr (SC) {
+        if constexpr (sizeof(AT) == 4) {  // (FP64 multiplies in the additions)
 #pragma unroll
-            for (int e = 0; e < 8; ++e) c[e] *= va[e];
-        }
-        if constexpr (SD && sizeof(AT) == 4) {  // (FP64 multiplies in the prefix)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) a[e] = mul_rn(va[e], a[e]);
+            for (int e = 0; e < 8; ++e) {
+                if constexpr (SC) c[e] *= va[e];
+                if constexpr (SD) a[e] = mul_rn(va[e], a[e]);
+            }
         }
         if (!whole) {  // positions past the last nonzero (zero times an infinity is no zero)
             const int nv = p.nnz - ps;
@@ -261,7 +260,13 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
         }
         if constexpr (SC) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) atomicAdd(acc + ix[e], c[e]);
+            for (int e = 0; e < 8; ++e) {
+                if constexpr (sizeof(AT) == 4) {
+                    atomicAdd(acc + ix[e], c[e]);
+                } else {
+                    acc_fma(acc + ix[e], va[e], c[e]);
+                }
+            }
         }
         if constexpr (SD) {  // into the order of the positions
 #pragma unroll
@@ -320,6 +325,8 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
                 const int reach = le ? lane - (31 - __clz(le)) : lane;
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) {
+                    // (FP64 additions are worth a vote)
+                    if (sizeof(AT) == 8 && !__any_sync(FULL, d <= reach)) break;
                     const AT o = __shfl_up_sync(FULL, s, d);
                     if (d <= reach) s += o;
                 }
