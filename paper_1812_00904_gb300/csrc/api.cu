@@ -539,11 +539,26 @@ static spmv_status run_row_blocks(spmv_plan_s *p, int kb, const void *const *in,
 
 static spmv_status run_dvalues(spmv_plan_s *p, const void *r, const void *x, void *g, cudaStream_t s) {
     if (p->nnz == 0) return SPMV_OK;
+    // CSC: g = r[row] * x[col] -> minor r, major x;  CSR: g = r[row] * x[col] -> minor x, major r
+    const bool csc = p->layout == SPMV_CSC_WIDE;
+    if (p->pass_sd) {
+        const PassGeometry geo = pass_geometry(p, false, true);
+        PassParams pp = pass_params(p);
+        pp.v = csc ? r : x;
+        pp.x = csc ? x : r;
+        pp.u = g;
+        pp.vec_bytes = (int)pass_vec_bytes(p);
+        pp.slots = geo.slots;
+        ProfScope ps(p, 4, s);
+        CUDA_TRY(p->val_t == SPMV_F64    ? launch_dvalues_f64(pp, p->ctas, geo.warps, (int)geo.smem, s)
+                 : p->val_t == SPMV_F32  ? launch_dvalues_f32(pp, p->ctas, geo.warps, (int)geo.smem, s)
+                 : p->val_t == SPMV_BF16 ? launch_dvalues_bf16(pp, p->ctas, geo.warps, (int)geo.smem, s)
+                                         : launch_dvalues_f16(pp, p->ctas, geo.warps, (int)geo.smem, s));
+        return SPMV_OK;
+    }
     LaunchArgs a;
     a.sp = base_params(p);
     a.sp.kb = 1;
-    // CSC: g = r[row] * x[col] -> minor r, major x;  CSR: g = r[row] * x[col] -> minor x, major r
-    const bool csc = p->layout == SPMV_CSC_WIDE;
     a.sp.vin[0] = csc ? r : x;
     a.sp.vin[1] = csc ? x : r;
     a.sp.vout[0] = g;

@@ -16,5 +16,8 @@ cudaError_t launch_mvdot_bf16(int kv, bool onchip, const PassParams &p, int grid
 cudaError_t launch_mvscatter_bf16(int kv, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
     return launch_mvscatter<__nv_bfloat16>(kv, p, grid, warps, smem, s);
 }
+cudaError_t launch_dvalues_bf16(const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return launch_dvalues<__nv_bfloat16, float>(p, grid, warps, smem, s);
+}
 
 }  // namespace gbk

@@ -16,5 +16,8 @@ cudaError_t launch_mvdot_f16(int kv, bool onchip, const PassParams &p, int grid,
 cudaError_t launch_mvscatter_f16(int kv, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
     return launch_mvscatter<__half>(kv, p, grid, warps, smem, s);
 }
+cudaError_t launch_dvalues_f16(const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return launch_dvalues<__half, float>(p, grid, warps, smem, s);
+}
 
 }  // namespace gbk

@@ -16,5 +16,8 @@ cudaError_t launch_mvdot_f32(int kv, bool onchip, const PassParams &p, int grid,
 cudaError_t launch_mvscatter_f32(int kv, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
     return launch_mvscatter<float>(kv, p, grid, warps, smem, s);
 }
+cudaError_t launch_dvalues_f32(const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return launch_dvalues<float, float>(p, grid, warps, smem, s);
+}
 
 }  // namespace gbk

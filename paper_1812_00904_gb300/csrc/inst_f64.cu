@@ -10,5 +10,8 @@ cudaError_t launch_pass_f64(bool sc, bool sd, const PassParams &p, int grid, int
                             cudaStream_t s) {
     return launch_pass<double, double>(sc, sd, p, grid, warps, smem, s);
 }
+cudaError_t launch_dvalues_f64(const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return launch_dvalues<double, double>(p, grid, warps, smem, s);
+}
 
 }  // namespace gbk

@@ -200,10 +200,15 @@ cudaError_t launch_stream_f64(int mode, int kb, const LaunchArgs &a);
 cudaError_t launch_stream_f32(int mode, int kb, const LaunchArgs &a);
 cudaError_t launch_stream_bf16(int mode, int kb, const LaunchArgs &a);
 cudaError_t launch_stream_f16(int mode, int kb, const LaunchArgs &a);
-// One-vector pass: the accumulating product (sc), the dot products (sd) or both.
+// One-vector pass: the accumulating product (sc), the dot products (sd) or both; and the values'
+// gradient (v the minor, x the major vector, u the gradient).
+cudaError_t launch_dvalues_f64(const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
 cudaError_t launch_pass_f64(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_dvalues_f32(const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
 cudaError_t launch_pass_f32(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_dvalues_bf16(const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
 cudaError_t launch_pass_bf16(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
+cudaError_t launch_dvalues_f16(const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
 cudaError_t launch_pass_f16(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s);
 
 // Accumulating and dot products of up to kv = 2, 4 or 8 vectors (32-bit accumulation).

@@ -24,7 +24,8 @@ namespace gbk {
 // A slot receives a step's indices, values and record, one bulk copy each (the nonzeros of a partial
 // last step are read from global memory instead), and a header: step, chunk << 2 | first << 1 |
 // last; step -1: no more work.
-template <typename VT> struct StepFeed {
+// VALS: the values too.
+template <typename VT, bool VALS = true> struct StepFeed {
     static constexpr int SLOT = pass_slot_bytes(sizeof(VT));
     static constexpr int OFF_VAL = 1024, OFF_REC = OFF_VAL + 256 * (int)sizeof(VT), OFF_HDR = OFF_REC + (int)sizeof(StepRec);
     const PassParams &p;
@@ -71,7 +72,7 @@ template <typename VT> struct StepFeed {
         uint32_t bytes = 0;
         if (fs < fe) {
             hdr = make_int2(fs, (fq << 2) | ffirst | (fs + 1 == fe ? 1 : 0));
-            bytes = sizeof(StepRec) + ((p.nnz >> 8) > fs ? 1024u + 256u * (uint32_t)sizeof(VT) : 0u);
+            bytes = sizeof(StepRec) + ((p.nnz >> 8) > fs ? 1024u + (VALS ? 256u * (uint32_t)sizeof(VT) : 0u) : 0u);
         }
         *reinterpret_cast<int2 *>(slot + OFF_HDR) = hdr;
         mbar_arrive_expect_tx(&bars[i], bytes);  // releases the header; the bulk bytes complete the phase
@@ -79,8 +80,9 @@ template <typename VT> struct StepFeed {
             bulk_g2s(slot + OFF_REC, p.steps + fs, sizeof(StepRec), &bars[i]);
             if ((p.nnz >> 8) > fs) {
                 bulk_g2s(slot, p.idx + (size_t)fs * 256, 1024u, &bars[i]);
-                bulk_g2s(slot + OFF_VAL, static_cast<const VT *>(p.vals) + (size_t)fs * 256,
-                         256u * (uint32_t)sizeof(VT), &bars[i]);
+                if constexpr (VALS)
+                    bulk_g2s(slot + OFF_VAL, static_cast<const VT *>(p.vals) + (size_t)fs * 256,
+                             256u * (uint32_t)sizeof(VT), &bars[i]);
             }
             ++fs;
             ffirst = 0;
@@ -716,6 +718,94 @@ cudaError_t launch_mvdot(int kv, bool onchip, const PassParams &p, int grid, int
                : kv == 4 ? launch_mvdot_one<VT, 4, false>(p, grid, warps, smem, s)
                          : launch_mvdot_one<VT, 8, false>(p, grid, warps, smem, s);
     }
+}
+
+// Two neighbouring values of the gradient, in the values' type, by one store.
+__device__ __forceinline__ void store2(float *g, float a, float b) { *reinterpret_cast<float2 *>(g) = make_float2(a, b); }
+__device__ __forceinline__ void store2(double *g, double a, double b) { *reinterpret_cast<double2 *>(g) = make_double2(a, b); }
+__device__ __forceinline__ void store2(__nv_bfloat16 *g, float a, float b) {
+    *reinterpret_cast<__nv_bfloat162 *>(g) = __halves2bfloat162(__float2bfloat16_rn(a), __float2bfloat16_rn(b));
+}
+__device__ __forceinline__ void store2(__half *g, float a, float b) {
+    *reinterpret_cast<__half2 *>(g) = __halves2half2(__float2half_rn(a), __float2half_rn(b));
+}
+
+// The gradient of r^T A x by the stored values, g[k] = minor[idx[k]] * major[seg(k)]: the minor
+// vector on chip, a lane taking positions 64 j + 2 lane and the next one (conflict-free index
+// loads, whole-line stores).  Reads 4 bytes and writes one value a nonzero; the streaming kernel,
+// 128 positions a step, took 108 us for 20M FP16 values (m = 8,003), this one 38.
+template <typename VT, typename XT, int WB>
+__global__ void __launch_bounds__(WB * 32, 1) dvalues_kernel(const __grid_constant__ PassParams p) {
+    using AT = typename Acc<VT>::type;
+    using Feed = StepFeed<VT, false>;
+    extern __shared__ __align__(128) unsigned char smem[];
+    XT *vs = reinterpret_cast<XT *>(smem);
+    const int lane = threadIdx.x & 31;
+    grid_release();
+    __shared__ int next_chunk;
+    Feed feed(p, smem + p.vec_bytes, &next_chunk);
+    {
+        constexpr int xa = 16 / (int)sizeof(XT);
+        const XT *src = static_cast<const XT *>(p.v);
+        const int n16 = p.n_minor / xa;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < n16; i += blockDim.x)
+            reinterpret_cast<float4 *>(vs)[i] = __ldg(reinterpret_cast<const float4 *>(src) + i);
+        for (int i = n16 * xa + threadIdx.x; i < p.n_minor; i += blockDim.x) vs[i] = __ldg(src + i);
+    }
+    __syncthreads();
+    const XT *xg = static_cast<const XT *>(p.x);
+    VT *g = static_cast<VT *>(p.u);
+    unsigned char *slot;
+    int2 hdr;
+    while (feed.next(slot, hdr)) {
+        const int ps = hdr.x << 8;
+        const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
+        const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);
+        const bool gaps = (bf.y & STEP_GAPS) != 0;
+        const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
+        auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
+        const int left = p.nnz - ps;
+        int ix[8];
+        AT x[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int pos = 64 * j + 2 * lane;
+            if (left >= 256) {
+                const int2 q = *reinterpret_cast<const int2 *>(slot + 4 * pos);
+                ix[2 * j] = q.x;
+                ix[2 * j + 1] = q.y;
+            } else {
+                ix[2 * j] = pos < left ? __ldg(p.idx + ps + pos) : 0;
+                ix[2 * j + 1] = pos + 1 < left ? __ldg(p.idx + ps + pos + 1) : 0;
+            }
+            const uint32_t w = rec->heads[pos >> 5];
+            const int b = pos & 31;  // (even: bit b + 1 exists)
+            const int c0 = base + rec->before[pos >> 5] + __popc(w & ((2u << b) - 1u));
+            const int c1 = c0 + ((w >> (b + 1)) & 1u);
+            x[2 * j] = static_cast<AT>(__ldg(xg + col_of(max(c0, 0))));
+            x[2 * j + 1] = static_cast<AT>(__ldg(xg + col_of(max(c1, 0))));
+        }
+        feed.release();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int pos = 64 * j + 2 * lane;
+            const AT a = static_cast<AT>(vs[ix[2 * j]]) * x[2 * j], c = static_cast<AT>(vs[ix[2 * j + 1]]) * x[2 * j + 1];
+            if (pos + 1 < left)
+                store2(g + ps + pos, a, c);
+            else if (pos < left)
+                g[ps + pos] = from_d<VT>(static_cast<double>(a));
+        }
+    }
+}
+
+template <typename VT, typename XT>
+cudaError_t launch_dvalues(const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    auto kern = dvalues_kernel<VT, XT, pass_warps(sizeof(VT))>;
+    static SmemLimit lim;
+    const cudaError_t e = ensure_smem_limit(kern, lim, smem);
+    if (e != cudaSuccess) return e;
+    return launch_overlapped(kern, dim3(grid), dim3(warps * 32), smem, s, p);
 }
 
 template <typename VT, typename XT, bool SC, bool SD>

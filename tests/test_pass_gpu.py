@@ -48,6 +48,12 @@ def _check(A, dtype, tile_items, what):
     short, ref_s, scale = ((y, oracle.spmv, oracle.abs_spmv) if A.layout == "csc" else (u, oracle.spvtm, oracle.abs_spvtm))
     arg = host_of(xd if A.layout == "csc" else vd)
     assert_close(host_of(short), ref_s(stored, arg), scale(stored, arg), TOL[dtype], f"{what}: pair")
+    r, z = dev_vec(synth.uniform_vector(A.m, 5), plan.vec_dtype), dev_vec(synth.uniform_vector(A.n, 6), plan.vec_dtype)
+    g = plan.dvalues(r, z)
+    assert torch.equal(g, ref.dvalues(r, z)), f"{what}: the values' gradient differs from the streaming kernel's"
+    exact = oracle.dvalues(stored, host_of(r), host_of(z))
+    unit = {torch.bfloat16: 2.0**-8, torch.float16: 2.0**-11}.get(dtype, 2.0**-23)
+    assert np.all(np.abs(host_of(g) - exact) <= unit * np.abs(exact) + 2.0**-24), f"{what}: dvalues"
     plan.check()
 
 
