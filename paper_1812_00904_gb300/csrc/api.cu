@@ -77,7 +77,10 @@ struct PassGeometry {
     size_t smem;
 };
 // tiles of a CTA: no more warps than these can work
-int cta_tiles(const spmv_plan_s *p) { return std::max(1, (p->ntiles + p->ctas - 1) / std::max(1, p->ctas)); }
+int cta_tiles(const spmv_plan_s *p) {
+    const int blocks = std::max(1, p->ctas * p->bpc);
+    return std::max(1, (p->ntiles + blocks - 1) / blocks);
+}
 PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1) {
     PassGeometry g;
     const size_t acc = sc ? align_up((size_t)p->n_minor * kv * p->sa, 128) : 0, vec = (sd ? pass_vec_bytes(p) : 0) + PASS_BAR_BYTES;
@@ -255,6 +258,8 @@ static PassParams pass_params(const spmv_plan_s *p) {
     pp.ntiles = p->ntiles;
     pp.spt = p->T / 256;
     pp.chunk_tiles = p->chunk_tiles;
+    pp.bpc = p->bpc;
+    pp.win = p->win;
     pp.part = p->part;
     pp.rec_left = p->rec_left;
     pp.rec_right = p->rec_right;
@@ -267,7 +272,9 @@ static PassParams pass_params(const spmv_plan_s *p) {
 
 // The one-vector pass of plan p: y_short += A x (sc) into the per-CTA partials, u = the dot
 // products with v (sd), or both; then the combine and the zone fix-up in one launch.
-static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *v, void *u, cudaStream_t s) {
+// The launches are timed as kernels 0 / 1 and id_dot / id_fix of plan `prof`.
+static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *v, void *u, cudaStream_t s,
+                            spmv_plan_s *prof, int id_dot = 2, int id_fix = 3) {
     const bool sc = y != nullptr, sd = u != nullptr;
     PassParams pp = pass_params(p);
     pp.acc_bytes = sc ? (int)pass_acc_bytes(p) : 0;
@@ -281,13 +288,13 @@ static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *
     const bool f64 = p->vec_t == SPMV_F64;
     {
         // a pass that serves both products counts as a launch of each, with half of its time
-        ProfScope ps0(p, 0, s, !sc ? 0.0 : sd ? 0.5 : 1.0), ps2(p, 2, s, !sd ? 0.0 : sc ? 0.5 : 1.0);
+        ProfScope ps0(prof, 0, s, !sc ? 0.0 : sd ? 0.5 : 1.0), ps2(prof, id_dot, s, !sd ? 0.0 : sc ? 0.5 : 1.0);
         CUDA_TRY(launch_pass(p, sc, sd, pp, g.warps, (int)g.smem, s));
     }
     const spmv_plan_s::ProcZones &pz = p->pz;
     const bool zones = sd && pz.z > 0;
     if (sc || zones) {
-        ProfScope ps1(p, 1, s, !sc ? 0.0 : zones ? 0.5 : 1.0), ps3(p, 3, s, !zones ? 0.0 : sc ? 0.5 : 1.0);
+        ProfScope ps1(prof, 1, s, !sc ? 0.0 : zones ? 0.5 : 1.0), ps3(prof, id_fix, s, !zones ? 0.0 : sc ? 0.5 : 1.0);
         if (sc && zones)
             CUDA_TRY(launch_combine_fixup(f64, p->part, p->ctas, p->n_minor, y, pz.zones, pz.z, p->rec_left, p->rec_right,
                                           pz.nproc, u, s));
@@ -308,7 +315,7 @@ spmv_status run_scatter(spmv_plan_s *p, int kb, const void *const *in, void *con
             for (int b = 0; b < kb; ++b) CUDA_TRY(cudaMemsetAsync(out[b], 0, out_bytes, s));
         return SPMV_OK;
     }
-    if (kb == 1 && p->pass_sc) return run_pass(p, in[0], out[0], nullptr, nullptr, s);
+    if (kb == 1 && p->pass_sc) return run_pass(p, in[0], out[0], nullptr, nullptr, s, p);
     if (p->pass_mv && p->pass_sc) return run_mvscatter(p, kb, in, out, s);
     if (!p->onchip && kb > 1) {
         for (int b = 0; b < kb; ++b) {
@@ -457,7 +464,7 @@ static spmv_status run_segdot_impl(spmv_plan_s *p, int kb, const void *const *in
             for (int b = 0; b < kb; ++b) CUDA_TRY(cudaMemsetAsync(out[b], 0, out_bytes, s));
         return SPMV_OK;
     }
-    if (kb == 1 && p->pass_sd) return run_pass(p, nullptr, nullptr, in[0], out[0], s);
+    if (kb == 1 && p->pass_sd) return run_pass(p, nullptr, nullptr, in[0], out[0], s, prof, id_dot, id_fix);
     const bool f64_onchip = p->val_t == SPMV_F64 && p->onchip && kb <= p->batch_width;
     if (kb > 1 && !f64_onchip) {
         const int grp = seg_group(p);
@@ -879,7 +886,9 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     }
     // the one-vector passes serve validated plans with whole-step tiles whose short vectors fit in
     // shared memory beside the staging slots of enough warps
-    if (!pi && nnz > 0 && p->T % 256 == 0 && !(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL))) {
+    if (pi && nnz > 0 && p->T % 256 == 0) {  // the row-sorted copy: its single-vector dot products
+        p->pass_sd = pass_fits(p, false, true);
+    } else if (nnz > 0 && p->T % 256 == 0 && !(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL))) {
         p->pass_sc = pass_fits(p, true, false);
         p->pass_sd = pass_fits(p, false, true);
         p->pass_pair = pass_fits(p, true, true);
@@ -1113,7 +1122,7 @@ static spmv_status pair_device(spmv_plan_s *p, const void *x, void *y, const voi
     // both short vectors on chip: one reading of the matrix serves both products
     if (p->pass_pair && !p->tplan) {
         const bool csc = p->layout == SPMV_CSC_WIDE;
-        return csc ? run_pass(p, x, y, v, u, s) : run_pass(p, v, u, x, y, s);
+        return csc ? run_pass(p, x, y, v, u, s, p) : run_pass(p, v, u, x, y, s, p);
     }
     if (!p->cstream) CUDA_TRY(cudaStreamCreateWithFlags(&p->cstream, cudaStreamNonBlocking));
     if (!p->ev_x) CUDA_TRY(cudaEventCreateWithFlags(&p->ev_x, cudaEventDisableTiming));

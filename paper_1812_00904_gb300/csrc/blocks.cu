@@ -129,12 +129,14 @@ spmv_status build_row_blocks(spmv_plan_s *p, int sms, cudaStream_t s) {
         const int nt = (int)((p->nnz + Tc - 1) / Tc);
         if (nt < sms) continue;
         const int mwp = (int)(((size_t)Tc + 8 + 31) / 32 + 3) / 4 * 4;
-        // the window budget: what the segmented pass leaves beside 16 warps of staging slots
+        // the window budget: what the pass leaves beside all of its warps' staging slots
+        // (whole-step tiles), or the streaming kernel beside 16 warps' slots
         const size_t slot = (size_t)p->S * (((size_t)Tc * 4 + 127) / 128 * 128 +
                                             ((size_t)Tc * p->sv + 127) / 128 * 128 + (size_t)mwp * 4 +
                                             ((size_t)p->mwq * 2 + 15) / 16 * 16 + 160);
-        const size_t budget =
-            (size_t)p->smem_max > BAR_BYTES + 16 * slot ? (size_t)p->smem_max - BAR_BYTES - 16 * slot : 0;
+        const size_t staging = Tc % 256 == 0 ? PASS_BAR_BYTES + 128 + (size_t)pass_warps(p->sv) * pass_slot_bytes(p->sv)
+                                             : BAR_BYTES + 16 * slot;
+        const size_t budget = (size_t)p->smem_max > staging ? (size_t)p->smem_max - staging : 0;
         const int64_t max_elems = (int64_t)(budget / p->sx);
         if (max_elems < 64) continue;
         int32_t *d_max = nullptr;

@@ -128,6 +128,8 @@ struct PassParams {
     void *part;              // SC: per-CTA partials [cta][n_minor]
     void *u;                 // SD: the long output
     void *rec_left, *rec_right;  // SD: carry records [proc], (hi, lo) pairs
+    int32_t bpc;             // SD over row-sorted blocks: blocks each CTA runs in turn, and per block its window
+    const int2 *win;         // (first element, length) of v (NULL: all of v)
     float *uv[VL_MAX];       // several vectors: their outputs (SD; v then being interleaved [entry][KV]),
     const void *xv[VL_MAX];  // their long inputs (SC)
     int32_t kb, nproc;       // several vectors: how many; records [b * nproc + proc]

@@ -33,26 +33,35 @@ template <typename VT, bool VALS = true> struct StepFeed {
     uint64_t *bars;
     unsigned char *slots;
     int *next_chunk;
-    const CtaChunks c;
+    CtaChunks c;
+    bool dead = false;  // a copy did not arrive in time: no more work
     // cursor of the copies: steps [fs, fe) of chunk fq are still to come (lane 0 alone keeps it)
     int fs = 0, fe = 0, fq = -1, ffirst = 0;
     int s = 0;        // slot of the warp's next step
     uint32_t ph = 0;  // phase parity of that slot's barrier
 
     __device__ __forceinline__ StepFeed(const PassParams &p_, unsigned char *area, int *next_chunk_)
-        : p(p_), lane(threadIdx.x & 31), next_chunk(next_chunk_),
-          c(cta_chunks(blockIdx.x, p_.ntiles, gridDim.x, p_.chunk_tiles)) {
+        : p(p_), lane(threadIdx.x & 31), next_chunk(next_chunk_) {
         const int warp = threadIdx.x >> 5;
         bars = reinterpret_cast<uint64_t *>(area) + warp * p.slots;
         slots = area + PASS_BAR_BYTES + warp * p.slots * SLOT;
-        if (threadIdx.x == 0) *next_chunk = 0;
         if (lane == 0) {
             for (int i = 0; i < p.slots; ++i) mbar_init(&bars[i], 1);
             fence_mbar_init();
         }
+    }
+
+    // Begin block gb of `blocks`; again: after another one, whose steps every warp has finished
+    // (plans with one slot a warp).  The first copies fly while the vectors are staged.
+    __device__ __forceinline__ void start(int gb, int blocks, bool again) {
+        c = cta_chunks(gb, p.ntiles, blocks, p.chunk_tiles);
+        if (threadIdx.x == 0) *next_chunk = 0;
         __syncthreads();
-        grid_wait();  // (values and vectors may come from the kernels before)
-        for (int i = 0; i < p.slots; ++i) issue(i);  // the first copies fly while the vectors are staged
+        if (!again) grid_wait();  // (values and vectors may come from the kernels before)
+        if (again) ph ^= 1u;      // the slot's last phase said "no more work"
+        if (dead) return;
+        for (int i = 0; i < p.slots; ++i) issue(i);
+        __syncwarp();
     }
 
     __device__ __forceinline__ void issue(int i) {
@@ -92,6 +101,7 @@ template <typename VT, bool VALS = true> struct StepFeed {
     // The next step's slot and header, or false: no more work (or a copy did not arrive in time,
     // which is reported; the copies still in flight are let land).
     __device__ __forceinline__ bool next(unsigned char *&slot, int2 &hdr) {
+        if (dead) return false;
         slot = slots + s * SLOT;
         bool ok = mbar_wait_bounded(&bars[s], ph, WAIT_LIMIT_NS);
         ok = __all_sync(FULL, ok);
@@ -101,6 +111,7 @@ template <typename VT, bool VALS = true> struct StepFeed {
                 const int rs = s + r < p.slots ? s + r : s + r - p.slots;
                 mbar_wait_bounded(&bars[rs], s + r < p.slots ? ph : ph ^ 1u, WAIT_LIMIT_NS);
             }
+            dead = true;
             return false;
         }
         hdr = *reinterpret_cast<const int2 *>(slot + OFF_HDR);
@@ -141,27 +152,41 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
     }
     __shared__ int next_chunk;
     Feed feed(p, smem + p.copies * p.acc_bytes + p.vec_bytes, &next_chunk);
-    if constexpr (SD) {
-        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x)
-            static_cast<XT *>(p.u)[p.emptylist[i]] = XT(0);
-        constexpr int xa = 16 / (int)sizeof(XT);
-        const XT *src = static_cast<const XT *>(p.v);
-        const int n16 = p.n_minor / xa;
-#pragma unroll 4
-        for (int i = threadIdx.x; i < n16; i += blockDim.x)
-            reinterpret_cast<float4 *>(vs)[i] = __ldg(reinterpret_cast<const float4 *>(src) + i);
-        for (int i = n16 * xa + threadIdx.x; i < p.n_minor; i += blockDim.x) vs[i] = __ldg(src + i);
-    }
-    __syncthreads();
-
     const XT *xg = static_cast<const XT *>(p.x);
     const int sh = (lane & 3) << 3;  // the lane's byte of its segment-start word
     const int sw = (lane >> 2) & 1;  // staggered shared-memory loads
+    unsigned char *slot;
+    int2 hdr;
+
+    // the row-sorted copy's blocks take turns, each with its window of the input; else one block a CTA
+    const int bpc = SD && !SC ? p.bpc : 1;
+#pragma unroll 1
+    for (int hb_ = 0; hb_ < bpc; ++hb_) {
+    const int gb = blockIdx.x * bpc + hb_;
+    if (hb_ > 0) __syncthreads();  // every warp is done with the block before
+    feed.start(gb, gridDim.x * bpc, hb_ > 0);
+    if constexpr (SD) {
+        if (hb_ == 0)
+            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x)
+                static_cast<XT *>(p.u)[p.emptylist[i]] = XT(0);
+        constexpr int xa = 16 / (int)sizeof(XT);
+        const XT *src = static_cast<const XT *>(p.v);
+        int len = p.n_minor;
+        if (!SC && p.win) {  // (windows begin on 16 bytes)
+            const int2 w = p.win[gb];
+            src += w.x;
+            len = min(w.y, p.n_minor);
+        }
+        const int n16 = len / xa;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < n16; i += blockDim.x)
+            reinterpret_cast<float4 *>(vs)[i] = __ldg(reinterpret_cast<const float4 *>(src) + i);
+        for (int i = n16 * xa + threadIdx.x; i < len; i += blockDim.x) vs[i] = __ldg(src + i);
+    }
+    __syncthreads();
 
     AT chi = AT(0), clo = AT(0);  // open segment's running sum (SD)
     int cfirst = -1;              // the chunk's first segment when its sum goes to the left record
-    unsigned char *slot;
-    int2 hdr;
     while (feed.next(slot, hdr)) {
         const int ps = hdr.x << 8;
         const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
@@ -369,6 +394,7 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
             }
         }
     }
+    }  // blocks
 
     if constexpr (SC) {
         __syncthreads();
@@ -428,6 +454,7 @@ __global__ void __launch_bounds__(WB * 32, 1) mvdot_kernel(const __grid_constant
     grid_release();
     __shared__ int next_chunk;
     Feed feed(p, smem + p.vec_bytes, &next_chunk);
+    feed.start(blockIdx.x, gridDim.x, false);
 
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x) {
         const int col = p.emptylist[i];
@@ -620,6 +647,7 @@ __global__ void __launch_bounds__(WB * 32, 1) mvscatter_kernel(const __grid_cons
     }
     __shared__ int next_chunk;
     Feed feed(p, smem + p.copies * p.acc_bytes, &next_chunk);
+    feed.start(blockIdx.x, gridDim.x, false);
     __syncthreads();
     const float *xb = static_cast<const float *>(p.xv[act ? b : 0]);
     acc += b;
@@ -744,6 +772,7 @@ __global__ void __launch_bounds__(WB * 32, 1) dvalues_kernel(const __grid_consta
     grid_release();
     __shared__ int next_chunk;
     Feed feed(p, smem + p.vec_bytes, &next_chunk);
+    feed.start(blockIdx.x, gridDim.x, false);
     {
         constexpr int xa = 16 / (int)sizeof(XT);
         const XT *src = static_cast<const XT *>(p.v);

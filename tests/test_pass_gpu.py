@@ -126,3 +126,25 @@ def test_several_vectors(short, layout, dtype):
                 assert_close(host_of(R[b]), ref(stored, z), scale(stored, z), TOL[dtype], f"{layout} {op} k={k} vector {b}")
                 if dots:
                     assert torch.equal(R[b], plan.spvtm(Z[b]) if op == pkg.SPMV_OP_VTA else plan.spmv(Z[b]))
+
+
+def test_row_blocks_in_turn():
+    """Windows of the long vector too wide for one block a CTA: several blocks in turn, each restaging
+    its window; the same bits as the streaming kernel's multi-vector pass over the same copy."""
+    rng = np.random.default_rng(12)
+    n = 5_000_000
+    deg = np.zeros(n, dtype=np.int64)
+    deg[rng.choice(n, 900_000, replace=False)] = 1
+    deg[rng.choice(n, 20, replace=False)] = 64
+    A = synth.random_matrix(64, n, "csc", degrees=deg, seed=3, duplicates=True)
+    for dtype in (torch.float64, torch.float32):
+        plan, stored = make_plan(A, dtype, flags=pkg.SPMV_PLAN_ROW_BLOCKS, tile_items=256)
+        info = plan.info()
+        if dtype == torch.float64:
+            assert info["row_blocks"] > info["ctas"], info
+        check_products(plan, stored, synth.uniform_vector(n, 1), synth.uniform_vector(64, 2), TOL[dtype], f"{dtype}")
+        X = torch.stack([dev_vec(synth.uniform_vector(n, 7 + b), plan.vec_dtype) for b in range(2)])
+        Y = plan.batch(pkg.SPMV_OP_AX, X)
+        for b in range(2):
+            assert torch.equal(Y[b], plan.spmv(X[b]))
+        plan.close()
