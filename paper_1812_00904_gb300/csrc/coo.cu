@@ -52,45 +52,106 @@ static_assert(RS_BINS == RS_THREADS, "one thread per digit in the tile's scan");
 
 __device__ __forceinline__ int digit_of(uint64_t key, int shift, int mask) { return (int)(key >> shift) & mask; }
 
-// err bit 1: major index outside [0, n_major); bit 4: minor index outside [0, n_minor).  vals: the
-// values of 4 or 2 bytes that become the payload, or NULL (input positions).
-template <typename W>
-__global__ void coo_keys_kernel(const int32_t *__restrict__ major, const int32_t *__restrict__ minor,
-                                const W *__restrict__ vals, int64_t nnz, int n_major, int n_minor,
-                                uint64_t *__restrict__ keys, uint32_t *__restrict__ pay, int32_t *err) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int bits = 0;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nnz; k += stride) {
-        const int32_t j = major[k], i = minor[k];
-        const bool okj = static_cast<uint32_t>(j) < static_cast<uint32_t>(n_major);
-        const bool oki = static_cast<uint32_t>(i) < static_cast<uint32_t>(n_minor);
-        if (!okj) bits |= 1;
-        if (!oki) bits |= 4;
-        keys[k] = (okj && oki) ? (uint64_t)j * (uint64_t)n_minor + (uint64_t)i : 0;
-        pay[k] = vals ? (uint32_t)vals[k] : (uint32_t)k;
+// The lanes of `live` with the same digit, by one vote per bit.  A match instruction takes a round for
+// each digit that differs (32 a warp for random keys): 174 us for a pass of 10M keys over the low 9
+// bits, 125 with the votes.
+__device__ __forceinline__ unsigned same_digit(int d, unsigned live) {
+    unsigned m = live;
+#pragma unroll
+    for (int b = 0; b < RS_BITS; ++b) {
+        const bool one = (d >> b) & 1;
+        const unsigned v = __ballot_sync(0xffffffffu, one);
+        m &= one ? v : ~v;
     }
-    if (bits) atomicOr(err, bits);
+    return m;
 }
 
-// hist[d * ntiles + tile] = number of keys of the tile whose digit is d
-__global__ void __launch_bounds__(RS_THREADS) rs_hist_kernel(const uint64_t *__restrict__ keys, int64_t nnz,
+// The triples as the caller has them and, after the sort, as the plan takes them.
+struct Triples {
+    const int32_t *major, *minor;
+    const void *vals;
+    int vbytes;  // 2, 4 or 8
+    int n_major, n_minor;
+    uint64_t recip;  // floor((2^64 - 1) / n_minor)
+    int32_t *out_major, *out_minor;
+    void *out_vals;
+};
+
+// The key of triple k; 0 with bit 1 (major index outside [0, n_major)) or bit 4 (minor index
+// outside [0, n_minor)) of `bad` set.
+__device__ __forceinline__ uint64_t triple_key(const Triples &t, int64_t k, int &bad) {
+    const int32_t j = t.major[k], i = t.minor[k];
+    const bool okj = static_cast<uint32_t>(j) < static_cast<uint32_t>(t.n_major);
+    const bool oki = static_cast<uint32_t>(i) < static_cast<uint32_t>(t.n_minor);
+    if (!okj) bad |= 1;
+    if (!oki) bad |= 4;
+    return okj && oki ? (uint64_t)j * (uint64_t)t.n_minor + (uint64_t)i : 0;
+}
+
+// Values of 2 and 4 bytes travel as the payload, those of 8 bytes are gathered by position at the end.
+__device__ __forceinline__ uint32_t triple_payload(const Triples &t, int64_t k) {
+    return t.vbytes == 4   ? static_cast<const uint32_t *>(t.vals)[k]
+           : t.vbytes == 2 ? (uint32_t)static_cast<const uint16_t *>(t.vals)[k]
+                           : (uint32_t)k;
+}
+
+// Key and payload to their triple's place.  The quotient by the reciprocal is the true one or one
+// less: key < 2^62, so that the reciprocal's error takes away less than one.
+__device__ __forceinline__ void triple_store(const Triples &t, int64_t pos, int64_t nnz, uint64_t key, uint32_t pay, int32_t *err) {
+    uint64_t j = __umul64hi(key, t.recip), i = key - j * (uint64_t)t.n_minor;
+    if (i >= (uint64_t)t.n_minor) {
+        ++j;
+        i -= (uint64_t)t.n_minor;
+    }
+    t.out_major[pos] = (int32_t)j;
+    t.out_minor[pos] = (int32_t)i;
+    if (t.vbytes == 4) {
+        static_cast<uint32_t *>(t.out_vals)[pos] = pay;
+    } else if (t.vbytes == 2) {
+        static_cast<uint16_t *>(t.out_vals)[pos] = (uint16_t)pay;
+    } else if (pay < nnz) {
+        static_cast<uint64_t *>(t.out_vals)[pos] = static_cast<const uint64_t *>(t.vals)[pay];
+    } else {
+        static_cast<uint64_t *>(t.out_vals)[pos] = 0;
+        atomicOr(err, 8);
+    }
+}
+
+// hist[d * ntiles + tile] = number of keys of the tile whose digit is d.  FIRST: the keys come from
+// the triples, whose indices are checked.
+template <bool FIRST>
+__global__ void __launch_bounds__(RS_THREADS) rs_hist_kernel(const uint64_t *__restrict__ keys,
+                                                             const __grid_constant__ Triples tr, int64_t nnz,
                                                              int shift, int mask, int ntiles,
-                                                             int32_t *__restrict__ hist) {
+                                                             int32_t *__restrict__ hist, int32_t *err) {
     __shared__ int h[RS_BINS];
     const int t = threadIdx.x;
     h[t] = 0;
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * RS_TILE;
+    uint64_t key[RS_ROUNDS];
+    int bad = 0;
 #pragma unroll
     for (int j = 0; j < RS_ROUNDS; ++j) {
         const int64_t k = base + (int64_t)j * RS_THREADS + t;
-        if (k < nnz) atomicAdd(&h[digit_of(keys[k], shift, mask)], 1);
+        key[j] = 0;
+        if (k < nnz) {
+            if constexpr (FIRST)
+                key[j] = triple_key(tr, k, bad);
+            else
+                key[j] = keys[k];
+        }
     }
+#pragma unroll
+    for (int j = 0; j < RS_ROUNDS; ++j)
+        if (base + (int64_t)j * RS_THREADS + t < nnz) atomicAdd(&h[digit_of(key[j], shift, mask)], 1);
+    if (FIRST && bad) atomicOr(err, bad);
     __syncthreads();
     if (t <= mask) hist[(int64_t)t * ntiles + blockIdx.x] = h[t];
 }
 
-// exclusive scan of n int32 values in place: per-block sums, one-block scan of the sums, block scans
+// exclusive scan of n int32 values in place: per-block sums, then block scans that each begin by
+// adding up the sums before theirs
 constexpr int SC_THREADS = 1024, SC_ITEMS = 4, SC_CHUNK = SC_THREADS * SC_ITEMS;
 
 __device__ int block_exclusive_scan(int v, int *warp_tot, int &total) {
@@ -131,19 +192,6 @@ __global__ void __launch_bounds__(SC_THREADS) scan_sums_kernel(const int32_t *__
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(SC_THREADS) scan_top_kernel(int32_t *__restrict__ sums, int nb) {
-    __shared__ int wt[32];
-    int carry = 0;
-    for (int b0 = 0; b0 < nb; b0 += SC_THREADS) {
-        const int b = b0 + (int)threadIdx.x;
-        const int v = b < nb ? sums[b] : 0;
-        int total;
-        const int ex = block_exclusive_scan(v, wt, total);
-        if (b < nb) sums[b] = carry + ex;
-        carry += total;
-    }
-}
-
 __global__ void __launch_bounds__(SC_THREADS) scan_apply_kernel(int32_t *__restrict__ a, int64_t n,
                                                                 const int32_t *__restrict__ sums) {
     __shared__ int wt[32];
@@ -153,8 +201,11 @@ __global__ void __launch_bounds__(SC_THREADS) scan_apply_kernel(int32_t *__restr
         v[e] = base + e < n ? a[base + e] : 0;
         tot += v[e];
     }
-    int total;
-    int run = sums[blockIdx.x] + block_exclusive_scan(tot, wt, total);
+    int before = 0, total;
+    for (int q = threadIdx.x; q < (int)blockIdx.x; q += SC_THREADS) before += sums[q];
+    block_exclusive_scan(before, wt, total);
+    before = total;
+    int run = before + block_exclusive_scan(tot, wt, total);
     for (int e = 0; e < SC_ITEMS; ++e) {
         if (base + e < n) a[base + e] = run;
         run += v[e];
@@ -162,14 +213,18 @@ __global__ void __launch_bounds__(SC_THREADS) scan_apply_kernel(int32_t *__restr
 }
 
 // Stable scatter of a tile: every warp ranks its keys among its own of the same digit
-// (__match_any_sync, counters per warp), a scan over warps and digits gives their order in the
-// tile, and the keys go through shared memory in that order, so that the keys of a digit (8 on
-// average, 64 bytes) are written side by side to offs[d * ntiles + tile] and on.  Bound by the
-// 24 bytes a key moves; without the reordering the single 8- and 4-byte writes took 162 us a pass
-// of 10M keys.
+// (same_digit, counters per warp), a scan over warps and digits gives their order in the tile, and
+// the keys go through shared memory in that order, so that the keys of a digit (8 on average, 64
+// bytes) are written side by side to offs[d * ntiles + tile] and on.  The first pass reads the
+// triples themselves and the last one writes the sorted triples.  The 24 bytes a key moves set the
+// floor, 35 us a pass of 10M keys; the passes take 80 to 125 (104 with match instructions, and
+// 140 more for making the keys and taking them apart in kernels of their own; 162 without the
+// reordering).
 constexpr size_t RS_SMEM = RS_TILE * 12 + RS_WARPS * RS_BINS * 2 + RS_BINS * 8;
+template <bool FIRST, bool LAST>
 __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const uint64_t *__restrict__ kin,
-                                                                const uint32_t *__restrict__ pin, int64_t nnz, int shift,
+                                                                const uint32_t *__restrict__ pin,
+                                                                const __grid_constant__ Triples tr, int64_t nnz, int shift,
                                                                 int mask, int ntiles, const int32_t *__restrict__ offs,
                                                                 uint64_t *__restrict__ kout, uint32_t *__restrict__ pout,
                                                                 int32_t *err) {
@@ -190,8 +245,14 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const uint64_t *
 #pragma unroll
     for (int j = 0; j < RS_ROUNDS; ++j) {
         const int i = w * (32 * RS_ROUNDS) + 32 * j + lane;
-        key[j] = i < n ? kin[base + i] : 0;
-        pl[j] = i < n ? pin[base + i] : 0;
+        if constexpr (FIRST) {
+            int bad = 0;  // (reported by the histogram)
+            key[j] = i < n ? triple_key(tr, base + i, bad) : 0;
+            pl[j] = i < n ? triple_payload(tr, base + i) : 0;
+        } else {
+            key[j] = i < n ? kin[base + i] : 0;
+            pl[j] = i < n ? pin[base + i] : 0;
+        }
     }
     __syncthreads();
     uint16_t *mine = wcnt + w * RS_BINS;
@@ -199,7 +260,7 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const uint64_t *
     for (int j = 0; j < RS_ROUNDS; ++j) {
         const bool live = w * (32 * RS_ROUNDS) + 32 * j + lane < n;
         const int d = digit_of(key[j], shift, mask);
-        const unsigned peers = __match_any_sync(0xffffffffu, live ? d : -1);
+        const unsigned peers = same_digit(d, __ballot_sync(0xffffffffu, live));
         const int before = __popc(peers & ((1u << lane) - 1u));
         rank[j] = live ? (uint16_t)(mine[d] + before) : (uint16_t)0;
         __syncwarp();
@@ -235,33 +296,13 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const uint64_t *
         const uint64_t k = skey[i];
         const int64_t pos = (int64_t)gdelta[digit_of(k, shift, mask)] + i;
         if (pos >= 0 && pos < nnz) {
-            kout[pos] = k;
-            pout[pos] = spay[i];
+            if constexpr (LAST) {
+                triple_store(tr, pos, nnz, k, spay[i], err);
+            } else {
+                kout[pos] = k;
+                pout[pos] = spay[i];
+            }
         } else {
-            atomicOr(err, 8);
-        }
-    }
-}
-
-// sorted keys -> major (for the pointer array) and minor indices; the values from the payload, or
-// gathered by it (8-byte values: vals not NULL)
-template <typename W>
-__global__ void coo_unpack_kernel(const uint64_t *__restrict__ keys, const uint32_t *__restrict__ pay, int64_t nnz,
-                                  int n_minor, const W *__restrict__ vals, int32_t *__restrict__ major,
-                                  int32_t *__restrict__ minor, W *__restrict__ ovals, int32_t *err) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nnz; k += stride) {
-        const uint64_t key = keys[k];
-        const uint64_t j = key / (uint64_t)n_minor;
-        major[k] = (int32_t)j;
-        minor[k] = (int32_t)(key - j * (uint64_t)n_minor);
-        const uint32_t src = pay[k];
-        if (!vals) {
-            ovals[k] = (W)src;
-        } else if (src < nnz) {
-            ovals[k] = vals[src];
-        } else {
-            ovals[k] = W(0);
             atomicOr(err, 8);
         }
     }
@@ -305,45 +346,43 @@ spmv_status coo_sort(CooSort &cs, const int32_t *major, const int32_t *minor, co
     cs.own_bytes = ib + up((size_t)nnz * sv);
     if (dev_alloc(&cs.own, cs.own_bytes) != cudaSuccess) return set_error(SPMV_ERR_OOM, "sorted triples");
 
-    if (sv == 2)
-        coo_keys_kernel<uint16_t><<<grid, 256, 0, s>>>(major, minor, static_cast<const uint16_t *>(vals), nnz, n_major, n_minor, ka, pa, err);
-    else
-        coo_keys_kernel<uint32_t><<<grid, 256, 0, s>>>(major, minor, sv == 4 ? static_cast<const uint32_t *>(vals) : nullptr, nnz,
-                                                       n_major, n_minor, ka, pa, err);
     const uint64_t span = (uint64_t)n_major * (uint64_t)n_minor;
     const int bits = span > 1 ? 64 - __builtin_clzll(span - 1) : 0;
-    const int passes = (bits + RS_BITS - 1) / RS_BITS;
-    static SmemLimit lim;
-    if (ensure_smem_limit(rs_scatter_kernel, lim, (int)RS_SMEM) != cudaSuccess) return set_error(SPMV_ERR_CUDA, "sort launch failed");
+    const int passes = std::max(1, (bits + RS_BITS - 1) / RS_BITS);
+    Triples tr = {};
+    tr.major = major;
+    tr.minor = minor;
+    tr.vals = vals;
+    tr.vbytes = sv;
+    tr.n_major = n_major;
+    tr.n_minor = n_minor;
+    tr.recip = ~0ull / (uint64_t)n_minor;
+    tr.out_minor = static_cast<int32_t *>(cs.own);
+    tr.out_vals = static_cast<char *>(cs.own) + ib;
     for (int q = 0, shift = 0; q < passes; ++q) {  // passes of equal width, give or take a bit
         const int width = (bits - shift + passes - q - 1) / (passes - q), mask = (1 << width) - 1;
         const int64_t nhq = (int64_t)(mask + 1) * ntiles;
         const int nscq = (int)((nhq + SC_CHUNK - 1) / SC_CHUNK);
-        rs_hist_kernel<<<ntiles, RS_THREADS, 0, s>>>(ka, nnz, shift, mask, ntiles, hist);
+        const bool first = q == 0, last = q == passes - 1;
+        auto histogram = first ? rs_hist_kernel<true> : rs_hist_kernel<false>;
+        static SmemLimit lim[4];
+        auto scatter = first ? (last ? rs_scatter_kernel<true, true> : rs_scatter_kernel<true, false>)
+                             : (last ? rs_scatter_kernel<false, true> : rs_scatter_kernel<false, false>);
+        if (ensure_smem_limit(scatter, lim[2 * first + last], (int)RS_SMEM) != cudaSuccess)
+            return set_error(SPMV_ERR_CUDA, "sort launch failed");
+        tr.out_major = reinterpret_cast<int32_t *>(pb2);  // (the last pass writes no payload)
+        histogram<<<ntiles, RS_THREADS, 0, s>>>(ka, tr, nnz, shift, mask, ntiles, hist, err);
         scan_sums_kernel<<<nscq, SC_THREADS, 0, s>>>(hist, nhq, sums);
-        scan_top_kernel<<<1, SC_THREADS, 0, s>>>(sums, nscq);
         scan_apply_kernel<<<nscq, SC_THREADS, 0, s>>>(hist, nhq, sums);
-        rs_scatter_kernel<<<ntiles, RS_THREADS, RS_SMEM, s>>>(ka, pa, nnz, shift, mask, ntiles, hist, kb2, pb2, err);
+        scatter<<<ntiles, RS_THREADS, RS_SMEM, s>>>(ka, pa, tr, nnz, shift, mask, ntiles, hist, kb2, pb2, err);
         std::swap(ka, kb2);
         std::swap(pa, pb2);
         shift += width;
     }
-    int32_t *omin = static_cast<int32_t *>(cs.own);
-    void *ovals = static_cast<char *>(cs.own) + ib;
-    int32_t *omaj = reinterpret_cast<int32_t *>(pb2);  // the free payload buffer
-    if (sv == 8)
-        coo_unpack_kernel<uint64_t><<<grid, 256, 0, s>>>(ka, pa, nnz, n_minor, static_cast<const uint64_t *>(vals), omaj,
-                                                         omin, static_cast<uint64_t *>(ovals), err);
-    else if (sv == 4)
-        coo_unpack_kernel<uint32_t><<<grid, 256, 0, s>>>(ka, pa, nnz, n_minor, nullptr, omaj, omin,
-                                                         static_cast<uint32_t *>(ovals), err);
-    else
-        coo_unpack_kernel<uint16_t><<<grid, 256, 0, s>>>(ka, pa, nnz, n_minor, nullptr, omaj, omin,
-                                                         static_cast<uint16_t *>(ovals), err);
     if (cudaGetLastError() != cudaSuccess) return set_error(SPMV_ERR_CUDA, "sort launch failed");
-    *major_sorted = omaj;
-    *minor_sorted = omin;
-    *vals_sorted = ovals;
+    *major_sorted = tr.out_major;
+    *minor_sorted = tr.out_minor;
+    *vals_sorted = tr.out_vals;
     return SPMV_OK;
 }
 
