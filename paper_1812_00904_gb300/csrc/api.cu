@@ -62,13 +62,14 @@ cudaError_t launch_pass(const spmv_plan_s *p, bool sc, bool sd, const PassParams
 }
 
 // Shared memory of a one-vector pass: the accumulator (sc), the input vector (sd), a staging slot for
-// each of as many warps as fit, and what is left over for more copies of the accumulator.  Measured on
-// the 200M-nonzero wide matrix (m = 20,000; us): more warps always help (pair 420 / 481 / 537 / 627
-// at 32 / 24 / 20 / 16 warps).  The dot products alone take two slots a warp (279 against 286
-// with one); with the accumulator one slot and the room for a second copy are better (317 against
-// 345: an addition is a compare-and-swap loop, repeated when another warp got in between).
-// On the tall matrix (n = 2,000) the accumulating pass takes 438 / 378 / 335 / 306 / 276 us with
-// 1 / 2 / 4 / 8 / 16 copies, the pair 433 / 412 / 399 / 391 / 381; 32 copies add nothing.
+// each of as many warps as fit, and what is left over for more copies of the accumulator.  More warps
+// always help: the pair, the accumulating product and the dot products of the 200M-nonzero wide
+// matrix (m = 20,000) take 590 / 427 / 374 us with 16 warps, 501 / 374 / 326 with 20, 449 / 341 / 301
+// with 24, 417 / 322 / 281 with 28, 389 / 305 / 263 with 32.  A second slot a warp is no gain
+// (dot products 269 to 280).  An addition is a compare-and-swap loop, repeated when another warp got
+// in between, so copies help where they fit: with 1 / 2 / 4 / 8 / 16 of them the accumulating
+// product of the 150M-nonzero tall matrix (n = 2,000) takes 450 / 393 / 348 / 318 / 281 us, the pair
+// 441 / 419 / 406 / 393 / 372; 32 add nothing.
 size_t pass_acc_bytes(const spmv_plan_s *p) { return align_up((size_t)p->n_minor * p->sa, 128); }
 size_t pass_vec_bytes(const spmv_plan_s *p) { return align_up((size_t)p->n_minor * p->sx, 128); }
 constexpr int PASS_MAX_COPIES = 16;
@@ -96,8 +97,8 @@ PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1) {
     return g;
 }
 // A pass runs with at least 8 warps (or all a CTA has tiles for): fewer leave it to the streaming
-// kernel.  The pair wants 20, below which its two products run faster one by one (317 + 279 us
-// with 32 warps each, against 537 with 20 and 627 with 16).
+// kernel.  The pair wants 20: with 16 its two products run faster one by one, each with 32 warps
+// (305 + 263 us against 590; 501 with 20).
 bool pass_fits(const spmv_plan_s *p, bool sc, bool sd) {
     return pass_geometry(p, sc, sd).warps >= std::min(sc && sd ? std::min(20, pass_warps(p->sv)) : 8, cta_tiles(p));
 }
@@ -383,7 +384,10 @@ static spmv_status run_mvscatter(spmv_plan_s *p, int kb, const void *const *in, 
 }
 
 // The dot products of kb = 2 .. 8 vectors of a plan with step records (32-bit accumulation), the
-// vectors interleaved; on chip when that leaves room for all but a quarter of the warps.
+// vectors interleaved; on chip when that leaves room for enough warps: half for 2 vectors (77 us
+// against 103 through L2, 25M nonzeros, 18 of 24 warps; 101 against 110 with 14), three quarters for 4
+// (15 of 20 warps: 101 either way; 13: 129 against 103), all but one for 8 (15 of 16 warps: 141
+// against 147; 14: 150 against 147).
 static spmv_status run_mvdot(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s) {
     const int kv = kb <= 2 ? 2 : kb <= 4 ? 4 : 8;
     spmv_status st = interleave_inputs(p, kv, kb, in, p->n_minor, s);
@@ -396,7 +400,7 @@ static spmv_status run_mvdot(spmv_plan_s *p, int kb, const void *const *in, void
     const int most = std::min(mvdot_warps(kv), cta_tiles(p));
     const size_t room = (size_t)p->smem_max - PASS_BAR_BYTES;
     const size_t fit = room > vec ? (room - vec) / slot : 0;
-    const bool onchip = fit >= (size_t)(most - most / 4);
+    const bool onchip = fit >= (size_t)(kv == 2 ? (most + 1) / 2 : kv == 4 ? most - most / 4 : most - most / 16);
     const int warps = onchip ? (int)std::min<size_t>(most, fit) : most;
     pp.slots = onchip ? (int)std::min<size_t>(PASS_MAX_SLOTS, fit / warps) : PASS_MAX_SLOTS;
     pp.vec_bytes = onchip ? (int)vec : 0;
@@ -893,12 +897,15 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
         p->pass_sd = pass_fits(p, false, true);
         p->pass_pair = pass_fits(p, true, true);
         p->pass_mv = p->sv != 8;
-        // vectors per accumulating pass: as many as leave room for nearly all of the warps' staging
+        // vectors per accumulating pass: as many as leave room for three quarters of the warps'
+        // staging.  One pass at 24 to 27 of 32 warps against two of half as many vectors (25M
+        // nonzeros, us): 2 vectors 120 / 136 (m = 22,500), 4 174 / 187 (11,300), 8 258 / 270 (5,500);
+        // at 18 to 20 warps 150 / 134 (24,200), 198 / 186 (11,800), 318 / 271 (5,900).
         if (p->pass_mv && p->pass_sc) {
             const int full = std::min(pass_warps(p->sv), cta_tiles(p));
             p->batch_width = 1;
             for (int kv : {8, 4, 2})
-                if (p->batch_width == 1 && pass_geometry(p, true, false, kv).warps >= full - full / 8) p->batch_width = kv;
+                if (p->batch_width == 1 && pass_geometry(p, true, false, kv).warps >= full - full / 4) p->batch_width = kv;
         }
     }
     const size_t part_bytes =

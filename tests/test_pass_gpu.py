@@ -128,6 +128,28 @@ def test_several_vectors(short, layout, dtype):
                     assert torch.equal(R[b], plan.spvtm(Z[b]) if op == pkg.SPMV_OP_VTA else plan.spmv(Z[b]))
 
 
+@pytest.mark.parametrize("layout", ["csc", "csr"])
+@pytest.mark.parametrize("short,k", [(5_500, 8), (6_252, 8), (11_400, 4), (22_500, 2), (25_500, 2)])
+def test_several_vectors_beside_few_warps(short, k, layout):
+    """CTAs with tiles for all their warps, and accumulators or interleaved vectors that leave room for
+    some of them only: the batch against the oracle, its dot products the single ones' bits."""
+    rng = np.random.default_rng(short)
+    deg = rng.integers(0, 80, 32_000)  # 1.26M nonzeros: 32 tiles a CTA
+    m, n = (short, len(deg)) if layout == "csc" else (len(deg), short)
+    A = synth.random_matrix(m, n, layout, degrees=deg, seed=k, duplicates=True)
+    plan, stored = make_plan(A, torch.float32, tile_items=256)
+    for op, ln, ref, scale in ((pkg.SPMV_OP_AX, n, oracle.spmv, oracle.abs_spmv),
+                               (pkg.SPMV_OP_VTA, m, oracle.spvtm, oracle.abs_spvtm)):
+        Z = torch.stack([dev_vec(synth.uniform_vector(ln, 10 + b), torch.float32) for b in range(k)])
+        R = plan.batch(op, Z)
+        plan.check()
+        for b in range(k):
+            z = host_of(Z[b])
+            assert_close(host_of(R[b]), ref(stored, z), scale(stored, z), TOL[torch.float32], f"{layout} {op} vector {b}")
+            if (op == pkg.SPMV_OP_VTA) == (layout == "csc"):
+                assert torch.equal(R[b], plan.spvtm(Z[b]) if op == pkg.SPMV_OP_VTA else plan.spmv(Z[b]))
+
+
 def test_row_blocks_in_turn():
     """Windows of the long vector too wide for one block a CTA: several blocks in turn, each restaging
     its window; the same bits as the streaming kernel's multi-vector pass over the same copy."""
