@@ -7,9 +7,15 @@
 // and tries again.  The allocations and frees go through a stream of the pool's own: memory is
 // handed out after that stream was waited for, so it can be used on any stream, and the caller
 // frees memory only when no work that uses it is pending.  Every call is safe from any thread.
+//
+// Blocks of more than half of what the pool keeps bypass it: a pool grows at 0.87 us per MB and gives
+// back at 2.5 (256 MB: 228 us and 1.0 ms; 2 GB: 1.7 and 13 ms), cudaMalloc and cudaFree take 56 + 197
+// us for 256 MB and 0.1 + 1.4 ms for 2 GB, while a kept block costs 2 us.  (A bank-ordered plan of
+// 200M nonzeros: 14.5 ms with its 2.4 GB from the pool, 13.0 without.)
 #include <cuda_runtime.h>
 
 #include <mutex>
+#include <unordered_set>
 
 #include "plan_impl.h"
 
@@ -17,6 +23,7 @@ namespace gbk {
 namespace {
 
 constexpr uint64_t POOL_KEEP = 512ull << 20;
+constexpr size_t POOL_MOST = POOL_KEEP / 2;  // bytes of a block from the pool
 
 struct DevicePool {
     std::once_flag once;
@@ -24,6 +31,9 @@ struct DevicePool {
     cudaStream_t stream = nullptr;
 };
 DevicePool g_pools[MAX_DEVICES];
+
+std::mutex g_large_mu;
+std::unordered_set<void *> g_large;  // the blocks that bypassed the pool
 
 DevicePool &pool_of(int device) {
     DevicePool &P = g_pools[device];
@@ -58,6 +68,22 @@ cudaError_t dev_alloc(void **p, size_t bytes) {
     if (device < 0 || device >= MAX_DEVICES) return cudaErrorInvalidDevice;
     DevicePool &P = pool_of(device);
     if (!P.pool) return cudaMalloc(p, bytes);
+    if (bytes > POOL_MOST) {
+        e = cudaMalloc(p, bytes);
+        if (e == cudaErrorMemoryAllocation) {  // what the pool keeps may make room
+            cudaGetLastError();
+            cudaStreamSynchronize(P.stream);
+            cudaMemPoolTrimTo(P.pool, 0);
+            e = cudaMalloc(p, bytes);
+        }
+        if (e != cudaSuccess) {
+            *p = nullptr;
+            return e;
+        }
+        std::lock_guard<std::mutex> lk(g_large_mu);
+        g_large.insert(*p);
+        return cudaSuccess;
+    }
     for (int attempt = 0; attempt < 2; ++attempt) {
         e = cudaMallocFromPoolAsync(p, bytes, P.pool, P.stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(P.stream);
@@ -74,7 +100,12 @@ cudaError_t dev_alloc(void **p, size_t bytes) {
 
 void dev_free(void *p, int device) {
     if (!p) return;
-    if (device >= 0 && device < MAX_DEVICES && g_pools[device].pool) {
+    bool large;
+    {
+        std::lock_guard<std::mutex> lk(g_large_mu);
+        large = g_large.erase(p) != 0;
+    }
+    if (!large && device >= 0 && device < MAX_DEVICES && g_pools[device].pool) {
         cudaFreeAsync(p, g_pools[device].stream);
     } else {
         cudaFree(p);
