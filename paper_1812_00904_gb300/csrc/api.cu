@@ -388,9 +388,12 @@ static spmv_status run_mvscatter(spmv_plan_s *p, int kb, const void *const *in, 
 // against 103 through L2, 25M nonzeros, 18 of 24 warps; 101 against 110 with 14), three quarters for 4
 // (15 of 20 warps: 101 either way; 13: 129 against 103), all but one for 8 (15 of 16 warps: 141
 // against 147; 14: 150 against 147).
-static spmv_status run_mvdot(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s) {
+// in_len: entries of each input (the vectors that a row-sorted copy's windows lie in).  The launches
+// are timed as kernels id_dot / id_fix of plan `prof`.
+static spmv_status run_mvdot(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s,
+                             spmv_plan_s *prof, int id_dot, int id_fix, int64_t in_len) {
     const int kv = kb <= 2 ? 2 : kb <= 4 ? 4 : 8;
-    spmv_status st = interleave_inputs(p, kv, kb, in, p->n_minor, s);
+    spmv_status st = interleave_inputs(p, kv, kb, in, in_len >= 0 ? in_len : p->n_minor, s);
     if (st != SPMV_OK) return st;
     PassParams pp = pass_params(p);
     pp.v = p->vt;
@@ -402,18 +405,19 @@ static spmv_status run_mvdot(spmv_plan_s *p, int kb, const void *const *in, void
     const size_t fit = room > vec ? (room - vec) / slot : 0;
     const bool onchip = fit >= (size_t)(kv == 2 ? (most + 1) / 2 : kv == 4 ? most - most / 4 : most - most / 16);
     const int warps = onchip ? (int)std::min<size_t>(most, fit) : most;
-    pp.slots = onchip ? (int)std::min<size_t>(PASS_MAX_SLOTS, fit / warps) : PASS_MAX_SLOTS;
+    // (one slot a warp where blocks take turns: StepFeed::start)
+    pp.slots = p->bpc > 1 ? 1 : onchip ? (int)std::min<size_t>(PASS_MAX_SLOTS, fit / warps) : PASS_MAX_SLOTS;
     pp.vec_bytes = onchip ? (int)vec : 0;
     const size_t smem = pp.vec_bytes + PASS_BAR_BYTES + (size_t)warps * pp.slots * slot;
     {
-        ProfScope ps(p, 2, s);
+        ProfScope ps(prof, id_dot, s);
         CUDA_TRY(p->val_t == SPMV_F32    ? launch_mvdot_f32(kv, onchip, pp, p->ctas, warps, (int)smem, s)
                  : p->val_t == SPMV_BF16 ? launch_mvdot_bf16(kv, onchip, pp, p->ctas, warps, (int)smem, s)
                                          : launch_mvdot_f16(kv, onchip, pp, p->ctas, warps, (int)smem, s));
     }
     const spmv_plan_s::ProcZones &pz = p->pz;
     if (pz.z > 0) {
-        ProfScope ps(p, 3, s);
+        ProfScope ps(prof, id_fix, s);
         CUDA_TRY(launch_fixup(false, pz.zones, pz.z, p->rec_left, p->rec_right, pz.nproc, kb, out, s));
     }
     return SPMV_OK;
@@ -475,7 +479,7 @@ static spmv_status run_segdot_impl(spmv_plan_s *p, int kb, const void *const *in
         for (int g0 = 0; g0 < kb; g0 += grp) {
             const int kg = std::min(grp, kb - g0);
             spmv_status st = kg == 1 ? run_segdot_impl(p, 1, in + g0, out + g0, s, prof, id_dot, id_fix, in_len)
-                                : p->pass_mv ? run_mvdot(p, kg, in + g0, out + g0, s)
+                                : p->pass_mv ? run_mvdot(p, kg, in + g0, out + g0, s, prof, id_dot, id_fix, in_len)
                                              : run_segdot_global(p, kg, in + g0, out + g0, s, prof, id_dot, id_fix, in_len);
             if (st != SPMV_OK) return st;
         }
@@ -517,7 +521,7 @@ spmv_status run_segdot(spmv_plan_s *p, int kb, const void *const *in, void *cons
 // windowed segmented pass writes every block's short vector into ypart (its fix-up completes
 // the entries split between chunks), then the blocks' vectors are added in FP64 in block
 // order (Sec. III step 2).  One vector runs with its windows on chip; several (seg_group per
-// pass) read their windows through L2 from an interleaved copy of the long vectors, into
+// pass) take theirs from an interleaved copy of the long vectors, on chip or through L2, into
 // per-block vectors [vector][block][n_minor] (a plan-owned buffer made on first use).
 static spmv_status run_row_blocks(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s) {
     spmv_plan_s *q = p->tplan;
@@ -749,7 +753,8 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
         p->T = opts->tile_items;
     } else {
         // (an unvalidated plan or one with its short vector in global memory never runs the
-        // one-vector passes, which want tiles of whole 256-position steps)
+        // passes, which want tiles of whole 256-position steps: of tiles of 104, as small matrices
+        // had, 60% of a step was padding)
         const int64_t fill = (int64_t)sms * 16 * 2;
         if (!(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL)))
             p->T = nnz < fill * 512 ? 256 : 512;
@@ -890,8 +895,9 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     }
     // the one-vector passes serve validated plans with whole-step tiles whose short vectors fit in
     // shared memory beside the staging slots of enough warps
-    if (pi && nnz > 0 && p->T % 256 == 0) {  // the row-sorted copy: its single-vector dot products
+    if (pi && nnz > 0 && p->T % 256 == 0) {  // the row-sorted copy: its dot products
         p->pass_sd = pass_fits(p, false, true);
+        p->pass_mv = p->pass_sd && p->sv != 8;
     } else if (nnz > 0 && p->T % 256 == 0 && !(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL))) {
         p->pass_sc = pass_fits(p, true, false);
         p->pass_sd = pass_fits(p, false, true);

@@ -1,6 +1,7 @@
-// One-vector passes over the nonzeros of a validated plan: the accumulating product (SC: acc[idx[k]] += val[k] * x[seg(k)], A_(i) x_(i) of Sec. III),
-// the dot products (SD: u[j] = sum_k val[k] * v[idx[k]], v^T A_(i) of Sec. IV-A), or both from
-// one reading of the matrix.
+// One-vector passes over the nonzeros of a validated plan: the accumulating product (SC: acc[idx[k]] +=
+// val[k] * x[seg(k)], A_(i) x_(i) of Sec. III), the dot products (SD: u[j] = sum_k val[k] * v[idx[k]],
+// v^T A_(i) of Sec. IV-A), or both from one reading of the matrix; the passes of several vectors and
+// the values' gradient over the same steps.
 //
 // The tiles, chunks (the processors of Sec. II), masks and carry records are those of the
 // streaming kernel, and the dot products are formed with its operations in its order (lane
@@ -131,6 +132,14 @@ template <typename VT, bool VALS = true> struct StepFeed {
     }
 };
 
+// 32 warps of 64 registers (FP64: 16 of 128) with one step of 256 nonzeros in flight each: 66 KB, more
+// than the latency of memory needs, and warps enough to hide the chains of a step (scan, additions).
+// SC and the pair are bound by the shared-memory pipe (76 to 92% of its cycles): an FP32 addition is a
+// load and a compare-and-swap that costs two, each with the bank conflicts of 32 rows.  SD alone
+// runs near the memory rate, FP64 at the rate of its pipe (2 operations a cycle per SM).  With the
+// combine and fix-up, streaming kernel before, this one now (us): 200M FP32 nonzeros, m = 20,000, bank
+// order: pair 640 -> 386, SC 362 -> 305, SD 303 -> 263; 150M, n = 2,000: pair 538 -> 369, SC 313 ->
+// 276, SD 242 -> 207; 8M FP64, n = 4,000: pair 121 -> 79, SC 62 -> 59, SD 69 -> 48.
 template <typename VT, typename XT, bool SC, bool SD, int WB>
 __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant__ PassParams p) {
     using AT = typename Acc<VT>::type;
@@ -161,240 +170,240 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
     // the row-sorted copy's blocks take turns, each with its window of the input; else one block a CTA
     const int bpc = SD && !SC ? p.bpc : 1;
 #pragma unroll 1
-    for (int hb_ = 0; hb_ < bpc; ++hb_) {
-    const int gb = blockIdx.x * bpc + hb_;
-    if (hb_ > 0) __syncthreads();  // every warp is done with the block before
-    feed.start(gb, gridDim.x * bpc, hb_ > 0);
-    if constexpr (SD) {
-        if (hb_ == 0)
-            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x)
-                static_cast<XT *>(p.u)[p.emptylist[i]] = XT(0);
-        constexpr int xa = 16 / (int)sizeof(XT);
-        const XT *src = static_cast<const XT *>(p.v);
-        int len = p.n_minor;
-        if (!SC && p.win) {  // (windows begin on 16 bytes)
-            const int2 w = p.win[gb];
-            src += w.x;
-            len = min(w.y, p.n_minor);
-        }
-        const int n16 = len / xa;
+    for (int turn = 0; turn < bpc; ++turn) {
+        const int gb = blockIdx.x * bpc + turn;
+        if (turn > 0) __syncthreads();  // every warp is done with the block before
+        feed.start(gb, gridDim.x * bpc, turn > 0);
+        if constexpr (SD) {
+            if (turn == 0)
+                for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x)
+                    static_cast<XT *>(p.u)[p.emptylist[i]] = XT(0);
+            constexpr int xa = 16 / (int)sizeof(XT);
+            const XT *src = static_cast<const XT *>(p.v);
+            int len = p.n_minor;
+            if (!SC && p.win) {  // (windows begin on 16 bytes)
+                const int2 w = p.win[gb];
+                src += w.x;
+                len = min(w.y, p.n_minor);
+            }
+            const int n16 = len / xa;
 #pragma unroll 4
-        for (int i = threadIdx.x; i < n16; i += blockDim.x)
-            reinterpret_cast<float4 *>(vs)[i] = __ldg(reinterpret_cast<const float4 *>(src) + i);
-        for (int i = n16 * xa + threadIdx.x; i < len; i += blockDim.x) vs[i] = __ldg(src + i);
-    }
-    __syncthreads();
+            for (int i = threadIdx.x; i < n16; i += blockDim.x)
+                reinterpret_cast<float4 *>(vs)[i] = __ldg(reinterpret_cast<const float4 *>(src) + i);
+            for (int i = n16 * xa + threadIdx.x; i < len; i += blockDim.x) vs[i] = __ldg(src + i);
+        }
+        __syncthreads();
 
-    AT chi = AT(0), clo = AT(0);  // open segment's running sum (SD)
-    int cfirst = -1;              // the chunk's first segment when its sum goes to the left record
-    while (feed.next(slot, hdr)) {
-        const int ps = hdr.x << 8;
-        const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
-        const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);  // first, flags
-        // the step's segments are columns (rows of a tall matrix) first, first + 1, ..; with empty
-        // ones between them they are counted by rank and looked up
-        const bool gaps = (bf.y & STEP_GAPS) != 0;
-        const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
-        auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
-        const bool whole = p.nnz - ps >= 256;
-        // With SD this lane takes positions 8 lane .. 8 lane + 7, register e holding position
-        // e ^ (4 sw) (staggered loads, which touch every bank exactly four times an instruction);
-        // SC alone takes positions 32 e + lane (consecutive lanes then hold distinct rows of a
-        // segment, and neighbouring entries of the long vector).
-        int ix[8];
-        AT va[8];
-        if (whole && !SD) {
-            const int32_t *is = reinterpret_cast<const int32_t *>(slot);
-            const VT *vv = reinterpret_cast<const VT *>(slot + Feed::OFF_VAL);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                ix[e] = is[32 * e + lane];
-                va[e] = to_acc<AT>(vv[32 * e + lane]);
-            }
-        } else if (whole) {
-            stag8_idx(reinterpret_cast<const int32_t *>(slot), 8 * lane, sw, ix);
-            Stag8<VT, AT>::run(slot + Feed::OFF_VAL, 8 * lane, sw, va);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int pos = ps + (SD ? 8 * lane + (e ^ (4 * sw)) : 32 * e + lane);
-                const bool in = pos < p.nnz;
-                ix[e] = in ? __ldg(p.idx + pos) : 0;
-                va[e] = in ? to_acc<AT>(static_cast<const VT *>(p.vals)[pos]) : AT(0);
-            }
-        }
-        uint32_t hb = 0;
-        int L = base;  // segment open before the lane's positions
-        uint32_t w[8];
-        if constexpr (SD) {
-            const uint32_t mw = rec->heads[lane >> 2];
-            hb = (mw >> sh) & 0xFFu;
-            L += rec->before[lane >> 2] + __popc(mw & ((1u << sh) - 1u));
-        } else {
-            const uint4 wa = reinterpret_cast<const uint4 *>(rec->heads)[0], wb = reinterpret_cast<const uint4 *>(rec->heads)[1];
-            w[0] = wa.x; w[1] = wa.y; w[2] = wa.z; w[3] = wa.w;
-            w[4] = wb.x; w[5] = wb.y; w[6] = wb.z; w[7] = wb.w;
-        }
-        feed.release();
-        const unsigned bal = SD ? __ballot_sync(FULL, hb != 0u) : static_cast<unsigned>(bf.y >> 16);  // 0: no head
-        AT a[8], c[8];
-        if constexpr (SC) {  // the long vector's entries
-            if (bal == 0u) {
-                const AT xv = static_cast<AT>(__ldg(xg + col_of(L)));
-#pragma unroll
-                for (int e = 0; e < 8; ++e) c[e] = xv;
-            } else if (!SD) {
-                const uint32_t lane_le = FULL >> (31 - lane);
+        AT chi = AT(0), clo = AT(0);  // open segment's running sum (SD)
+        int cfirst = -1;              // the chunk's first segment when its sum goes to the left record
+        while (feed.next(slot, hdr)) {
+            const int ps = hdr.x << 8;
+            const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
+            const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);  // first, flags
+            // the step's segments are columns (rows of a tall matrix) first, first + 1, ..; with empty
+            // ones between them they are counted by rank and looked up
+            const bool gaps = (bf.y & STEP_GAPS) != 0;
+            const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
+            auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
+            const bool whole = p.nnz - ps >= 256;
+            // With SD this lane takes positions 8 lane .. 8 lane + 7, register e holding position
+            // e ^ (4 sw) (staggered loads, which touch every bank exactly four times an instruction);
+            // SC alone takes positions 32 e + lane (consecutive lanes then hold distinct rows of a
+            // segment, and neighbouring entries of the long vector).
+            int ix[8];
+            AT va[8];
+            if (whole && !SD) {
+                const int32_t *is = reinterpret_cast<const int32_t *>(slot);
+                const VT *vv = reinterpret_cast<const VT *>(slot + Feed::OFF_VAL);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
-                    c[e] = static_cast<AT>(__ldg(xg + col_of(L + __popc(w[e] & lane_le))));
-                    L += __popc(w[e]);
+                    ix[e] = is[32 * e + lane];
+                    va[e] = to_acc<AT>(vv[32 * e + lane]);
                 }
+            } else if (whole) {
+                stag8_idx(reinterpret_cast<const int32_t *>(slot), 8 * lane, sw, ix);
+                Stag8<VT, AT>::run(slot + Feed::OFF_VAL, 8 * lane, sw, va);
             } else {
-                const int nlo = __popc(hb & 0xFu);
-                const uint32_t h1 = sw ? hb >> 4 : hb, h2 = sw ? hb : hb >> 4;
-                int cc = sw ? L + nlo : L;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
-                    if (e == 4) cc = sw ? L : L + nlo;
-                    cc += ((e < 4 ? h1 : h2) >> (e & 3)) & 1u;
-                    // (-1 in the first step: empty segments before the first nonzero, whose head counts)
-                    c[e] = static_cast<AT>(__ldg(xg + col_of(cc)));
+                    const int pos = ps + (SD ? 8 * lane + (e ^ (4 * sw)) : 32 * e + lane);
+                    const bool in = pos < p.nnz;
+                    ix[e] = in ? __ldg(p.idx + pos) : 0;
+                    va[e] = in ? to_acc<AT>(static_cast<const VT *>(p.vals)[pos]) : AT(0);
                 }
             }
-        }
-        if constexpr (SD) {
-            if (hdr.y & 2) cfirst = (bf.y & STEP_NEED_LEFT) ? bf.x : -1;  // (a column)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) a[e] = static_cast<AT>(vs[ix[e]]);
-        }
-        if constexpr (sizeof(AT) == 4) {  // (FP64 multiplies in the additions)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                if constexpr (SC) c[e] *= va[e];
-                if constexpr (SD) a[e] = mul_rn(va[e], a[e]);
-            }
-        }
-        if (!whole) {  // positions past the last nonzero (zero times an infinity is no zero)
-            const int nv = p.nnz - ps;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                if ((SD ? 8 * lane + (e ^ (4 * sw)) : 32 * e + lane) >= nv) {
-                    if constexpr (SD) a[e] = AT(0);
-                    if constexpr (SC) c[e] = AT(0);
-                }
-            }
-        }
-        if constexpr (SC) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                if constexpr (sizeof(AT) == 4) {
-                    atomicAdd(acc + ix[e], c[e]);
-                } else {
-                    acc_fma(acc + ix[e], va[e], c[e]);
-                }
-            }
-        }
-        if constexpr (SD) {  // into the order of the positions
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const AT lo = sw ? a[e + 4] : a[e];
-                a[e + 4] = sw ? a[e] : a[e + 4];
-                a[e] = lo;
-                if constexpr (sizeof(AT) == 8) {
-                    const AT vl = sw ? va[e + 4] : va[e];
-                    va[e + 4] = sw ? va[e] : va[e + 4];
-                    va[e] = vl;
-                }
-            }
-        }
-        if constexpr (SD) {
-            // position e's term (FP32: its product) added to s, or alone where a segment starts
-            auto next_term = [&](int e, AT s, bool restart) -> AT {
-                if constexpr (sizeof(AT) == 8) {
-                    return seg_term(va[e], a[e], s, restart);
-                } else {
-                    return restart ? a[e] : s + a[e];
-                }
-            };
-            auto first_term = [&](int e) -> AT { return next_term(e, AT(0), true); };
-            if (bal == 0u) {
-                // the open segment runs through the step: butterfly total, compensated carry
-                AT s = first_term(0);
-#pragma unroll
-                for (int e = 1; e < 8; ++e) s = next_term(e, s, false);
-#pragma unroll
-                for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(FULL, s, d);
-                carry_in(chi, clo, s);
+            uint32_t hb = 0;
+            int L = base;  // segment open before the lane's positions
+            uint32_t w[8];
+            if constexpr (SD) {
+                const uint32_t mw = rec->heads[lane >> 2];
+                hb = (mw >> sh) & 0xFFu;
+                L += rec->before[lane >> 2] + __popc(mw & ((1u << sh) - 1u));
             } else {
-                // lane prefix restarted at every head; f: what the lane's first head closes
-                const uint32_t h1 = hb & (0u - hb), hr = hb ^ h1;
-                AT s = first_term(0), f = AT(0);
+                const uint4 wa = reinterpret_cast<const uint4 *>(rec->heads)[0], wb = reinterpret_cast<const uint4 *>(rec->heads)[1];
+                w[0] = wa.x; w[1] = wa.y; w[2] = wa.z; w[3] = wa.w;
+                w[4] = wb.x; w[5] = wb.y; w[6] = wb.z; w[7] = wb.w;
+            }
+            feed.release();
+            const unsigned bal = SD ? __ballot_sync(FULL, hb != 0u) : static_cast<unsigned>(bf.y >> 16);  // 0: no head
+            AT a[8], c[8];
+            if constexpr (SC) {  // the long vector's entries
+                if (bal == 0u) {
+                    const AT xv = static_cast<AT>(__ldg(xg + col_of(L)));
 #pragma unroll
-                for (int e = 1; e < 8; ++e) {
-                    if ((h1 >> e) & 1u) f = s;
-                    s = next_term(e, s, (hb >> e) & 1u);
+                    for (int e = 0; e < 8; ++e) c[e] = xv;
+                } else if (!SD) {
+                    const uint32_t lane_le = FULL >> (31 - lane);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        c[e] = static_cast<AT>(__ldg(xg + col_of(L + __popc(w[e] & lane_le))));
+                        L += __popc(w[e]);
+                    }
+                } else {
+                    const int nlo = __popc(hb & 0xFu);
+                    const uint32_t h1 = sw ? hb >> 4 : hb, h2 = sw ? hb : hb >> 4;
+                    int cc = sw ? L + nlo : L;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        if (e == 4) cc = sw ? L : L + nlo;
+                        cc += ((e < 4 ? h1 : h2) >> (e & 3)) & 1u;
+                        // (-1 in the first step: empty segments before the first nonzero, whose head counts)
+                        c[e] = static_cast<AT>(__ldg(xg + col_of(cc)));
+                    }
                 }
-                if (hr) {  // segments inside the lane: closed by its later heads
-                    AT q = first_term(0);
-                    int cc = L;
+            }
+            if constexpr (SD) {
+                if (hdr.y & 2) cfirst = (bf.y & STEP_NEED_LEFT) ? bf.x : -1;  // (a column)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) a[e] = static_cast<AT>(vs[ix[e]]);
+            }
+            if constexpr (sizeof(AT) == 4) {  // (FP64 multiplies in the additions)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    if constexpr (SC) c[e] *= va[e];
+                    if constexpr (SD) a[e] = mul_rn(va[e], a[e]);
+                }
+            }
+            if (!whole) {  // positions past the last nonzero (zero times an infinity is no zero)
+                const int nv = p.nnz - ps;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    if ((SD ? 8 * lane + (e ^ (4 * sw)) : 32 * e + lane) >= nv) {
+                        if constexpr (SD) a[e] = AT(0);
+                        if constexpr (SC) c[e] = AT(0);
+                    }
+                }
+            }
+            if constexpr (SC) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    if constexpr (sizeof(AT) == 4) {
+                        atomicAdd(acc + ix[e], c[e]);
+                    } else {
+                        acc_fma(acc + ix[e], va[e], c[e]);
+                    }
+                }
+            }
+            if constexpr (SD) {  // into the order of the positions
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const AT lo = sw ? a[e + 4] : a[e];
+                    a[e + 4] = sw ? a[e] : a[e + 4];
+                    a[e] = lo;
+                    if constexpr (sizeof(AT) == 8) {
+                        const AT vl = sw ? va[e + 4] : va[e];
+                        va[e + 4] = sw ? va[e] : va[e + 4];
+                        va[e] = vl;
+                    }
+                }
+            }
+            if constexpr (SD) {
+                // position e's term (FP32: its product) added to s, or alone where a segment starts
+                auto next_term = [&](int e, AT s, bool restart) -> AT {
+                    if constexpr (sizeof(AT) == 8) {
+                        return seg_term(va[e], a[e], s, restart);
+                    } else {
+                        return restart ? a[e] : s + a[e];
+                    }
+                };
+                auto first_term = [&](int e) -> AT { return next_term(e, AT(0), true); };
+                if (bal == 0u) {
+                    // the open segment runs through the step: butterfly total, compensated carry
+                    AT s = first_term(0);
+#pragma unroll
+                    for (int e = 1; e < 8; ++e) s = next_term(e, s, false);
+#pragma unroll
+                    for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(FULL, s, d);
+                    carry_in(chi, clo, s);
+                } else {
+                    // lane prefix restarted at every head; f: what the lane's first head closes
+                    const uint32_t h1 = hb & (0u - hb), hr = hb ^ h1;
+                    AT s = first_term(0), f = AT(0);
 #pragma unroll
                     for (int e = 1; e < 8; ++e) {
-                        if ((hr >> e) & 1u) {
-                            ++cc;
-                            static_cast<XT *>(p.u)[col_of(cc)] = static_cast<XT>(q);
-                        }
-                        q = next_term(e, q, (hb >> e) & 1u);
+                        if ((h1 >> e) & 1u) f = s;
+                        s = next_term(e, s, (hb >> e) & 1u);
                     }
-                }
-                // segmented scan of the lanes' open sums
-                const unsigned le = bal & (FULL >> (31 - lane));
-                const int reach = le ? lane - (31 - __clz(le)) : lane;
+                    if (hr) {  // segments inside the lane: closed by its later heads
+                        AT q = first_term(0);
+                        int cc = L;
 #pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    // (FP64 additions are worth a vote)
-                    if (sizeof(AT) == 8 && !__any_sync(FULL, d <= reach)) break;
-                    const AT o = __shfl_up_sync(FULL, s, d);
-                    if (d <= reach) s += o;
-                }
-                AT before = __shfl_up_sync(FULL, s, 1);  // open sum at the end of the previous lane
-                if (lane == 0) before = AT(0);
-                if (hb && L >= 0) {  // (-1: empty segments before the first nonzero)
-                    const AT lead = before + ((bal & ((1u << lane) - 1u)) ? AT(0) : chi + clo);
-                    const AT v = f + lead;
-                    const int col = col_of(L);
-                    if (col == cfirst)
-                        static_cast<AT2 *>(p.rec_left)[feed.c.proc0 + (hdr.y >> 2)] = make_pair2(v, AT(0));
-                    else
-                        static_cast<XT *>(p.u)[col] = static_cast<XT>(v);
-                }
-                chi = __shfl_sync(FULL, s, 31);
-                clo = AT(0);
-            }
-        }
-        if constexpr (SD) {
-            // a segment that ends with the tile is complete; the open one goes on in the chunk's
-            // next tile or, at the end of the chunk, to the right record
-            const bool ends = (bf.y & STEP_ENDS) != 0, chunk_last = (hdr.y & 1) != 0;
-            if (ends || chunk_last) {
-                if (lane == 0) {
-                    const int last = col_of(base + (bf.y >> 16));
-                    if (ends) {
-                        const AT v = chi + clo;
-                        if (last == cfirst)
+                        for (int e = 1; e < 8; ++e) {
+                            if ((hr >> e) & 1u) {
+                                ++cc;
+                                static_cast<XT *>(p.u)[col_of(cc)] = static_cast<XT>(q);
+                            }
+                            q = next_term(e, q, (hb >> e) & 1u);
+                        }
+                    }
+                    // segmented scan of the lanes' open sums
+                    const unsigned le = bal & (FULL >> (31 - lane));
+                    const int reach = le ? lane - (31 - __clz(le)) : lane;
+#pragma unroll
+                    for (int d = 1; d < 32; d <<= 1) {
+                        // (FP64 additions are worth a vote)
+                        if (sizeof(AT) == 8 && !__any_sync(FULL, d <= reach)) break;
+                        const AT o = __shfl_up_sync(FULL, s, d);
+                        if (d <= reach) s += o;
+                    }
+                    AT before = __shfl_up_sync(FULL, s, 1);  // open sum at the end of the previous lane
+                    if (lane == 0) before = AT(0);
+                    if (hb && L >= 0) {  // (-1: empty segments before the first nonzero)
+                        const AT lead = before + ((bal & ((1u << lane) - 1u)) ? AT(0) : chi + clo);
+                        const AT v = f + lead;
+                        const int col = col_of(L);
+                        if (col == cfirst)
                             static_cast<AT2 *>(p.rec_left)[feed.c.proc0 + (hdr.y >> 2)] = make_pair2(v, AT(0));
                         else
-                            static_cast<XT *>(p.u)[last] = static_cast<XT>(v);
-                    } else if (bf.y & STEP_NEED_RIGHT) {
-                        static_cast<AT2 *>(p.rec_right)[feed.c.proc0 + (hdr.y >> 2)] = make_pair2(chi, clo);
+                            static_cast<XT *>(p.u)[col] = static_cast<XT>(v);
                     }
+                    chi = __shfl_sync(FULL, s, 31);
+                    clo = AT(0);
                 }
-                chi = AT(0);
-                clo = AT(0);
+            }
+            if constexpr (SD) {
+                // a segment that ends with the tile is complete; the open one goes on in the chunk's
+                // next tile or, at the end of the chunk, to the right record
+                const bool ends = (bf.y & STEP_ENDS) != 0, chunk_last = (hdr.y & 1) != 0;
+                if (ends || chunk_last) {
+                    if (lane == 0) {
+                        const int last = col_of(base + (bf.y >> 16));
+                        if (ends) {
+                            const AT v = chi + clo;
+                            if (last == cfirst)
+                                static_cast<AT2 *>(p.rec_left)[feed.c.proc0 + (hdr.y >> 2)] = make_pair2(v, AT(0));
+                            else
+                                static_cast<XT *>(p.u)[last] = static_cast<XT>(v);
+                        } else if (bf.y & STEP_NEED_RIGHT) {
+                            static_cast<AT2 *>(p.rec_right)[feed.c.proc0 + (hdr.y >> 2)] = make_pair2(chi, clo);
+                        }
+                    }
+                    chi = AT(0);
+                    clo = AT(0);
+                }
             }
         }
     }
-    }  // blocks
 
     if constexpr (SC) {
         __syncthreads();
@@ -444,7 +453,10 @@ template <int KV, bool ONCHIP> __device__ __forceinline__ void mv_gather(const f
 // nonzero's KV entries (32 bytes for 8 vectors), GP positions' loads are in flight together, and
 // the products, prefixes and scans of a vector are those of pass_kernel, so each vector's result
 // equals its single product bit for bit.  Lane b keeps vector b's carry.  With the vectors read
-// through L2 (8 of m = 20,000 are 640 KB) the gathers set the pace.
+// through L2 (8 of m = 20,000 are 640 KB) the gathers set the pace: one line a cycle and SM from the
+// L1 tags.  8 vectors, 50M nonzeros: 261 us (streaming kernel 410); on chip (m = 5,500) 124 for 25M.
+// 8 vectors over the row-sorted copy of 200M nonzeros (windows of 38,466 columns): 1,436 us with the
+// combine (streaming kernel 2,763); 2 vectors 559 (1,254).
 template <typename VT, int KV, bool ONCHIP, int WB>
 __global__ void __launch_bounds__(WB * 32, 1) mvdot_kernel(const __grid_constant__ PassParams p) {
     using Feed = StepFeed<VT>;
@@ -454,173 +466,181 @@ __global__ void __launch_bounds__(WB * 32, 1) mvdot_kernel(const __grid_constant
     grid_release();
     __shared__ int next_chunk;
     Feed feed(p, smem + p.vec_bytes, &next_chunk);
-    feed.start(blockIdx.x, gridDim.x, false);
-
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x) {
-        const int col = p.emptylist[i];
-        for (int b = 0; b < p.kb; ++b) p.uv[b][col] = 0.f;
-    }
-    const float *vt = static_cast<const float *>(p.v);
-    if constexpr (ONCHIP) {
-        const int n8 = p.n_minor * KV / 2;  // in pairs of values
-#pragma unroll 4
-        for (int i = threadIdx.x; i < n8; i += blockDim.x)
-            reinterpret_cast<float2 *>(smem)[KV == 8 ? i ^ ((i >> 3) & 2) : i] = __ldg(reinterpret_cast<const float2 *>(vt) + i);
-        vt = reinterpret_cast<const float *>(smem);
-        __syncthreads();
-    }
     const int sh = (lane & 3) << 3;
     const int sw = (lane >> 2) & 1;
-    float chi = 0.f, clo = 0.f;  // vector `lane`'s open segment
-    int cfirst = -1;
     unsigned char *slot;
     int2 hdr;
-    while (feed.next(slot, hdr)) {
-        const int ps = hdr.x << 8;
-        const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
-        const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);
-        const bool gaps = (bf.y & STEP_GAPS) != 0;
-        const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
-        auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
-        const bool whole = p.nnz - ps >= 256;
-        int ix[8];
-        float va[8];
-        if (whole) {
-            stag8_idx(reinterpret_cast<const int32_t *>(slot), 8 * lane, sw, ix);
-            Stag8<VT, float>::run(slot + Feed::OFF_VAL, 8 * lane, sw, va);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {  // into the order of the positions
-                const int i0 = sw ? ix[e + 4] : ix[e];
-                const float v0 = sw ? va[e + 4] : va[e];
-                ix[e + 4] = sw ? ix[e] : ix[e + 4];
-                va[e + 4] = sw ? va[e] : va[e + 4];
-                ix[e] = i0;
-                va[e] = v0;
-            }
-        } else {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int pos = ps + 8 * lane + e;
-                const bool in = pos < p.nnz;
-                ix[e] = in ? __ldg(p.idx + pos) : 0;
-                va[e] = in ? to_f<VT>(static_cast<const VT *>(p.vals)[pos]) : 0.f;
-            }
-        }
-        const uint32_t mw = rec->heads[lane >> 2];
-        const uint32_t hb = (mw >> sh) & 0xFFu;
-        const int L = base + rec->before[lane >> 2] + __popc(mw & ((1u << sh) - 1u));
-        feed.release();
-        const unsigned bal = __ballot_sync(FULL, hb != 0u);
-        const int proc = feed.c.proc0 + (hdr.y >> 2);
-        if (hdr.y & 2) cfirst = (bf.y & STEP_NEED_LEFT) ? bf.x : -1;
 
-        // the lane's prefix s, restarted at every head; f: what its first head closes; segments
-        // inside the lane are closed by its later heads
-        const uint32_t h1 = hb & (0u - hb), hr = hb ^ h1;
-        float s[KV], f[KV];
-        int cc = L;
-#pragma unroll
-        for (int b = 0; b < KV; ++b) s[b] = f[b] = 0.f;
-#pragma unroll
-        for (int e0 = 0; e0 < 8; e0 += GP) {
-            float w[GP][KV];
-#pragma unroll
-            for (int g = 0; g < GP; ++g) mv_gather<KV, ONCHIP>(vt, ix[e0 + g], w[g]);
-            if (!whole) {  // past the last nonzero (zero times an infinity is no zero)
-#pragma unroll
-                for (int g = 0; g < GP; ++g)
-                    if (8 * lane + e0 + g >= p.nnz - ps) {
-#pragma unroll
-                        for (int b = 0; b < KV; ++b) w[g][b] = 0.f;
-                    }
+    // the row-sorted copy's blocks take turns, each with its window of the vectors; else one block a CTA
+#pragma unroll 1
+    for (int turn = 0; turn < p.bpc; ++turn) {
+        const int gb = blockIdx.x * p.bpc + turn;
+        if (turn > 0) __syncthreads();  // every warp is done with the block before
+        feed.start(gb, gridDim.x * p.bpc, turn > 0);
+        if (turn == 0)
+            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x) {
+                const int col = p.emptylist[i];
+                for (int b = 0; b < p.kb; ++b) p.uv[b][col] = 0.f;
             }
+        const int2 w = p.win ? p.win[gb] : make_int2(0, p.n_minor);  // (windows begin on four entries)
+        const float *vt = static_cast<const float *>(p.v) + (size_t)w.x * KV;
+        if constexpr (ONCHIP) {
+            const int n8 = min(w.y, p.n_minor) * KV / 2;  // in pairs of values
+#pragma unroll 4
+            for (int i = threadIdx.x; i < n8; i += blockDim.x)
+                reinterpret_cast<float2 *>(smem)[KV == 8 ? i ^ ((i >> 3) & 2) : i] = __ldg(reinterpret_cast<const float2 *>(vt) + i);
+            vt = reinterpret_cast<const float *>(smem);
+            __syncthreads();
+        }
+        float chi = 0.f, clo = 0.f;  // vector `lane`'s open segment
+        int cfirst = -1;
+        while (feed.next(slot, hdr)) {
+            const int ps = hdr.x << 8;
+            const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
+            const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);
+            const bool gaps = (bf.y & STEP_GAPS) != 0;
+            const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
+            auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
+            const bool whole = p.nnz - ps >= 256;
+            int ix[8];
+            float va[8];
+            if (whole) {
+                stag8_idx(reinterpret_cast<const int32_t *>(slot), 8 * lane, sw, ix);
+                Stag8<VT, float>::run(slot + Feed::OFF_VAL, 8 * lane, sw, va);
 #pragma unroll
-            for (int g = 0; g < GP; ++g) {
-                const int e = e0 + g;
-                if (e > 0) {
-                    if ((hr >> e) & 1u) {
-                        const int col = col_of(++cc);
+                for (int e = 0; e < 4; ++e) {  // into the order of the positions
+                    const int i0 = sw ? ix[e + 4] : ix[e];
+                    const float v0 = sw ? va[e + 4] : va[e];
+                    ix[e + 4] = sw ? ix[e] : ix[e + 4];
+                    va[e + 4] = sw ? va[e] : va[e + 4];
+                    ix[e] = i0;
+                    va[e] = v0;
+                }
+            } else {
 #pragma unroll
-                        for (int b = 0; b < KV; ++b)
-                            if (b < p.kb) p.uv[b][col] = s[b];
+                for (int e = 0; e < 8; ++e) {
+                    const int pos = ps + 8 * lane + e;
+                    const bool in = pos < p.nnz;
+                    ix[e] = in ? __ldg(p.idx + pos) : 0;
+                    va[e] = in ? to_f<VT>(static_cast<const VT *>(p.vals)[pos]) : 0.f;
+                }
+            }
+            const uint32_t mw = rec->heads[lane >> 2];
+            const uint32_t hb = (mw >> sh) & 0xFFu;
+            const int L = base + rec->before[lane >> 2] + __popc(mw & ((1u << sh) - 1u));
+            feed.release();
+            const unsigned bal = __ballot_sync(FULL, hb != 0u);
+            const int proc = feed.c.proc0 + (hdr.y >> 2);
+            if (hdr.y & 2) cfirst = (bf.y & STEP_NEED_LEFT) ? bf.x : -1;
+
+            // the lane's prefix s, restarted at every head; f: what its first head closes; segments
+            // inside the lane are closed by its later heads
+            const uint32_t h1 = hb & (0u - hb), hr = hb ^ h1;
+            float s[KV], f[KV];
+            int cc = L;
+#pragma unroll
+            for (int b = 0; b < KV; ++b) s[b] = f[b] = 0.f;
+#pragma unroll
+            for (int e0 = 0; e0 < 8; e0 += GP) {
+                float w[GP][KV];
+#pragma unroll
+                for (int g = 0; g < GP; ++g) mv_gather<KV, ONCHIP>(vt, ix[e0 + g], w[g]);
+                if (!whole) {  // past the last nonzero (zero times an infinity is no zero)
+#pragma unroll
+                    for (int g = 0; g < GP; ++g)
+                        if (8 * lane + e0 + g >= p.nnz - ps) {
+#pragma unroll
+                            for (int b = 0; b < KV; ++b) w[g][b] = 0.f;
+                        }
+                }
+#pragma unroll
+                for (int g = 0; g < GP; ++g) {
+                    const int e = e0 + g;
+                    if (e > 0) {
+                        if ((hr >> e) & 1u) {
+                            const int col = col_of(++cc);
+#pragma unroll
+                            for (int b = 0; b < KV; ++b)
+                                if (b < p.kb) p.uv[b][col] = s[b];
+                        }
+                        if ((h1 >> e) & 1u) {
+#pragma unroll
+                            for (int b = 0; b < KV; ++b) f[b] = s[b];
+                        }
                     }
-                    if ((h1 >> e) & 1u) {
+                    const bool restart = e == 0 || ((hb >> e) & 1u);
 #pragma unroll
-                        for (int b = 0; b < KV; ++b) f[b] = s[b];
+                    for (int b = 0; b < KV; ++b) {
+                        const float q = mul_rn(va[e], w[g][b]);
+                        s[b] = restart ? q : s[b] + q;
                     }
                 }
-                const bool restart = e == 0 || ((hb >> e) & 1u);
+            }
+            if (bal == 0u) {
+                // butterfly totals, the vectors halved between the lanes as long as there are several
+                // (the same pairs are added as by a butterfly of every vector); lane b gets vector b's
+                int n = KV, d = 16;
+#pragma unroll
+                for (; n > 1; n >>= 1, d >>= 1) {
+                    const bool up = (lane & d) != 0;
+#pragma unroll
+                    for (int j = 0; j < KV / 2; ++j)
+                        if (j < n / 2) {
+                            const float mine = up ? s[j + n / 2] : s[j], other = up ? s[j] : s[j + n / 2];
+                            s[j] = mine + __shfl_xor_sync(FULL, other, d);
+                        }
+                }
+#pragma unroll
+                for (; d >= 1; d >>= 1) s[0] += __shfl_xor_sync(FULL, s[0], d);
+                carry_in(chi, clo, __shfl_sync(FULL, s[0], (lane * (32 / KV)) & 31));
+            } else {
+                const unsigned le = bal & (FULL >> (31 - lane));
+                const int reach = le ? lane - (31 - __clz(le)) : lane;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    if (!__any_sync(FULL, d <= reach)) break;
+#pragma unroll
+                    for (int b = 0; b < KV; ++b) {
+                        const float o = __shfl_up_sync(FULL, s[b], d);
+                        if (d <= reach) s[b] += o;
+                    }
+                }
+                const float carry = chi + clo;
+                const bool own = hb && L >= 0, inner = (bal & ((1u << lane) - 1u)) != 0u;
+                const int col = own ? col_of(L) : 0;
+                clo = 0.f;
 #pragma unroll
                 for (int b = 0; b < KV; ++b) {
-                    const float q = mul_rn(va[e], w[g][b]);
-                    s[b] = restart ? q : s[b] + q;
-                }
-            }
-        }
-        if (bal == 0u) {
-            // butterfly totals, the vectors halved between the lanes as long as there are several
-            // (the same pairs are added as by a butterfly of every vector); lane b gets vector b's
-            int n = KV, d = 16;
-#pragma unroll
-            for (; n > 1; n >>= 1, d >>= 1) {
-                const bool up = (lane & d) != 0;
-#pragma unroll
-                for (int j = 0; j < KV / 2; ++j)
-                    if (j < n / 2) {
-                        const float mine = up ? s[j + n / 2] : s[j], other = up ? s[j] : s[j + n / 2];
-                        s[j] = mine + __shfl_xor_sync(FULL, other, d);
+                    float before = __shfl_up_sync(FULL, s[b], 1);
+                    if (lane == 0) before = 0.f;
+                    const float cb = __shfl_sync(FULL, carry, b), end = __shfl_sync(FULL, s[b], 31);
+                    if (own && b < p.kb) {
+                        const float v = f[b] + (before + (inner ? 0.f : cb));
+                        if (col == cfirst)
+                            static_cast<float2 *>(p.rec_left)[(size_t)b * p.nproc + proc] = make_float2(v, 0.f);
+                        else
+                            p.uv[b][col] = v;
                     }
-            }
-#pragma unroll
-            for (; d >= 1; d >>= 1) s[0] += __shfl_xor_sync(FULL, s[0], d);
-            carry_in(chi, clo, __shfl_sync(FULL, s[0], (lane * (32 / KV)) & 31));
-        } else {
-            const unsigned le = bal & (FULL >> (31 - lane));
-            const int reach = le ? lane - (31 - __clz(le)) : lane;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                if (!__any_sync(FULL, d <= reach)) break;
-#pragma unroll
-                for (int b = 0; b < KV; ++b) {
-                    const float o = __shfl_up_sync(FULL, s[b], d);
-                    if (d <= reach) s[b] += o;
+                    if (lane == b) chi = end;
                 }
             }
-            const float carry = chi + clo;
-            const bool own = hb && L >= 0, inner = (bal & ((1u << lane) - 1u)) != 0u;
-            const int col = own ? col_of(L) : 0;
-            clo = 0.f;
-#pragma unroll
-            for (int b = 0; b < KV; ++b) {
-                float before = __shfl_up_sync(FULL, s[b], 1);
-                if (lane == 0) before = 0.f;
-                const float cb = __shfl_sync(FULL, carry, b), end = __shfl_sync(FULL, s[b], 31);
-                if (own && b < p.kb) {
-                    const float v = f[b] + (before + (inner ? 0.f : cb));
-                    if (col == cfirst)
-                        static_cast<float2 *>(p.rec_left)[(size_t)b * p.nproc + proc] = make_float2(v, 0.f);
-                    else
-                        p.uv[b][col] = v;
+            const bool ends = (bf.y & STEP_ENDS) != 0, chunk_last = (hdr.y & 1) != 0;
+            if (ends || chunk_last) {
+                if (lane < p.kb) {
+                    const int last = col_of(base + (bf.y >> 16));
+                    if (ends) {
+                        const float v = chi + clo;
+                        if (last == cfirst)
+                            static_cast<float2 *>(p.rec_left)[(size_t)lane * p.nproc + proc] = make_float2(v, 0.f);
+                        else
+                            p.uv[lane][last] = v;
+                    } else if (bf.y & STEP_NEED_RIGHT) {
+                        static_cast<float2 *>(p.rec_right)[(size_t)lane * p.nproc + proc] = make_float2(chi, clo);
+                    }
                 }
-                if (lane == b) chi = end;
+                chi = 0.f;
+                clo = 0.f;
             }
-        }
-        const bool ends = (bf.y & STEP_ENDS) != 0, chunk_last = (hdr.y & 1) != 0;
-        if (ends || chunk_last) {
-            if (lane < p.kb) {
-                const int last = col_of(base + (bf.y >> 16));
-                if (ends) {
-                    const float v = chi + clo;
-                    if (last == cfirst)
-                        static_cast<float2 *>(p.rec_left)[(size_t)lane * p.nproc + proc] = make_float2(v, 0.f);
-                    else
-                        p.uv[lane][last] = v;
-                } else if (bf.y & STEP_NEED_RIGHT) {
-                    static_cast<float2 *>(p.rec_right)[(size_t)lane * p.nproc + proc] = make_float2(chi, clo);
-                }
-            }
-            chi = 0.f;
-            clo = 0.f;
         }
     }
 }
@@ -628,8 +648,10 @@ __global__ void __launch_bounds__(WB * 32, 1) mvdot_kernel(const __grid_constant
 // The accumulating product of up to KV = 2, 4 or 8 vectors in one reading of the matrix (32-bit
 // accumulation), the accumulators interleaved [row][KV] on chip.  KV lanes take one nonzero, a
 // vector each, four nonzeros in a row per load; 32 / KV nonzeros per addition then meet fewer
-// bank conflicts than 32 rows of one vector do, and the nonzeros are staged once.  The partials
-// go out as [cta][vector][row].
+// bank conflicts than 32 rows of one vector do (additions at 980, 1,160, 1,450 G/s for KV = 2, 4, 8
+// against 800; a 64- or 128-bit compare-and-swap over 2 or 4 vectors is no faster), and the nonzeros
+// are staged once.  8 vectors of 20,000 rows, 50M nonzeros, two a pass: 603 us (866 one by one in the
+// streaming kernel).  The partials go out as [cta][vector][row].
 template <typename VT, int KV, int WB>
 __global__ void __launch_bounds__(WB * 32, 1) mvscatter_kernel(const __grid_constant__ PassParams p) {
     using Feed = StepFeed<VT>;

@@ -170,3 +170,25 @@ def test_row_blocks_in_turn():
         for b in range(2):
             assert torch.equal(Y[b], plan.spmv(X[b]))
         plan.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=str)
+@pytest.mark.parametrize("m,n,blocks_in_turn", [(64, 9_000_000, True), (300, 400_000, False), (2_000, 60_000, False)])
+def test_row_blocks_of_several_vectors(m, n, blocks_in_turn, dtype):
+    """Batches over the row-sorted copy, windows on chip and read through L2, one block a CTA and several
+    in turn: every vector the single product's bits."""
+    rng = np.random.default_rng(m)
+    deg = np.zeros(n, dtype=np.int64)
+    deg[rng.choice(n, min(n, 1_500_000) * 9 // 10, replace=False)] = 1
+    deg[rng.choice(n, min(n, 40_000), replace=False)] += int(max(2, 8 * 152 * m * 1.3 // 40_000))
+    A = synth.random_matrix(m, n, "csc", degrees=deg, seed=3, duplicates=True)
+    plan, stored = make_plan(A, dtype, flags=pkg.SPMV_PLAN_ROW_BLOCKS, tile_items=256)
+    info = plan.info()
+    assert info["row_blocks"] > 0 and (info["row_blocks"] > info["ctas"]) == blocks_in_turn, info
+    X = torch.stack([dev_vec(synth.uniform_vector(n, 7 + b), torch.float32) for b in range(9)])
+    single = [plan.spmv(X[b]) for b in range(9)]
+    for k in (2, 3, 4, 7, 9):
+        Y = plan.batch(pkg.SPMV_OP_AX, X[:k])
+        plan.check()
+        for b in range(k):
+            assert torch.equal(Y[b], single[b]), f"k={k} vector {b}"
