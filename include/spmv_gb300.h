@@ -122,12 +122,17 @@ typedef struct spmv_plan_s *spmv_plan_t;
 /* Optional tuning of a plan; zero fields take the defaults. */
 typedef struct {
     int32_t chunks;        /* P, the number of reporting chunks (Sec. II); 0 = min(tiles, 16 per SM) */
-    int32_t warps_per_cta; /* most warps per CTA, 1..24 (at most 16 run the multi-vector passes);
+    int32_t warps_per_cta; /* streaming kernel (plans without validation, tiles of other sizes than
+                              multiples of 256, short vectors too long for the chip, FP64 batches):
+                              most warps per CTA, 1..24 (at most 16 run the multi-vector passes);
                               0 = 24; every pass runs as many as its staging slots fit in shared
-                              memory (up to 16 warps with 128 registers a thread, more with 80) */
-    int32_t tile_items;    /* nonzeros per execution tile, a multiple of 8 in [8, 992]; 0 = 512, or
-                              down to 64 when nnz < 32 x 512 per SM (about two tiles per warp) */
-    int32_t stages;        /* staging slots per warp (tiles in flight + 1), 2..4; 0 = 2 */
+                              memory (up to 16 warps with 128 registers a thread, more with 80).
+                              The passes of validated plans take 32 (FP64 16) or as many as fit. */
+    int32_t tile_items;    /* nonzeros per execution tile, a multiple of 8 in [8, 992]; 0 = 512;
+                              when nnz < 32 x 512 per SM, 256 for validated plans, else down to 64
+                              (about two tiles per warp) */
+    int32_t stages;        /* staging slots per warp of the streaming kernel (tiles in flight + 1),
+                              2..4; 0 = 2 */
     int32_t chunk_tiles;   /* consecutive tiles a warp streams as one processor, 1..64 (segments that
                               run on between them are carried in registers; overlap zones arise only
                               between chunks); 0 = 8.  The last MAX(24 (C + 1)) tiles of every CTA
@@ -277,7 +282,8 @@ spmv_status spmv_check(spmv_plan_t plan, void *stream);
  * combine, 2 = chunk dot (SpVTM local), 3 = zone fixup, 4 = dvalues,
  * 5 = row-block dot (the SpMV local step over the row-sorted copy), 6 = its zone fixup.
  * One pass that serves both products of a spmv_pair counts as a launch of kernel 0 and of
- * kernel 2, with half of its time each.
+ * kernel 2, with half of its time each; one launch that combines and fixes up counts so for
+ * kernels 1 and 3.
  * Synchronizes the device.  *ms = summed event time, *launches = number of
  * timed launches.  Timing brackets every launch with two events, which waits
  * for each kernel to drain before the next starts: a profiled sequence of

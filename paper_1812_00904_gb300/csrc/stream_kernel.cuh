@@ -1,4 +1,8 @@
-// Streaming kernel: the nonzeros are cut into equal-count tiles of T nonzeros;
+// Streaming kernel, the general path: any tile size, plans that were not validated, short vectors
+// that do not fit on chip, FP64 batches.  (The other products of validated plans run in
+// pass_kernel.cuh, over the same tiles, chunks and records.)
+//
+// The nonzeros are cut into equal-count tiles of T nonzeros;
 // each CTA takes a contiguous range of tiles by the Sec. II rule and cuts it into
 // chunks: nb chunks of C consecutive tiles, then a tail of single-tile chunks
 // (at least MAX_WARPS (C + 1) tiles, when the CTA has that many).  The chunks are
