@@ -64,11 +64,11 @@ cudaError_t launch_pass(const spmv_plan_s *p, bool sc, bool sd, const PassParams
 // Shared memory of a one-vector pass: the accumulator (sc), the input vector (sd), a staging slot for
 // each of as many warps as fit, and what is left over for more copies of the accumulator.  More warps
 // always help: the pair, the accumulating product and the dot products of the 200M-nonzero wide
-// matrix (m = 20,000) take 590 / 427 / 374 us with 16 warps, 501 / 374 / 326 with 20, 449 / 341 / 301
-// with 24, 417 / 322 / 281 with 28, 389 / 305 / 263 with 32.  A second slot a warp is no gain
+// matrix (m = 20,000) take 590 / 403 / 374 us with 16 warps, 501 / 355 / 326 with 20, 449 / 325 / 301
+// with 24, 417 / 309 / 281 with 28, 389 / 294 / 261 with 32.  A second slot a warp is no gain
 // (dot products 269 to 280).  An addition is a compare-and-swap loop, repeated when another warp got
 // in between, so copies help where they fit: with 1 / 2 / 4 / 8 / 16 of them the accumulating
-// product of the 150M-nonzero tall matrix (n = 2,000) takes 450 / 393 / 348 / 318 / 281 us, the pair
+// product of the 150M-nonzero tall matrix (n = 2,000) takes 348 / 318 / 302 / 290 / 262 us, the pair
 // 441 / 419 / 406 / 393 / 372; 32 add nothing.
 size_t pass_acc_bytes(const spmv_plan_s *p) { return align_up((size_t)p->n_minor * p->sa, 128); }
 size_t pass_vec_bytes(const spmv_plan_s *p) { return align_up((size_t)p->n_minor * p->sx, 128); }
@@ -98,7 +98,7 @@ PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1) {
 }
 // A pass runs with at least 8 warps (or all a CTA has tiles for): fewer leave it to the streaming
 // kernel.  The pair wants 20: with 16 its two products run faster one by one, each with 32 warps
-// (305 + 263 us against 590; 501 with 20).
+// (294 + 261 us against 590; 501 with 20).
 bool pass_fits(const spmv_plan_s *p, bool sc, bool sd) {
     return pass_geometry(p, sc, sd).warps >= std::min(sc && sd ? std::min(20, pass_warps(p->sv)) : 8, cta_tiles(p));
 }

@@ -121,17 +121,19 @@ __device__ __forceinline__ float seg_term(float v, float w, float s, bool restar
 __device__ __forceinline__ double seg_term(double v, double w, double s, bool restart) {
     return fma(v, w, restart ? 0.0 : s);
 }
-// *acc += v x on an FP64 accumulator in shared memory, the product fused into the addition of the
-// compare-and-swap loop: the FP64 pipe takes 16 cycles an instruction and a warp, also on every
-// repetition (8M nonzeros, n = 4,000: 54 us with the product apart, 50 with it fused).
-__device__ __forceinline__ void acc_fma(double *acc, double v, double x) {
+// One attempt at *acc += v x (FP64, the product fused into the addition: its pipe takes 16 cycles an
+// instruction and a warp) or *acc += x (FP32, x the product), acc in shared memory; false: another
+// addition to the same place came between.
+__device__ __forceinline__ bool try_add(double *acc, double v, double x) {
     unsigned long long *a = reinterpret_cast<unsigned long long *>(acc);
-    unsigned long long seen = *reinterpret_cast<volatile unsigned long long *>(a), was;
-    do {
-        was = seen;
-        seen = atomicCAS(a, was, static_cast<unsigned long long>(__double_as_longlong(
-                                     fma(v, x, __longlong_as_double(static_cast<long long>(was))))));
-    } while (seen != was);
+    const unsigned long long was = *reinterpret_cast<volatile unsigned long long *>(a);
+    return atomicCAS(a, was, static_cast<unsigned long long>(__double_as_longlong(
+                                 fma(v, x, __longlong_as_double(static_cast<long long>(was)))))) == was;
+}
+__device__ __forceinline__ bool try_add(float *acc, float, float x) {
+    unsigned *a = reinterpret_cast<unsigned *>(acc);
+    const unsigned was = *reinterpret_cast<volatile unsigned *>(a);
+    return atomicCAS(a, was, __float_as_uint(__uint_as_float(was) + x)) == was;
 }
 // hi + lo += t, compensated (TwoSum: hi takes the rounded sum, lo gathers its rounding
 // errors).  A sum that is infinite or NaN carries no error term, so that hi + lo stays what the

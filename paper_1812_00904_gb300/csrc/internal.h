@@ -141,9 +141,9 @@ struct PassParams {
 constexpr int PASS_BAR_BYTES = 512;  // slot barriers, PASS_MAX_SLOTS for each of up to 32 warps
 constexpr int PASS_MAX_SLOTS = 2;
 __host__ __device__ constexpr int pass_slot_bytes(int val_bytes) { return 1024 + 256 * val_bytes + (int)sizeof(StepRec) + 16; }
-// Most warps of a pass: 32 of 64 registers a thread; FP64 needs more registers, and its passes lose
-// with more warps (8M nonzeros, n = 4,000, with 16 / 20 / 24 / 32: dot products 48 / 48 / 48 / 49
-// us, accumulating 59 / 63 / 65 / 71, whose compare-and-swap loops meet each other).
+// Most warps of a pass: 32 of 64 registers a thread; FP64 needs more registers, and its passes gain
+// little from more warps (8M nonzeros, n = 4,000, with 16 / 20 / 24: dot products 48 / 48 / 49 us,
+// accumulating 42 / 41 / 40, the pair 76 / 77 / 77).
 constexpr int pass_warps(int val_bytes) { return val_bytes != 8 ? 32 : 16; }
 
 // Most warps of the dot products of KV vectors (128, 96 and 80 registers a thread).

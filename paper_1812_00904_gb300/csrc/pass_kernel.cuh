@@ -138,13 +138,20 @@ template <typename VT, bool VALS = true> struct StepFeed {
 // load and a compare-and-swap that costs two, each with the bank conflicts of 32 rows.  SD alone
 // runs near the memory rate, FP64 at the rate of its pipe (2 operations a cycle per SM).  With the
 // combine and fix-up, streaming kernel before, this one now (us): 200M FP32 nonzeros, m = 20,000, bank
-// order: pair 640 -> 386, SC 362 -> 305, SD 303 -> 263; 150M, n = 2,000: pair 538 -> 369, SC 313 ->
-// 276, SD 242 -> 207; 8M FP64, n = 4,000: pair 121 -> 79, SC 62 -> 59, SD 69 -> 48.
+// order: pair 640 -> 386, SC 362 -> 294, SD 303 -> 261; 150M, n = 2,000: pair 538 -> 369, SC 313 ->
+// 262, SD 242 -> 207; 8M FP64, n = 4,000: pair 121 -> 76, SC 62 -> 42, SD 69 -> 48.
 template <typename VT, typename XT, bool SC, bool SD, int WB>
 __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant__ PassParams p) {
     using AT = typename Acc<VT>::type;
     using AT2 = typename Pair<AT>::type;
     using Feed = StepFeed<VT>;
+    // SC's additions are one attempt each, and what failed (another warp's addition to the same place came
+    // between) is tried again after the eight, every lane at its own next one: a loop around each
+    // addition repeated nearly all of them for the sake of single lanes (FP64, 8M nonzeros, n = 4,000:
+    // 2.3 compare-and-swaps an addition, 16 cycles of the FP64 pipe each; 59 us, now 42; FP32, 10M, m =
+    // 15,000: 40 -> 33; 200M, m = 20,000: 305 -> 294).  The FP32 pair has no registers left for it (402
+    // against 391), and KV lanes to a nonzero meet too seldom (wide batch of 8: 695 against 670).
+    constexpr bool DEFER = sizeof(AT) == 8 || !SD;
     extern __shared__ __align__(128) unsigned char smem[];
     // this warp's copy of the accumulator (warps share p.copies of them)
     AT *acc = reinterpret_cast<AT *>(smem + (threadIdx.x >> 5) % p.copies * p.acc_bytes);
@@ -295,13 +302,27 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
                 }
             }
             if constexpr (SC) {
+                [[maybe_unused]] unsigned failed = 0u;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
-                    if constexpr (sizeof(AT) == 4) {
+                    if constexpr (!DEFER) {
                         atomicAdd(acc + ix[e], c[e]);
-                    } else {
-                        acc_fma(acc + ix[e], va[e], c[e]);
+                    } else if (!try_add(acc + ix[e], va[e], c[e])) {
+                        failed |= 1u << e;
                     }
+                }
+                while (failed) {  // each lane its next failed addition
+                    const int e = __ffs(failed) - 1;
+                    int r = ix[0];
+                    AT v = va[0], x = c[0];
+#pragma unroll
+                    for (int q = 1; q < 8; ++q)
+                        if (e == q) {
+                            r = ix[q];
+                            v = va[q];
+                            x = c[q];
+                        }
+                    if (try_add(acc + r, v, x)) failed &= failed - 1u;
                 }
             }
             if constexpr (SD) {  // into the order of the positions
