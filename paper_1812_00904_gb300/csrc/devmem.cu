@@ -33,7 +33,8 @@ struct DevicePool {
 DevicePool g_pools[MAX_DEVICES];
 
 std::mutex g_large_mu;
-std::unordered_set<void *> g_large;  // the blocks that bypassed the pool
+// the blocks that bypassed the pool (never destroyed: plans may be freed while the process ends)
+std::unordered_set<void *> &g_large = *new std::unordered_set<void *>;
 
 DevicePool &pool_of(int device) {
     DevicePool &P = g_pools[device];
