@@ -82,17 +82,22 @@ int cta_tiles(const spmv_plan_s *p) {
     const int blocks = std::max(1, p->ctas * p->bpc);
     return std::max(1, (p->ntiles + blocks - 1) / blocks);
 }
+// Warps that a CTA's copies of the short vectors ask for, 512 elements each (staged, zeroed, written
+// out), even if it has fewer tiles: 103 CTAs of one tile and one warp each took 20 us more for 45,889
+// elements than the streaming kernel.
+int copy_warps(const spmv_plan_s *p, int kv) { return (int)std::min<int64_t>(32, ((int64_t)p->n_minor * kv + 511) / 512); }
 PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1) {
     PassGeometry g;
     const size_t acc = sc ? align_up((size_t)p->n_minor * kv * p->sa, 128) : 0, vec = (sd ? pass_vec_bytes(p) : 0) + PASS_BAR_BYTES;
     const size_t slot = pass_slot_bytes(p->sv), all = (size_t)p->smem_max;
     const size_t fit = all > acc + vec ? (all - acc - vec) / slot : 0;
-    g.warps = (int)std::min<size_t>(std::min(pass_warps(p->sv), cta_tiles(p)), fit);
+    const int most_warps = pass_warps(p->sv), work = std::min(most_warps, cta_tiles(p));
+    g.warps = (int)std::min<size_t>(std::max(work, std::min(most_warps, copy_warps(p, kv))), fit);
     g.slots = 1;
     const size_t rest = vec + (size_t)g.warps * g.slots * slot;
     g.copies = 1;
     const int most = p->sv == 8 ? 2 : PASS_MAX_COPIES;  // (adding up FP64 copies costs more than they save)
-    while (sc && 2 * g.copies <= std::min(g.warps, most) && 2 * g.copies * acc + rest <= all) g.copies *= 2;
+    while (sc && 2 * g.copies <= std::min({g.warps, work, most}) && 2 * g.copies * acc + rest <= all) g.copies *= 2;
     g.smem = g.copies * acc + rest;
     return g;
 }
@@ -404,7 +409,7 @@ static spmv_status run_mvdot(spmv_plan_s *p, int kb, const void *const *in, void
     const size_t room = (size_t)p->smem_max - PASS_BAR_BYTES;
     const size_t fit = room > vec ? (room - vec) / slot : 0;
     const bool onchip = fit >= (size_t)(kv == 2 ? (most + 1) / 2 : kv == 4 ? most - most / 4 : most - most / 16);
-    const int warps = onchip ? (int)std::min<size_t>(most, fit) : most;
+    const int warps = onchip ? (int)std::min<size_t>(std::max(most, std::min(mvdot_warps(kv), copy_warps(p, kv))), fit) : most;
     // (one slot a warp where blocks take turns: StepFeed::start)
     pp.slots = p->bpc > 1 ? 1 : onchip ? (int)std::min<size_t>(PASS_MAX_SLOTS, fit / warps) : PASS_MAX_SLOTS;
     pp.vec_bytes = onchip ? (int)vec : 0;

@@ -80,6 +80,17 @@ def test_length_of_the_short_vector(short, dtype):
     _check(A, dtype, 256, f"short={short}")
 
 
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32, torch.bfloat16], ids=str)
+@pytest.mark.parametrize("short,nnz", [(513, 200), (9_451, 2_000), (22_000, 30_000), (45_889, 26_428)])
+def test_few_tiles_beside_a_long_short_vector(short, nnz, dtype):
+    """More warps move the short vectors than there are tiles to work on."""
+    rng = np.random.default_rng(short)
+    deg = np.minimum(rng.integers(1, 2_000, 300), short)
+    deg = deg[: np.searchsorted(np.cumsum(deg), nnz) + 1]
+    for layout, m, n in (("csc", short, len(deg)), ("csr", len(deg), short)):
+        _check(synth.random_matrix(m, n, layout, degrees=deg, seed=5, duplicates=True), dtype, 256, f"{layout} {short}")
+
+
 def test_in_a_graph_and_with_changed_values():
     """A captured pair replays on new vectors and on values changed in place (the plan borrows them)."""
     rng = np.random.default_rng(8)
