@@ -51,9 +51,8 @@ template <typename T> __device__ __forceinline__ void two_sum(T &s, T &c, T v) {
 // 2: beta = sum / gamma, gamma = sum.  (As two kernels, the first over 608 blocks whatever the
 // length, 11 + 4 us for 400,000 FP64 elements and 6 + 4 for 4,000, and a launch more.)
 template <typename T>
-__global__ void __launch_bounds__(DOT_THREADS) dot_kernel(const T *__restrict__ a, const T *__restrict__ b, int64_t len,
-                                                          double *__restrict__ part, int what, CgScalars *sc,
-                                                          int *done) {
+__global__ void __launch_bounds__(DOT_THREADS) dot_kernel(const T *a, const T *b, int64_t len, double *part, int what,
+                                                          CgScalars *sc, int *done) {
     __shared__ T sh_s[DOT_THREADS], sh_c[DOT_THREADS];
     __shared__ bool last;
     grid_release();
@@ -112,23 +111,24 @@ __global__ void __launch_bounds__(DOT_THREADS) dot_kernel(const T *__restrict__ 
 
 // x += alpha p (n entries), r -= alpha q (m entries)
 template <typename T>
-__global__ void xr_update_kernel(T *__restrict__ x, const T *__restrict__ p, int64_t n, T *__restrict__ r,
-                                 const T *__restrict__ q, int64_t m, const CgScalars *sc) {
+__global__ void xr_update_kernel(T *x, const T *p, int64_t n, T *r, const T *q, int64_t m, const CgScalars *sc) {
     grid_release();
     grid_wait();
     const T alpha = (T)sc->alpha;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t len = n > m ? n : m;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += stride) {
-        if (i < n) x[i] += alpha * p[i];
-        if (i < m) r[i] -= alpha * q[i];
+        // (the four loads first: the pointers may alias as far as the compiler knows)
+        const bool in_x = i < n, in_r = i < m;
+        const T xi = in_x ? x[i] : T(0), pi = in_x ? p[i] : T(0), ri = in_r ? r[i] : T(0), qi = in_r ? q[i] : T(0);
+        if (in_x) x[i] = xi + alpha * pi;
+        if (in_r) r[i] = ri - alpha * qi;
     }
 }
 
 // p = s + beta p (beta = 0 copies)
 template <typename T>
-__global__ void p_update_kernel(T *__restrict__ p, const T *__restrict__ s, int64_t n, const CgScalars *sc,
-                                int first) {
+__global__ void p_update_kernel(T *p, const T *s, int64_t n, const CgScalars *sc, int first) {
     grid_release();
     grid_wait();
     const T beta = first ? T(0) : (T)sc->beta;

@@ -39,6 +39,40 @@ __device__ __forceinline__ void fence_mbar_init() {
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Loads of a kernel launched with programmatic serialization.  What the kernel before may write
+// (vectors, values, indices, partials, scalars) is still being written while this one is already
+// resident, so the non-coherent path (__ldg, const __restrict__) is not allowed for it: PTX wants data
+// that nobody writes during the whole kernel.  call_load is a plain global load that stays behind
+// grid_wait (both are volatile).  plan_load may take the non-coherent path: plan memory is written
+// before the plan's creation returns and never again.  (Plain loads cost nothing measurable: see the
+// figures at the kernels, all taken with them.)
+__device__ __forceinline__ int32_t call_load(const int32_t *p) {
+    int32_t v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float call_load(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double call_load(const double *p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 call_load(const float2 *p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 call_load(const float4 *p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+template <typename T> __device__ __forceinline__ T plan_load(const T *p) { return __ldg(p); }
+
 // Orders this thread's earlier generic-proxy shared-memory accesses before later async-proxy (bulk copy) ones.
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

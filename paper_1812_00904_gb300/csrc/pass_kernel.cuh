@@ -196,8 +196,8 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
             const int n16 = len / xa;
 #pragma unroll 4
             for (int i = threadIdx.x; i < n16; i += blockDim.x)
-                reinterpret_cast<float4 *>(vs)[i] = __ldg(reinterpret_cast<const float4 *>(src) + i);
-            for (int i = n16 * xa + threadIdx.x; i < len; i += blockDim.x) vs[i] = __ldg(src + i);
+                reinterpret_cast<float4 *>(vs)[i] = call_load(reinterpret_cast<const float4 *>(src) + i);
+            for (int i = n16 * xa + threadIdx.x; i < len; i += blockDim.x) vs[i] = call_load(src + i);
         }
         __syncthreads();
 
@@ -210,8 +210,8 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
             // the step's segments are columns (rows of a tall matrix) first, first + 1, ..; with empty
             // ones between them they are counted by rank and looked up
             const bool gaps = (bf.y & STEP_GAPS) != 0;
-            const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
-            auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
+            const int base = gaps && bf.x >= 0 ? plan_load(p.rank + bf.x) : bf.x;
+            auto col_of = [&](int c) { return gaps ? plan_load(p.seglist + c) : c; };
             const bool whole = p.nnz - ps >= 256;
             // With SD this lane takes positions 8 lane .. 8 lane + 7, register e holding position
             // e ^ (4 sw) (staggered loads, which touch every bank exactly four times an instruction);
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
                 for (int e = 0; e < 8; ++e) {
                     const int pos = ps + (SD ? 8 * lane + (e ^ (4 * sw)) : 32 * e + lane);
                     const bool in = pos < p.nnz;
-                    ix[e] = in ? __ldg(p.idx + pos) : 0;
+                    ix[e] = in ? call_load(p.idx + pos) : 0;
                     va[e] = in ? to_acc<AT>(static_cast<const VT *>(p.vals)[pos]) : AT(0);
                 }
             }
@@ -256,14 +256,14 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
             AT a[8], c[8];
             if constexpr (SC) {  // the long vector's entries
                 if (bal == 0u) {
-                    const AT xv = static_cast<AT>(__ldg(xg + col_of(L)));
+                    const AT xv = static_cast<AT>(call_load(xg + col_of(L)));
 #pragma unroll
                     for (int e = 0; e < 8; ++e) c[e] = xv;
                 } else if (!SD) {
                     const uint32_t lane_le = FULL >> (31 - lane);
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        c[e] = static_cast<AT>(__ldg(xg + col_of(L + __popc(w[e] & lane_le))));
+                        c[e] = static_cast<AT>(call_load(xg + col_of(L + __popc(w[e] & lane_le))));
                         L += __popc(w[e]);
                     }
                 } else {
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
                         if (e == 4) cc = sw ? L : L + nlo;
                         cc += ((e < 4 ? h1 : h2) >> (e & 3)) & 1u;
                         // (-1 in the first step: empty segments before the first nonzero, whose head counts)
-                        c[e] = static_cast<AT>(__ldg(xg + col_of(cc)));
+                        c[e] = static_cast<AT>(call_load(xg + col_of(cc)));
                     }
                 }
             }
@@ -450,17 +450,17 @@ template <int KV, bool ONCHIP> __device__ __forceinline__ void mv_gather(const f
     const float *q = vt + (size_t)i * KV;
     const int hs = ONCHIP && KV == 8 ? (i >> 2) & 1 : 0;
     if constexpr (!ONCHIP && KV == 8) {
-        asm volatile("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                      : "=f"(w[0]), "=f"(w[1]), "=f"(w[2]), "=f"(w[3]), "=f"(w[4]), "=f"(w[5]), "=f"(w[6]), "=f"(w[7])
                      : "l"(q));
     } else if constexpr (KV == 2) {
-        const float2 t = ONCHIP ? *reinterpret_cast<const float2 *>(q) : __ldg(reinterpret_cast<const float2 *>(q));
+        const float2 t = ONCHIP ? *reinterpret_cast<const float2 *>(q) : call_load(reinterpret_cast<const float2 *>(q));
         w[0] = t.x;
         w[1] = t.y;
     } else {
 #pragma unroll
         for (int h = 0; h < KV / 4; ++h) {
-            const float4 t = ONCHIP ? reinterpret_cast<const float4 *>(q)[h ^ hs] : __ldg(reinterpret_cast<const float4 *>(q) + h);
+            const float4 t = ONCHIP ? reinterpret_cast<const float4 *>(q)[h ^ hs] : call_load(reinterpret_cast<const float4 *>(q) + h);
             w[4 * h] = t.x;
             w[4 * h + 1] = t.y;
             w[4 * h + 2] = t.z;
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(WB * 32, 1) mvdot_kernel(const __grid_constant
             const int n8 = min(w.y, p.n_minor) * KV / 2;  // in pairs of values
 #pragma unroll 4
             for (int i = threadIdx.x; i < n8; i += blockDim.x)
-                reinterpret_cast<float2 *>(smem)[KV == 8 ? i ^ ((i >> 3) & 2) : i] = __ldg(reinterpret_cast<const float2 *>(vt) + i);
+                reinterpret_cast<float2 *>(smem)[KV == 8 ? i ^ ((i >> 3) & 2) : i] = call_load(reinterpret_cast<const float2 *>(vt) + i);
             vt = reinterpret_cast<const float *>(smem);
             __syncthreads();
         }
@@ -520,8 +520,8 @@ __global__ void __launch_bounds__(WB * 32, 1) mvdot_kernel(const __grid_constant
             const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
             const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);
             const bool gaps = (bf.y & STEP_GAPS) != 0;
-            const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
-            auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
+            const int base = gaps && bf.x >= 0 ? plan_load(p.rank + bf.x) : bf.x;
+            auto col_of = [&](int c) { return gaps ? plan_load(p.seglist + c) : c; };
             const bool whole = p.nnz - ps >= 256;
             int ix[8];
             float va[8];
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(WB * 32, 1) mvdot_kernel(const __grid_constant
                 for (int e = 0; e < 8; ++e) {
                     const int pos = ps + 8 * lane + e;
                     const bool in = pos < p.nnz;
-                    ix[e] = in ? __ldg(p.idx + pos) : 0;
+                    ix[e] = in ? call_load(p.idx + pos) : 0;
                     va[e] = in ? to_f<VT>(static_cast<const VT *>(p.vals)[pos]) : 0.f;
                 }
             }
@@ -701,8 +701,8 @@ __global__ void __launch_bounds__(WB * 32, 1) mvscatter_kernel(const __grid_cons
         const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
         const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);
         const bool gaps = (bf.y & STEP_GAPS) != 0;
-        const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
-        auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
+        const int base = gaps && bf.x >= 0 ? plan_load(p.rank + bf.x) : bf.x;
+        auto col_of = [&](int c) { return gaps ? plan_load(p.seglist + c) : c; };
         const int left = p.nnz - ps;  // (256 or more but in a partial last step)
         int cprev = -1;
         float x = 0.f;
@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(WB * 32, 1) mvscatter_kernel(const __grid_cons
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const bool in = pos + i < left;
-                    row[i] = in ? __ldg(p.idx + ps + pos + i) : -1;
+                    row[i] = in ? call_load(p.idx + ps + pos + i) : -1;
                     v[i] = in ? to_f<VT>(static_cast<const VT *>(p.vals)[ps + pos + i]) : 0.f;
                 }
             }
@@ -730,7 +730,7 @@ __global__ void __launch_bounds__(WB * 32, 1) mvscatter_kernel(const __grid_cons
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 c += (hb >> i) & 1u;
-                if (c != cprev) x = __ldg(xb + col_of(c));
+                if (c != cprev) x = call_load(xb + col_of(c));
                 cprev = c;
                 xs[i] = x;
             }
@@ -822,8 +822,8 @@ __global__ void __launch_bounds__(WB * 32, 1) dvalues_kernel(const __grid_consta
         const int n16 = p.n_minor / xa;
 #pragma unroll 4
         for (int i = threadIdx.x; i < n16; i += blockDim.x)
-            reinterpret_cast<float4 *>(vs)[i] = __ldg(reinterpret_cast<const float4 *>(src) + i);
-        for (int i = n16 * xa + threadIdx.x; i < p.n_minor; i += blockDim.x) vs[i] = __ldg(src + i);
+            reinterpret_cast<float4 *>(vs)[i] = call_load(reinterpret_cast<const float4 *>(src) + i);
+        for (int i = n16 * xa + threadIdx.x; i < p.n_minor; i += blockDim.x) vs[i] = call_load(src + i);
     }
     __syncthreads();
     const XT *xg = static_cast<const XT *>(p.x);
@@ -835,8 +835,8 @@ __global__ void __launch_bounds__(WB * 32, 1) dvalues_kernel(const __grid_consta
         const StepRec *rec = reinterpret_cast<const StepRec *>(slot + Feed::OFF_REC);
         const int2 bf = *reinterpret_cast<const int2 *>(&rec->first);
         const bool gaps = (bf.y & STEP_GAPS) != 0;
-        const int base = gaps && bf.x >= 0 ? __ldg(p.rank + bf.x) : bf.x;
-        auto col_of = [&](int c) { return gaps ? __ldg(p.seglist + c) : c; };
+        const int base = gaps && bf.x >= 0 ? plan_load(p.rank + bf.x) : bf.x;
+        auto col_of = [&](int c) { return gaps ? plan_load(p.seglist + c) : c; };
         const int left = p.nnz - ps;
         int ix[8];
         AT x[8];
@@ -848,15 +848,15 @@ __global__ void __launch_bounds__(WB * 32, 1) dvalues_kernel(const __grid_consta
                 ix[2 * j] = q.x;
                 ix[2 * j + 1] = q.y;
             } else {
-                ix[2 * j] = pos < left ? __ldg(p.idx + ps + pos) : 0;
-                ix[2 * j + 1] = pos + 1 < left ? __ldg(p.idx + ps + pos + 1) : 0;
+                ix[2 * j] = pos < left ? call_load(p.idx + ps + pos) : 0;
+                ix[2 * j + 1] = pos + 1 < left ? call_load(p.idx + ps + pos + 1) : 0;
             }
             const uint32_t w = rec->heads[pos >> 5];
             const int b = pos & 31;  // (even: bit b + 1 exists)
             const int c0 = base + rec->before[pos >> 5] + __popc(w & ((2u << b) - 1u));
             const int c1 = c0 + ((w >> (b + 1)) & 1u);
-            x[2 * j] = static_cast<AT>(__ldg(xg + col_of(max(c0, 0))));
-            x[2 * j + 1] = static_cast<AT>(__ldg(xg + col_of(max(c1, 0))));
+            x[2 * j] = static_cast<AT>(call_load(xg + col_of(max(c0, 0))));
+            x[2 * j + 1] = static_cast<AT>(call_load(xg + col_of(max(c1, 0))));
         }
         feed.release();
 #pragma unroll

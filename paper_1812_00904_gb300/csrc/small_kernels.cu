@@ -155,7 +155,7 @@ cudaError_t launch_combine_fixup(bool f64, const void *part, int nparts, int n_m
 // consecutive entries of every vector: coalesced reads of each vector into shared memory,
 // then coalesced writes of the interleaved rows.
 template <typename XT, int KB>
-__global__ void __launch_bounds__(256) interleave_kernel(InPtrs in, int kb, int64_t len, XT *__restrict__ out) {
+__global__ void __launch_bounds__(256) interleave_kernel(InPtrs in, int kb, int64_t len, XT *out) {
     constexpr int IT = 256;
     constexpr int RS = KB + 1;  // padded row: no bank conflicts in either phase
     __shared__ XT sh[IT * RS];
