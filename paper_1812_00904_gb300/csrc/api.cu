@@ -605,20 +605,21 @@ spmv_status run_op(spmv_plan_s *p, int op, int k, const void *const *in, void *c
 
 namespace gbk {
 
-void plan_free(spmv_plan_s *p) {
+void plan_free(spmv_plan_s *p, bool idle) {
     if (!p) return;
-    plan_free(p->tplan);
+    plan_free(p->tplan, idle);
+    auto give_back = [&](void *mem) { dev_free(mem, p->device, idle); };
     if (p->vt) cudaFree(p->vt);
     if (p->ypart_k) cudaFree(p->ypart_k);
-    dev_free(p->bws, p->device);
-    dev_free(p->bown, p->device);
+    give_back(p->bws);
+    give_back(p->bown);
     for (auto &pr : p->prof) {
         cudaEventDestroy(pr.a);
         cudaEventDestroy(pr.b);
     }
-    dev_free(p->ws, p->device);
-    dev_free(p->ws2, p->device);
-    dev_free(p->ws_seg, p->device);
+    give_back(p->ws);
+    give_back(p->ws2);
+    give_back(p->ws_seg);
     if (p->hin) cudaFree(p->hin);
     if (p->hout) cudaFree(p->hout);
     if (p->hv) cudaFree(p->hv);
@@ -628,8 +629,8 @@ void plan_free(spmv_plan_s *p) {
     if (p->cstream) cudaStreamDestroy(p->cstream);
     if (p->hg) cudaFree(p->hg);
     if (p->ynorm) cudaFree(p->ynorm);
-    dev_free(p->owned_ptr, p->device);
-    dev_free(p->owned_nz, p->device);
+    give_back(p->owned_ptr);
+    give_back(p->owned_nz);
     delete p;
 }
 
@@ -640,8 +641,7 @@ namespace {
 struct PlanGuard {  // a plan whose creation failed: its set-up may still be running
     spmv_plan_s *p;
     ~PlanGuard() {
-        if (p) cudaDeviceSynchronize();
-        plan_free(p);
+        if (p) plan_free(p, cudaDeviceSynchronize() == cudaSuccess);
     }
 };
 
@@ -1013,8 +1013,14 @@ extern "C" {
 
 spmv_status spmv_plan_destroy(spmv_plan_t plan) {
     if (!plan) return SPMV_OK;
-    cudaDeviceSynchronize();
-    plan_free(plan);
+    // wait for the device that owns the plan's memory (the current one belongs to the thread and may be
+    // another); while it cannot be waited for, as during a stream capture, its kernels may still run and the
+    // plan's pooled blocks are kept out of the pool for good
+    int current = plan->device;
+    const bool elsewhere = cudaGetDevice(&current) == cudaSuccess && current != plan->device;
+    if (elsewhere) cudaSetDevice(plan->device);
+    plan_free(plan, cudaDeviceSynchronize() == cudaSuccess);
+    if (elsewhere) cudaSetDevice(current);
     return SPMV_OK;
 }
 

@@ -228,7 +228,7 @@ spmv_status build_row_blocks(spmv_plan_s *p, int sms, cudaStream_t s) {
                      p->flags & SPMV_PLAN_BANK_ORDER, &o, &pi);
     if (st != SPMV_OK) return st;
     if (!q->onchip || q->ctas * q->bpc != G) {  // the windows must sit in shared memory, block by block
-        plan_free(q);
+        plan_free(q, true);  // (its set-up has been waited for)
         return SPMV_OK;
     }
     q->win = win;

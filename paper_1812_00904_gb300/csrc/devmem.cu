@@ -99,7 +99,7 @@ cudaError_t dev_alloc(void **p, size_t bytes) {
     return e;
 }
 
-void dev_free(void *p, int device) {
+void dev_free(void *p, int device, bool idle) {
     if (!p) return;
     bool large;
     {
@@ -107,7 +107,9 @@ void dev_free(void *p, int device) {
         large = g_large.erase(p) != 0;
     }
     if (!large && device >= 0 && device < MAX_DEVICES && g_pools[device].pool) {
-        cudaFreeAsync(p, g_pools[device].stream);
+        // (cudaFree waits for the device by itself, the pool for nothing: memory that may still be in use
+        // must not go back to it)
+        if (idle) cudaFreeAsync(p, g_pools[device].stream);
     } else {
         cudaFree(p);
     }

@@ -112,9 +112,10 @@ struct spmv_plan_s {
 namespace gbk {
 
 // Device memory from the current device's pool (devmem.cu): usable on any stream once returned;
-// freed when no work that uses it is pending on `device`.
+// freed when no work that uses it is pending on `device`, or with idle = false (a pooled block then
+// stays allocated).
 cudaError_t dev_alloc(void **p, size_t bytes);
-void dev_free(void *p, int device);
+void dev_free(void *p, int device, bool idle = true);
 
 // Internal overrides of a plan made by the library itself.
 struct PlanInternal {
@@ -125,7 +126,8 @@ struct PlanInternal {
 spmv_status plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nnz, int32_t layout, const int32_t *ptr,
                         const int32_t *idx, const void *vals, int32_t val_dtype, int32_t vec_dtype, cudaStream_t s,
                         uint32_t flags, const spmv_plan_opts *opts, const PlanInternal *pi);
-void plan_free(spmv_plan_s *p);
+// idle: no work that uses the plan is pending on its device.
+void plan_free(spmv_plan_s *p, bool idle);
 // Build the row-sorted block copy of a finished plan (blocks.cu); leaves the plan unchanged
 // when the copy would not pay or its windows do not fit on chip.
 spmv_status build_row_blocks(spmv_plan_s *p, int sms, cudaStream_t s);
