@@ -101,6 +101,18 @@ __host__ __device__ inline CtaChunks cta_chunks(int g, int ntiles, int ctas, int
     return c;
 }
 
+// Element-wise loops over segments, of which there may be 2^31 - 65: a thread's elements first,
+// first + step, .. below n, counted in 64 bits (a 32-bit counter wraps when its last step crosses 2^31).
+template <typename F> __host__ __device__ inline void strided(int64_t first, int64_t step, int64_t n, F f) {
+    for (int64_t i = first; i < n; i += step) f(i);
+}
+// The blocks that rank the nonempty segments take SEG_BLOCK segments each, every thread SEG_IPT in a row.
+constexpr int SEG_IPT = 2, SEG_BLOCK = 512;
+__host__ __device__ inline int seg_rank_blocks(int n_major) { return (int)(((int64_t)n_major + SEG_BLOCK - 1) / SEG_BLOCK); }
+__host__ __device__ inline int64_t seg_rank_first(unsigned block, unsigned thread) {
+    return (int64_t)block * SEG_BLOCK + (int64_t)thread * SEG_IPT;
+}
+
 // What the one-vector passes (pass_kernel.cuh) read per step of 256 nonzeros beside them.
 struct alignas(16) StepRec {
     uint32_t heads[8];  // bit i of word j: a segment starts at position 32 j + i (the tile's masks)
@@ -249,7 +261,6 @@ cudaError_t launch_validate(const int32_t *ptr, const int32_t *idx, int n_major,
 // the empty segments in order; blk: seg_rank_blocks(n_major) ints of scratch.
 cudaError_t launch_seg_ranks(const int32_t *pptr, int n_major, int32_t *rank, int32_t *seglist, int32_t *emptylist,
                              int32_t *blk, int32_t *total, cudaStream_t s);
-int seg_rank_blocks(int n_major);
 // The step records of tiles of 256 spt nonzeros, from their masks and descriptors.
 cudaError_t launch_steps(const TileMeta *meta, const uint32_t *masks, int mwp, int ntiles, int spt,
                          const int32_t *seglist, StepRec *steps, cudaStream_t s);

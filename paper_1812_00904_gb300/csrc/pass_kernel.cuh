@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
         feed.start(gb, gridDim.x * bpc, turn > 0);
         if constexpr (SD) {
             if (turn == 0)
-                for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x)
-                    static_cast<XT *>(p.u)[p.emptylist[i]] = XT(0);
+                strided((int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, p.nempty,
+                        [&](int64_t i) { static_cast<XT *>(p.u)[p.emptylist[i]] = XT(0); });
             constexpr int xa = 16 / (int)sizeof(XT);
             const XT *src = static_cast<const XT *>(p.v);
             int len = p.n_minor;
@@ -499,10 +499,10 @@ __global__ void __launch_bounds__(WB * 32, 1) mvdot_kernel(const __grid_constant
         if (turn > 0) __syncthreads();  // every warp is done with the block before
         feed.start(gb, gridDim.x * p.bpc, turn > 0);
         if (turn == 0)
-            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.nempty; i += gridDim.x * blockDim.x) {
+            strided((int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, p.nempty, [&](int64_t i) {
                 const int col = p.emptylist[i];
                 for (int b = 0; b < p.kb; ++b) p.uv[b][col] = 0.f;
-            }
+            });
         const int2 w = p.win ? p.win[gb] : make_int2(0, p.n_minor);  // (windows begin on four entries)
         const float *vt = static_cast<const float *>(p.v) + (size_t)w.x * KV;
         if constexpr (ONCHIP) {

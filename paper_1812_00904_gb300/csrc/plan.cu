@@ -372,12 +372,12 @@ size_t setup_scratch_bytes(int P) {
 }
 
 // The nonempty segments in order and their ranks, for matrices with empty ones: every block
-// counts its SU_ITEMS segments, one block scans the counts, every block writes its part.
+// counts its SEG_BLOCK segments, one block scans the counts, every block writes its part.
 __global__ void __launch_bounds__(SU_THREADS) seg_count_kernel(const int32_t *__restrict__ pptr, int n_major,
                                                                int32_t *__restrict__ blk) {
-    const int j0 = blockIdx.x * SU_ITEMS + threadIdx.x * SU_IPT;
+    const int64_t j0 = seg_rank_first(blockIdx.x, threadIdx.x);
     int c = 0;
-    for (int i = 0; i < SU_IPT && j0 + i < n_major; ++i) c += pptr[j0 + i + 1] > pptr[j0 + i];
+    for (int i = 0; i < SEG_IPT && j0 + i < n_major; ++i) c += pptr[j0 + i + 1] > pptr[j0 + i];
     int total;
     block_exclusive(c, 0, AddOp(), &total);
     if (threadIdx.x == 0) blk[blockIdx.x] = total;
@@ -386,13 +386,13 @@ __global__ void __launch_bounds__(SU_THREADS) seg_rank_kernel(const int32_t *__r
                                                               const int32_t *__restrict__ blk, int32_t *__restrict__ rank,
                                                               int32_t *__restrict__ seglist,
                                                               int32_t *__restrict__ emptylist) {
-    const int j0 = blockIdx.x * SU_ITEMS + threadIdx.x * SU_IPT;
+    const int64_t j0 = seg_rank_first(blockIdx.x, threadIdx.x);
     int c = 0;
-    for (int i = 0; i < SU_IPT && j0 + i < n_major; ++i) c += pptr[j0 + i + 1] > pptr[j0 + i];
+    for (int i = 0; i < SEG_IPT && j0 + i < n_major; ++i) c += pptr[j0 + i + 1] > pptr[j0 + i];
     int total;
     int r = blk[blockIdx.x] + block_exclusive(c, 0, AddOp(), &total);
-    for (int i = 0; i < SU_IPT && j0 + i < n_major; ++i) {
-        const int j = j0 + i;
+    for (int i = 0; i < SEG_IPT && j0 + i < n_major; ++i) {
+        const int j = (int)(j0 + i);
         rank[j] = r;
         if (pptr[j + 1] > pptr[j])
             seglist[r++] = j;
@@ -402,10 +402,9 @@ __global__ void __launch_bounds__(SU_THREADS) seg_rank_kernel(const int32_t *__r
     }
 }
 
-int seg_rank_blocks(int n_major) { return (n_major + SU_ITEMS - 1) / SU_ITEMS; }
-
 cudaError_t launch_seg_ranks(const int32_t *pptr, int n_major, int32_t *rank, int32_t *seglist, int32_t *emptylist,
                              int32_t *blk, int32_t *total, cudaStream_t s) {
+    static_assert(SEG_BLOCK == SU_THREADS * SEG_IPT, "segments of a block");
     const int nb = seg_rank_blocks(n_major);
     if (nb <= 0) return cudaSuccess;
     seg_count_kernel<<<nb, SU_THREADS, 0, s>>>(pptr, n_major, blk);

@@ -2,6 +2,7 @@
 // entries of a log.  Linked with the library's host code (plans, routing, memory, serving) compiled by g++.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 #include <map>
@@ -75,6 +76,28 @@ void *fake_alloc(size_t n) {
     void *p = nullptr;
     take(&p, n, false);
     return p;
+}
+// segments seen once and in range: by the blocks that rank them, and by thread `thread` of `threads` in a strided loop
+int64_t fake_ranked_segments(int n_major, unsigned block, int64_t *lowest) {
+    int64_t n = 0;
+    *lowest = INT64_MAX;
+    for (unsigned t = 0; t < gbk::SEG_BLOCK / gbk::SEG_IPT; ++t) {
+        const int64_t j0 = gbk::seg_rank_first(block, t);
+        for (int i = 0; i < gbk::SEG_IPT && j0 + i < n_major; ++i, ++n) *lowest = std::min(*lowest, j0 + i);
+    }
+    return n;
+}
+int fake_rank_blocks(int n_major) { return gbk::seg_rank_blocks(n_major); }
+int64_t fake_strided(int64_t thread, int64_t threads, int64_t n, int64_t *lowest, int64_t *highest) {
+    int64_t seen = 0;
+    *lowest = INT64_MAX;
+    *highest = -1;
+    gbk::strided(thread, threads, n, [&](int64_t i) {
+        *lowest = std::min(*lowest, i);
+        *highest = std::max(*highest, i);
+        ++seen;
+    });
+    return seen;
 }
 
 // ---- the runtime
@@ -168,7 +191,6 @@ int stream_processors(int ntiles, int T, int nnz, int ctas, int C, int32_t *nzb)
     return np;
 }
 
-int seg_rank_blocks(int n_major) { return (n_major + 511) / 512; }
 spmv_status build_row_blocks(spmv_plan_s *, int, cudaStream_t) { return SPMV_OK; }
 cudaError_t launch_bank_order(const int32_t *, int, int, const int32_t *, const void *, int, int32_t *, void *, int32_t *,
                               int, int, cudaStream_t) { return cudaSuccess; }
