@@ -227,7 +227,10 @@ spmv_status build_row_blocks(spmv_plan_s *p, int sms, cudaStream_t s) {
     st = plan_create(&q, (int64_t)nseg, wmax, p->nnz, SPMV_CSR_TALL, bptr, sidx, svals, p->val_t, p->vec_t, s,
                      p->flags & SPMV_PLAN_BANK_ORDER, &o, &pi);
     if (st != SPMV_OK) return st;
-    if (!q->onchip || q->ctas * q->bpc != G) {  // the windows must sit in shared memory, block by block
+    // the windows must sit in shared memory, block by block: beside the staging of the pass that runs the
+    // copy (whole-step tiles; the budget above), else of the streaming kernel.  (q->onchip alone speaks of the
+    // streaming kernel's accumulating pass, which the copy never runs and which stages more.)
+    if (!(q->pass_sd || q->onchip) || q->ctas * q->bpc != G) {
         plan_free(q, true);  // (its set-up has been waited for)
         return SPMV_OK;
     }
