@@ -233,9 +233,11 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
             } else {
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
-                    const int pos = ps + (SD ? 8 * lane + (e ^ (4 * sw)) : 32 * e + lane);
+                    const int at = SD ? 8 * lane + (e ^ (4 * sw)) : 32 * e + lane, pos = ps + at;
                     const bool in = pos < p.nnz;
-                    ix[e] = in ? call_load(p.idx + pos) : 0;
+                    // (the pair adds zeros for the positions past the end: to places of their own, for 243
+                    // additions to one place took 10 us)
+                    ix[e] = in ? call_load(p.idx + pos) : SC && SD ? at % p.n_minor : 0;
                     va[e] = in ? to_acc<AT>(static_cast<const VT *>(p.vals)[pos]) : AT(0);
                 }
             }
