@@ -148,7 +148,8 @@ typedef struct {
     int32_t tiles;             /* execution tiles */
     int32_t zones;             /* z, overlap zones (Sec. II), z <= P-1 */
     int32_t max_zone_size;     /* V = max |S_k| (Sec. IV-A) */
-    int32_t short_on_chip;     /* 1 if the short vector lives in shared memory */
+    int32_t short_on_chip;     /* 1 if the short vector lives in shared memory (a long one, beside few
+                                  nonzeros, only as the input of the dot products) */
     int32_t batch_width;       /* vectors per pass of the accumulating direction of spmv_batch (1..8) */
     int64_t max_chunk_nnz, min_chunk_nnz;
     double imbalance;          /* Delta = P (max - min) / Z (Sec. VI), 0 when Z = 0 */

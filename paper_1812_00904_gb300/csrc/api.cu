@@ -75,6 +75,7 @@ size_t pass_vec_bytes(const spmv_plan_s *p) { return align_up((size_t)p->n_minor
 constexpr int PASS_MAX_COPIES = 16;
 struct PassGeometry {
     int warps, slots, copies;
+    int fit;  // warps whose staging shared memory holds beside one copy
     size_t smem;
 };
 // tiles of a CTA: no more warps than these can work
@@ -92,7 +93,8 @@ PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1) {
     const size_t slot = pass_slot_bytes(p->sv), all = (size_t)p->smem_max;
     const size_t fit = all > acc + vec ? (all - acc - vec) / slot : 0;
     const int most_warps = pass_warps(p->sv), work = std::min(most_warps, cta_tiles(p));
-    g.warps = (int)std::min<size_t>(std::max(work, std::min(most_warps, copy_warps(p, kv))), fit);
+    g.fit = (int)std::min<size_t>(fit, 1024);
+    g.warps = std::min(std::max(work, std::min(most_warps, copy_warps(p, kv))), g.fit);
     g.slots = 1;
     const size_t rest = vec + (size_t)g.warps * g.slots * slot;
     g.copies = 1;
@@ -101,11 +103,28 @@ PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1) {
     g.smem = g.copies * acc + rest;
     return g;
 }
-// A pass runs with at least 8 warps (or all a CTA has tiles for): fewer leave it to the streaming
-// kernel.  The pair wants 20: with 16 its two products run faster one by one, each with 32 warps
-// (294 + 261 us against 590; 501 with 20).
+// A pass runs with at least 8 warps, or with all that its tiles and the moving of its short vectors ask
+// for; fewer leave it to the streaming kernel, also where a CTA has a tile or two.  Dot products, us,
+// pass / streaming kernel, with 4, 6, 8 and 10 warps (FP32, m = 55,500 to 52,400): 20,000 nonzeros 10.3 /
+// 7.6, 8.7 / 7.8, 7.8 / 7.8, 7.4 / 7.9; 500,000 13.8 / 11.8, 11.3 / 15.5, 9.6 / 13.2, 9.3 / 12.9; 2.4M
+// 25.3 / 24.2, 19.0 / 24.1, 15.8 / 24.2, 14.1 / 24.2; one warp 26.5 / 7.6 for 20,000.  The pair wants 20:
+// with 16 its two products run faster one by one, each with 32 warps (294 + 261 us against 590 on the
+// 200M-nonzero matrix; 501 with 20).
 bool pass_fits(const spmv_plan_s *p, bool sc, bool sd) {
-    return pass_geometry(p, sc, sd).warps >= std::min(sc && sd ? std::min(20, pass_warps(p->sv)) : 8, cta_tiles(p));
+    const int least = sc && sd ? std::min(20, pass_warps(p->sv)) : 8;
+    return pass_geometry(p, sc, sd).warps >= std::min(least, std::max(cta_tiles(p), copy_warps(p, 1)));
+}
+// The accumulating product of a validated plan whose short vector leaves the pass fewer than all its
+// warps: with few nonzeros for the CTAs' copies of that vector (zeroed, written out and added up, 152 x
+// 50,000 elements), one copy in global memory is faster.  Where the lines cross, in nonzeros per element
+// of the copies: FP32 8 / 10 / 12 / 16 / 20 / 24 / 31 warps 0.95 / 0.73 / 0.63 / 0.55 / 0.54 / 0.58 / 0.54,
+// FP64 8 / 10 / 12 / 14 warps 1.2 / 0.93 / 0.63 / 0.56.  (us, pass / global: FP32, 10 warps, m = 52,400:
+// 500,000 nonzeros 30.7 / 11.3, 2.4M 36.5 / 23, 5M 44.2 / 42, 20M 94 / 132; 24 warps, m = 45,000: 25.7 /
+// 11.2, 29.9 / 23.0, 34.8 / 38.5.)  Short vectors that leave room for all warps stay on chip.
+bool scatter_off_chip(const spmv_plan_s *p) {
+    const int fit = pass_geometry(p, true, false).fit;
+    if (fit >= pass_warps(p->sv) || fit < 1) return false;
+    return (double)p->nnz < (double)p->ctas * p->n_minor * std::max(0.55, 8.0 / fit);
 }
 
 int kb_template(int kb) { return kb <= 1 ? 1 : kb <= 2 ? 2 : kb <= 4 ? 4 : 8; }
@@ -323,7 +342,8 @@ spmv_status run_scatter(spmv_plan_s *p, int kb, const void *const *in, void *con
     }
     if (kb == 1 && p->pass_sc) return run_pass(p, in[0], out[0], nullptr, nullptr, s, p);
     if (p->pass_mv && p->pass_sc) return run_mvscatter(p, kb, in, out, s);
-    if (!p->onchip && kb > 1) {
+    const bool onchip = p->onchip && !p->sc_global;
+    if (!onchip && kb > 1) {
         for (int b = 0; b < kb; ++b) {
             spmv_status st = run_scatter(p, 1, in + b, out + b, s);
             if (st != SPMV_OK) return st;
@@ -334,9 +354,9 @@ spmv_status run_scatter(spmv_plan_s *p, int kb, const void *const *in, void *con
     a.sp = base_params(p);
     a.sp.kb = kb;
     for (int b = 0; b < kb; ++b) a.sp.vin[b] = in[b];
-    set_geometry(p, a, MODE_SCATTER, kb_template(kb), p->onchip);
+    set_geometry(p, a, MODE_SCATTER, kb_template(kb), onchip);
     a.sp.part = p->part;
-    if (!p->onchip) CUDA_TRY(cudaMemsetAsync(p->part, 0, (size_t)p->n_minor * sizeof(double), s));
+    if (!onchip) CUDA_TRY(cudaMemsetAsync(p->part, 0, (size_t)p->n_minor * sizeof(double), s));
     a.stream = s;
     {
         ProfScope ps(p, 0, s);
@@ -345,7 +365,7 @@ spmv_status run_scatter(spmv_plan_s *p, int kb, const void *const *in, void *con
     {
         ProfScope ps(p, 1, s);
         const bool f64 = p->vec_t == SPMV_F64;
-        CUDA_TRY(launch_combine(f64, f64 || !p->onchip, p->part, p->onchip ? p->ctas : 1, p->n_minor, kb, out, s));
+        CUDA_TRY(launch_combine(f64, f64 || !onchip, p->part, onchip ? p->ctas : 1, p->n_minor, kb, out, s));
     }
     return SPMV_OK;
 }
@@ -904,7 +924,8 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
         p->pass_sd = pass_fits(p, false, true);
         p->pass_mv = p->pass_sd && p->sv != 8;
     } else if (nnz > 0 && p->T % 256 == 0 && !(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL))) {
-        p->pass_sc = pass_fits(p, true, false);
+        p->sc_global = scatter_off_chip(p);
+        p->pass_sc = !p->sc_global && pass_fits(p, true, false);
         p->pass_sd = pass_fits(p, false, true);
         p->pass_pair = pass_fits(p, true, true);
         p->pass_mv = p->sv != 8;
@@ -921,8 +942,8 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     }
     const size_t part_bytes =
         (pi && pi->segdot_only) ? 16
-                                : std::max(p->onchip ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa
-                                                     : (size_t)p->n_minor * sizeof(double),
+                                : std::max(p->onchip && !p->sc_global ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa
+                                                                      : (size_t)p->n_minor * sizeof(double),
                                            p->pass_sc || p->pass_pair ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa : (size_t)0);
     // ranks of the nonempty segments, when some are empty
     int32_t *&rank = p->segrank;

@@ -47,6 +47,7 @@ struct spmv_plan_s {
     uint32_t *masks = nullptr;
     // one-vector passes (pass_kernel.cuh): which products they serve (the short vectors fit on chip)
     bool pass_sc = false, pass_sd = false, pass_pair = false;
+    bool sc_global = false;  // the accumulating product keeps its short vector in global memory (few nonzeros)
     bool pass_mv = false;  // the dot products of several vectors run in mvdot_kernel
     gbk::StepRec *steps = nullptr;
     // nonempty / empty segments and ranks among the nonempty (when some are empty)

@@ -138,7 +138,7 @@ cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cu
     return memcpy(d, s, n), cudaSuccess;
 }
 cudaError_t cudaMemset(void *d, int v, size_t n) { return memset(d, v, n), cudaSuccess; }
-cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) { return memset(d, v, n), cudaSuccess; }
+cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) { return memset(d, v, n), cudaSuccess; }  // (plan memory)
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *) {
     memset(a, 0, sizeof(*a));
     a->type = cudaMemoryTypeDevice;

@@ -37,6 +37,10 @@ class HostLib:
         self.lib.spmv_plan_ex.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int64, ctypes.c_int64, ctypes.c_int32,
                                           ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32,
                                           ctypes.c_int32, ctypes.c_void_p, ctypes.c_uint32, ctypes.c_void_p]
+        for name, vectors in (("spmv", 2), ("spvtm", 2), ("spmv_pair", 4), ("spmv_dvalues", 3)):
+            getattr(self.lib, name).argtypes = [ctypes.c_void_p] * (vectors + 2)
+        self.lib.spmv_batch.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_void_p, ctypes.c_int64,
+                                        ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
         self.lib.spmv_last_error.restype = ctypes.c_char_p
         self.reset()
 
@@ -64,3 +68,19 @@ class HostLib:
                                    F64 if val == F64 else F32, None, flags, opts)
         assert st == 0, self.lib.spmv_last_error().decode()
         return out
+
+    def launches(self, plan, call, *extra):
+        """The kernels that a call on device vectors launches: [(name, warps of a CTA, CTAs)]."""
+        self.log()
+        vectors = {"spmv": 2, "spvtm": 2, "spmv_pair": 4, "spmv_dvalues": 3}
+        if call == "batch":
+            op, k, ld_in, ld_out = extra
+            st = self.lib.spmv_batch(plan, op, k, 0x100000, ld_in, 0x200000, ld_out, None)
+        else:
+            st = getattr(self.lib, call)(plan, *(0x100000 * (i + 1) for i in range(vectors[call])), None)
+        assert st == 0, self.lib.spmv_last_error().decode()
+        return [(" ".join(w[:-2]), int(w[-2]), int(w[-1])) for w in (line.split() for line in self.log())
+                if len(w) > 2 and w[-1].isdigit() and w[-2].isdigit()]
+
+    def close(self, plan):
+        self.lib.spmv_plan_destroy(plan)
