@@ -98,7 +98,10 @@ PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1) {
     g.slots = 1;
     const size_t rest = vec + (size_t)g.warps * g.slots * slot;
     g.copies = 1;
-    const int most = p->sv == 8 ? 2 : PASS_MAX_COPIES;  // (adding up FP64 copies costs more than they save)
+    // adding up FP64 copies costs more than they save, but for a second one with four nonzeros or more to an
+    // element (one / two copies, us: m = 4,000, 50,000 nonzeros 7.4 / 8.5, 1M 11.5 / 12.2, 8M 40.2 / 39.3;
+    // m = 300, 500,000 11.0 / 10.0)
+    const int most = p->sv != 8 ? PASS_MAX_COPIES : p->nnz >= (int64_t)4 * p->ctas * p->n_minor ? 2 : 1;
     while (sc && 2 * g.copies <= std::min({g.warps, work, most}) && 2 * g.copies * acc + rest <= all) g.copies *= 2;
     g.smem = g.copies * acc + rest;
     return g;
@@ -126,6 +129,16 @@ bool scatter_off_chip(const spmv_plan_s *p) {
     if (fit >= pass_warps(p->sv) || fit < 1) return false;
     return (double)p->nnz < (double)p->ctas * p->n_minor * std::max(0.55, 8.0 / fit);
 }
+
+// FP64 batches of small matrices accumulate with a pass for each vector in one launch: in the streaming
+// kernel's pass over several vectors a few tiles of 256 nonzeros a CTA leave most warps without work.  As
+// many vectors as keep the partials within F64_PARTIALS, on matrices of at most F64_TILES tiles a CTA.
+// 8 vectors, us, streaming kernel with tiles of 256 / of the size it chose for itself / the passes: m = 300,
+// 4,800 nonzeros 20.1 / 13.2 / 6.3, 93,000 23.7 / 17.8 / 13.0; m = 1,000, 49,000 26.9 / 17.4 / 10.6; m =
+// 8,000, 4,900 60 / 52 / 21, 97,000 88 / 67 / 68.  Beyond the line: m = 40, 144,000 39 / 34 / 22, 357,000
+// 70 / 80 / 85; m = 300, 184,000 26 / 28 / 19, 459,000 45 / 50 / 50.
+constexpr int F64_TILES = 6;
+constexpr size_t F64_PARTIALS = 32 << 20;
 
 int kb_template(int kb) { return kb <= 1 ? 1 : kb <= 2 ? 2 : kb <= 4 ? 4 : 8; }
 
@@ -305,6 +318,7 @@ static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *
     pp.acc_bytes = sc ? (int)pass_acc_bytes(p) : 0;
     pp.vec_bytes = sd ? (int)pass_vec_bytes(p) : 0;
     pp.x = x;
+    pp.xv[0] = x;
     pp.v = v;
     pp.u = u;
     const PassGeometry g = pass_geometry(p, sc, sd);
@@ -333,6 +347,24 @@ static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *
 
 static spmv_status run_mvscatter(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s);
 
+// The accumulating product of kb FP64 vectors, a pass for each in one launch, then the combine.
+static spmv_status run_scatter_f64(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s) {
+    const PassGeometry g = pass_geometry(p, true, false);
+    PassParams pp = pass_params(p);
+    pp.acc_bytes = (int)pass_acc_bytes(p);
+    pp.kb = kb;
+    for (int b = 0; b < kb; ++b) pp.xv[b] = in[b];
+    pp.slots = g.slots;
+    pp.copies = g.copies;
+    {
+        ProfScope ps(p, 0, s);
+        CUDA_TRY(launch_pass(p, true, false, pp, g.warps, (int)g.smem, s));
+    }
+    ProfScope ps(p, 1, s);
+    CUDA_TRY(launch_combine(true, true, p->part, p->ctas, p->n_minor, kb, out, s));
+    return SPMV_OK;
+}
+
 spmv_status run_scatter(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s) {
     const size_t out_bytes = (size_t)p->n_minor * p->sx;
     if (p->nnz == 0 || p->n_major == 0) {
@@ -342,6 +374,7 @@ spmv_status run_scatter(spmv_plan_s *p, int kb, const void *const *in, void *con
     }
     if (kb == 1 && p->pass_sc) return run_pass(p, in[0], out[0], nullptr, nullptr, s, p);
     if (p->pass_mv && p->pass_sc) return run_mvscatter(p, kb, in, out, s);
+    if (kb > 1 && p->f64_width > 1) return run_scatter_f64(p, kb, in, out, s);
     const bool onchip = p->onchip && !p->sc_global;
     if (!onchip && kb > 1) {
         for (int b = 0; b < kb; ++b) {
@@ -613,8 +646,9 @@ spmv_status run_op(spmv_plan_s *p, int op, int k, const void *const *in, void *c
     const bool scatter = (op == SPMV_OP_AX) == (p->layout == SPMV_CSC_WIDE);
     if (scatter && p->tplan && p->nnz > 0) return run_row_blocks(p, k, in, out, s);
     if (!scatter) return run_segdot(p, k, in, out, s);
-    for (int g0 = 0; g0 < k; g0 += p->batch_width) {
-        const int kb = std::min(p->batch_width, k - g0);
+    const int width = std::max(p->batch_width, p->f64_width);
+    for (int g0 = 0; g0 < k; g0 += width) {
+        const int kb = std::min(width, k - g0);
         spmv_status st = run_scatter(p, kb, in + g0, out + g0, s);
         if (st != SPMV_OK) return st;
     }
@@ -940,11 +974,15 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
                 if (p->batch_width == 1 && pass_geometry(p, true, false, kv).warps >= full - full / 4) p->batch_width = kv;
         }
     }
+    if (p->sv == 8 && p->pass_sc && cta_tiles(p) <= F64_TILES) {
+        p->f64_width = KB_MAX;
+        while (p->f64_width > 1 && (size_t)p->ctas * p->f64_width * p->n_minor * 8 > F64_PARTIALS) p->f64_width /= 2;
+    }
     const size_t part_bytes =
         (pi && pi->segdot_only) ? 16
                                 : std::max(p->onchip && !p->sc_global ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa
                                                                       : (size_t)p->n_minor * sizeof(double),
-                                           p->pass_sc || p->pass_pair ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa : (size_t)0);
+                                           p->pass_sc || p->pass_pair ? (size_t)p->ctas * std::max(p->batch_width, p->f64_width) * p->n_minor * p->sa : (size_t)0);
     // ranks of the nonempty segments, when some are empty
     int32_t *&rank = p->segrank;
     if ((p->pass_sc || p->pass_sd || p->pass_pair || p->pass_mv) && p->nempty > 0) {

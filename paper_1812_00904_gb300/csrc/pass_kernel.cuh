@@ -168,7 +168,8 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
     }
     __shared__ int next_chunk;
     Feed feed(p, smem + p.copies * p.acc_bytes + p.vec_bytes, &next_chunk);
-    const XT *xg = static_cast<const XT *>(p.x);
+    // (FP64 batches: a grid row for each vector)
+    const XT *xg = static_cast<const XT *>(SC && !SD && sizeof(AT) == 8 ? p.xv[blockIdx.y] : p.x);
     const int sh = (lane & 3) << 3;  // the lane's byte of its segment-start word
     const int sw = (lane >> 2) & 1;  // staggered shared-memory loads
     unsigned char *slot;
@@ -430,7 +431,7 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
 
     if constexpr (SC) {
         __syncthreads();
-        AT *part = static_cast<AT *>(p.part) + (size_t)blockIdx.x * p.n_minor;
+        AT *part = static_cast<AT *>(p.part) + ((size_t)blockIdx.x * gridDim.y + blockIdx.y) * p.n_minor;
         const AT *acc0 = reinterpret_cast<const AT *>(smem);
         if (p.copies == 1) {
             for (int i = threadIdx.x; i < p.n_minor; i += blockDim.x) part[i] = acc0[i];
@@ -889,7 +890,8 @@ cudaError_t launch_pass_one(const PassParams &p, int grid, int warps, int smem, 
     static SmemLimit lim;
     const cudaError_t e = ensure_smem_limit(kern, lim, smem);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(kern, dim3(grid), dim3(warps * 32), smem, s, p);
+    const int vectors = SC && !SD && sizeof(VT) == 8 ? std::max(1, p.kb) : 1;
+    return launch_overlapped(kern, dim3(grid, vectors), dim3(warps * 32), smem, s, p);
 }
 
 template <typename VT, typename XT>

@@ -5,6 +5,7 @@ import pytest
 from host_lib import BF16, F16, F32, F64, HostLib
 
 SLOT = {F32: 2112, BF16: 1600, F16: 1600, F64: 3136}
+MOST = {F32: 32, BF16: 32, F16: 32, F64: 16}
 ROOM = 232448 - 1024 - 512
 
 
@@ -19,13 +20,11 @@ def m_for(val, warps, vectors=1):
     return (ROOM - warps * SLOT[val]) // (8 if val == F64 else 4) // vectors // 32 * 32
 
 
-@pytest.mark.parametrize("val", [F32, BF16, F16, F64])
 @pytest.mark.parametrize("nnz", [5_000, 38_000, 400_000, 3_000_000, 30_000_000])
-@pytest.mark.parametrize("warps", [1, 4, 7, 8, 12, 16, 20, 31, 32])
+@pytest.mark.parametrize("val,warps", [(v, w) for v in (F32, BF16, F16, F64) for w in (1, 4, 7, 8, 12, 16, 20, 31, 32)
+                                       if w <= MOST[v]])
 def test_a_pass_has_the_warps_its_vectors_need(host, val, nnz, warps):
-    most = 16 if val == F64 else 32
-    if warps > most:
-        pytest.skip("more warps than the pass takes")
+    most = MOST[val]
     host.reset()
     m = m_for(val, warps)
     plan = host.plan(m, 1_000, nnz, val)
@@ -39,13 +38,10 @@ def test_a_pass_has_the_warps_its_vectors_need(host, val, nnz, warps):
     host.close(plan)
 
 
-@pytest.mark.parametrize("val", [F32, BF16, F64])
 @pytest.mark.parametrize("nnz", [5_000, 150_000, 3_000_000])
-@pytest.mark.parametrize("warps", [1, 8, 16, 19, 20, 32])
+@pytest.mark.parametrize("val,warps", [(v, w) for v in (F32, BF16, F64) for w in (1, 8, 16, 19, 20, 32) if w <= MOST[v]])
 def test_the_pair_is_one_pass_with_enough_warps(host, val, nnz, warps):
-    most, least = (16, 16) if val == F64 else (32, 20)
-    if warps > most:
-        pytest.skip("more warps than the pass takes")
+    least = 16 if val == F64 else 20
     host.reset()
     plan = host.plan(m_for(val, warps, vectors=2), 1_000, nnz, val)
     kernels = [k for k, _, _ in host.launches(plan, "spmv_pair")]
@@ -62,3 +58,14 @@ def test_short_vectors_with_room_for_all_warps_stay_on_chip(host, val, m):
         assert host.launches(plan, "spvtm")[0][0] == "pass segdot"
         assert host.launches(plan, "spmv_pair")[0][0] == ("pass pair" if m < 20_000 else "pass segdot")
         host.close(plan)
+
+
+@pytest.mark.parametrize("m,nnz,launches", [(300, 4_877, 1), (4_000, 60_000, 2), (15_000, 5_000, 1), (12_000, 100_000, 4),
+                                            (300, 233_472, 1), (300, 233_473, 0), (300, 8_000_000, 0)])
+def test_f64_batches_of_small_matrices_take_a_pass_for_each_vector(host, m, nnz, launches):
+    host.reset()
+    plan = host.plan(m, 1_000, nnz, F64)
+    kernels = [k for k, _, _ in host.launches(plan, "batch", 0, 8, 1_000, m)]
+    assert kernels.count("pass scatter") == launches
+    assert ("stream scatter" in kernels) == (launches == 0)
+    host.close(plan)
