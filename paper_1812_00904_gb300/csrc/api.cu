@@ -70,7 +70,13 @@ cudaError_t launch_pass(const spmv_plan_s *p, bool sc, bool sd, const PassParams
 // in between, so copies help where they fit: with 1 / 2 / 4 / 8 / 16 of them the accumulating
 // product of the 150M-nonzero tall matrix (n = 2,000) takes 348 / 318 / 302 / 290 / 262 us, the pair
 // 441 / 419 / 406 / 393 / 372; 32 add nothing.
-size_t pass_acc_bytes(const spmv_plan_s *p) { return align_up((size_t)p->n_minor * p->sa, 128); }
+// One-vector SC into very short vectors: an element for every lane of a warp (pass_kernel's LANES).  The
+// FP32 pair's additions stand conflicts better (one row, 5,000 nonzeros 16 us) and stay as they are.
+constexpr int PASS_LANES_MOST = 32;
+bool pass_lanes(const spmv_plan_s *p, bool sc, bool sd) { return sc && (!sd || p->sv == 8) && p->n_minor <= PASS_LANES_MOST; }
+size_t pass_acc_bytes(const spmv_plan_s *p, bool sd) {
+    return align_up((size_t)p->n_minor * (pass_lanes(p, true, sd) ? 32 : 1) * p->sa, 128);
+}
 size_t pass_vec_bytes(const spmv_plan_s *p) { return align_up((size_t)p->n_minor * p->sx, 128); }
 constexpr int PASS_MAX_COPIES = 16;
 struct PassGeometry {
@@ -87,14 +93,17 @@ int cta_tiles(const spmv_plan_s *p) {
 // out), even if it has fewer tiles: 103 CTAs of one tile and one warp each took 20 us more for 45,889
 // elements than the streaming kernel.
 int copy_warps(const spmv_plan_s *p, int kv) { return (int)std::min<int64_t>(32, ((int64_t)p->n_minor * kv + 511) / 512); }
-PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1) {
+// rows: vectors that take a grid row each (FP64 batches), which share the SMs: fewer warps each to move them
+// (8 vectors of 8,000, 97,000 nonzeros 68 us with 16 warps, which fill an SM, 56 with 2).
+PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1, int rows = 1) {
     PassGeometry g;
-    const size_t acc = sc ? align_up((size_t)p->n_minor * kv * p->sa, 128) : 0, vec = (sd ? pass_vec_bytes(p) : 0) + PASS_BAR_BYTES;
+    const bool lanes = kv == 1 && pass_lanes(p, sc, sd);  // (a warp for every two rows' sums over the lanes)
+    const size_t acc = sc ? align_up((size_t)p->n_minor * (lanes ? 32 : kv) * p->sa, 128) : 0, vec = (sd ? pass_vec_bytes(p) : 0) + PASS_BAR_BYTES;
     const size_t slot = pass_slot_bytes(p->sv), all = (size_t)p->smem_max;
     const size_t fit = all > acc + vec ? (all - acc - vec) / slot : 0;
     const int most_warps = pass_warps(p->sv), work = std::min(most_warps, cta_tiles(p));
     g.fit = (int)std::min<size_t>(fit, 1024);
-    g.warps = std::min(std::max(work, std::min(most_warps, copy_warps(p, kv))), g.fit);
+    g.warps = std::min(std::max(work, std::min(most_warps, copy_warps(p, lanes ? 256 : kv)) / rows), g.fit);
     g.slots = 1;
     const size_t rest = vec + (size_t)g.warps * g.slots * slot;
     g.copies = 1;
@@ -135,7 +144,7 @@ bool scatter_off_chip(const spmv_plan_s *p) {
 // many vectors as keep the partials within F64_PARTIALS, on matrices of at most F64_TILES tiles a CTA.
 // 8 vectors, us, streaming kernel with tiles of 256 / of the size it chose for itself / the passes: m = 300,
 // 4,800 nonzeros 20.1 / 13.2 / 6.3, 93,000 23.7 / 17.8 / 13.0; m = 1,000, 49,000 26.9 / 17.4 / 10.6; m =
-// 8,000, 4,900 60 / 52 / 21, 97,000 88 / 67 / 68.  Beyond the line: m = 40, 144,000 39 / 34 / 22, 357,000
+// 8,000, 4,900 60 / 52 / 20, 97,000 88 / 67 / 56.  Beyond the line: m = 40, 144,000 39 / 34 / 22, 357,000
 // 70 / 80 / 85; m = 300, 184,000 26 / 28 / 19, 459,000 45 / 50 / 50.
 constexpr int F64_TILES = 6;
 constexpr size_t F64_PARTIALS = 32 << 20;
@@ -315,7 +324,8 @@ static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *
                             spmv_plan_s *prof, int id_dot = 2, int id_fix = 3) {
     const bool sc = y != nullptr, sd = u != nullptr;
     PassParams pp = pass_params(p);
-    pp.acc_bytes = sc ? (int)pass_acc_bytes(p) : 0;
+    pp.acc_bytes = sc ? (int)pass_acc_bytes(p, sd) : 0;
+    pp.lanes = pass_lanes(p, sc, sd);
     pp.vec_bytes = sd ? (int)pass_vec_bytes(p) : 0;
     pp.x = x;
     pp.xv[0] = x;
@@ -349,9 +359,10 @@ static spmv_status run_mvscatter(spmv_plan_s *p, int kb, const void *const *in, 
 
 // The accumulating product of kb FP64 vectors, a pass for each in one launch, then the combine.
 static spmv_status run_scatter_f64(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s) {
-    const PassGeometry g = pass_geometry(p, true, false);
+    const PassGeometry g = pass_geometry(p, true, false, 1, kb);
     PassParams pp = pass_params(p);
-    pp.acc_bytes = (int)pass_acc_bytes(p);
+    pp.acc_bytes = (int)pass_acc_bytes(p, false);
+    pp.lanes = pass_lanes(p, true, false);
     pp.kb = kb;
     for (int b = 0; b < kb; ++b) pp.xv[b] = in[b];
     pp.slots = g.slots;

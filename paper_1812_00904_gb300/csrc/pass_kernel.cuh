@@ -140,7 +140,10 @@ template <typename VT, bool VALS = true> struct StepFeed {
 // combine and fix-up, streaming kernel before, this one now (us): 200M FP32 nonzeros, m = 20,000, bank
 // order: pair 640 -> 386, SC 362 -> 294, SD 303 -> 261; 150M, n = 2,000: pair 538 -> 369, SC 313 ->
 // 262, SD 242 -> 207; 8M FP64, n = 4,000: pair 121 -> 76, SC 62 -> 42, SD 69 -> 48.
-template <typename VT, typename XT, bool SC, bool SD, int WB>
+// LANES: SC into very short vectors (PASS_LANES_MOST elements): every lane has an element of its own for
+// each row, [row][lane], so that the lanes of a warp never add to the same place (one row, 51,000
+// nonzeros: 58 us FP64 and 48 FP32 without, the streaming kernel 31 and 26).
+template <typename VT, typename XT, bool SC, bool SD, bool LANES, int WB>
 __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant__ PassParams p) {
     using AT = typename Acc<VT>::type;
     using AT2 = typename Pair<AT>::type;
@@ -154,7 +157,8 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
     constexpr bool DEFER = sizeof(AT) == 8 || !SD;
     extern __shared__ __align__(128) unsigned char smem[];
     // this warp's copy of the accumulator (warps share p.copies of them)
-    AT *acc = reinterpret_cast<AT *>(smem + (threadIdx.x >> 5) % p.copies * p.acc_bytes);
+    AT *acc = reinterpret_cast<AT *>(smem + (threadIdx.x >> 5) % p.copies * p.acc_bytes) + (LANES ? threadIdx.x & 31 : 0);
+    auto place = [&](int row) { return acc + (LANES ? 32 * row : row); };
     XT *vs = reinterpret_cast<XT *>(smem + p.copies * p.acc_bytes);
     const int lane = threadIdx.x & 31;
     // the combine and the zone fix-up may be launched: their blocks find room as this grid's CTAs end
@@ -309,8 +313,8 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     if constexpr (!DEFER) {
-                        atomicAdd(acc + ix[e], c[e]);
-                    } else if (!try_add(acc + ix[e], va[e], c[e])) {
+                        atomicAdd(place(ix[e]), c[e]);
+                    } else if (!try_add(place(ix[e]), va[e], c[e])) {
                         failed |= 1u << e;
                     }
                 }
@@ -325,7 +329,7 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
                             v = va[q];
                             x = c[q];
                         }
-                    if (try_add(acc + r, v, x)) failed &= failed - 1u;
+                    if (try_add(place(r), v, x)) failed &= failed - 1u;
                 }
             }
             if constexpr (SD) {  // into the order of the positions
@@ -433,7 +437,15 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
         __syncthreads();
         AT *part = static_cast<AT *>(p.part) + ((size_t)blockIdx.x * gridDim.y + blockIdx.y) * p.n_minor;
         const AT *acc0 = reinterpret_cast<const AT *>(smem);
-        if (p.copies == 1) {
+        if constexpr (LANES) {  // (a warp takes a row: its 32 sums, then a butterfly)
+            for (int i = threadIdx.x; i < 32 * p.n_minor; i += blockDim.x) {
+                AT t = acc0[i];
+                for (int r = 1; r < p.copies; ++r) t += acc0[r * (p.acc_bytes / (int)sizeof(AT)) + i];
+#pragma unroll
+                for (int d = 16; d >= 1; d >>= 1) t += __shfl_xor_sync(FULL, t, d);
+                if (lane == 0) part[i >> 5] = t;
+            }
+        } else if (p.copies == 1) {
             for (int i = threadIdx.x; i < p.n_minor; i += blockDim.x) part[i] = acc0[i];
         } else {
             for (int i = threadIdx.x; i < p.n_minor; i += blockDim.x) {
@@ -883,10 +895,10 @@ cudaError_t launch_dvalues(const PassParams &p, int grid, int warps, int smem, c
     return launch_overlapped(kern, dim3(grid), dim3(warps * 32), smem, s, p);
 }
 
-template <typename VT, typename XT, bool SC, bool SD>
+template <typename VT, typename XT, bool SC, bool SD, bool LANES>
 cudaError_t launch_pass_one(const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
     constexpr int WB = pass_warps(sizeof(VT));
-    auto kern = pass_kernel<VT, XT, SC, SD, WB>;
+    auto kern = pass_kernel<VT, XT, SC, SD, LANES, WB>;
     static SmemLimit lim;
     const cudaError_t e = ensure_smem_limit(kern, lim, smem);
     if (e != cudaSuccess) return e;
@@ -896,9 +908,15 @@ cudaError_t launch_pass_one(const PassParams &p, int grid, int warps, int smem, 
 
 template <typename VT, typename XT>
 cudaError_t launch_pass(bool sc, bool sd, const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
-    if (sc && sd) return launch_pass_one<VT, XT, true, true>(p, grid, warps, smem, s);
-    if (sc) return launch_pass_one<VT, XT, true, false>(p, grid, warps, smem, s);
-    return launch_pass_one<VT, XT, false, true>(p, grid, warps, smem, s);
+    if (sc && sd) {
+        if constexpr (sizeof(VT) == 8)
+            if (p.lanes) return launch_pass_one<VT, XT, true, true, true>(p, grid, warps, smem, s);
+        return launch_pass_one<VT, XT, true, true, false>(p, grid, warps, smem, s);
+    }
+    if (sc)
+        return p.lanes ? launch_pass_one<VT, XT, true, false, true>(p, grid, warps, smem, s)
+                       : launch_pass_one<VT, XT, true, false, false>(p, grid, warps, smem, s);
+    return launch_pass_one<VT, XT, false, true, false>(p, grid, warps, smem, s);
 }
 
 }  // namespace gbk
