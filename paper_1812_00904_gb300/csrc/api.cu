@@ -119,12 +119,16 @@ PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1, i
 // for; fewer leave it to the streaming kernel, also where a CTA has a tile or two.  Dot products, us,
 // pass / streaming kernel, with 4, 6, 8 and 10 warps (FP32, m = 55,500 to 52,400): 20,000 nonzeros 10.3 /
 // 7.6, 8.7 / 7.8, 7.8 / 7.8, 7.4 / 7.9; 500,000 13.8 / 11.8, 11.3 / 15.5, 9.6 / 13.2, 9.3 / 12.9; 2.4M
-// 25.3 / 24.2, 19.0 / 24.1, 15.8 / 24.2, 14.1 / 24.2; one warp 26.5 / 7.6 for 20,000.  The pair wants 20:
-// with 16 its two products run faster one by one, each with 32 warps (294 + 261 us against 590 on the
-// 200M-nonzero matrix; 501 with 20).
+// 25.3 / 24.2, 19.0 / 24.1, 15.8 / 24.2, 14.1 / 24.2; one warp 26.5 / 7.6 for 20,000.  The pair wants 20
+// on large matrices: with 16 its two products run faster one by one, each with 32 warps (294 + 261 us
+// against 590 on the 200M-nonzero matrix; 501 with 20).  On smaller ones fewer will do (one pass / two,
+// us, FP32 with 6, 8, 12 and 16 warps): 20,000 nonzeros 19.0 / 17.9, 17.7 / 17.9, 16.2 / 17.3, 15.7 /
+// 16.9; 300,000 25.9 / 24.5, 23.0 / 24.1, 21.5 / 23.6, 20.9 / 23.1; 2.4M 40 / 31, 35 / 31, 30.2 / 30.5,
+// 28.0 / 29.9; 8M 82 / 50, 66 / 50, 52.5 / 50.3, 46.8 / 49.6.
 bool pass_fits(const spmv_plan_s *p, bool sc, bool sd) {
-    const int least = sc && sd ? std::min(20, pass_warps(p->sv)) : 8;
-    return pass_geometry(p, sc, sd).warps >= std::min(least, std::max(cta_tiles(p), copy_warps(p, 1)));
+    const int tiles = cta_tiles(p);
+    const int least = !(sc && sd) || tiles <= 8 ? 8 : tiles <= 64 ? 12 : std::min(20, pass_warps(p->sv));
+    return pass_geometry(p, sc, sd).warps >= std::min(least, std::max(tiles, copy_warps(p, 1)));
 }
 // The accumulating product of a validated plan whose short vector leaves the pass fewer than all its
 // warps: with few nonzeros for the CTAs' copies of that vector (zeroed, written out and added up, 152 x

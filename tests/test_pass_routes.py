@@ -38,10 +38,11 @@ def test_a_pass_has_the_warps_its_vectors_need(host, val, nnz, warps):
     host.close(plan)
 
 
-@pytest.mark.parametrize("nnz", [5_000, 150_000, 3_000_000])
-@pytest.mark.parametrize("val,warps", [(v, w) for v in (F32, BF16, F64) for w in (1, 8, 16, 19, 20, 32) if w <= MOST[v]])
-def test_the_pair_is_one_pass_with_enough_warps(host, val, nnz, warps):
-    least = 16 if val == F64 else 20
+@pytest.mark.parametrize("nnz,least", [(5_000, 8), (311_296, 8), (311_297, 12), (3_000_000, 12), (30_000_000, 20)])
+@pytest.mark.parametrize("val,warps", [(v, w) for v in (F32, BF16, F64) for w in (1, 7, 8, 11, 12, 16, 19, 20, 32)
+                                       if w <= MOST[v]])
+def test_the_pair_is_one_pass_with_enough_warps(host, val, nnz, least, warps):
+    least = min(least, MOST[val])
     host.reset()
     plan = host.plan(m_for(val, warps, vectors=2), 1_000, nnz, val)
     kernels = [k for k, _, _ in host.launches(plan, "spmv_pair")]
