@@ -212,8 +212,14 @@ spmv_status spmv_plan_coo(spmv_plan_t *out, int64_t m, int64_t n, int64_t nnz, i
                           const int32_t *rows, const int32_t *cols, const void *vals, int32_t val_dtype,
                           int32_t vec_dtype, void *stream, uint32_t flags, const spmv_plan_opts *opts);
 
-/* Release the plan's workspace.  Accepts NULL.  The caller's arrays are untouched. */
+/* Release the plan's workspace.  Accepts NULL.  The caller's arrays are untouched.  Waits for the
+ * plan's device, whichever device is current.  Up to 512 MB per device of what plans held is kept
+ * for the next plan (the library gives it back when an allocation of its own fails). */
 spmv_status spmv_plan_destroy(spmv_plan_t plan);
+
+/* Give the memory that the library keeps for later plans back to the current device, so that other
+ * allocators can have it.  Plans that exist keep theirs.  Callable from any thread. */
+spmv_status spmv_release_memory(void);
 
 /* Copy the plan summary into *info (host memory). */
 spmv_status spmv_plan_info(spmv_plan_t plan, spmv_plan_info_t *info);

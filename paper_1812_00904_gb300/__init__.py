@@ -16,7 +16,7 @@ from ._lib import (SPMV_BF16, SPMV_CSC_WIDE, SPMV_CSR_TALL, SPMV_F16, SPMV_F32, 
                    SPMV_PLAN_ROW_BLOCKS, SPMV_PLAN_SHORT_IN_GLOBAL, SpmvError)
 
 __all__ = [
-    "spmv_plan", "spmv_plan_ex", "spmv_plan_coo", "spmv_plan_destroy", "spmv_plan_info", "spmv_plan_chunks", "spmv", "spvtm", "spmv_pair",
+    "spmv_plan", "spmv_plan_ex", "spmv_plan_coo", "spmv_plan_destroy", "spmv_release_memory", "spmv_plan_info", "spmv_plan_chunks", "spmv", "spvtm", "spmv_pair",
     "spmv_batch", "spmv_dvalues", "spmv_noalloc", "spmv_normal", "spmv_cgls", "spmv_check", "spmv_plan_export", "spmv_profile_read", "spmv_profile_reset", "spmv_profile_enable", "spmv_last_error",
     "spmv_version", "serve_create", "serve_register", "serve_register_host", "serve_submit", "serve_poll",
     "serve_wait", "serve_stats", "serve_destroy", "Plan", "SparseMatVec", "sparse_matvec", "SpmvError",
@@ -89,6 +89,11 @@ def spmv_plan_coo(m, n, nnz, layout, rows, cols, vals, val_dtype, vec_dtype, str
 
 def spmv_plan_destroy(plan):
     _lib.call("spmv_plan_destroy", plan)
+
+
+def spmv_release_memory():
+    """Give the device memory that the library keeps for later plans (at most 512 MB) back to the current device."""
+    _lib.call("spmv_release_memory")
 
 
 def spmv_plan_info(plan) -> dict:

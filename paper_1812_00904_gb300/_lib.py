@@ -84,6 +84,7 @@ SIGNATURES = {
     "spmv_plan_coo": (_I32, [ctypes.POINTER(_P), _I64, _I64, _I64, _I32, _P, _P, _P, _I32, _I32, _P, _U32,
                              ctypes.POINTER(spmv_plan_opts)]),
     "spmv_plan_destroy": (_I32, [_P]),
+    "spmv_release_memory": (_I32, []),
     "spmv_plan_info": (_I32, [_P, ctypes.POINTER(spmv_plan_info_t)]),
     "spmv_plan_chunks": (_I32, [_P, ctypes.POINTER(spmv_chunk_t), _I32]),
     "spmv": (_I32, [_P, _P, _P, _P]),

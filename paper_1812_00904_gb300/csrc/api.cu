@@ -427,7 +427,7 @@ static spmv_status interleave_inputs(spmv_plan_s *p, int kbt, int kb, const void
         if (p->vt) cudaFree(p->vt);
         p->vt = nullptr;
         p->vt_bytes = 0;
-        CUDA_TRY(cudaMalloc(&p->vt, need));
+        CUDA_TRY(dev_malloc(&p->vt, need));
         p->vt_bytes = need;
     }
     CUDA_TRY(launch_interleave(p->vec_t == SPMV_F64, kbt, kb, in, len, p->vt, s));
@@ -611,7 +611,7 @@ static spmv_status run_row_blocks(spmv_plan_s *p, int kb, const void *const *in,
                 if (p->ypart_k) cudaFree(p->ypart_k);
                 p->ypart_k = nullptr;
                 p->ypart_k_bytes = 0;
-                CUDA_TRY(cudaMalloc(&p->ypart_k, need));
+                CUDA_TRY(dev_malloc(&p->ypart_k, need));
                 p->ypart_k_bytes = need;
             }
             base = p->ypart_k;
@@ -729,8 +729,8 @@ spmv_status with_staging(spmv_plan_s *p, const void *in, size_t in_bytes, void *
     }
     std::lock_guard<std::mutex> lk(p->host_mu);
     const size_t cap = (size_t)std::max(p->m, p->n) * p->sx + 16;
-    if (!p->hin) CUDA_TRY(cudaMalloc(&p->hin, cap));
-    if (!p->hout) CUDA_TRY(cudaMalloc(&p->hout, cap));
+    if (!p->hin) CUDA_TRY(dev_malloc(&p->hin, cap));
+    if (!p->hout) CUDA_TRY(dev_malloc(&p->hout, cap));
     const void *din = in;
     void *dout = out;
     if (ki == PK_HOST) {
@@ -1098,6 +1098,11 @@ spmv_status spmv_plan_destroy(spmv_plan_t plan) {
     return SPMV_OK;
 }
 
+spmv_status spmv_release_memory(void) {
+    CUDA_TRY(dev_release());
+    return SPMV_OK;
+}
+
 spmv_status spmv_plan_info(spmv_plan_t p, spmv_plan_info_t *info) {
     if (!p || !info) return set_error(SPMV_ERR_INVALID_ARG, "null argument");
     std::memset(info, 0, sizeof(*info));
@@ -1174,7 +1179,7 @@ static spmv_status pair_staged(spmv_plan_s *p, const void *x, void *y, const voi
     const size_t cap = (size_t)std::max(p->m, p->n) * p->sx + 16;
     const size_t xb = (size_t)p->n * p->sx, yb = (size_t)p->m * p->sx;
     for (void **b : {&p->hin, &p->hout, &p->hv, &p->hu})
-        if (!*b) CUDA_TRY(cudaMalloc(b, cap));
+        if (!*b) CUDA_TRY(dev_malloc(b, cap));
     if (!p->cstream) CUDA_TRY(cudaStreamCreateWithFlags(&p->cstream, cudaStreamNonBlocking));
     if (!p->ev_x) CUDA_TRY(cudaEventCreateWithFlags(&p->ev_x, cudaEventDisableTiming));
     if (!p->ev_u) CUDA_TRY(cudaEventCreateWithFlags(&p->ev_u, cudaEventDisableTiming));
@@ -1297,9 +1302,9 @@ spmv_status spmv_dvalues(spmv_plan_t p, const void *r, const void *x, void *g, v
     }
     std::lock_guard<std::mutex> lk(p->host_mu);
     const size_t cap = (size_t)std::max(p->m, p->n) * p->sx + 16;
-    if (!p->hin) CUDA_TRY(cudaMalloc(&p->hin, cap));
-    if (!p->hout) CUDA_TRY(cudaMalloc(&p->hout, cap));
-    if (!p->hg) CUDA_TRY(cudaMalloc(&p->hg, (size_t)p->nnz * p->sv + 16));
+    if (!p->hin) CUDA_TRY(dev_malloc(&p->hin, cap));
+    if (!p->hout) CUDA_TRY(dev_malloc(&p->hout, cap));
+    if (!p->hg) CUDA_TRY(dev_malloc(&p->hg, (size_t)p->nnz * p->sv + 16));
     const void *dr = r, *dx = x;
     void *dg = g;
     if (kr == PK_HOST) {

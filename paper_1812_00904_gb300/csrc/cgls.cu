@@ -247,7 +247,7 @@ spmv_status spmv_normal(spmv_plan_t p, const void *x, void *u, void *y, void *st
     void *yb = y;
     if (!yb) {
         std::lock_guard<std::mutex> lk(p->host_mu);
-        if (!p->ynorm) CG_TRY(cudaMalloc(&p->ynorm, (size_t)std::max<int64_t>(p->m, 1) * p->sx + 16));
+        if (!p->ynorm) CG_TRY(dev_malloc(&p->ynorm, (size_t)std::max<int64_t>(p->m, 1) * p->sx + 16));
         yb = p->ynorm;
     }
     const void *xin = x;

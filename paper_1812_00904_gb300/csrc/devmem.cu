@@ -3,8 +3,9 @@
 // cudaMalloc and cudaFree take about 100 us each on this machine (a plan makes eight, a CGLS call
 // two: 0.8 of the 2.4 ms of ingesting 10M triples, 0.2 of the 1.0 ms of a short CGLS run).  The
 // pool keeps up to POOL_KEEP bytes of freed memory for the next plan and gives everything beyond
-// back to the device at its next synchronisation; when an allocation fails it gives all of it back
-// and tries again.  The allocations and frees go through a stream of the pool's own: memory is
+// back to the device at its next synchronisation; when an allocation of the library fails, whether
+// from the pool or beside it, it gives all of it back and tries again, and spmv_release_memory gives
+// it back for others.  The allocations and frees go through a stream of the pool's own: memory is
 // handed out after that stream was waited for, so it can be used on any stream, and the caller
 // frees memory only when no work that uses it is pending.  Every call is safe from any thread.
 //
@@ -61,6 +62,30 @@ DevicePool &pool_of(int device) {
 
 }  // namespace
 
+cudaError_t dev_release() {
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    if (device < 0 || device >= MAX_DEVICES) return cudaErrorInvalidDevice;
+    DevicePool &P = pool_of(device);
+    if (!P.pool) return cudaSuccess;
+    e = cudaStreamSynchronize(P.stream);
+    return e == cudaSuccess ? cudaMemPoolTrimTo(P.pool, 0) : e;
+}
+
+cudaError_t dev_malloc(void **p, size_t bytes) {
+    *p = nullptr;
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {  // what the pool keeps may make room
+        cudaGetLastError();
+        *p = nullptr;
+        dev_release();
+        e = cudaMalloc(p, bytes);
+    }
+    if (e != cudaSuccess) *p = nullptr;
+    return e;
+}
+
 cudaError_t dev_alloc(void **p, size_t bytes) {
     *p = nullptr;
     int device = 0;
@@ -70,17 +95,8 @@ cudaError_t dev_alloc(void **p, size_t bytes) {
     DevicePool &P = pool_of(device);
     if (!P.pool) return cudaMalloc(p, bytes);
     if (bytes > POOL_MOST) {
-        e = cudaMalloc(p, bytes);
-        if (e == cudaErrorMemoryAllocation) {  // what the pool keeps may make room
-            cudaGetLastError();
-            cudaStreamSynchronize(P.stream);
-            cudaMemPoolTrimTo(P.pool, 0);
-            e = cudaMalloc(p, bytes);
-        }
-        if (e != cudaSuccess) {
-            *p = nullptr;
-            return e;
-        }
+        e = dev_malloc(p, bytes);
+        if (e != cudaSuccess) return e;
         std::lock_guard<std::mutex> lk(g_large_mu);
         g_large.insert(*p);
         return cudaSuccess;
@@ -91,10 +107,7 @@ cudaError_t dev_alloc(void **p, size_t bytes) {
         if (e != cudaErrorMemoryAllocation) break;
         cudaGetLastError();
         *p = nullptr;
-        if (attempt == 0) {
-            cudaStreamSynchronize(P.stream);
-            cudaMemPoolTrimTo(P.pool, 0);
-        }
+        if (attempt == 0) dev_release();
     }
     return e;
 }

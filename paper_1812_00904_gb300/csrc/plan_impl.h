@@ -118,6 +118,10 @@ namespace gbk {
 // stays allocated).
 cudaError_t dev_alloc(void **p, size_t bytes);
 void dev_free(void *p, int device, bool idle = true);
+// Memory beside the pool (freed with cudaFree), which makes room by what the pool keeps if need be.
+cudaError_t dev_malloc(void **p, size_t bytes);
+// Give what the current device's pool keeps back to the device.
+cudaError_t dev_release();
 
 // Internal overrides of a plan made by the library itself.
 struct PlanInternal {

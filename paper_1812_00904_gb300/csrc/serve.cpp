@@ -232,9 +232,9 @@ struct serve_s {
             M.d_ptr = M.d_idx = M.d_vals = nullptr;
             return s;
         };
-        if (cudaMalloc(&M.d_ptr, (size_t)(major + 1) * 4) != cudaSuccess) return fail(SPMV_ERR_OOM);
-        if (cudaMalloc(&M.d_idx, std::max<size_t>(16, (size_t)M.nnz * 4)) != cudaSuccess) return fail(SPMV_ERR_OOM);
-        if (cudaMalloc(&M.d_vals, std::max<size_t>(16, (size_t)M.nnz * dsize(M.val_t))) != cudaSuccess)
+        if (gbk::dev_malloc(&M.d_ptr, (size_t)(major + 1) * 4) != cudaSuccess) return fail(SPMV_ERR_OOM);
+        if (gbk::dev_malloc(&M.d_idx, std::max<size_t>(16, (size_t)M.nnz * 4)) != cudaSuccess) return fail(SPMV_ERR_OOM);
+        if (gbk::dev_malloc(&M.d_vals, std::max<size_t>(16, (size_t)M.nnz * dsize(M.val_t))) != cudaSuccess)
             return fail(SPMV_ERR_OOM);
         cudaStream_t s = admit_stream;
         if (cudaMemcpyAsync(M.d_ptr, M.h_ptr, (size_t)(major + 1) * 4, cudaMemcpyHostToDevice, s) != cudaSuccess ||
