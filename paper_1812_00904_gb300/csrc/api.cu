@@ -771,54 +771,11 @@ spmv_status spmv_plan_ex(spmv_plan_t *out, int64_t m, int64_t n, int64_t nnz, in
 
 }  // extern "C"
 
-spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nnz, int32_t layout, const int32_t *ptr,
-                             const int32_t *idx, const void *vals, int32_t val_dtype, int32_t vec_dtype,
-                             cudaStream_t s, uint32_t flags, const spmv_plan_opts *opts, const PlanInternal *pi) {
-    if (!out) return set_error(SPMV_ERR_INVALID_ARG, "out is NULL");
-    *out = nullptr;
-    if (layout != SPMV_CSC_WIDE && layout != SPMV_CSR_TALL) return set_error(SPMV_ERR_INVALID_ARG, "bad layout");
-    if (m < 0 || n < 0 || nnz < 0 || m >= (1ll << 31) - 64 || n >= (1ll << 31) - 64 || nnz >= (1ll << 31) - 64)
-        return set_error(SPMV_ERR_INVALID_ARG, "m, n and nnz must lie in [0, 2^31 - 64)");
-    if (dtype_size(val_dtype) == 0 || dtype_size(vec_dtype) == 0)
-        return set_error(SPMV_ERR_INVALID_ARG, "unknown dtype");
-    if (!pair_supported(val_dtype, vec_dtype))
-        return set_error(SPMV_ERR_UNSUPPORTED, "supported (values, vectors): (f64,f64) (f32,f32) (bf16,f32) (f16,f32)");
-    if (!ptr) return set_error(SPMV_ERR_INVALID_ARG, "ptr is NULL");
-    if (nnz > 0 && (!idx || !vals)) return set_error(SPMV_ERR_INVALID_ARG, "idx/vals are NULL");
-    if (nnz > 0 && (layout == SPMV_CSC_WIDE ? m : n) == 0)
-        return set_error(SPMV_ERR_BAD_MATRIX, "nonzeros need a nonempty indexed dimension");
-    if (!aligned16(ptr) || (nnz > 0 && (!aligned16(idx) || !aligned16(vals))))
-        return set_error(SPMV_ERR_INVALID_ARG, "ptr, idx and vals must be 16-byte aligned device pointers");
-    for (const void *q : {(const void *)ptr, (const void *)idx, vals}) {
-        if (q && classify(q) != PK_DEVICE)
-            return set_error(SPMV_ERR_INVALID_ARG, "ptr, idx and vals must be device pointers");
-    }
-    spmv_plan_s *p = new (std::nothrow) spmv_plan_s();
-    if (!p) return set_error(SPMV_ERR_OOM, "host allocation failed");
-    PlanGuard guard{p};
-    CUDA_TRY(cudaGetDevice(&p->device));
-    p->m = m;
-    p->n = n;
-    p->nnz = nnz;
-    p->layout = layout;
-    p->val_t = val_dtype;
-    p->vec_t = vec_dtype;
-    p->flags = flags;
-    p->prof_on = (flags & SPMV_PLAN_PROFILE) != 0;
-    p->n_major = (int)(layout == SPMV_CSC_WIDE ? n : m);
-    p->n_minor = (int)(layout == SPMV_CSC_WIDE ? m : n);
-    p->ptr = ptr;
-    p->idx = idx;
-    p->vals = vals;
-    p->sv = dtype_size(val_dtype);
-    p->sx = dtype_size(vec_dtype);
-    p->sa = (val_dtype == SPMV_F64) ? 8 : 4;
-
-    int sms = 0, smem_max = 0;
-    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
-    CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
-    smem_max -= 1024;  // static shared memory and slack
-
+// Everything about a plan that its shape, types and options decide: tiles, warps, processors and which
+// passes serve it (p holds the shape and the types).
+static spmv_status plan_configure(spmv_plan_s *p, uint32_t flags, const spmv_plan_opts *opts, const PlanInternal *pi, int sms,
+                                  int smem_max) {
+    const int64_t nnz = p->nnz;
     // ---- launch configuration: tiles of T nonzeros, up to W warps per CTA, S staging slots per warp
     // default tile: 512 nonzeros (two whole 256-position steps); smaller when the matrix has
     // too few nonzeros to give every warp of a full wave about two tiles
@@ -848,6 +805,7 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     p->x_cap = (int)align_up((size_t)p->T / 4 + 16, 8);  // columns of a tile's window (fall back to global beyond)
     p->smem_max = smem_max;
     p->W = W;
+    p->pptr_len = (int)align_up((size_t)p->n_major + 1 + 8, 4);
     // the short vector on chip when it leaves room for at least 4 warps of the scatter pass
     p->onchip = !(flags & SPMV_PLAN_SHORT_IN_GLOBAL);
     if (p->onchip && warps_for(p, MODE_SCATTER, 1) < std::min(W, 4)) p->onchip = false;
@@ -876,31 +834,180 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
         p->max_chunk = q + (nnz % p->P ? 1 : 0);
         p->min_chunk = q;
     }
+    p->ntiles = (int)nt64;
+    const int nt = p->ntiles;
+    p->ctas = (pi && pi->ctas > 0) ? std::min(pi->ctas, std::max(nt, 1)) : std::max(1, std::min(sms, nt));
+    p->bpc = (pi && pi->blocks_per_cta > 1 && (int64_t)p->ctas * pi->blocks_per_cta <= nt) ? pi->blocks_per_cta : 1;
+    p->chunk_tiles = (opts && opts->chunk_tiles > 0) ? opts->chunk_tiles : CHUNK_TILES;
+    // processors (chunks of tiles) of the streaming passes
+    p->pz.nproc = stream_processors(nt, p->T, (int)nnz, p->ctas * p->bpc, p->chunk_tiles, nullptr);
+    p->max_nproc = std::max(1, p->pz.nproc);
+    // the one-vector passes serve validated plans with whole-step tiles whose short vectors fit in
+    // shared memory beside the staging slots of enough warps
+    if (pi && nnz > 0 && p->T % 256 == 0) {  // the row-sorted copy: its dot products
+        p->pass_sd = pass_fits(p, false, true);
+        p->pass_mv = p->pass_sd && p->sv != 8;
+    } else if (nnz > 0 && p->T % 256 == 0 && !(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL))) {
+        p->sc_global = scatter_off_chip(p);
+        p->pass_sc = !p->sc_global && pass_fits(p, true, false);
+        p->pass_sd = pass_fits(p, false, true);
+        p->pass_pair = pass_fits(p, true, true);
+        p->pass_mv = p->sv != 8;
+        // vectors per accumulating pass: as many as leave room for three quarters of the warps'
+        // staging.  One pass at 24 to 27 of 32 warps against two of half as many vectors (25M
+        // nonzeros, us): 2 vectors 120 / 136 (m = 22,500), 4 174 / 187 (11,300), 8 258 / 270 (5,500);
+        // at 18 to 20 warps 150 / 134 (24,200), 198 / 186 (11,800), 318 / 271 (5,900).
+        if (p->pass_mv && p->pass_sc) {
+            const int full = std::min(pass_warps(p->sv), cta_tiles(p));
+            p->batch_width = 1;
+            for (int kv : {8, 4, 2})
+                if (p->batch_width == 1 && pass_geometry(p, true, false, kv).warps >= full - full / 4) p->batch_width = kv;
+        }
+    }
+    if (p->sv == 8 && p->pass_sc && cta_tiles(p) <= F64_TILES) {
+        p->f64_width = KB_MAX;
+        while (p->f64_width > 1 && (size_t)p->ctas * p->f64_width * p->n_minor * 8 > F64_PARTIALS) p->f64_width /= 2;
+    }
+    return SPMV_OK;
+}
 
-    // ---- workspace, part 1: pointer copy, reporting chunks, counters
-    p->pptr_len = (int)align_up((size_t)p->n_major + 1 + 8, 4);
+// The plan's device memory: offsets and sizes of its blocks.
+struct PlanLayout {
+    size_t o_pptr, o_aux, o_chunks, o_zones, o_counts, o_sscr, o_err, ws1;  // pointer copy, reporting chunks, counters
+    // tiles (descriptors, masks, steps), processor zones, records, partial sums; then set-up only
+    size_t o_meta, o_masks, o_pfx, o_steps, o_pz, o_recl, o_recr,
+        o_part, o_tnzb, o_taux, o_pnzb, o_paux, o_pdev, o_pscr, ws2;
+    size_t rec_bytes;
+    size_t seg;   // ranks and lists of the segments, when some are empty
+    bool passes;  // step records
+};
+static PlanLayout plan_layout(const spmv_plan_s *p, const PlanInternal *pi) {
+    PlanLayout L;
     size_t off = 0;
     auto carve = [&](size_t bytes) {
         const size_t o = off;
         off = align_up(off + bytes, 256);
         return o;
     };
-    const size_t o_pptr = carve((size_t)p->pptr_len * 4);
-    const size_t o_aux = carve((size_t)p->P * sizeof(ChunkAux));
-    const size_t o_chunks = carve((size_t)p->P * sizeof(ChunkDev));
-    const size_t o_zones = carve((size_t)p->P * sizeof(ZoneDev));
-    const size_t o_counts = carve(128);
-    const size_t o_sscr = carve(setup_scratch_bytes(p->P));
-    const size_t o_err = carve(16);
-    const size_t ws1 = off;
-    CUDA_TRY(dev_alloc(&p->ws, ws1));
+    L.o_pptr = carve((size_t)p->pptr_len * 4);
+    L.o_aux = carve((size_t)p->P * sizeof(ChunkAux));
+    L.o_chunks = carve((size_t)p->P * sizeof(ChunkDev));
+    L.o_zones = carve((size_t)p->P * sizeof(ZoneDev));
+    L.o_counts = carve(128);
+    L.o_sscr = carve(setup_scratch_bytes(p->P));
+    L.o_err = carve(16);
+    L.ws1 = off;
+    const int nt = p->ntiles;
+    const size_t part_bytes =
+        (pi && pi->segdot_only) ? 16
+                                : std::max(p->onchip && !p->sc_global ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa
+                                                                      : (size_t)p->n_minor * sizeof(double),
+                                           p->pass_sc || p->pass_pair ? (size_t)p->ctas * std::max(p->batch_width, p->f64_width) * p->n_minor * p->sa : (size_t)0);
+    L.passes = p->pass_sc || p->pass_sd || p->pass_pair || p->pass_mv;
+    L.seg = L.passes ? ((size_t)p->n_major * 2 + 1 + seg_rank_blocks(p->n_major) + 4) * 4 : 0;
+    L.rec_bytes = (size_t)VL_MAX * p->max_nproc * 2 * p->sa;  // any segmented pass: up to VL_MAX vectors
+    off = 0;
+    L.o_meta = carve((size_t)(nt + 1) * sizeof(TileMeta));
+    L.o_masks = carve((size_t)std::max(nt, 1) * p->mwp * 4);
+    L.o_pfx = carve((size_t)std::max(nt, 1) * p->mwq * 2);
+    L.o_steps = carve(L.passes ? (size_t)nt * (p->T / 256) * sizeof(StepRec) : 0);
+    L.o_pz = carve((size_t)p->max_nproc * sizeof(ZoneDev));
+    L.o_recl = carve(L.rec_bytes);
+    L.o_recr = carve(L.rec_bytes);
+    L.o_part = carve(std::max(part_bytes, (size_t)16));
+    // set-up only
+    L.o_tnzb = carve((size_t)(nt + 1) * 4);
+    L.o_taux = carve((size_t)std::max(nt, 1) * sizeof(ChunkAux));
+    L.o_pnzb = carve((size_t)(p->max_nproc + 1) * 4);
+    L.o_paux = carve((size_t)p->max_nproc * sizeof(ChunkAux));
+    L.o_pdev = carve((size_t)p->max_nproc * sizeof(ChunkDev));
+    L.o_pscr = carve(setup_scratch_bytes(p->max_nproc));
+    L.ws2 = off;
+    return L;
+}
+
+// The device of a plan: its SMs and the shared memory a CTA may use (less static memory and slack).
+static cudaError_t device_limits(int device, int &sms, int &smem_max) {
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    smem_max -= 1024;
+    return e;
+}
+
+static void plan_shape(spmv_plan_s *p, int64_t m, int64_t n, int64_t nnz, int32_t layout, int32_t val_dtype, int32_t vec_dtype) {
+    p->m = m;
+    p->n = n;
+    p->nnz = nnz;
+    p->layout = layout;
+    p->val_t = val_dtype;
+    p->vec_t = vec_dtype;
+    p->n_major = (int)(layout == SPMV_CSC_WIDE ? n : m);
+    p->n_minor = (int)(layout == SPMV_CSC_WIDE ? m : n);
+    p->sv = dtype_size(val_dtype);
+    p->sx = dtype_size(vec_dtype);
+    p->sa = (val_dtype == SPMV_F64) ? 8 : 4;
+}
+
+uint64_t gbk::plan_bytes_most(int device, int64_t m, int64_t n, int64_t nnz, int32_t layout, int32_t val_dtype, int32_t vec_dtype) {
+    if (m < 0 || n < 0 || nnz < 0 || std::max({m, n, nnz}) >= (1ll << 31) - 64 || !pair_supported(val_dtype, vec_dtype)) return 0;
+    spmv_plan_s p;
+    plan_shape(&p, m, n, nnz, layout, val_dtype, vec_dtype);
+    int sms = 0, smem_max = 0;
+    if (device_limits(device, sms, smem_max) != cudaSuccess) return 0;
+    if (plan_configure(&p, 0, nullptr, nullptr, sms, smem_max) != SPMV_OK) return 0;
+    const PlanLayout L = plan_layout(&p, nullptr);
+    return plan_footprint(&p) + L.ws1 + L.ws2 + L.seg;
+}
+
+spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nnz, int32_t layout, const int32_t *ptr,
+                             const int32_t *idx, const void *vals, int32_t val_dtype, int32_t vec_dtype,
+                             cudaStream_t s, uint32_t flags, const spmv_plan_opts *opts, const PlanInternal *pi) {
+    if (!out) return set_error(SPMV_ERR_INVALID_ARG, "out is NULL");
+    *out = nullptr;
+    if (layout != SPMV_CSC_WIDE && layout != SPMV_CSR_TALL) return set_error(SPMV_ERR_INVALID_ARG, "bad layout");
+    if (m < 0 || n < 0 || nnz < 0 || m >= (1ll << 31) - 64 || n >= (1ll << 31) - 64 || nnz >= (1ll << 31) - 64)
+        return set_error(SPMV_ERR_INVALID_ARG, "m, n and nnz must lie in [0, 2^31 - 64)");
+    if (dtype_size(val_dtype) == 0 || dtype_size(vec_dtype) == 0)
+        return set_error(SPMV_ERR_INVALID_ARG, "unknown dtype");
+    if (!pair_supported(val_dtype, vec_dtype))
+        return set_error(SPMV_ERR_UNSUPPORTED, "supported (values, vectors): (f64,f64) (f32,f32) (bf16,f32) (f16,f32)");
+    if (!ptr) return set_error(SPMV_ERR_INVALID_ARG, "ptr is NULL");
+    if (nnz > 0 && (!idx || !vals)) return set_error(SPMV_ERR_INVALID_ARG, "idx/vals are NULL");
+    if (nnz > 0 && (layout == SPMV_CSC_WIDE ? m : n) == 0)
+        return set_error(SPMV_ERR_BAD_MATRIX, "nonzeros need a nonempty indexed dimension");
+    if (!aligned16(ptr) || (nnz > 0 && (!aligned16(idx) || !aligned16(vals))))
+        return set_error(SPMV_ERR_INVALID_ARG, "ptr, idx and vals must be 16-byte aligned device pointers");
+    for (const void *q : {(const void *)ptr, (const void *)idx, vals}) {
+        if (q && classify(q) != PK_DEVICE)
+            return set_error(SPMV_ERR_INVALID_ARG, "ptr, idx and vals must be device pointers");
+    }
+    spmv_plan_s *p = new (std::nothrow) spmv_plan_s();
+    if (!p) return set_error(SPMV_ERR_OOM, "host allocation failed");
+    PlanGuard guard{p};
+    CUDA_TRY(cudaGetDevice(&p->device));
+    plan_shape(p, m, n, nnz, layout, val_dtype, vec_dtype);
+    p->flags = flags;
+    p->prof_on = (flags & SPMV_PLAN_PROFILE) != 0;
+    p->ptr = ptr;
+    p->idx = idx;
+    p->vals = vals;
+
+    int sms = 0, smem_max = 0;
+    CUDA_TRY(device_limits(p->device, sms, smem_max));
+
+    spmv_status st = plan_configure(p, flags, opts, pi, sms, smem_max);
+    if (st != SPMV_OK) return st;
+
+    // ---- workspace, part 1: pointer copy, reporting chunks, counters
+    const PlanLayout L = plan_layout(p, pi);
+    CUDA_TRY(dev_alloc(&p->ws, L.ws1));
     char *w1 = static_cast<char *>(p->ws);
-    p->pptr = reinterpret_cast<int32_t *>(w1 + o_pptr);
-    p->aux = reinterpret_cast<ChunkAux *>(w1 + o_aux);
-    p->chunks = reinterpret_cast<ChunkDev *>(w1 + o_chunks);
-    p->zones = reinterpret_cast<ZoneDev *>(w1 + o_zones);
-    p->counts = reinterpret_cast<int32_t *>(w1 + o_counts);
-    p->err = reinterpret_cast<int32_t *>(w1 + o_err);
+    p->pptr = reinterpret_cast<int32_t *>(w1 + L.o_pptr);
+    p->aux = reinterpret_cast<ChunkAux *>(w1 + L.o_aux);
+    p->chunks = reinterpret_cast<ChunkDev *>(w1 + L.o_chunks);
+    p->zones = reinterpret_cast<ZoneDev *>(w1 + L.o_zones);
+    p->counts = reinterpret_cast<int32_t *>(w1 + L.o_counts);
+    p->err = reinterpret_cast<int32_t *>(w1 + L.o_err);
     CUDA_TRY(cudaMemsetAsync(p->counts, 0, 128, s));
     CUDA_TRY(cudaMemsetAsync(p->err, 0, 16, s));
 
@@ -950,116 +1057,53 @@ spmv_status gbk::plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nn
     CUDA_TRY(cudaEventRecord(e0, s));
     CUDA_TRY(launch_pad_ptr(ptr, p->pptr, p->n_major, (int)nnz, p->pptr_len, s));
     CUDA_TRY(launch_chunks(p->pptr, p->n_major, (int)nnz, p->P, nullptr, p->T, p->aux, s));
-    CUDA_TRY(launch_setup(p->aux, p->P, p->chunks, p->zones, p->counts, static_cast<char *>(p->ws) + o_sscr, s));
-    p->ntiles = (int)nt64;
-
+    CUDA_TRY(launch_setup(p->aux, p->P, p->chunks, p->zones, p->counts, static_cast<char *>(p->ws) + L.o_sscr, s));
     // ---- workspace, part 2: tiles (descriptors, masks), processor zones, records and partial sums
     const int nt = p->ntiles;
-    p->ctas = (pi && pi->ctas > 0) ? std::min(pi->ctas, std::max(nt, 1)) : std::max(1, std::min(sms, nt));
-    p->bpc = (pi && pi->blocks_per_cta > 1 && (int64_t)p->ctas * pi->blocks_per_cta <= nt) ? pi->blocks_per_cta : 1;
-    p->chunk_tiles = (opts && opts->chunk_tiles > 0) ? opts->chunk_tiles : CHUNK_TILES;
-    // processors (chunks of tiles) of the streaming passes and their nonzero boundaries
-    std::vector<int32_t> pnzb;
-    {
-        spmv_plan_s::ProcZones &pz = p->pz;
-        pz.nproc = stream_processors(nt, p->T, (int)nnz, p->ctas * p->bpc, p->chunk_tiles, nullptr);
-        pnzb.resize((size_t)pz.nproc + 1);
-        stream_processors(nt, p->T, (int)nnz, p->ctas * p->bpc, p->chunk_tiles, pnzb.data());
-        p->max_nproc = std::max(1, pz.nproc);
-    }
-    // the one-vector passes serve validated plans with whole-step tiles whose short vectors fit in
-    // shared memory beside the staging slots of enough warps
-    if (pi && nnz > 0 && p->T % 256 == 0) {  // the row-sorted copy: its dot products
-        p->pass_sd = pass_fits(p, false, true);
-        p->pass_mv = p->pass_sd && p->sv != 8;
-    } else if (nnz > 0 && p->T % 256 == 0 && !(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL))) {
-        p->sc_global = scatter_off_chip(p);
-        p->pass_sc = !p->sc_global && pass_fits(p, true, false);
-        p->pass_sd = pass_fits(p, false, true);
-        p->pass_pair = pass_fits(p, true, true);
-        p->pass_mv = p->sv != 8;
-        // vectors per accumulating pass: as many as leave room for three quarters of the warps'
-        // staging.  One pass at 24 to 27 of 32 warps against two of half as many vectors (25M
-        // nonzeros, us): 2 vectors 120 / 136 (m = 22,500), 4 174 / 187 (11,300), 8 258 / 270 (5,500);
-        // at 18 to 20 warps 150 / 134 (24,200), 198 / 186 (11,800), 318 / 271 (5,900).
-        if (p->pass_mv && p->pass_sc) {
-            const int full = std::min(pass_warps(p->sv), cta_tiles(p));
-            p->batch_width = 1;
-            for (int kv : {8, 4, 2})
-                if (p->batch_width == 1 && pass_geometry(p, true, false, kv).warps >= full - full / 4) p->batch_width = kv;
-        }
-    }
-    if (p->sv == 8 && p->pass_sc && cta_tiles(p) <= F64_TILES) {
-        p->f64_width = KB_MAX;
-        while (p->f64_width > 1 && (size_t)p->ctas * p->f64_width * p->n_minor * 8 > F64_PARTIALS) p->f64_width /= 2;
-    }
-    const size_t part_bytes =
-        (pi && pi->segdot_only) ? 16
-                                : std::max(p->onchip && !p->sc_global ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa
-                                                                      : (size_t)p->n_minor * sizeof(double),
-                                           p->pass_sc || p->pass_pair ? (size_t)p->ctas * std::max(p->batch_width, p->f64_width) * p->n_minor * p->sa : (size_t)0);
+    std::vector<int32_t> pnzb((size_t)p->pz.nproc + 1);  // nonzero boundaries of the processors
+    stream_processors(nt, p->T, (int)nnz, p->ctas * p->bpc, p->chunk_tiles, pnzb.data());
     // ranks of the nonempty segments, when some are empty
     int32_t *&rank = p->segrank;
-    if ((p->pass_sc || p->pass_sd || p->pass_pair || p->pass_mv) && p->nempty > 0) {
+    if (L.passes && p->nempty > 0) {
         const int nfull = p->n_major - p->nempty, nblk = seg_rank_blocks(p->n_major);
-        const size_t seg_bytes = ((size_t)p->n_major * 2 + 1 + nblk + 4) * 4;
-        CUDA_TRY(dev_alloc(&p->ws_seg, seg_bytes));
+        CUDA_TRY(dev_alloc(&p->ws_seg, L.seg));
         p->seglist = static_cast<int32_t *>(p->ws_seg);
         p->emptylist = p->seglist + nfull;
         rank = p->emptylist + p->nempty;
         int32_t *blk = rank + p->n_major + 1;
         CUDA_TRY(launch_seg_ranks(p->pptr, p->n_major, rank, p->seglist, p->emptylist, blk, blk + nblk, s));
-        p->ws_bytes = seg_bytes;
+        p->ws_bytes = L.seg;
     }
-    const size_t rec_bytes = (size_t)VL_MAX * p->max_nproc * 2 * p->sa;  // any segmented pass: up to VL_MAX vectors
-    off = 0;
-    const size_t o_meta = carve((size_t)(nt + 1) * sizeof(TileMeta));
-    const size_t o_masks = carve((size_t)std::max(nt, 1) * p->mwp * 4);
-    const size_t o_pfx = carve((size_t)std::max(nt, 1) * p->mwq * 2);
-    const bool passes = p->pass_sc || p->pass_sd || p->pass_pair || p->pass_mv;
-    const size_t o_steps = carve(passes ? (size_t)nt * (p->T / 256) * sizeof(StepRec) : 0);
-    const size_t o_pz = carve((size_t)p->max_nproc * sizeof(ZoneDev));
-    const size_t o_recl = carve(rec_bytes);
-    const size_t o_recr = carve(rec_bytes);
-    const size_t o_part = carve(std::max(part_bytes, (size_t)16));
-    // set-up only
-    const size_t o_tnzb = carve((size_t)(nt + 1) * 4);
-    const size_t o_taux = carve((size_t)std::max(nt, 1) * sizeof(ChunkAux));
-    const size_t o_pnzb = carve((size_t)(p->max_nproc + 1) * 4);
-    const size_t o_paux = carve((size_t)p->max_nproc * sizeof(ChunkAux));
-    const size_t o_pdev = carve((size_t)p->max_nproc * sizeof(ChunkDev));
-    const size_t o_pscr = carve(setup_scratch_bytes(p->max_nproc));
-    const size_t ws2 = off;
-    CUDA_TRY(dev_alloc(&p->ws2, ws2));
-    p->ws_bytes += ws1 + ws2;
+    CUDA_TRY(dev_alloc(&p->ws2, L.ws2));
+    p->ws_bytes += L.ws1 + L.ws2;
     char *w2 = static_cast<char *>(p->ws2);
-    p->meta = reinterpret_cast<TileMeta *>(w2 + o_meta);
-    p->masks = reinterpret_cast<uint32_t *>(w2 + o_masks);
-    p->pfx = reinterpret_cast<uint16_t *>(w2 + o_pfx);
-    p->steps = passes ? reinterpret_cast<StepRec *>(w2 + o_steps) : nullptr;
-    p->rec_left = w2 + o_recl;
-    p->rec_right = w2 + o_recr;
-    p->part = w2 + o_part;
-    int32_t *tnzb = reinterpret_cast<int32_t *>(w2 + o_tnzb);
-    ChunkAux *taux = reinterpret_cast<ChunkAux *>(w2 + o_taux);
-    int32_t *dpnzb = reinterpret_cast<int32_t *>(w2 + o_pnzb);
-    ChunkAux *paux = reinterpret_cast<ChunkAux *>(w2 + o_paux);
-    ChunkDev *pdev = reinterpret_cast<ChunkDev *>(w2 + o_pdev);
+    p->meta = reinterpret_cast<TileMeta *>(w2 + L.o_meta);
+    p->masks = reinterpret_cast<uint32_t *>(w2 + L.o_masks);
+    p->pfx = reinterpret_cast<uint16_t *>(w2 + L.o_pfx);
+    p->steps = L.passes ? reinterpret_cast<StepRec *>(w2 + L.o_steps) : nullptr;
+    p->rec_left = w2 + L.o_recl;
+    p->rec_right = w2 + L.o_recr;
+    p->part = w2 + L.o_part;
+    int32_t *tnzb = reinterpret_cast<int32_t *>(w2 + L.o_tnzb);
+    ChunkAux *taux = reinterpret_cast<ChunkAux *>(w2 + L.o_taux);
+    int32_t *dpnzb = reinterpret_cast<int32_t *>(w2 + L.o_pnzb);
+    ChunkAux *paux = reinterpret_cast<ChunkAux *>(w2 + L.o_paux);
+    ChunkDev *pdev = reinterpret_cast<ChunkDev *>(w2 + L.o_pdev);
     if (nt > 0) {
         // execution tiles: bounds, first/last segments, owned end events; masks and descriptors
         CUDA_TRY(launch_tile_bounds(nt, p->T, (int)nnz, tnzb, s));
         CUDA_TRY(launch_chunks(p->pptr, p->n_major, (int)nnz, nt, tnzb, p->T, taux, s));
         CUDA_TRY(launch_masks(p->pptr, taux, nt, (int)nnz, p->n_major, p->mwp, p->masks, p->mwq, p->pfx, p->meta, rank, s));
-        if (passes) CUDA_TRY(launch_steps(p->meta, p->masks, p->mwp, nt, p->T / 256, p->seglist, p->steps, s));
+        if (L.passes) CUDA_TRY(launch_steps(p->meta, p->masks, p->mwp, nt, p->T / 256, p->seglist, p->steps, s));
         // the Sec. IV-B set-up over the processors (chunks) gives their overlap zones
         spmv_plan_s::ProcZones &pz = p->pz;
-        pz.zones = reinterpret_cast<ZoneDev *>(w2 + o_pz);
+        pz.zones = reinterpret_cast<ZoneDev *>(w2 + L.o_pz);
         CUDA_TRY(cudaMemcpyAsync(dpnzb, pnzb.data(), ((size_t)pz.nproc + 1) * 4, cudaMemcpyHostToDevice, s));
         CUDA_TRY(launch_chunks(p->pptr, p->n_major, (int)nnz, pz.nproc, dpnzb, p->T, paux, s));
-        CUDA_TRY(launch_setup(paux, pz.nproc, pdev, pz.zones, p->counts + 8, w2 + o_pscr, s));
+        CUDA_TRY(launch_setup(paux, pz.nproc, pdev, pz.zones, p->counts + 8, w2 + L.o_pscr, s));
     }
-    CUDA_TRY(cudaMemsetAsync(p->rec_left, 0, rec_bytes, s));
-    CUDA_TRY(cudaMemsetAsync(p->rec_right, 0, rec_bytes, s));
+    CUDA_TRY(cudaMemsetAsync(p->rec_left, 0, L.rec_bytes, s));
+    CUDA_TRY(cudaMemsetAsync(p->rec_right, 0, L.rec_bytes, s));
     CUDA_TRY(cudaEventRecord(e1, s));
     // zone counts of the reporting chunks ([0] z, [2] V) and of the processor tables ([8 + 4i])
     int32_t counts[32] = {0};

@@ -145,6 +145,9 @@ spmv_status run_segdot(spmv_plan_s *p, int kb, const void *const *in, void *cons
 // op product on device vectors, any k (split into passes of batch_width)
 spmv_status run_op(spmv_plan_s *p, int op, int k, const void *const *in, void *const *out, cudaStream_t s);
 size_t plan_footprint(const spmv_plan_s *p);
+// The largest plan_footprint that a matrix of that shape can have on the device with the default
+// options (reached when some segment is empty); 0: no such plan.
+uint64_t plan_bytes_most(int device, int64_t m, int64_t n, int64_t nnz, int32_t layout, int32_t val_dtype, int32_t vec_dtype);
 // Plan-owned copy of idx/vals, permuted within each segment so that one warp instruction of the
 // streaming kernels meets distinct shared-memory banks (banks: 32, or 16 for 8-byte vectors).
 cudaError_t launch_bank_order(const int32_t *ptr, int n_major, int nnz, const int32_t *idx, const void *vals,

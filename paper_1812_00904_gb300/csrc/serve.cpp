@@ -54,6 +54,7 @@ struct Matrix {
     const int32_t *h_ptr = nullptr, *h_idx = nullptr;
     const void *h_vals = nullptr;
     void *d_ptr = nullptr, *d_idx = nullptr, *d_vals = nullptr;
+    uint64_t need = 0;       // most device bytes that the matrix and its plan can take
     uint64_t footprint = 0;  // device bytes counted against the budget (reserved while admitting)
     uint64_t last_use = 0;
     bool inflight = false;
@@ -129,19 +130,12 @@ struct serve_s {
         st.resident_matrices--;
     }
 
-    uint64_t estimate(const Matrix &M) const {
-        const int64_t major = M.layout == SPMV_CSC_WIDE ? M.n : M.m;
-        const int64_t minor = M.layout == SPMV_CSC_WIDE ? M.m : M.n;
-        return (uint64_t)M.nnz * (4 + dsize(M.val_t)) + (uint64_t)(major + 1) * 8 +
-               std::min<uint64_t>((uint64_t)minor * 32, 232448) * 160 + (4u << 20);
-    }
-
     // Start making matrix `id` resident: reserve its bytes (evicting idle host matrices) and
     // hand it to the admission thread.  False if it cannot start now; *err set if it never can.
     bool start_admission(int id, spmv_status *err) {
         Matrix &M = mats[id];
         *err = SPMV_OK;
-        const uint64_t need = estimate(M);
+        const uint64_t need = M.need;
         if (need > budget) {
             *err = SPMV_ERR_BUSY;
             return false;
@@ -457,8 +451,11 @@ spmv_status serve_register_host(serve_t s, int64_t m, int64_t n, int64_t nnz, in
         return gbk::set_error(SPMV_ERR_INVALID_ARG, "null argument");
     if (layout != SPMV_CSC_WIDE && layout != SPMV_CSR_TALL) return gbk::set_error(SPMV_ERR_INVALID_ARG, "bad layout");
     if (m < 0 || n < 0 || nnz < 0) return gbk::set_error(SPMV_ERR_INVALID_ARG, "negative size");
-    std::lock_guard<std::mutex> lk(s->mu);
     Matrix M;
+    M.need = gbk::plan_bytes_most(s->device, m, n, nnz, layout, val_dtype, vec_dtype);
+    if (!M.need)  // (its admission will fail with the plan's own error)
+        M.need = (uint64_t)nnz * (4 + dsize(val_dtype)) + (uint64_t)((layout == SPMV_CSC_WIDE ? n : m) + 1) * 8;
+    std::lock_guard<std::mutex> lk(s->mu);
     M.m = m;
     M.n = n;
     M.nnz = nnz;
