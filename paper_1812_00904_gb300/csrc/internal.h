@@ -204,6 +204,17 @@ cudaError_t launch_overlapped(void (*kern)(Params...), dim3 grid, dim3 block, si
     return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
 }
 
+// The combine and fix-up kernel: blocks of FIN_X x FIN_ROWS threads.  The dynamic shared memory that each of
+// `blocks` of them asks for so that no SM takes more than its share: with s of them to an SM, 1 / s of what
+// an SM has, less 4 KB (a block's static memory, what the system reserves, rounding).
+constexpr int FIN_X = 32, FIN_ROWS = 8;
+inline int finish_request(int64_t blocks, int sms, int smem_most) {
+    const int64_t per_sm = (blocks + sms - 1) / sms;
+    if (per_sm < 1 || per_sm >= 2048 / (FIN_X * FIN_ROWS)) return 0;
+    const int64_t request = (smem_most - 7 * 1024) / per_sm - 4096;
+    return request > 0 ? (int)request : 0;
+}
+
 struct LaunchArgs {
     StreamParams sp;
     int grid, block, smem;

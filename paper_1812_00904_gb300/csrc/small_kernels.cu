@@ -39,7 +39,7 @@ struct FinishArgs {
     const void *rec_left, *rec_right;
     OutPtrs short_out, long_out;
 };
-constexpr int FIN_X = 32, FIN_ROWS = 8, FIN_CB = 10;
+constexpr int FIN_CB = 10;
 template <typename XT, typename PT, typename RT>
 __global__ void __launch_bounds__(FIN_X * FIN_ROWS) finish_kernel(const __grid_constant__ FinishArgs p) {
     __shared__ double sh_s[FIN_ROWS][FIN_X];
@@ -79,23 +79,42 @@ __global__ void __launch_bounds__(FIN_X * FIN_ROWS) finish_kernel(const __grid_c
     }
 }
 
+// SMs and most shared memory of a CTA of the current device (asked once per device).
+static cudaError_t device_shape(int &sms, int &most) {
+    static std::atomic<int> known[MAX_DEVICES][2];
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    if (device < 0 || device >= MAX_DEVICES) return cudaErrorInvalidDevice;
+    sms = known[device][0].load(std::memory_order_relaxed);
+    most = known[device][1].load(std::memory_order_relaxed);
+    if (sms > 0 && most > 0) return cudaSuccess;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    if (e != cudaSuccess) return e;
+    known[device][0].store(sms, std::memory_order_relaxed);
+    known[device][1].store(most, std::memory_order_relaxed);
+    return cudaSuccess;
+}
+
 // Launched with programmatic serialization: its blocks may become resident while the pass before
 // drains (they wait in griddepcontrol.wait), which hides the launch.  They would all settle on
 // the SMs that come free first and share those SMs' FP64 pipes (19 us instead of 7 for 20,000
 // elements); each asks for so much shared memory that no SM takes more than its share of them.
 template <typename XT, typename PT, typename RT>
 cudaError_t launch_finish(FinishArgs &p, int kb, cudaStream_t s) {
-    constexpr int SMS = 152, ALL = 220 * 1024, RESIDENT = 2048 / (FIN_X * FIN_ROWS);
     p.comb_blocks = (p.n_minor + FIN_X - 1) / FIN_X;
     const int64_t blocks = p.comb_blocks + ((int64_t)p.z + FIN_X * FIN_ROWS - 1) / (FIN_X * FIN_ROWS);
     if (blocks <= 0) return cudaSuccess;
-    const int64_t per_sm = (blocks * kb + SMS - 1) / SMS;
+    int sms = 0, most = 0;
+    cudaError_t e = device_shape(sms, most);
+    if (e != cudaSuccess) return e;
     auto kern = finish_kernel<XT, PT, RT>;
     static SmemLimit lim;
-    const size_t smem = per_sm < RESIDENT ? ALL / per_sm - 4096 : 0;
-    const cudaError_t e = ensure_smem_limit(kern, lim, (int)smem);
+    const int smem = finish_request(blocks * kb, sms, most);
+    e = ensure_smem_limit(kern, lim, smem);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(kern, dim3((unsigned)blocks, kb), dim3(FIN_X * FIN_ROWS), smem, s, p);
+    return launch_overlapped(kern, dim3((unsigned)blocks, kb), dim3(FIN_X * FIN_ROWS), (size_t)smem, s, p);
 }
 
 static void out_ptrs(OutPtrs &o, void *const *out, int kb) {
@@ -193,7 +212,6 @@ cudaError_t launch_interleave(bool f64, int kbt, int kb, const void *const *in, 
         else if (kbt == 4) return launch_overlapped(interleave_kernel<float, 4>, dim3(grid), dim3(256), 0, s, ip, kb, len, o);
         else return launch_overlapped(interleave_kernel<float, 8>, dim3(grid), dim3(256), 0, s, ip, kb, len, o);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace gbk

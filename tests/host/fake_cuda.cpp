@@ -90,6 +90,7 @@ int64_t fake_ranked_segments(int n_major, unsigned block, int64_t *lowest) {
 uint64_t fake_plan_bytes_most(int64_t m, int64_t n, int64_t nnz, int val, int vec) {
     return gbk::plan_bytes_most(0, m, n, nnz, SPMV_CSC_WIDE, val, vec);
 }
+int fake_finish_request(int64_t blocks, int sm_count, int smem_most) { return gbk::finish_request(blocks, sm_count, smem_most); }
 int fake_rank_blocks(int n_major) { return gbk::seg_rank_blocks(n_major); }
 int64_t fake_strided(int64_t thread, int64_t threads, int64_t n, int64_t *lowest, int64_t *highest) {
     int64_t seen = 0;
