@@ -330,6 +330,7 @@ static spmv_status run_pass(spmv_plan_s *p, const void *x, void *y, const void *
     PassParams pp = pass_params(p);
     pp.acc_bytes = sc ? (int)pass_acc_bytes(p, sd) : 0;
     pp.lanes = pass_lanes(p, sc, sd);
+    for (pp.spread = 255; pp.spread >= p->n_minor; pp.spread >>= 1) {}
     pp.vec_bytes = sd ? (int)pass_vec_bytes(p) : 0;
     pp.x = x;
     pp.xv[0] = x;

@@ -135,6 +135,7 @@ struct PassParams {
     int32_t nnz, n_minor, ntiles, spt, chunk_tiles;
     int32_t slots;           // staging slots per warp
     int32_t lanes;           // SC: 1 = an element of the accumulator for every lane
+    int32_t spread;          // pair: a mask of up to 255 below n_minor (places for a last step's empty positions)
     int32_t copies;          // copies of the accumulator (a power of two), shared by the warps in turn
     int32_t acc_bytes, vec_bytes;  // shared memory of one accumulator (0 without SC) and of the input (0 without SD)
     const void *x, *v;       // the long input (SC), the short input (SD)

@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(WB * 32, 1) pass_kernel(const __grid_constant_
                     const bool in = pos < p.nnz;
                     // (the pair adds zeros for the positions past the end: to places of their own, for 243
                     // additions to one place took 10 us)
-                    ix[e] = in ? call_load(p.idx + pos) : SC && SD ? at % p.n_minor : 0;
+                    ix[e] = in ? call_load(p.idx + pos) : SC && SD ? at & p.spread : 0;
                     va[e] = in ? to_acc<AT>(static_cast<const VT *>(p.vals)[pos]) : AT(0);
                 }
             }
