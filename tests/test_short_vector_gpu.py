@@ -1,4 +1,4 @@
-"""Short vectors of a few elements (an accumulator element for every lane up to 32 of them), against the oracle."""
+"""Short vectors of a few elements (an accumulator element for every lane up to 32 of them, FP64 pairs up to 64), against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("layout", ["csc", "csr"])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16, torch.float16, torch.float64], ids=str)
-@pytest.mark.parametrize("minor", [1, 2, 3, 16, 31, 32, 33])
+@pytest.mark.parametrize("minor", [1, 2, 3, 16, 31, 32, 33, 64, 65])
 @pytest.mark.parametrize("nnz", [1, 255, 5_003, 600_001])
 def test_products(minor, nnz, dtype, layout):
     major = max(4, nnz // 20 // 4 * 4)
