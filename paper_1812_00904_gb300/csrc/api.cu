@@ -111,10 +111,10 @@ PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1, i
     g.slots = 1;
     const size_t rest = vec + (size_t)g.warps * g.slots * slot;
     g.copies = 1;
-    // adding up FP64 copies costs more than they save, but for a second one with four nonzeros or more to an
-    // element (one / two copies, us: m = 4,000, 50,000 nonzeros 7.4 / 8.5, 1M 11.5 / 12.2, 8M 40.2 / 39.3;
-    // m = 300, 500,000 11.0 / 10.0)
-    const int most = p->sv != 8 ? PASS_MAX_COPIES : p->nnz >= (int64_t)4 * p->ctas * p->n_minor ? 2 : 1;
+    // Copies are worth their adding up with four nonzeros or more to an element, FP64 a second one alone.
+    // FP64 one / two copies, us: m = 4,000, 50,000 nonzeros 7.4 / 8.5, 1M 11.5 / 12.2, 8M 40.2 / 39.3; m = 300,
+    // 500,000 11.0 / 10.0.  FP32, 8 vectors of 2,000, 50,000 nonzeros: 21.7 / 22.9.
+    const int most = p->nnz < (int64_t)4 * p->ctas * p->n_minor ? 1 : p->sv == 8 ? 2 : PASS_MAX_COPIES;
     while (sc && 2 * g.copies <= std::min({g.warps, work, most}) && 2 * g.copies * acc + rest <= all) g.copies *= 2;
     g.smem = g.copies * acc + rest;
     return g;
