@@ -107,7 +107,7 @@ PassGeometry pass_geometry(const spmv_plan_s *p, bool sc, bool sd, int kv = 1, i
     const size_t fit = all > acc + vec ? (all - acc - vec) / slot : 0;
     const int most_warps = pass_warps(p->sv), work = std::min(most_warps, cta_tiles(p));
     g.fit = (int)std::min<size_t>(fit, 1024);
-    g.warps = std::min(std::max(work, std::min(most_warps, copy_warps(p, lanes ? 256 : kv)) / rows), g.fit);
+    g.warps = std::min(std::max(work, sc || sd ? std::min(most_warps, copy_warps(p, lanes ? 256 : kv)) / rows : 0), g.fit);
     g.slots = 1;
     const size_t rest = vec + (size_t)g.warps * g.slots * slot;
     g.copies = 1;
@@ -634,13 +634,14 @@ static spmv_status run_dvalues(spmv_plan_s *p, const void *r, const void *x, voi
     if (p->nnz == 0) return SPMV_OK;
     // CSC: g = r[row] * x[col] -> minor r, major x;  CSR: g = r[row] * x[col] -> minor x, major r
     const bool csc = p->layout == SPMV_CSC_WIDE;
-    if (p->pass_sd) {
-        const PassGeometry geo = pass_geometry(p, false, true);
+    if (p->pass_dv) {
+        // (a minor vector too long for the chip: no copy of it, all warps that the tiles ask for)
+        const PassGeometry geo = pass_geometry(p, false, p->pass_sd);
         PassParams pp = pass_params(p);
         pp.v = csc ? r : x;
         pp.x = csc ? x : r;
         pp.u = g;
-        pp.vec_bytes = (int)pass_vec_bytes(p);
+        pp.vec_bytes = p->pass_sd ? (int)pass_vec_bytes(p) : 0;
         pp.slots = geo.slots;
         ProfScope ps(p, 4, s);
         CUDA_TRY(p->val_t == SPMV_F64    ? launch_dvalues_f64(pp, p->ctas, geo.warps, (int)geo.smem, s)
@@ -858,6 +859,7 @@ static spmv_status plan_configure(spmv_plan_s *p, uint32_t flags, const spmv_pla
         p->pass_sd = pass_fits(p, false, true);
         p->pass_pair = pass_fits(p, true, true);
         p->pass_mv = p->sv != 8;
+        p->pass_dv = true;
         // vectors per accumulating pass: as many as leave room for three quarters of the warps'
         // staging.  One pass at 24 to 27 of 32 warps against two of half as many vectors (25M
         // nonzeros, us): 2 vectors 120 / 136 (m = 22,500), 4 174 / 187 (11,300), 8 258 / 270 (5,500);
@@ -908,7 +910,7 @@ static PlanLayout plan_layout(const spmv_plan_s *p, const PlanInternal *pi) {
                                 : std::max(p->onchip && !p->sc_global ? (size_t)p->ctas * p->batch_width * p->n_minor * p->sa
                                                                       : (size_t)p->n_minor * sizeof(double),
                                            p->pass_sc || p->pass_pair ? (size_t)p->ctas * std::max(p->batch_width, p->f64_width) * p->n_minor * p->sa : (size_t)0);
-    L.passes = p->pass_sc || p->pass_sd || p->pass_pair || p->pass_mv;
+    L.passes = p->pass_sc || p->pass_sd || p->pass_pair || p->pass_mv || p->pass_dv;
     L.seg = L.passes ? ((size_t)p->n_major * 2 + 1 + seg_rank_blocks(p->n_major) + 4) * 4 : 0;
     L.rec_bytes = (size_t)VL_MAX * p->max_nproc * 2 * p->sa;  // any segmented pass: up to VL_MAX vectors
     off = 0;

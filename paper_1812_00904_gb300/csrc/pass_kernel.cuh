@@ -819,8 +819,9 @@ __device__ __forceinline__ void store2(__half *g, float a, float b) {
 // The gradient of r^T A x by the stored values, g[k] = minor[idx[k]] * major[seg(k)]: the minor
 // vector on chip, a lane taking positions 64 j + 2 lane and the next one (conflict-free index
 // loads, whole-line stores).  Reads 4 bytes and writes one value a nonzero; the streaming kernel,
-// 128 positions a step, took 108 us for 20M FP16 values (m = 8,003), this one 38.
-template <typename VT, typename XT, int WB>
+// 128 positions a step, took 108 us for 20M FP16 values (m = 8,003), this one 38.  A minor vector too
+// long for the chip is read through L2.
+template <typename VT, typename XT, bool ONCHIP, int WB>
 __global__ void __launch_bounds__(WB * 32, 1) dvalues_kernel(const __grid_constant__ PassParams p) {
     using AT = typename Acc<VT>::type;
     using Feed = StepFeed<VT, false>;
@@ -831,9 +832,16 @@ __global__ void __launch_bounds__(WB * 32, 1) dvalues_kernel(const __grid_consta
     __shared__ int next_chunk;
     Feed feed(p, smem + p.vec_bytes, &next_chunk);
     feed.start(blockIdx.x, gridDim.x, false);
-    {
+    const XT *vg = static_cast<const XT *>(p.v);
+    auto minor = [&](int i) -> AT {
+        if constexpr (ONCHIP)
+            return static_cast<AT>(vs[i]);
+        else
+            return static_cast<AT>(call_load(vg + i));
+    };
+    if constexpr (ONCHIP) {
         constexpr int xa = 16 / (int)sizeof(XT);
-        const XT *src = static_cast<const XT *>(p.v);
+        const XT *src = vg;
         const int n16 = p.n_minor / xa;
 #pragma unroll 4
         for (int i = threadIdx.x; i < n16; i += blockDim.x)
@@ -877,7 +885,7 @@ __global__ void __launch_bounds__(WB * 32, 1) dvalues_kernel(const __grid_consta
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int pos = 64 * j + 2 * lane;
-            const AT a = static_cast<AT>(vs[ix[2 * j]]) * x[2 * j], c = static_cast<AT>(vs[ix[2 * j + 1]]) * x[2 * j + 1];
+            const AT a = minor(ix[2 * j]) * x[2 * j], c = minor(ix[2 * j + 1]) * x[2 * j + 1];
             if (pos + 1 < left)
                 store2(g + ps + pos, a, c);
             else if (pos < left)
@@ -886,13 +894,20 @@ __global__ void __launch_bounds__(WB * 32, 1) dvalues_kernel(const __grid_consta
     }
 }
 
-template <typename VT, typename XT>
-cudaError_t launch_dvalues(const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
-    auto kern = dvalues_kernel<VT, XT, pass_warps(sizeof(VT))>;
+template <typename VT, typename XT, bool ONCHIP>
+cudaError_t launch_dvalues_one(const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    auto kern = dvalues_kernel<VT, XT, ONCHIP, pass_warps(sizeof(VT))>;
     static SmemLimit lim;
     const cudaError_t e = ensure_smem_limit(kern, lim, smem);
     if (e != cudaSuccess) return e;
     return launch_overlapped(kern, dim3(grid), dim3(warps * 32), smem, s, p);
+}
+
+// (p.vec_bytes: 0 for a minor vector in global memory)
+template <typename VT, typename XT>
+cudaError_t launch_dvalues(const PassParams &p, int grid, int warps, int smem, cudaStream_t s) {
+    return p.vec_bytes ? launch_dvalues_one<VT, XT, true>(p, grid, warps, smem, s)
+                       : launch_dvalues_one<VT, XT, false>(p, grid, warps, smem, s);
 }
 
 template <typename VT, typename XT, bool SC, bool SD, bool LANES>

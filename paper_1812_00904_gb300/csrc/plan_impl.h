@@ -49,6 +49,7 @@ struct spmv_plan_s {
     bool pass_sc = false, pass_sd = false, pass_pair = false;
     bool sc_global = false;  // the accumulating product keeps its short vector in global memory (few nonzeros)
     int f64_width = 0;       // FP64: vectors of an accumulating launch with a pass for each (0, 1: not used)
+    bool pass_dv = false;  // the values' gradient runs in dvalues_kernel
     bool pass_mv = false;  // the dot products of several vectors run in mvdot_kernel
     gbk::StepRec *steps = nullptr;
     // nonempty / empty segments and ranks among the nonempty (when some are empty)
