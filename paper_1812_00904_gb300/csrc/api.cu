@@ -501,7 +501,8 @@ static spmv_status run_mvdot(spmv_plan_s *p, int kb, const void *const *in, void
     return SPMV_OK;
 }
 
-// Several vectors of a segmented pass in one streaming of the nonzeros, read from the
+// Several vectors' dot products in the streaming kernel, which plans without step records and FP64
+// plans use (the others: run_mvdot): one streaming of the nonzeros, the vectors read from the
 // interleaved copy vt through L2: FP64 with MODE_SEGDOT (2..KB_MAX vectors), the other value
 // types with MODE_VSEG (2..VL_MAX vectors, one per lane of a lane group).  Either way every
 // vector's sums are formed exactly as in its single-vector pass.
@@ -539,9 +540,10 @@ static spmv_status run_segdot_global(spmv_plan_s *p, int kb, const void *const *
 static int seg_group(const spmv_plan_s *p) { return p->val_t == SPMV_F64 ? KB_MAX : VL_MAX; }
 
 // The segmented pass (and its zone fix-up) of plan p; the launches are timed as kernels
-// id_dot / id_fix of plan `prof`.  One vector runs with the short vector on chip when it fits;
-// several run through run_segdot_global (FP64: on chip instead while batch_width holds them),
-// seg_group(p) per pass.
+// id_dot / id_fix of plan `prof`.  One vector goes to the pass where that serves the plan (pass_sd), else
+// to the streaming kernel, with the short vector on chip when it fits.  Several, seg_group(p) at a time,
+// go to run_mvdot (plans with step records, 32-bit accumulation) or run_segdot_global; FP64 ones
+// stay on chip in the streaming kernel while batch_width holds them.
 static spmv_status run_segdot_impl(spmv_plan_s *p, int kb, const void *const *in, void *const *out, cudaStream_t s,
                                    spmv_plan_s *prof, int id_dot, int id_fix, int64_t in_len) {
     const size_t out_bytes = (size_t)p->n_major * p->sx;
@@ -789,9 +791,11 @@ static spmv_status plan_configure(spmv_plan_s *p, uint32_t flags, const spmv_pla
     if (opts && opts->tile_items) {
         p->T = opts->tile_items;
     } else {
-        // (an unvalidated plan or one with its short vector in global memory never runs the
+        // (an unvalidated plan or one made to keep its short vector in global memory never runs the
         // passes, which want tiles of whole 256-position steps: of tiles of 104, as small matrices
-        // had, 60% of a step was padding)
+        // had, 60% of a step was padding.  A validated plan whose short vector does not fit keeps 256
+        // as well: the streaming kernel is as fast with them or faster (FP32, m = 60,000, 290,000 nonzeros,
+        // us, tiles of 256 / 64: accumulating 10.7 / 13.0, dot products 8.4 / 12.0, of 8 vectors 10.7 / 24.5))
         const int64_t fill = (int64_t)sms * 16 * 2;
         if (!(flags & (SPMV_PLAN_NO_VALIDATE | SPMV_PLAN_SHORT_IN_GLOBAL)))
             p->T = nnz < fill * 512 ? 256 : 512;

@@ -199,7 +199,7 @@ spmv_status build_row_blocks(spmv_plan_s *p, int sms, cudaStream_t s) {
     const int32_t *smaj = nullptr;
     int32_t *sidx = nullptr;
     void *svals = nullptr;
-    spmv_status st = coo_sort(cs, bmaj, bmin, p->vals, p->sv, p->nnz, (int)nseg, wmax, sms * 8, p->err, s, &smaj,
+    spmv_status st = coo_sort(cs, bmaj, bmin, p->vals, p->sv, p->nnz, (int)nseg, wmax, p->err, s, &smaj,
                               &sidx, &svals);
     if (st == SPMV_OK) {
         ce = launch_coo_ptr(smaj, p->nnz, (int)nseg, bptr, sms * 8, s);

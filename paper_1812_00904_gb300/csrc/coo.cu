@@ -327,7 +327,7 @@ cudaError_t launch_coo_ptr(const int32_t *major_sorted, int64_t nnz, int n_major
 // plan-owned block, the sorted major indices to the temporary one; all three come back through
 // the out-parameters.  Range errors are reported through `err` (read by the caller after a sync).
 spmv_status coo_sort(CooSort &cs, const int32_t *major, const int32_t *minor, const void *vals, int sv, int64_t nnz,
-                     int n_major, int n_minor, int grid, int32_t *err, cudaStream_t s, const int32_t **major_sorted,
+                     int n_major, int n_minor, int32_t *err, cudaStream_t s, const int32_t **major_sorted,
                      int32_t **minor_sorted, void **vals_sorted) {
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     const int ntiles = (int)((nnz + RS_TILE - 1) / RS_TILE);
@@ -439,7 +439,7 @@ extern "C" spmv_status spmv_plan_coo(spmv_plan_t *out, int64_t m, int64_t n, int
     if (unsorted && nnz > 0) {
         int32_t *omin = nullptr;
         void *ovals = nullptr;
-        const spmv_status st = coo_sort(cs, major, minor, vals, dsize(val_dtype), nnz, n_major, n_minor, grid, err, s,
+        const spmv_status st = coo_sort(cs, major, minor, vals, dsize(val_dtype), nnz, n_major, n_minor, err, s,
                                         &maj_use, &omin, &ovals);
         if (st != SPMV_OK) {
             free_ptr();

@@ -128,7 +128,7 @@ cudaError_t dev_release();
 struct PlanInternal {
     int ctas = 0;             // CTAs of every pass (0: one per SM, at most one per tile)
     int blocks_per_cta = 1;   // blocks of tiles each CTA runs in turn
-    bool segdot_only = false; // only single-vector segmented passes will run
+    bool segdot_only = false; // only dot products will run (of one vector or several)
 };
 spmv_status plan_create(spmv_plan_s **out, int64_t m, int64_t n, int64_t nnz, int32_t layout, const int32_t *ptr,
                         const int32_t *idx, const void *vals, int32_t val_dtype, int32_t vec_dtype, cudaStream_t s,
@@ -168,7 +168,7 @@ struct CooSort {
 // Stable LSD radix sort of the triples by (major, minor) on `s`: sorted minor indices and values
 // in cs.own, sorted major indices in a buffer inside cs.tmp.  Range errors set bits 1 / 4 of err.
 spmv_status coo_sort(CooSort &cs, const int32_t *major, const int32_t *minor, const void *vals, int sv, int64_t nnz,
-                     int n_major, int n_minor, int grid, int32_t *err, cudaStream_t s, const int32_t **major_sorted,
+                     int n_major, int n_minor, int32_t *err, cudaStream_t s, const int32_t **major_sorted,
                      int32_t **minor_sorted, void **vals_sorted);
 // ptr[j] = number of entries of the sorted major-index array below j, j = 0..n_major.
 cudaError_t launch_coo_ptr(const int32_t *major_sorted, int64_t nnz, int n_major, int32_t *ptr, int grid,
