@@ -777,8 +777,8 @@ def run_ours(args):
                               "bytes (the matrix twice), frac_of_hbm_read the bytes read once" if fused else
                               "the two products side by side on two streams"), "l2": "inputs larger than L2 (no flush)",
                           "parallelism": f"replicas x{world}", "chunks": info["chunks"], "ctas": info["ctas"],
-                          "warps_per_cta": info["warps_per_cta"], "tile_items": info["tile_items"],
-                          "stages": info["stages"], "zones": info["zones"],
+                          "tile_items": info["tile_items"], "zones": info["zones"],
+                          "streaming_kernel": {"warps_per_cta": info["warps_per_cta"], "stages": info["stages"]},
                           "nonzero_order": "stored" if args.stored_order else
                           "bank order (plan-owned copy, permuted within each column)",
                           "plan_setup_ms": round(info["setup_ms"], 3),

@@ -144,13 +144,15 @@ typedef struct {
     int64_t m, n, nnz;
     int32_t layout, val_dtype, vec_dtype;
     int32_t chunks;            /* P */
-    int32_t ctas, warps_per_cta, tile_items, stages;
+    int32_t ctas, warps_per_cta, tile_items, stages;  /* warps_per_cta and stages: of the streaming kernel
+                                  (spmv_plan_opts), also where the passes of validated plans run, which
+                                  have one slot a warp and as many warps as spmv_plan_opts says */
     int32_t tiles;             /* execution tiles */
     int32_t zones;             /* z, overlap zones (Sec. II), z <= P-1 */
     int32_t max_zone_size;     /* V = max |S_k| (Sec. IV-A) */
     int32_t short_on_chip;     /* 1 if the short vector lives in shared memory (a long one, beside few
                                   nonzeros, only as the input of the dot products) */
-    int32_t batch_width;       /* vectors per pass of the accumulating direction of spmv_batch (1..8) */
+    int32_t batch_width;       /* vectors per launch of the accumulating direction of spmv_batch (1..8) */
     int64_t max_chunk_nnz, min_chunk_nnz;
     double imbalance;          /* Delta = P (max - min) / Z (Sec. VI), 0 when Z = 0 */
     int64_t workspace_bytes;   /* device bytes owned by the plan */

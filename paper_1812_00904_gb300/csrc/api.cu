@@ -1176,7 +1176,7 @@ spmv_status spmv_plan_info(spmv_plan_t p, spmv_plan_info_t *info) {
     info->zones = p->z;
     info->max_zone_size = p->vmax;
     info->short_on_chip = p->onchip ? 1 : 0;
-    info->batch_width = p->batch_width;
+    info->batch_width = p->sc_global ? 1 : std::max(p->batch_width, p->f64_width);
     info->max_chunk_nnz = p->max_chunk;
     info->min_chunk_nnz = p->min_chunk;
     info->imbalance = p->nnz > 0 ? (double)p->P * (double)(p->max_chunk - p->min_chunk) / (double)p->nnz : 0.0;
