@@ -1144,11 +1144,14 @@ spmv_status spmv_plan_destroy(spmv_plan_t plan) {
     if (!plan) return SPMV_OK;
     // wait for the device that owns the plan's memory (the current one belongs to the thread and may be
     // another); while it cannot be waited for, as during a stream capture, its kernels may still run and the
-    // plan's pooled blocks are kept out of the pool for good
+    // plan's pooled blocks go back to the pool with those of a later plan
     int current = plan->device;
     const bool elsewhere = cudaGetDevice(&current) == cudaSuccess && current != plan->device;
     if (elsewhere) cudaSetDevice(plan->device);
-    plan_free(plan, cudaDeviceSynchronize() == cudaSuccess);
+    const int device = plan->device;
+    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+    if (idle) dev_free_late(device);
+    plan_free(plan, idle);
     if (elsewhere) cudaSetDevice(current);
     return SPMV_OK;
 }

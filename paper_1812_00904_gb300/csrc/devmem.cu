@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include <mutex>
+#include <unordered_map>
 #include <unordered_set>
 
 #include "plan_impl.h"
@@ -36,6 +37,8 @@ DevicePool g_pools[MAX_DEVICES];
 std::mutex g_large_mu;
 // the blocks that bypassed the pool (never destroyed: plans may be freed while the process ends)
 std::unordered_set<void *> &g_large = *new std::unordered_set<void *>;
+// pooled blocks freed while they might still be in use, by device (under g_large_mu)
+std::unordered_multimap<int, void *> &g_late = *new std::unordered_multimap<int, void *>;
 
 DevicePool &pool_of(int device) {
     DevicePool &P = g_pools[device];
@@ -121,11 +124,23 @@ void dev_free(void *p, int device, bool idle) {
     }
     if (!large && device >= 0 && device < MAX_DEVICES && g_pools[device].pool) {
         // (cudaFree waits for the device by itself, the pool for nothing: memory that may still be in use
-        // must not go back to it)
-        if (idle) cudaFreeAsync(p, g_pools[device].stream);
+        // must not go back to it yet)
+        if (idle) {
+            cudaFreeAsync(p, g_pools[device].stream);
+        } else {
+            std::lock_guard<std::mutex> lk(g_large_mu);
+            g_late.emplace(device, p);
+        }
     } else {
         cudaFree(p);
     }
+}
+
+void dev_free_late(int device) {
+    std::lock_guard<std::mutex> lk(g_large_mu);
+    const auto late = g_late.equal_range(device);
+    for (auto it = late.first; it != late.second; ++it) cudaFreeAsync(it->second, g_pools[device].stream);
+    g_late.erase(late.first, late.second);
 }
 
 }  // namespace gbk

@@ -116,9 +116,10 @@ namespace gbk {
 
 // Device memory from the current device's pool (devmem.cu): usable on any stream once returned;
 // freed when no work that uses it is pending on `device`, or with idle = false (a pooled block then
-// stays allocated).
+// stays allocated until dev_free_late, which is called when nothing is pending on the device).
 cudaError_t dev_alloc(void **p, size_t bytes);
 void dev_free(void *p, int device, bool idle = true);
+void dev_free_late(int device);
 // Memory beside the pool (freed with cudaFree), which makes room by what the pool keeps if need be.
 cudaError_t dev_malloc(void **p, size_t bytes);
 // Give what the current device's pool keeps back to the device.

@@ -33,3 +33,8 @@ def test_memory_stays_out_of_the_pool_when_the_wait_fails(host):
     host.lib.spmv_plan_destroy(plan)
     assert "pool free" not in host.log()
     host.lib.fake_fail_sync(0)
+    plan = host.plan(300, 5_000, 40_000)
+    host.log()
+    host.lib.spmv_plan_destroy(plan)
+    log = host.log()
+    assert log.count("pool free") == 4 and log[0] == "sync device 0"  # (both plans' two blocks)
