@@ -138,7 +138,7 @@ template <typename VT, bool VALS = true> struct StepFeed {
 // load and a compare-and-swap that costs two, each with the bank conflicts of 32 rows.  SD alone
 // runs near the memory rate, FP64 at the rate of its pipe (2 operations a cycle per SM).  With the
 // combine and fix-up, streaming kernel before, this one now (us): 200M FP32 nonzeros, m = 20,000, bank
-// order: pair 640 -> 386, SC 362 -> 294, SD 303 -> 261; 150M, n = 2,000: pair 538 -> 369, SC 313 ->
+// order: pair 640 -> 386, SC 362 -> 294, SD 303 -> 261; 150M, n = 2,000: pair 538 -> 372, SC 313 ->
 // 262, SD 242 -> 207; 8M FP64, n = 4,000: pair 121 -> 76, SC 62 -> 42, SD 69 -> 48.
 // LANES: SC into very short vectors (PASS_LANES_MOST elements): every lane has an element of its own for
 // each row, [row][lane], so that the lanes of a warp never add to the same place (one row, 51,000
