@@ -61,15 +61,6 @@ cudaError_t launch_pass(const spmv_plan_s *p, bool sc, bool sd, const PassParams
     }
 }
 
-// Shared memory of a one-vector pass: the accumulator (sc), the input vector (sd), a staging slot for
-// each of as many warps as fit, and what is left over for more copies of the accumulator.  More warps
-// always help: the pair, the accumulating product and the dot products of the 200M-nonzero wide
-// matrix (m = 20,000) take 590 / 403 / 374 us with 16 warps, 501 / 355 / 326 with 20, 449 / 325 / 301
-// with 24, 417 / 309 / 281 with 28, 389 / 294 / 261 with 32.  A second slot a warp is no gain
-// (dot products 269 to 280).  An addition is a compare-and-swap loop, repeated when another warp got
-// in between, so copies help where they fit: with 1 / 2 / 4 / 8 / 16 of them the accumulating
-// product of the 150M-nonzero tall matrix (n = 2,000) takes 348 / 318 / 302 / 290 / 262 us, the pair
-// 441 / 419 / 406 / 393 / 372; 32 add nothing.
 // One-vector SC into very short vectors: an element for every lane of a warp (pass_kernel's LANES).  The
 // FP32 pair's additions stand conflicts better (one row, 5,000 nonzeros 16 us) and stay as they are.
 // The FP64 pair, whose eight places of a lane lie side by side, still gains at 64 (40 rows, 5,000 nonzeros
@@ -82,6 +73,16 @@ size_t pass_acc_bytes(const spmv_plan_s *p, bool sd) {
     return align_up((size_t)p->n_minor * (pass_lanes(p, true, sd) ? 32 : 1) * p->sa, 128);
 }
 size_t pass_vec_bytes(const spmv_plan_s *p) { return align_up((size_t)p->n_minor * p->sx, 128); }
+
+// Shared memory of a one-vector pass: the accumulator (sc), the input vector (sd), a staging slot for
+// each of as many warps as fit, and what is left over for more copies of the accumulator.  More warps
+// always help: the pair, the accumulating product and the dot products of the 200M-nonzero wide
+// matrix (m = 20,000) take 590 / 403 / 374 us with 16 warps, 501 / 355 / 326 with 20, 449 / 325 / 301
+// with 24, 417 / 309 / 281 with 28, 389 / 294 / 261 with 32.  A second slot a warp is no gain
+// (dot products 269 to 280).  An addition is a compare-and-swap loop, repeated when another warp got
+// in between, so copies help where they fit: with 1 / 2 / 4 / 8 / 16 of them the accumulating
+// product of the 150M-nonzero tall matrix (n = 2,000) takes 348 / 318 / 302 / 290 / 262 us, the pair
+// 441 / 419 / 406 / 393 / 372; 32 add nothing.
 constexpr int PASS_MAX_COPIES = 16;
 struct PassGeometry {
     int warps, slots, copies;
